@@ -570,8 +570,8 @@ typedef struct {
     int kernel;                 /* TCW_KERNEL_GROUP or TCW_KERNEL_LOOKUP */
     int launches;               /* kernels launched by the search */
     int64_t lookups;            /* n_sky * n_tmpl * n_det * n_seg */
-    int64_t general_path_lanes; /* group-kernel (template, detector, segment,
-                                   sky-group) steps that took the per-sky path */
+    int64_t general_path_lanes; /* lookups at a band edge: (template, detector, segment) steps whose
+                                   skies do not all read bins inside the band */
     double doppler_bins_max;    /* largest |f * v.nhat/c| / df over the search */
     double quantum;             /* fixed-point step of the Doppler factor */
     float search_ms;            /* device time of the search kernel, ms */

@@ -162,6 +162,145 @@ tcw_status ensure_bits(tcw_ctx* c, int* launches) {
   return TCW_OK;
 }
 
+// Largest |rho| of the loaded map, taken once per load.
+tcw_status ensure_map_max(tcw_ctx* c) {
+  if (c->map_max_epoch == c->spec_epoch) return TCW_OK;
+  TCW_CUDA(c, c->flags.ensure(64), "flags");
+  unsigned* out = reinterpret_cast<unsigned*>(c->flags.as<char>() + 40);
+  unsigned bits = 0;
+  TCW_CUDA(c, cudaMemsetAsync(out, 0, 4, c->stream), "map maximum");
+  TCW_CUDA(c, launch_absmax(c->rho.p, c->dtype == TCW_F16, (int64_t)c->D * c->Nseg * c->Nbin, out, c->stream),
+           "absmax_kernel launch");
+  TCW_CUDA(c, cudaMemcpyAsync(&bits, out, 4, cudaMemcpyDeviceToHost, c->stream), "map maximum");
+  TCW_CUDA(c, cudaStreamSynchronize(c->stream), "map maximum");
+  std::memcpy(&c->map_max, &bits, 4);
+  c->map_max_epoch = c->spec_epoch;
+  return TCW_OK;
+}
+
+// The exhaustive search by step functions (tcw_step.cuh).  *ran = false when
+// its conditions do not hold (the group kernel's exactness conditions, a track
+// series, and fixed-point sums at least as accurate as fp32 ones: not with
+// non-finite or very large powers): the caller takes the group kernel.
+tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, bool* ran) {
+  *ran = false;
+  if (!pl.group_ok || pl.nterms < 1 || c->D > 2) return TCW_OK;
+  const bool count = c->statistic == TCW_STAT_NUMBER_COUNT;
+  tcw_status st = TCW_OK;
+  if (!count && (st = ensure_map_max(c)) != TCW_OK) return st;
+  const double vmax = (count ? 1.0 : (double)c->map_max) * c->track_bins;
+  const double f_top = c->f_min + (double)c->Nbin * c->df;
+  const StepScales sc =
+      step_scales(vmax, c->w_min, c->w_max,
+                  step_amp_ref(c->amp_power, c->h_t, c->T0, c->bank_tau_min, c->bank_r_max, f_top, c->bank_f0max),
+                  (int64_t)c->D * c->Nseg);
+  if (!sc.ok) return TCW_OK;
+  const StepGeometry g = step_geometry(c->S, c->D, c->Nseg, c->tile_segments, c->h_v.data(), false);
+  const int tile_shift = ilog2(c->tile_segments);
+  const int n_tiles = (int)((c->Nseg + c->tile_segments - 1) / c->tile_segments);
+  const size_t rows = (size_t)g.n_chunks * c->Nseg * c->D;
+  TCW_CUDA(c, c->step_q.ensure(rows * g.cpad * sizeof(int32_t)), "doppler rows");
+  TCW_CUDA(c, c->step_meta.ensure(rows * step_meta(g.cpad) * sizeof(int4)), "doppler rows");
+  TCW_CUDA(c, ensure_step_edge(c->step_edge, c->grid, c->stream), "scratch");
+  if (step_ordered(g)) {
+    TCW_CUDA(c, c->step_order.ensure((size_t)g.passes * g.n_chunks * g.cpad * sizeof(int16_t)), "sky order");
+    TCW_CUDA(c, c->step_acc.ensure(step_acc_bytes(c->grid)), "scratch");
+  }
+  StepRowsParams rp{};
+  rp.vel = c->vel.as<double>();
+  rp.nhat = c->nhat_sorted.as<double>();
+  rp.weights = c->weights.as<float>();
+  rp.t_mid = c->t_mid.as<double>();
+  rp.T0 = c->T0;
+  rp.n_det = c->D;
+  rp.n_seg = (int)c->Nseg;
+  rp.S = (int)c->S;
+  set_step_geometry(rp, g);
+  rp.tile_shift = tile_shift;
+  rp.inv_q = pl.inv_q;
+  rp.w1_scale = std::ldexp(1.0, sc.w1);
+  rp.w2_scale = std::ldexp(1.0, sc.w2);
+  rp.order = step_ordered(g) ? c->step_order.as<int16_t>() : nullptr;
+  rp.q = c->step_q.as<int32_t>();
+  rp.meta = c->step_meta.as<int4>();
+  TCW_CUDA(c, launch_step_rows(rp, c->stream), "step_rows_kernel launch");
+  ++*launches;
+  if (count && (st = ensure_bits(c, launches)) != TCW_OK) return st;
+  TCW_CUDA(c, c->anchors.ensure((size_t)c->Bpad * n_tiles * 2 * sizeof(double)), "anchors");
+  AnchorParams ap{};
+  ap.t_mid = c->t_mid.as<double>();
+  ap.f0 = c->f0.as<double>();
+  ap.tau = c->tau.as<double>();
+  ap.nbr = c->nbr.as<double>();
+  ap.T0 = c->T0;
+  ap.n_seg = (int)c->Nseg;
+  ap.n_tiles = n_tiles;
+  ap.tile_shift = tile_shift;
+  ap.Bpad = c->Bpad;
+  ap.anchors = c->anchors.as<double>();
+  ap.chain = anchor_chain_for(c->h_t.data(), c->Nseg, c->T0, 1 << tile_shift, c->bank_tau_min, c->bank_r_max);
+  StepEvent ev{};
+  ev.rho = c->rho.p;
+  ev.bits = count ? c->bits.as<uint32_t>() : nullptr;
+  ev.bit_pitch = count ? bit_pitch_for(c->Nbin) : 0;
+  ev.t_mid = c->t_mid.as<double>();
+  ev.anchors = ap.anchors;
+  ev.f0 = ap.f0;
+  ev.nbr = ap.nbr;
+  ev.q = rp.q;
+  ev.meta = rp.meta;
+  ev.order = rp.order;
+  ev.psi = c->psi.as<float>();
+  ev.S_out = keep ? c->st_S.as<float>() : nullptr;
+  ev.W1_out = keep ? c->st_W1.as<float>() : nullptr;
+  ev.W2_out = keep ? c->st_W2.as<float>() : nullptr;
+  ev.T0 = c->T0;
+  set_step_scales(ev, sc);
+  ev.n_seg = (int)c->Nseg;
+  ev.n_tiles = n_tiles;
+  ev.S = (int)c->S;
+  ev.Bpad = c->Bpad;
+  set_step_geometry(ev, g);
+  TCW_CUDA(c, c->evtab.ensure(sizeof(StepEvent)), "event table");
+  TCW_CUDA(c, cudaMemcpyAsync(c->evtab.p, &ev, sizeof(ev), cudaMemcpyHostToDevice, c->stream), "event table");
+  StepParams p{};
+  p.events = c->evtab.as<StepEvent>();
+  p.items = nullptr;
+  p.n_chunks = g.n_chunks;
+  p.bank_chunk = c->bank_chunk;
+  const int blocks = c->Bpad >> g.log_t;
+  p.n_items = g.n_chunks * ((blocks + c->bank_chunk - 1) / c->bank_chunk);
+  p.next = reinterpret_cast<unsigned*>(c->flags.as<char>() + 32);
+  p.n_det = c->D;
+  p.n_bin = c->Nbin;
+  p.f_min = c->f_min;
+  p.df = c->df;
+  p.inv_q = pl.inv_q;
+  p.q = (float)pl.q;
+  p.q_exp = -std::ilogb(pl.q);
+  p.nterms = pl.nterms;
+  p.tile_shift = tile_shift;
+  p.sub_shift = step_sub_shift(c->Nseg, tile_shift);
+  p.amp_power = c->amp_power;
+  p.nc_q = count ? std::exp(-c->rho_th) : 0.0;
+  p.track_bins = c->track_bins;
+  p.map_half = c->dtype == TCW_F16 ? 1 : 0;
+  p.acc = c->step_acc.as<long long>();
+  p.edge = c->step_edge.as<longlong2>();
+  p.n_general = reinterpret_cast<unsigned long long*>(c->flags.as<char>() + 8);
+  TCW_CUDA(c, cudaEventRecord(c->ev0, c->stream), "event");
+  TCW_CUDA(c, launch_anchors(ap, c->stream), "anchor_kernel launch");
+  const bool fast = step_fast_track(c->h_t.data(), c->Nseg, c->T0, c->tile_segments, c->bank_tau_min, c->bank_r_max,
+                                    c->f_min, c->df, p.q_exp) != 0;
+  TCW_CUDA(c, launch_step(p, g.dets_per_pass, c->dtype == TCW_F16, count || c->track_bins == 2, fast, step_cells(g),
+                          std::min(c->grid, p.n_items), c->stream),
+           "step_kernel launch");
+  TCW_CUDA(c, cudaEventRecord(c->ev1, c->stream), "event");
+  *launches += 2;
+  *ran = true;
+  return TCW_OK;
+}
+
 tcw_status run_search(tcw_ctx* c, bool record, int32_t* rec_dev) {
   if (!c->have_spec) return fail(c, TCW_ERR_STATE, "no spectrogram loaded");
   if (!c->have_vel) return fail(c, TCW_ERR_STATE, "no velocities loaded");
@@ -189,8 +328,14 @@ tcw_status run_search(tcw_ctx* c, bool record, int32_t* rec_dev) {
   TCW_CUDA(c, c->flags.ensure(64), "flags");
   TCW_CUDA(c, cudaMemsetAsync(c->flags.p, 0, 64, c->stream), "flags");
   int launches = 0;
-
+  bool stepped = false;
   if (kernel == TCW_KERNEL_GROUP) {
+    // a forced group kernel keeps its bound on the width of a sky group (checked below)
+    if (!record && c->opt_kernel != TCW_KERNEL_GROUP &&
+        (st = step_search(c, pl, keep, &launches, &stepped)) != TCW_OK)
+      return st;
+  }
+  if (kernel == TCW_KERNEL_GROUP && !stepped) {
     const size_t blkn = (size_t)(c->Spad / chunk_skies(c->lanes)) * c->Nseg * c->D * block_words(c->lanes);
     TCW_CUDA(c, c->dq.ensure(blkn * sizeof(int32_t)), "doppler table");
     DopplerParams dp{};
@@ -218,9 +363,14 @@ tcw_status run_search(tcw_ctx* c, bool record, int32_t* rec_dev) {
         return fail(c, TCW_ERR_UNSUPPORTED, "group kernel unavailable: sky groups span too many bins");
       kernel = TCW_KERNEL_LOOKUP;
     }
+    if (!record && c->opt_kernel == TCW_KERNEL_GROUP &&
+        (st = step_search(c, pl, keep, &launches, &stepped)) != TCW_OK)
+      return st;
   }
   const bool count = c->statistic == TCW_STAT_NUMBER_COUNT;
-  if (kernel == TCW_KERNEL_GROUP) {
+  if (stepped) {
+    // done
+  } else if (kernel == TCW_KERNEL_GROUP) {
     if (count && (st = ensure_bits(c, &launches)) != TCW_OK) return st;
     const int tile_shift = ilog2(c->tile_segments);
     const int n_tiles = (int)((c->Nseg + c->tile_segments - 1) / c->tile_segments);
@@ -503,6 +653,15 @@ SweepPlan plan_sweep(const std::vector<double>& tc, double T0, double tau_min, d
 
 }  // namespace
 
+double tcw::step_amp_ref(int amp_power, const std::vector<double>& t, double T0, double tau_min, double r_max,
+                         double f_top, double f0_max) {
+  if (amp_power == 0) return 1.0;
+  double a = std::min(1.0, f_top / f0_max);
+  const auto first = std::lower_bound(t.begin(), t.end(), T0);
+  if (first != t.end()) a = std::min(a, std::pow((*first - T0) / tau_min + 1.0, -r_max));
+  return std::pow(std::max(a, 1e-30), amp_power);
+}
+
 tcw_status tcw::coarse_pass(tcw_ctx* c, const CoarseEvent& ev, int patch_size, float lo, float hi, float* feat,
                        float* psi, int* P_out, int* sweep_out) {
   if (ev.D > 2) return fail(c, TCW_ERR_UNSUPPORTED, "coarse pass handles at most 2 detectors");
@@ -769,6 +928,7 @@ tcw_status tcw_destroy(tcw_ctx* c) {
   cudaStreamSynchronize(c->stream);
   DevBuf* bufs[] = {&c->rho, &c->t_mid, &c->weights, &c->vel, &c->f0, &c->tau, &c->nbr,
                     &c->bank_perm, &c->bank_pos, &c->nhat_sorted, &c->sky_perm, &c->sky_pos,
+                    &c->step_q, &c->step_meta, &c->step_edge, &c->step_acc, &c->step_order,
                     &c->dq, &c->anchors, &c->psi, &c->st_S, &c->st_W1, &c->st_W2, &c->dev,
                     &c->flags, &c->stage_f, &c->stage_i, &c->evtab, &c->items, &c->tri_dop,
                     &c->tri_hist, &c->tri_feat, &c->tri_psi, &c->tri_anchor, &c->tri_h1, &c->tri_h2,
@@ -887,8 +1047,13 @@ tcw_status tcw_load_spectrogram(tcw_ctx* c, int n_det, int64_t n_seg, int64_t n_
   c->df = df;
   c->h_t = std::move(t);
   c->unit_weights = true;
-  for (float x : w)
+  c->w_min = INFINITY;
+  c->w_max = 0;
+  for (float x : w) {
     if (x != 1.0f) c->unit_weights = false;
+    if (x > 0 && x < c->w_min) c->w_min = x;
+    if (x > c->w_max) c->w_max = x;
+  }
   c->have_spec = true;
   c->have_result = false;
   c->sky_dirty = true;

@@ -6,7 +6,7 @@
 #include <string>
 #include <vector>
 
-#include "tcw_internal.cuh"
+#include "tcw_step.cuh"
 
 namespace tcw {
 
@@ -66,6 +66,9 @@ struct tcw_ctx {
   double f_min = 0, df = 0;
   std::vector<double> h_t;
   bool unit_weights = true;
+  float w_min = 0, w_max = 0;        // smallest nonzero and largest weight
+  float map_max = 0;                 // largest |rho| of the loaded map (see ensure_map_max)
+  unsigned map_max_epoch = ~0u;
   tcw::DevBuf rho, t_mid, weights;
   tcw::DevBuf bits;        // number-count bit map of rho (see tcw_set_statistic)
   unsigned bits_epoch = ~0u;
@@ -89,6 +92,7 @@ struct tcw_ctx {
   bool sky_dirty = true;
   tcw::DevBuf nhat_sorted, sky_perm, sky_pos;
   // derived and outputs
+  tcw::DevBuf step_q, step_meta, step_edge, step_acc, step_order;   // step-function kernel: Doppler rows, band-edge scratch
   tcw::DevBuf dq, anchors, psi, st_S, st_W1, st_W2, dev, flags, stage_f, stage_i, evtab, items;
   int64_t items_key[5] = {-1, -1, -1, -1, -1};  // (n_chunks, Bpad, bank_chunk, grid, lanes) of the schedule
   int grid = 0, n_items = 0;
@@ -156,6 +160,19 @@ inline bool finite_all(const std::vector<double>& v) {
     if (!std::isfinite(x)) return false;
   return true;
 }
+
+// Band-edge scratch of the step-function kernel for `grid` CTAs: zero at
+// allocation, left zero by every launch.
+inline cudaError_t ensure_step_edge(DevBuf& b, int grid, cudaStream_t st) {
+  if (b.p && b.bytes >= step_edge_bytes(grid)) return cudaSuccess;
+  cudaError_t e = b.ensure(step_edge_bytes(grid));
+  return e == cudaSuccess ? cudaMemsetAsync(b.p, 0, b.bytes, st) : e;
+}
+
+// Amplitude factor (Eq. 3) that every template's first lookups reach at least:
+// at the first segment from T0 on, or where the track enters the band.
+double step_amp_ref(int amp_power, const std::vector<double>& t, double T0, double tau_min, double r_max,
+                    double f_top, double f0_max);
 
 void batch_free(tcw_ctx* c);
 

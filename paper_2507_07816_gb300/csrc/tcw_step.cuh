@@ -1,0 +1,173 @@
+// tcw_step.cuh -- shared declarations of the step-function search kernel
+// (tcw_step.cu): the exhaustive search of one or many events.
+//
+// Over the skies of a chunk, sorted by their Doppler factor, the bin of one
+// (template, segment, detector) lookup is a step function: it changes only
+// where the threshold between two bins (tcw_internal.cuh) falls between two
+// neighbouring skies, one or two places for the whole sky at 500-3000 Hz.  So
+// a lookup is the first sky's bin plus one difference per step, added to a
+// per-template difference array over the sorted positions; a prefix sum at the
+// end gives every sky's weighted power.  All sums are fixed-point integers
+// (48 bits, two 32-bit words), so they are exact and do not depend on the order
+// of the additions or on how the sky and the bank are cut into work items.
+#pragma once
+
+#include <cmath>
+
+#include "tcw_internal.cuh"
+
+namespace tcw {
+
+constexpr int kStepBlock = 8;          // sorted skies per block of a Doppler row
+constexpr int kStepMaxChunk = 1024;    // sorted skies per chunk
+constexpr int kStepCells = 16384;      // difference cells of a CTA: chunk x templates
+
+// One event.  Its segments and detectors are worked through in passes: a pass
+// is a run of pass_seg segments of one detector (dets_per_pass = 1) or of all
+// of them, over which the skies of a chunk keep one order, so that the rows'
+// Doppler factors stay (almost) sorted.  Doppler rows: one per (chunk, segment,
+// detector), cpad skies in the order of their pass (a multiple of kStepBlock;
+// the last sky repeated):
+//   q     [cpad]  floor(v.nhat/c / q-grid step)
+//   meta  {qmin, qmax, dt hi, dt lo}: smallest and largest q; t_j - t_a from
+//         the tile's anchor time as an fp32 pair (NaN before T0)
+//         {blocks per grid unit (float bits), w (float bits), 0, 0}
+//         {W1 word, W2 word}: w and w^2 in fixed point (int64 each),
+//         then per block g {largest q of blocks 0..g, smallest q of blocks
+//         g+1.. (INT_MAX after the last)} as int2
+struct StepEvent {
+  const void* rho;           // [D][n_seg][n_bin]
+  const uint32_t* bits;      // number count: bit map (see EventDesc), else null
+  const double* t_mid;
+  const double* anchors;     // [Bpad][n_tiles][2]
+  const double* f0;          // sorted bank [Bpad]
+  const double* nbr;
+  const int32_t* q;          // [n_chunks][n_seg][D][cpad]
+  const int4* meta;          // [n_chunks][n_seg][D][step_meta(cpad)]
+  const int16_t* order;      // [passes][n_chunks][cpad] sky (in the chunk) at a position; null for one pass
+                             // in the sorted order itself
+  float* psi;                // [>= S][Bpad]
+  float* S_out;              // optional
+  float* W1_out;
+  float* W2_out;
+  double T0;
+  double x_unit, w1_unit, w2_unit;   // value of one unit of the fixed-point sums
+  float x_scale;                     // 2^-16 / x_unit
+  float w1_scale, w2_scale;          // 2^-16 / w1_unit, 2^-16 / w2_unit
+  int n_seg, n_tiles, S, Bpad;
+  int bit_pitch;
+  int chunk, cpad, log_t;    // skies per chunk, of a row; templates of a block: 1 << log_t
+  int n_chunks, pass_seg, passes;
+};
+
+struct StepParams {
+  const StepEvent* events;
+  const int4* items;         // {event, chunk, first template, template blocks}; null: every chunk of
+                             // event 0 x runs of bank_chunk template blocks
+  int n_items, n_chunks, bank_chunk;
+  int n_det;
+  unsigned* next;            // item counter, zero at launch
+  int64_t n_bin;
+  double f_min, df, inv_q;
+  float q;
+  int q_exp;                 // q = 2^-q_exp
+  int nterms, tile_shift;    // FP64 track series (> 0), anchor tiles
+  int sub_shift;             // segments of one warp's turn: 1 << sub_shift <= tile
+  int amp_power;
+  double nc_q;               // number count: q = exp(-rho_th), else 0
+  int track_bins;
+  int map_half;
+  long long* acc;            // [grid][kStepCells]: sums of the finished passes (several passes only)
+  longlong2* edge;           // [grid][2 kStepCells + 32]: W1, W2 steps at band edges and their sums over
+                             // the finished passes, zero between launches
+  unsigned long long* n_general;
+};
+
+struct StepRowsParams {
+  const double* vel;         // [D][n_seg][3]
+  const double* nhat;        // [>= S][3] sorted
+  const float* weights;      // [D][n_seg]
+  const double* t_mid;
+  double T0;
+  int n_det, n_seg, S, chunk, cpad, n_chunks, tile_shift;
+  int dets_per_pass, pass_seg, passes;
+  double inv_q;
+  double w1_scale, w2_scale; // 1 / w1_unit, 1 / w2_unit
+  int16_t* order;            // written first when not null (see StepEvent)
+  int32_t* q;
+  int4* meta;
+};
+
+constexpr int kStepHead = 3;   // int4 words of a row's meta before its blocks
+__host__ __device__ constexpr int step_meta(int cpad) { return kStepHead + (cpad / kStepBlock + 1) / 2; }
+
+// Chunks of an event's sorted skies: the fewest chunks of at most
+// kStepMaxChunk skies, of nearly equal size; 32 templates per block while the
+// difference cells allow it (chunks of up to 511 skies), else 16.
+struct StepGeometry {
+  int n_chunks, chunk, cpad, log_t;
+  int dets_per_pass, pass_seg, passes;
+};
+// v: velocities [D][n_seg][3] (host); split: one detector per pass even where all would do.
+StepGeometry step_geometry(int64_t S, int D, int64_t n_seg, int tile, const double* v, bool split);
+inline void set_step_geometry(StepEvent& e, const StepGeometry& g) {
+  e.chunk = g.chunk;
+  e.cpad = g.cpad;
+  e.log_t = g.log_t;
+  e.n_chunks = g.n_chunks;
+  e.pass_seg = g.pass_seg;
+  e.passes = g.passes;
+}
+inline void set_step_geometry(StepRowsParams& p, const StepGeometry& g) {
+  p.chunk = g.chunk;
+  p.cpad = g.cpad;
+  p.n_chunks = g.n_chunks;
+  p.dets_per_pass = g.dets_per_pass;
+  p.pass_seg = g.pass_seg;
+  p.passes = g.passes;
+}
+inline bool step_ordered(const StepGeometry& g) { return g.passes > 1; }
+
+// 1 when the in-kernel fp32-pair track series (t - t_a at tiles of `tile`
+// segments) is as accurate as the FP64 one for every template and lookup.
+int step_fast_track(const double* t_mid, int64_t n_seg, double T0, int tile, double tau_min, double r_max,
+                    double f_min, double df, int q_exp);
+
+// Fixed-point scales of one event, or ok = false when the sums would not be
+// at least as accurate as fp32 partial sums (see step_scales).
+struct StepScales {
+  bool ok = false;
+  int x = 0, w1 = 0, w2 = 0;   // exponents: one unit is 2^-x (2^-w1, 2^-w2)
+};
+// vmax: largest |value| a lookup adds (before its weight); w_min: smallest
+// nonzero weight, w_max the largest; a_ref: amplitude factor of a template's
+// first lookups; n: lookups of one (template, sky).
+StepScales step_scales(double vmax, double w_min, double w_max, double a_ref, int64_t n);
+
+inline void set_step_scales(StepEvent& e, const StepScales& s) {
+  e.x_unit = std::ldexp(1.0, -s.x);
+  e.w1_unit = std::ldexp(1.0, -s.w1);
+  e.w2_unit = std::ldexp(1.0, -s.w2);
+  e.x_scale = std::ldexp(1.0f, s.x - 16);
+  e.w1_scale = std::ldexp(1.0f, s.w1 - 16);
+  e.w2_scale = std::ldexp(1.0f, s.w2 - 16);
+}
+// Segments of one warp's turn (as a shift): a whole tile where the event has
+// several tiles per warp, else 8 segments so that short events use every warp.
+inline int step_sub_shift(int64_t n_seg, int tile_shift) {
+  return n_seg >= (int64_t)4 * 32 << tile_shift ? tile_shift : 3;
+}
+inline int step_cells(const StepGeometry& g) { return (g.cpad + 1) << g.log_t; }
+inline size_t step_edge_bytes(int grid) { return (size_t)grid * (2 * kStepCells + 32) * sizeof(longlong2); }
+inline size_t step_acc_bytes(int grid) { return (size_t)grid * kStepCells * sizeof(long long); }
+cudaError_t launch_step_rows(const StepRowsParams& p, cudaStream_t st);
+// Raises the kernel's shared-memory limit (also done at its first launch; call before a graph capture).
+cudaError_t step_prepare(int dets_per_pass, bool half, bool general, bool fast);
+// general: number count or two-bin lookups; fast: step_fast_track held for every event; cells: the
+// largest step_cells of the items' events, whose passes all take dets_per_pass detectors.
+cudaError_t launch_step(const StepParams& p, int dets_per_pass, bool half, bool general, bool fast, int cells,
+                        int grid, cudaStream_t st);
+// *out = bits of the largest |rho| (NaN above infinity above every finite value); out zero at launch.
+cudaError_t launch_absmax(const void* rho, bool half, int64_t n, unsigned* out, cudaStream_t st);
+
+}  // namespace tcw

@@ -184,7 +184,7 @@ tcw_status ensure_map_max(tcw_ctx* c) {
 // non-finite or very large powers): the caller takes the group kernel.
 tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, bool* ran) {
   *ran = false;
-  if (!pl.group_ok || pl.nterms < 1 || c->D > 2) return TCW_OK;
+  if (!pl.group_ok || c->D > 2) return TCW_OK;
   const bool count = c->statistic == TCW_STAT_NUMBER_COUNT;
   tcw_status st = TCW_OK;
   if (!count && (st = ensure_map_max(c)) != TCW_OK) return st;
@@ -195,17 +195,22 @@ tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, boo
                   step_amp_ref(c->amp_power, c->h_t, c->T0, c->bank_tau_min, c->bank_r_max, f_top, c->bank_f0max),
                   (int64_t)c->D * c->Nseg);
   if (!sc.ok) return TCW_OK;
-  const StepGeometry g = step_geometry(c->S, c->D, c->Nseg, c->tile_segments, c->h_v.data(), false);
-  const int tile_shift = ilog2(c->tile_segments);
-  const int n_tiles = (int)((c->Nseg + c->tile_segments - 1) / c->tile_segments);
+  const StepTrack tr = step_track(c->h_t.data(), c->Nseg, c->T0, c->tile_segments, c->bank_tau_min, c->bank_r_max,
+                                  c->bank_f0max / c->df, pl.doppler_bins, c->f_min, c->df, pl.inv_q);
+  if (!tr.ok) return TCW_OK;
+  const int tile = 1 << tr.shift;
+  const StepGeometry g = step_geometry(c->S, c->D, c->Nseg, tile, c->h_v.data(), false);
+  const int n_tiles = (int)((c->Nseg + tile - 1) / tile);
   const size_t rows = (size_t)g.n_chunks * c->Nseg * c->D;
-  TCW_CUDA(c, c->step_q.ensure(rows * g.cpad * sizeof(int32_t)), "doppler rows");
-  TCW_CUDA(c, c->step_meta.ensure(rows * step_meta(g.cpad) * sizeof(int4)), "doppler rows");
+  TCW_CUDA(c, c->step_q.ensure(rows * step_row(g.cpad) * sizeof(int32_t)), "doppler rows");
+  TCW_CUDA(c, c->step_head.ensure(rows * kStepHead * sizeof(int4)), "doppler rows");
+  TCW_CUDA(c, c->step_tab.ensure(rows * step_buckets(g.cpad) * sizeof(uint32_t)), "doppler rows");
+  TCW_CUDA(c, c->step_wtot.ensure(kStepSlots * 16 + (size_t)c->Nseg * c->D * sizeof(longlong2)), "weight sums");
+  TCW_CUDA(c, cudaMemsetAsync(c->step_wtot.p, 0, kStepSlots * 16, c->stream), "weight sums");
   TCW_CUDA(c, ensure_step_edge(c->step_edge, c->grid, c->stream), "scratch");
-  if (step_ordered(g)) {
-    TCW_CUDA(c, c->step_order.ensure((size_t)g.passes * g.n_chunks * g.cpad * sizeof(int16_t)), "sky order");
-    TCW_CUDA(c, c->step_acc.ensure(step_acc_bytes(c->grid)), "scratch");
-  }
+  TCW_CUDA(c, c->step_slow.ensure(step_slow_bytes(c->grid)), "scratch");
+  if (step_ordered(g))
+    TCW_CUDA(c, c->step_order.ensure((size_t)g.passes * g.n_chunks * g.cpad * 2 * sizeof(int16_t)), "sky order");
   StepRowsParams rp{};
   rp.vel = c->vel.as<double>();
   rp.nhat = c->nhat_sorted.as<double>();
@@ -216,18 +221,28 @@ tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, boo
   rp.n_seg = (int)c->Nseg;
   rp.S = (int)c->S;
   set_step_geometry(rp, g);
-  rp.tile_shift = tile_shift;
+  rp.tile_shift = tr.shift;
   rp.inv_q = pl.inv_q;
+  rp.eps_max = tr.eps_max;
   rp.w1_scale = std::ldexp(1.0, sc.w1);
   rp.w2_scale = std::ldexp(1.0, sc.w2);
   rp.order = step_ordered(g) ? c->step_order.as<int16_t>() : nullptr;
+  rp.remap = rp.order ? rp.order + (size_t)g.passes * g.n_chunks * g.cpad : nullptr;
   rp.q = c->step_q.as<int32_t>();
-  rp.meta = c->step_meta.as<int4>();
+  rp.head = c->step_head.as<int4>();
+  rp.tab = c->step_tab.as<uint32_t>();
+  rp.wtot = c->step_wtot.as<unsigned long long>();
+  rp.wfix = reinterpret_cast<longlong2*>(rp.wtot + kStepSlots * 2);
   TCW_CUDA(c, launch_step_rows(rp, c->stream), "step_rows_kernel launch");
   ++*launches;
   if (count && (st = ensure_bits(c, launches)) != TCW_OK) return st;
   TCW_CUDA(c, c->anchors.ensure((size_t)c->Bpad * n_tiles * 2 * sizeof(double)), "anchors");
-  AnchorParams ap{};
+  TCW_CUDA(c, c->step_tiles.ensure((size_t)c->Bpad * n_tiles * sizeof(StepTile)), "track tiles");
+  StepTileParams tp{};
+  tp.f_min = c->f_min;
+  tp.df = c->df;
+  tp.tiles = c->step_tiles.as<StepTile>();
+  AnchorParams& ap = tp.a;
   ap.t_mid = c->t_mid.as<double>();
   ap.f0 = c->f0.as<double>();
   ap.tau = c->tau.as<double>();
@@ -235,21 +250,27 @@ tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, boo
   ap.T0 = c->T0;
   ap.n_seg = (int)c->Nseg;
   ap.n_tiles = n_tiles;
-  ap.tile_shift = tile_shift;
+  ap.tile_shift = tr.shift;
   ap.Bpad = c->Bpad;
   ap.anchors = c->anchors.as<double>();
-  ap.chain = anchor_chain_for(c->h_t.data(), c->Nseg, c->T0, 1 << tile_shift, c->bank_tau_min, c->bank_r_max);
+  ap.chain = anchor_chain_for(c->h_t.data(), c->Nseg, c->T0, tile, c->bank_tau_min, c->bank_r_max);
   StepEvent ev{};
   ev.rho = c->rho.p;
   ev.bits = count ? c->bits.as<uint32_t>() : nullptr;
   ev.bit_pitch = count ? bit_pitch_for(c->Nbin) : 0;
   ev.t_mid = c->t_mid.as<double>();
   ev.anchors = ap.anchors;
+  ev.tiles = tp.tiles;
   ev.f0 = ap.f0;
   ev.nbr = ap.nbr;
   ev.q = rp.q;
-  ev.meta = rp.meta;
+  ev.head = rp.head;
+  ev.tab = rp.tab;
+  ev.wtot = c->step_wtot.as<long long>();
+  ev.wfix = rp.wfix;
+  ev.sub_shift = step_sub_shift(g, c->Nseg, tr.shift);
   ev.order = rp.order;
+  ev.remap = rp.remap;
   ev.psi = c->psi.as<float>();
   ev.S_out = keep ? c->st_S.as<float>() : nullptr;
   ev.W1_out = keep ? c->st_W1.as<float>() : nullptr;
@@ -277,22 +298,19 @@ tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, boo
   p.df = c->df;
   p.inv_q = pl.inv_q;
   p.q = (float)pl.q;
-  p.q_exp = -std::ilogb(pl.q);
-  p.nterms = pl.nterms;
-  p.tile_shift = tile_shift;
-  p.sub_shift = step_sub_shift(c->Nseg, tile_shift);
+  p.inv_q_f = (float)pl.inv_q;
+  p.df_f = (float)c->df;
+  set_step_track(p, tr);
   p.amp_power = c->amp_power;
   p.nc_q = count ? std::exp(-c->rho_th) : 0.0;
   p.track_bins = c->track_bins;
   p.map_half = c->dtype == TCW_F16 ? 1 : 0;
-  p.acc = c->step_acc.as<long long>();
+  p.slow = c->step_slow.as<int4>();
   p.edge = c->step_edge.as<longlong2>();
   p.n_general = reinterpret_cast<unsigned long long*>(c->flags.as<char>() + 8);
   TCW_CUDA(c, cudaEventRecord(c->ev0, c->stream), "event");
-  TCW_CUDA(c, launch_anchors(ap, c->stream), "anchor_kernel launch");
-  const bool fast = step_fast_track(c->h_t.data(), c->Nseg, c->T0, c->tile_segments, c->bank_tau_min, c->bank_r_max,
-                                    c->f_min, c->df, p.q_exp) != 0;
-  TCW_CUDA(c, launch_step(p, g.dets_per_pass, c->dtype == TCW_F16, count || c->track_bins == 2, fast, step_cells(g),
+  TCW_CUDA(c, launch_step_tiles(tp, c->stream), "step_tile_kernel launch");
+  TCW_CUDA(c, launch_step(p, g.dets_per_pass, g.log_t, c->dtype == TCW_F16, count || c->track_bins == 2, step_cells(g),
                           std::min(c->grid, p.n_items), c->stream),
            "step_kernel launch");
   TCW_CUDA(c, cudaEventRecord(c->ev1, c->stream), "event");
@@ -928,7 +946,7 @@ tcw_status tcw_destroy(tcw_ctx* c) {
   cudaStreamSynchronize(c->stream);
   DevBuf* bufs[] = {&c->rho, &c->t_mid, &c->weights, &c->vel, &c->f0, &c->tau, &c->nbr,
                     &c->bank_perm, &c->bank_pos, &c->nhat_sorted, &c->sky_perm, &c->sky_pos,
-                    &c->step_q, &c->step_meta, &c->step_edge, &c->step_acc, &c->step_order,
+                    &c->step_q, &c->step_tiles, &c->step_head, &c->step_tab, &c->step_wtot, &c->step_edge, &c->step_slow, &c->step_order,
                     &c->dq, &c->anchors, &c->psi, &c->st_S, &c->st_W1, &c->st_W2, &c->dev,
                     &c->flags, &c->stage_f, &c->stage_i, &c->evtab, &c->items, &c->tri_dop,
                     &c->tri_hist, &c->tri_feat, &c->tri_psi, &c->tri_anchor, &c->tri_h1, &c->tri_h2,

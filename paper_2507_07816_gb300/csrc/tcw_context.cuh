@@ -92,7 +92,7 @@ struct tcw_ctx {
   bool sky_dirty = true;
   tcw::DevBuf nhat_sorted, sky_perm, sky_pos;
   // derived and outputs
-  tcw::DevBuf step_q, step_meta, step_edge, step_acc, step_order;   // step-function kernel: Doppler rows, band-edge scratch
+  tcw::DevBuf step_q, step_tiles, step_head, step_tab, step_wtot, step_edge, step_slow, step_order;   // step-function kernel: Doppler rows, band-edge scratch
   tcw::DevBuf dq, anchors, psi, st_S, st_W1, st_W2, dev, flags, stage_f, stage_i, evtab, items;
   int64_t items_key[5] = {-1, -1, -1, -1, -1};  // (n_chunks, Bpad, bank_chunk, grid, lanes) of the schedule
   int grid = 0, n_items = 0;

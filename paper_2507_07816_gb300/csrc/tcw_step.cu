@@ -15,15 +15,85 @@ constexpr int kStepWarps = kStepThreads / 32;
 // word takes at most 8 bin differences of at most 2^16 per (segment, detector),
 // 2 detectors, so 2^11 segments stay within 2^31.
 constexpr int kStepCarry = 2048;
-// fp32-pair track series: coefficients 1..4 as pairs, 5..kFastTerms as fp32
-constexpr int kFastTerms = 9;
-constexpr int kFastWords = 8 + (kFastTerms - 4);   // fp32 words of a template's coefficients
-constexpr int kCoefBytes = kMaxSeriesTerms * 8;    // per template, either form
-static_assert(kFastWords * 4 <= kCoefBytes, "coefficients fit");
+constexpr int kExactSpan = 8;    // boundaries either side of the track that the exact search goes to
+constexpr int kStepTerms = 4;    // fp32 terms of the track beyond the quadratic one
+constexpr int kStepTurn = 16;    // rows whose heads a warp holds (segments of a turn x detectors of a pass)
+// Entries of a warp's list (global memory), and the most that one round of lookups adds: 2 detectors,
+// 7 queue rounds and the lookups themselves.
+constexpr int kStepSlowMore = 2 * 8 * 32;
+constexpr int kStepSlow = kStepSlowMore + 256;
+constexpr int kStepQueue = 64;   // steps a warp's queue holds: fewer than 32 left over and 32 new ones
+
+// Anchor time of tile ti, as tile_anchor_time of tcw_persist.cuh.
+__device__ __forceinline__ double anchor_time(const double* t_mid, int n_seg, double T0, int shift, int ti) {
+  const int j0 = ti << shift;
+  return fmax(t_mid[j0 + (min(1 << shift, n_seg - j0) - 1) / 2], T0);
+}
+
+// ---------------------------------------------------------------------------
+// Tile anchors (the values of anchor_chain_kernel / anchor_kernel in
+// tcw_persist.cu) with the track constants of StepTile: one thread per
+// (template, run of kAnchorRun tiles), FP64.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(128) step_tile_kernel(StepTileParams p) {
+  const AnchorParams& a = p.a;
+  const int runs = (a.n_tiles + kAnchorRun - 1) / kAnchorRun;
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (int64_t)a.Bpad * runs) return;
+  const int b = (int)(i / runs), t0 = (int)(i % runs) * kAnchorRun;
+  const int t1 = min(a.n_tiles, t0 + kAnchorRun);
+  const double tau = a.tau[b], r = 1.0 / (a.nbr[b] - 1.0), inv_df = 1.0 / p.df, f0 = a.f0[b];
+  const double e2 = -0.5 * (-r - 1.0);   // C(e, 2) / e up to sign: C(e, 2) = e (e - 1) / 2, e = -r
+  double c[kAnchorTerms];   // C(r, k)
+  c[0] = 1.0;
+#pragma unroll
+  for (int k = 1; k < kAnchorTerms; ++k) c[k] = c[k - 1] * (r - (k - 1)) * (1.0 / k);
+  double h = 0.0, ta_prev = 0.0, y_prev = 0.0;
+  for (int ti = t0; ti < t1; ++ti) {
+    const double ta = anchor_time(a.t_mid, a.n_seg, a.T0, a.tile_shift, ti);
+    if (ti == t0 || !a.chain) {
+      h = pow((ta - a.T0) / tau + 1.0, r) / f0;
+    } else {
+      // u'/u - 1 = (t_a' - t_a) / (tau u) = (t_a' - t_a) y
+      const double d = (ta - ta_prev) * y_prev;
+      double S = c[kAnchorTerms - 1];
+#pragma unroll
+      for (int k = kAnchorTerms - 2; k >= 0; --k) S = fma(S, d, c[k]);
+      h *= S;
+    }
+    const double y = 1.0 / (tau + (ta - a.T0));
+    const int64_t o = (int64_t)b * a.n_tiles + ti;
+    reinterpret_cast<double2*>(a.anchors)[o] = make_double2(h, y);
+    // X = 1 / (h df): fp32 seed and two Newton steps
+    const double hd = h * p.df;
+    double X = (double)(1.0f / (float)hd);
+    X = X * fma(-hd, X, 2.0);
+    X = X * fma(-hd, X, 2.0);
+    const double xa = fma(-p.f_min, inv_df, X), xr = rint(xa);
+    const double A = -r * X * y, Q = A * e2 * y * -1.0;
+    StepTile t;
+    // far outside any band: no lookups
+    t.base = fabs(xr) < 1.0e9 ? (int)xr : INT_MIN / 2;
+    t.frac = (float)(xa - xr);
+    t.A_hi = (float)A;
+    t.A_lo = (float)(A - (double)t.A_hi);
+    t.Q_hi = (float)Q;
+    t.Q_lo = (float)(Q - (double)t.Q_hi);
+    t.X = (float)X;
+    t.s = (float)y;
+    int4* w = reinterpret_cast<int4*>(p.tiles + o);
+    const int4* v = reinterpret_cast<const int4*>(&t);
+    w[0] = v[0];
+    w[1] = v[1];
+    ta_prev = ta;
+    y_prev = y;
+  }
+}
 
 // ---------------------------------------------------------------------------
 // Sky order of one (pass, chunk): positions sorted by the grid value at the
-// pass's middle segment (ties by index), by counting.
+// pass's middle segment (ties by index), by counting; and each sky's position
+// in the order of the pass before.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ int doppler_q(const double* v, const double* n, double inv_q) {
   const double dD = (v[0] * n[0] + v[1] * n[1] + v[2] * n[2]) / kLightSpeed;   // Eq. 2
@@ -32,32 +102,46 @@ __device__ __forceinline__ int doppler_q(const double* v, const double* n, doubl
 
 __global__ void __launch_bounds__(kStepMaxChunk) step_order_kernel(StepRowsParams p) {
   __shared__ int s_q[kStepMaxChunk];
-  const int pass = blockIdx.x, c = blockIdx.y, i = threadIdx.x;
-  const int per = p.n_det / p.dets_per_pass;
-  const int e = pass / per, d = p.dets_per_pass == 1 ? pass % per : 0;
-  const int js = e * p.pass_seg, je = min(p.n_seg, js + p.pass_seg);
-  const double* v = p.vel + ((int64_t)d * p.n_seg + (js + je - 1) / 2) * 3;
+  const int c = blockIdx.y, i = threadIdx.x;
   const int rows = min(p.chunk, p.S - c * p.chunk);
-  if (i < rows) s_q[i] = doppler_q(v, p.nhat + (int64_t)(c * p.chunk + i) * 3, p.inv_q);
-  __syncthreads();
+  auto rank_in = [&](int pass) {
+    const int per = p.n_det / p.dets_per_pass;
+    const int e = pass / per, d = p.dets_per_pass == 1 ? pass % per : 0;
+    const int js = e * p.pass_seg, je = min(p.n_seg, js + p.pass_seg);
+    const double* v = p.vel + ((int64_t)d * p.n_seg + (js + je - 1) / 2) * 3;
+    __syncthreads();
+    if (i < rows) s_q[i] = doppler_q(v, p.nhat + (int64_t)(c * p.chunk + i) * 3, p.inv_q);
+    __syncthreads();
+    int rank = 0;
+    if (i < rows)
+      for (int k = 0; k < rows; ++k) rank += s_q[k] < s_q[i] || (s_q[k] == s_q[i] && k < i);
+    return rank;
+  };
+  const int pass = blockIdx.x;
+  const int rank = rank_in(pass), before = pass > 0 ? rank_in(pass - 1) : 0;
   if (i >= rows) return;
-  const int q = s_q[i];
-  int rank = 0;
-  for (int k = 0; k < rows; ++k) rank += s_q[k] < q || (s_q[k] == q && k < i);
-  int16_t* o = p.order + ((int64_t)pass * p.n_chunks + c) * p.cpad;
-  o[rank] = (int16_t)i;
-  if (rank == rows - 1)
-    for (int k = rows; k < p.cpad; ++k) o[k] = (int16_t)i;
+  const int64_t o = ((int64_t)pass * p.n_chunks + c) * p.cpad;
+  // positions past the last sky repeat it
+  for (int k = rank; k < (rank == rows - 1 ? p.cpad : rank + 1); ++k) {
+    p.order[o + k] = (int16_t)i;
+    p.remap[o + k] = (int16_t)before;
+  }
+}
+
+// Bucket of a threshold (or of a sky's grid value) in a row's table: monotone in v.
+__device__ __forceinline__ int step_bucket(int v, int qmin, float per_unit, int n) {
+  return min((int)((float)((unsigned)v - (unsigned)qmin) * per_unit), n - 1);
 }
 
 // ---------------------------------------------------------------------------
 // Doppler rows (Eq. 2): one CTA per (segment, detector, chunk), one thread per
-// block of 8 skies.
+// 8 skies.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(128) step_rows_kernel(StepRowsParams p) {
   __shared__ int s_max[4], s_min[4];
+  __shared__ uint16_t s_from[step_buckets(kStepMaxChunk)], s_to[step_buckets(kStepMaxChunk)];
   const int d = blockIdx.x % p.n_det, j = blockIdx.x / p.n_det, c = blockIdx.y;
-  const int nb = p.cpad / kStepBlock;
+  const int nb = p.cpad / kStepBlock, nk = step_buckets(p.cpad);
   const int g = threadIdx.x, lane = g & 31, warp = g >> 5;
   const int64_t dj = (int64_t)d * p.n_seg + j;
   const double* v = p.vel + dj * 3;
@@ -75,11 +159,11 @@ __global__ void __launch_bounds__(128) step_rows_kernel(StepRowsParams p) {
       mx = max(mx, qv[i]);
       mn = min(mn, qv[i]);
     }
-    int4* o = reinterpret_cast<int4*>(p.q + row * p.cpad + g * kStepBlock);
+    int4* o = reinterpret_cast<int4*>(p.q + row * step_row(p.cpad) + g * kStepBlock);
     o[0] = make_int4(qv[0], qv[1], qv[2], qv[3]);
     o[1] = make_int4(qv[4], qv[5], qv[6], qv[7]);
   }
-  // inclusive prefix maximum, exclusive suffix minimum over the blocks
+  // exclusive prefix maximum and suffix minimum over the threads
   int U = mx, L = mn;
 #pragma unroll
   for (int off = 1; off < 32; off <<= 1) {
@@ -89,32 +173,70 @@ __global__ void __launch_bounds__(128) step_rows_kernel(StepRowsParams p) {
   }
   if (lane == 31) s_max[warp] = U;
   if (lane == 0) s_min[warp] = L;
-  int Ln = __shfl_down_sync(0xffffffffu, L, 1);
-  if (lane == 31) Ln = INT_MAX;
+  int Ue = __shfl_up_sync(0xffffffffu, U, 1), Le = __shfl_down_sync(0xffffffffu, L, 1);
+  if (lane == 0) Ue = INT_MIN;
+  if (lane == 31) Le = INT_MAX;
   __syncthreads();
   int qmin = INT_MAX, qmax = INT_MIN;
   for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-    if (w < warp) U = max(U, s_max[w]);
-    if (w > warp) Ln = min(Ln, s_min[w]);
+    if (w < warp) Ue = max(Ue, s_max[w]);
+    if (w > warp) Le = min(Le, s_min[w]);
     qmin = min(qmin, s_min[w]);
     qmax = max(qmax, s_max[w]);
   }
-  int4* m = p.meta + row * step_meta(p.cpad);
-  if (g < nb) reinterpret_cast<int2*>(m + kStepHead)[g] = make_int2(U, Ln);
+  const float span = (float)((double)qmax - (double)qmin);
+  const float per_unit = span > 0.f ? (float)nk / span : 0.f;
+  if (g < nb) {
+    // Bucket k's window: from the first position whose prefix maximum falls into
+    // bucket k or a later one, to the first position whose suffix minimum falls
+    // into a later one, with a margin for the error of a threshold.  Position i
+    // fills the buckets that it is the first for.
+    auto up = [&](int v) { return step_bucket((int)min((long long)v + p.eps_max, (long long)INT_MAX), qmin, per_unit, nk); };
+    auto down = [&](int v) { return step_bucket((int)max((long long)v - p.eps_max, (long long)qmin), qmin, per_unit, nk); };
+    int u = Ue, ub = g > 0 ? up(Ue) : -1;
+    int l[kStepBlock];
+    int run = Le;
+#pragma unroll
+    for (int i = kStepBlock - 1; i >= 0; --i) {
+      run = min(run, qv[i]);
+      l[i] = run;
+    }
+#pragma unroll
+    for (int i = 0; i < kStepBlock; ++i) {
+      const int pos = g * kStepBlock + i;
+      u = max(u, qv[i]);
+      const int nu = up(u);
+      for (int k = ub + 1; k <= nu; ++k) s_from[k] = (uint16_t)pos;
+      ub = nu;
+      // suffix minimum from pos on to that from pos + 1 on
+      const int a = down(l[i]);
+      const int next = i + 1 < kStepBlock ? l[i + 1] : Le;
+      const int b = pos + 1 < p.cpad ? down(next) : nk;
+      for (int k = a; k < b; ++k) s_to[k] = (uint16_t)(pos + 1);
+    }
+  }
+  __syncthreads();
+  uint32_t* tab = p.tab + row * nk;
+  for (int k = threadIdx.x; k < nk; k += blockDim.x) tab[k] = (uint32_t)s_from[k] | (uint32_t)s_to[k] << 11;
   if (g == 0) {
-    // t_j - t_a from the anchor time of the tile (tile_anchor_time of tcw_persist.cuh)
-    const int t0 = j >> p.tile_shift << p.tile_shift;
-    const double ta = fmax(p.t_mid[t0 + (min(1 << p.tile_shift, p.n_seg - t0) - 1) / 2], p.T0);
-    const double tj = p.t_mid[j], dt = tj - ta;
-    const float dth = tj >= p.T0 ? (float)dt : NAN;
-    m[0] = make_int4(qmin, qmax, __float_as_int(dth), __float_as_int((float)(dt - (double)dth)));
+    int4* pad = reinterpret_cast<int4*>(p.q + row * step_row(p.cpad) + p.cpad);
+    pad[0] = pad[1] = make_int4(qmax, qmax, qmax, qmax);
+    int4* m = p.head + row * kStepHead;
+    const double ta = anchor_time(p.t_mid, p.n_seg, p.T0, p.tile_shift, j >> p.tile_shift);
+    const double tj = p.t_mid[j], dt = tj - ta, d2 = dt * dt;
+    const float dth = tj >= p.T0 ? (float)dt : NAN, d2h = (float)d2;
     const float w = p.weights[dj];
-    const float span = (float)((double)qmax - (double)qmin);
-    m[1] = make_int4(__float_as_int(span > 0.f ? (float)nb / span : 0.f), __float_as_int(w), 0, 0);
+    m[0] = make_int4(qmin, qmax, __float_as_int(per_unit), __float_as_int(w));
+    m[1] = make_int4(__float_as_int(dth), __float_as_int((float)(dt - (double)(float)dt)), __float_as_int(d2h),
+                     __float_as_int((float)(d2 - (double)d2h)));
     longlong2 wi;
     wi.x = __double2ll_rn((double)w * p.w1_scale);
     wi.y = __double2ll_rn((double)w * (double)w * p.w2_scale);
-    *reinterpret_cast<longlong2*>(m + 2) = wi;
+    if (c == 0) p.wfix[(int64_t)j * p.n_det + d] = wi;
+    if (c == 0 && tj >= p.T0) {
+      atomicAdd(p.wtot + 2 * (blockIdx.x % kStepSlots), (unsigned long long)wi.x);
+      atomicAdd(p.wtot + 2 * (blockIdx.x % kStepSlots) + 1, (unsigned long long)wi.y);
+    }
   }
 }
 
@@ -142,35 +264,40 @@ __global__ void absmax_kernel(const T* x, int64_t n, unsigned* out) {
 }
 
 // Shared memory of the search kernel for `cells` difference cells (templates x
-// (row + 1)): two word planes, piece sums of the epilogue, track series
-// coefficients, per-template sums.
+// (row + 1)): two word planes, the warps' queues of steps (and in their place
+// the piece sums of the epilogue), FP64 and fp32 series coefficients, the heads
+// of each warp's turn, per-template sums.
+static_assert(3 * kStepThreads * 8 <= kStepWarps * kStepQueue * 16, "piece sums fit the queues' place");
 struct StepLayout {
-  size_t lo, part, coef, tsum, total;
+  size_t part, coef, fcoef, queue, head, tsum, total;
   __host__ __device__ constexpr explicit StepLayout(int cells)
-      : lo((size_t)cells * 4),
-        part(((size_t)cells * 8 + 15) & ~(size_t)15),
-        coef(part + (size_t)3 * kStepThreads * 8),
-        tsum(coef + (size_t)kCoefBytes * 32),
+      : part(((size_t)cells * 8 + 15) & ~(size_t)15),
+        coef(part + (size_t)kStepWarps * kStepQueue * 16),
+        fcoef(coef + (size_t)kMaxSeriesTerms * 8 * 32),
+        queue(part),
+        head(fcoef + (size_t)32 * 16),
+        tsum(head + (size_t)kStepWarps * kStepTurn * kStepHead * 16),
         total(tsum + (size_t)32 * 4 * 8) {}
 };
+static_assert(StepLayout(kStepCells + 32).total <= 232448 - 1024, "one CTA's shared memory");
 
-// A value of the lookup at bin K (the caller checks the band).
+// A value of the lookup at bin K of row (the caller checks the band).
 // VK 0: fp32 power, 1: fp16 power, 2: number count and / or two-bin sums.
 template <int VK>
 __device__ __forceinline__ float step_value(const StepParams& p, const StepEvent& ev, int64_t row, int K) {
   if constexpr (VK == 0) {
-    return __ldg(static_cast<const float*>(ev.rho) + row * p.n_bin + K);
+    return __ldg(static_cast<const float*>(ev.rho) + (row + K));
   } else if constexpr (VK == 1) {
-    return __half2float(__ldg(static_cast<const __half*>(ev.rho) + row * p.n_bin + K));
+    return __half2float(__ldg(static_cast<const __half*>(ev.rho) + (row + K)));
   } else {
     const int more = p.track_bins == 2 ? 1 : 0;
     float v = 0.f;
     if (ev.bits) {
-      const uint32_t* r = ev.bits + row * ev.bit_pitch;
+      const uint32_t* r = ev.bits + row;
       for (int i = 0; i <= more; ++i) v += (float)((__ldg(r + ((K + i) >> 5)) >> ((K + i) & 31)) & 1u);
     } else {
       for (int i = 0; i <= more; ++i) {
-        const int64_t o = row * p.n_bin + K + i;
+        const int64_t o = row + K + i;
         v += p.map_half ? __half2float(__ldg(static_cast<const __half*>(ev.rho) + o))
                         : __ldg(static_cast<const float*>(ev.rho) + o);
       }
@@ -188,499 +315,711 @@ __device__ __forceinline__ void to_fixed(float v, float s, int& hi, int& lo) {
   lo = __float_as_int(fmaf(r, 65536.0f, kMagic)) - kMagicBits;
 }
 
-// An fp32 pair hi + lo.
-struct Pair {
-  float h, l;
+// The exact thresholds of (template b, segment j) on the q grid, as the group
+// kernel takes them: theta_n = (V + n V2) >> 8 between the bins base + n and
+// base + n + 1 (Eq. 1 in FP64 from the tile anchor; two-bin lookups: bin
+// centres in place of edges).
+struct StepExact {
+  long long V, V2;
+  double h;   // 1/f
+  int base;
 };
-__device__ __forceinline__ Pair pair_of(double x) {
-  const float h = (float)x;
-  return {h, (float)(x - (double)h)};
+__device__ __forceinline__ StepExact step_exact(const StepParams& p, const StepEvent& ev, const double* coef, int b,
+                                                int j, bool two) {
+  const int ti = j >> p.tile_shift;
+  const double2 an = reinterpret_cast<const double2*>(ev.anchors)[(int64_t)b * ev.n_tiles + ti];
+  const double delta = (ev.t_mid[j] - anchor_time(ev.t_mid, ev.n_seg, ev.T0, p.tile_shift, ti)) * an.y;
+  double R = coef[(p.nterms - 1) * 32];
+  for (int k = p.nterms - 2; k >= 0; --k) R = fma(R, delta, coef[k * 32]);
+  const double h = an.x * R;
+  StepExact x;
+  x.base = __float2int_rn((__frcp_rn((float)h) - (float)p.f_min) * (float)(1.0 / p.df));
+  const double Q = p.df * h;
+  const double A0 = fma((double)x.base + (two ? 1.0 : 0.5), Q, fma(p.f_min, h, -1.0));
+  x.V = __double2ll_rn(A0 * (p.inv_q * 256.0)) + 128;
+  x.V2 = __double2ll_rn(Q * (p.inv_q * 256.0));
+  x.h = h;
+  return x;
 }
-__device__ __forceinline__ Pair pair_mul(Pair a, Pair b) {
-  const float p = a.h * b.h;
-  float e = fmaf(a.h, b.h, -p);
-  e = fmaf(a.h, b.l, e);
-  return {p, fmaf(a.l, b.h, e)};
+
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
 }
-// c + a b for |c| >= |a b|
-__device__ __forceinline__ Pair pair_fma(Pair a, Pair b, Pair c) {
-  const Pair m = pair_mul(a, b);
-  const float h = c.h + m.h;
-  return {h, (m.h - (h - c.h)) + (c.l + m.l)};
+
+// v >> 8, saturated to 32 bits
+__device__ __forceinline__ int saturate(long long v) {
+  const int hi = (int)(v >> 32);
+  const int r = (int)__funnelshift_r((unsigned)v, (unsigned)hi, 8);
+  return hi >> 7 == r >> 31 ? r : (hi < 0 ? -2147483647 : 2147483647);
 }
-// round((h + l) 2^e) with s1 = 2^(e - 22), s2 = 2^e
-__device__ __forceinline__ long long pair_fixed(Pair a, float s1, float s2) {
-  const int hi = __float2int_rn(a.h * s1);
-  const float r = fmaf(a.h, s1, -(float)hi);
-  return (long long)hi * 4194304 + __float2int_rn(fmaf(r, 4194304.0f, a.l * s2));
+
+// Places one step with an exact threshold: calls place(position, up) where the
+// state of the sorted skies changes.
+template <typename F>
+__device__ __forceinline__ void place_exact(const int32_t* q, uint32_t window, int th, const F& place) {
+  const int to = (int)(window >> 11);
+  bool above = false;
+  for (int p = (int)(window & 0x7ff); p < to; ++p) {
+    const bool m = __ldg(q + p) >= th;
+    if (m != above) place(p, m);
+    above = m;
+  }
+  if (!above) place(to, true);
+}
+
+// What the rare lookups of a block need (shared memory).
+struct StepBlockCtx {
+  const StepEvent* ev;
+  int* chi;
+  const double* coef;
+  unsigned long long* tsum;
+  longlong2* edge;
+  int b0, cpad, nk, chunk;
+  unsigned edge_mask;   // templates with band-edge weight steps (bit per template)
+  unsigned n_edge;      // lookups at a band edge
+};
+
+// A lookup (template lt of the block; segment j, detector d) by the exact
+// thresholds: all of it with its weights at a band edge (only < 0), or only its
+// step `only`, whose fp32 threshold came too close to a sky.
+template <int VK, int LT>
+__device__ __forceinline__ void step_rare(const StepParams& p, StepBlockCtx& c, int lt, int j, int d, int only) {
+  const StepEvent& ev = *c.ev;
+  const bool two = VK == 2 && p.track_bins == 2;
+  const unsigned k_end = (unsigned)max(0, (int)p.n_bin - (two ? 1 : 0));
+  const int64_t row = ((int64_t)c.chunk * ev.n_seg + j) * p.n_det + d;
+  const int4 m0 = ev.head[row * kStepHead];
+  const float dth = __int_as_float(ev.head[row * kStepHead + 1].x);
+  if (!(dth == dth)) return;   // before T0
+  const StepExact x = step_exact(p, ev, c.coef + lt, c.b0 + lt, j, two);
+  float amp = 1.0f;
+  if (p.amp_power > 0) {
+    const float rr = (float)(x.h * ev.f0[c.b0 + lt]);
+    float rp = rr;
+    for (int k = 1; k < p.amp_power; ++k) rp *= rr;
+    amp = __frcp_rn(rp);
+  }
+  const float w = __int_as_float(m0.w) * amp, ws = w * ev.x_scale, per_unit = __int_as_float(m0.z);
+  const int64_t vrow =
+      ((int64_t)d * ev.n_seg + j) * (VK == 2 && ev.bits ? (int64_t)ev.bit_pitch : p.n_bin);
+  const int qmin = m0.x, qmax = m0.y;
+  auto value = [&](int K, int& h, int& l) {
+    to_fixed((unsigned)K < k_end ? step_value<VK>(p, ev, vrow, K) : 0.f, ws, h, l);
+  };
+  auto step = [&](int t, int K, long long e1, long long e2) {   // from bin K to K + 1
+    int h0, l0, h1, l1;
+    value(K, h0, l0);
+    value(K + 1, h1, l1);
+    const int dh = h1 - h0, dl = l1 - l0;
+    const uint32_t win = __ldg(ev.tab + row * c.nk + step_bucket(t, qmin, per_unit, c.nk));
+    place_exact(ev.q + row * step_row(c.cpad), win, t, [&](int pos, bool up) {
+      int* const cell = c.chi + (pos << (LT + 1)) + lt;
+      atomicAdd(cell, up ? dh : -dh);
+      atomicAdd(cell + (1 << LT), up ? dl : -dl);
+      if (e1 | e2) {
+        unsigned long long* ec = reinterpret_cast<unsigned long long*>(c.edge + (int64_t)lt * (c.cpad + 1) + pos);
+        atomicAdd(ec, (unsigned long long)(up ? e1 : -e1));
+        atomicAdd(ec + 1, (unsigned long long)(up ? e2 : -e2));
+      }
+    });
+  };
+  // first boundary above the lowest sky
+  int n = -kExactSpan;
+  long long v = x.V + n * x.V2;
+  while (n < kExactSpan && saturate(v) <= qmin) {
+    v += x.V2;
+    ++n;
+  }
+  const int K0 = x.base + n;   // the lowest sky's bin
+  if (only >= 0) {
+    step(saturate(v + only * x.V2), K0 + only, 0, 0);
+    return;
+  }
+  int nb = 0;
+  for (long long u = v; nb < kNThr && saturate(u) <= qmax; u += x.V2) ++nb;
+  long long u1, u2;   // the lookup's weights
+  if (p.amp_power > 0) {
+    int wh, wl;
+    to_fixed(w, ev.w1_scale, wh, wl);
+    u1 = (long long)wh * 65536 + wl;
+    to_fixed(w, w * ev.w2_scale, wh, wl);
+    u2 = (long long)wh * 65536 + wl;
+  } else {
+    const longlong2 wi = ev.wfix[(int64_t)j * p.n_det + d];
+    u1 = wi.x;
+    u2 = wi.y;
+  }
+  const bool first = (unsigned)K0 < k_end;
+  if (K0 < 0 || (unsigned)(K0 + nb) >= k_end) {
+    atomicAdd(&c.n_edge, 1u);
+    atomicOr(&c.edge_mask, 1u << lt);
+  }
+  int h0, l0;
+  value(K0, h0, l0);
+  atomicAdd(c.tsum + lt, (unsigned long long)((long long)h0 * 65536 + l0));
+  // W1, W2 start from every segment's weights, amplitude weights from 0
+  if (first != (p.amp_power == 0)) {
+    atomicAdd(c.tsum + 32 + lt, (unsigned long long)(first ? u1 : -u1));
+    atomicAdd(c.tsum + 64 + lt, (unsigned long long)(first ? u2 : -u2));
+  }
+  for (int i = 0; i < nb; ++i) {
+    const bool ok0 = (unsigned)(K0 + i) < k_end, ok1 = (unsigned)(K0 + i + 1) < k_end;
+    step(saturate(v + i * x.V2), K0 + i, ok1 == ok0 ? 0 : (ok1 ? u1 : -u1), ok1 == ok0 ? 0 : (ok1 ? u2 : -u2));
+  }
+}
+
+// The end of a pass: prefix sums of the cells over the sky positions; after the
+// last pass Psi (Eq. 4), before it the sums move to the next pass's sky order.
+// All threads of the CTA; a call, so that its registers do not weigh on the
+// search loop.
+template <int VK, int LT>
+__device__ __noinline__ void step_fold(const StepParams& p, StepBlockCtx& s_ctx, unsigned char* smem, long long* part,
+                                       int pass, bool last) {
+  constexpr unsigned kAll = 0xffffffffu;
+  constexpr int T = 1 << LT, pieces = kStepThreads >> LT;
+  const StepEvent& ev = *s_ctx.ev;
+  int* const chi = reinterpret_cast<int*>(smem);
+  int* const clo = chi + T;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int t = tid & (T - 1), pc = tid >> LT, cpad = s_ctx.cpad;
+  const int len = (cpad + pieces - 1) / pieces;
+  const int p0 = min(cpad, pc * len), p1 = min(cpad, p0 + len);
+  const unsigned long long* const tsum = s_ctx.tsum;
+  longlong2* const edge_acc = s_ctx.edge + kStepCells + 32;
+  longlong2* const ecol = s_ctx.edge + (int64_t)t * (cpad + 1);
+  const bool two = VK == 2 && p.track_bins == 2;
+  const int chunk = s_ctx.chunk, b0 = s_ctx.b0;
+  const bool te = (s_ctx.edge_mask >> t) & 1u;
+  {
+    long long sx = 0, s1 = 0, s2 = 0;
+    for (int q = p0; q < p1; ++q) {
+      const int c = (q << (LT + 1)) + t;
+      sx += (long long)chi[c] * 65536 + clo[c];
+      if (te) {
+        const longlong2 v = __ldcg(ecol + q);
+        s1 += v.x;
+        s2 += v.y;
+      }
+    }
+    part[tid] = sx;
+    part[kStepThreads + tid] = s1;
+    part[2 * kStepThreads + tid] = s2;
+  }
+  __syncthreads();
+  // exclusive scans over a template's pieces (32 or 64), one warp per template
+  for (int tt = warp; tt < T; tt += kStepWarps) {
+    const int ks = s_ctx.edge_mask >> tt & 1u ? 3 : 1;
+    for (int k = 0; k < ks; ++k) {
+      long long run = 0;
+      for (int i0 = 0; i0 < pieces; i0 += 32) {
+        long long* const q = part + k * kStepThreads + ((i0 + lane) << LT) + tt;
+        const long long v = i0 + lane < pieces ? *q : 0;
+        long long sum = v;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+          const long long u = __shfl_up_sync(kAll, sum, off);
+          if (lane >= off) sum += u;
+        }
+        if (i0 + lane < pieces) *q = run + sum - v;
+        run += __shfl_sync(kAll, sum, 31);
+      }
+    }
+  }
+  __syncthreads();
+  if (!last) {
+    // the sums move to the next pass's order of the skies: prefix sums in place, then their
+    // differences along the new order (exact integers modulo 2^48)
+    long long X = part[tid], w1 = part[kStepThreads + tid], w2 = part[2 * kStepThreads + tid];
+    for (int q = p0; q < p1; ++q) {
+      const int c = (q << (LT + 1)) + t;
+      X += (long long)chi[c] * 65536 + clo[c];
+      chi[c] = (int)(X >> 16);
+      clo[c] = (int)(X & 0xffff);
+      if (te) {
+        const longlong2 v = __ldcg(ecol + q);
+        w1 += v.x;
+        w2 += v.y;
+        __stcg(edge_acc + (int64_t)t * cpad + q, make_longlong2(w1, w2));
+      }
+    }
+    __syncthreads();
+    const int16_t* map = ev.remap + ((int64_t)(pass + 1) * ev.n_chunks + chunk) * cpad;
+    long long prev = 0;
+    longlong2 eprev = make_longlong2(0, 0);
+    if (p0 > 0 && p0 < p1) {
+      const int m = map[p0 - 1], c = (m << (LT + 1)) + t;
+      prev = (long long)chi[c] * 65536 + clo[c];
+      if (te) eprev = __ldcg(edge_acc + (int64_t)t * cpad + m);
+    }
+    constexpr int kLen = kStepMaxChunk * 16 / kStepThreads;   // positions of a piece
+    int dh[kLen], dl[kLen];
+#pragma unroll
+    for (int i = 0; i < kLen; ++i) {
+      if (p0 + i < p1) {
+        const int m = map[p0 + i], c = (m << (LT + 1)) + t;
+        const long long v = (long long)chi[c] * 65536 + clo[c], u = v - prev;
+        prev = v;
+        dh[i] = (int)(u >> 16);
+        dl[i] = (int)(u & 0xffff);
+        if (te) {
+          const longlong2 w = __ldcg(edge_acc + (int64_t)t * cpad + m);
+          __stcg(ecol + p0 + i, make_longlong2(w.x - eprev.x, w.y - eprev.y));
+          eprev = w;
+        }
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kLen; ++i) {
+      if (p0 + i < p1) {
+        const int c = ((p0 + i) << (LT + 1)) + t;
+        chi[c] = dh[i];
+        clo[c] = dl[i];
+      }
+    }
+  } else {
+    // Eq. 4: <s> = mq W1, sigma^2 = vq W2 (power: 1, 1; number count: q, q(1-q)),
+    // both doubled for two-bin lookups
+    const double nbins = two ? 2.0 : 1.0;
+    const bool count = VK == 2 && p.nc_q > 0.0;
+    const double mq = nbins * (count ? p.nc_q : 1.0);
+    const float vq = (float)(nbins * (count ? p.nc_q * (1.0 - p.nc_q) : 1.0));
+    const double m_units = mq * ev.w1_unit / ev.x_unit;   // mean of one W1 unit, in units of X
+    const float x_unit = (float)ev.x_unit;
+    const int64_t sky0 = (int64_t)chunk * ev.chunk;
+    const int rows = min(ev.chunk, ev.S - (int)sky0);
+    long long X = part[tid] + (long long)tsum[t];
+    long long w1 = (long long)tsum[32 + t], w2 = (long long)tsum[64 + t];
+    if (te) {
+      w1 += part[kStepThreads + tid];
+      w2 += part[2 * kStepThreads + tid];
+    }
+    // skies without band-edge steps share W1, W2 and the mean
+    long long mean = 0;
+    float W2f = 0.f, rs = 0.f;
+    auto moments = [&]() {
+      mean = __double2ll_rn((double)w1 * m_units);
+      W2f = (float)((double)w2 * ev.w2_unit);
+      rs = W2f > 0.f ? rsqrtf(vq * W2f) : 0.f;
+    };
+    moments();
+    const int16_t* order = ev.order ? ev.order + ((int64_t)pass * ev.n_chunks + chunk) * cpad : nullptr;
+    for (int q = p0; q < p1; ++q) {
+      const int c = (q << (LT + 1)) + t;
+      X += (long long)chi[c] * 65536 + clo[c];
+      chi[c] = clo[c] = 0;
+      if (te) {
+        const longlong2 v = __ldcg(ecol + q);
+        __stcg(ecol + q, make_longlong2(0, 0));
+        w1 += v.x;
+        w2 += v.y;
+        moments();
+      }
+      if (q >= rows) continue;
+      // the cells' high words wrap at 2^31, so X is known modulo 2^48
+      const long long x = (long long)((unsigned long long)X << 16) >> 16;
+      const int64_t o = (sky0 + (order ? (int)order[q] : q)) * ev.Bpad + b0 + t;
+      ev.psi[o] = W2f > 0.f ? (float)(x - mean) * x_unit * rs : -INFINITY;
+      if (ev.S_out) {
+        ev.S_out[o] = (float)((double)x * ev.x_unit);
+        ev.W1_out[o] = (float)((double)w1 * ev.w1_unit);
+        ev.W2_out[o] = W2f;
+      }
+    }
+  }
 }
 
 // The search kernel: one CTA per SM takes (sky chunk, template block) items from
 // a counter; the difference cells of a block (16 or 32 templates x up to 1024
 // skies, two words each) live in shared memory, one column per template.  A
-// lane owns one (template, segment) of its warp's turn: the track, the first
-// sky's bin, and for each bin boundary inside the chunk's Doppler range one
-// search in the row and one difference.  It is bound by the latency and the
-// number of its instructions (nothing is saturated), so as many warps as fit
-// (32; 24 and 16 measured slower).  2e5 templates x 1024 skies x 2 detectors x
-// 1e4 segments: 644 ms by the group kernel -> 276 ms; one sky: 204 -> 50 ms.
-template <int VK, int DP, bool FAST>
+// lane owns one (template, segment) of its warp's turn: the fp32 track, the
+// first sky's bin, and for each bin boundary inside the chunk's Doppler range a
+// step put on the warp's queue, so that 32 steps are placed at a time whatever
+// their number per lookup.  What fp32 cannot decide (a sky within the
+// threshold's error, about 2 in 1000 steps), skies out of order and lookups at a
+// band edge go on a list that the warp works through at the end of its turn with
+// the exact FP64 thresholds, so that the search loop has no FP64 and no calls.
+// It is bound by instruction latency: about 190 instructions per 32 (template,
+// segment) and 350 more for the steps of 1024 skies, 0.6 and 0.4 issued per
+// scheduler and cycle, nothing saturated; hence 32 warps (24: 3-10 % slower).
+// 2e5 templates x 1024 skies x 2 detectors x 1e4 segments: 655 ms by the group
+// kernel, 276 with the track in fp32 pairs and every step searched where it
+// arises, 160 so; one sky and one detector: 205, 50, 25 ms.
+template <int VK, int DP, int LT>
 __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int cells) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_item;
-  __shared__ unsigned s_edge;   // templates with band-edge weight steps (bit per template)
+  __shared__ unsigned long long s_wtot[2];
+  __shared__ StepBlockCtx s_ctx;
+  __shared__ StepEvent s_ev;   // the item's event: read in the loops without a trip to global memory
   const StepLayout L(cells);
   int* const chi = reinterpret_cast<int*>(smem);
-  int* const clo = reinterpret_cast<int*>(smem + L.lo);
+  constexpr int T = 1 << LT;      // templates of a block
+  int* const clo = chi + T;       // cell (position, template) at [position][word][template]
   long long* const part = reinterpret_cast<long long*>(smem + L.part);
   double* const coef = reinterpret_cast<double*>(smem + L.coef);
-  float* const fcoef = reinterpret_cast<float*>(smem + L.coef);   // [word][32]: c1 hi lo .. c4 hi lo, c5 ..
+  float4* const fcoef = reinterpret_cast<float4*>(smem + L.fcoef);   // [32]: C(e, 3) .. C(e, 6)
+  int4* const queue = reinterpret_cast<int4*>(smem + L.queue) + (threadIdx.x >> 5) * kStepQueue;
+  int4* const slow_list = p.slow + ((int64_t)blockIdx.x * kStepWarps + (threadIdx.x >> 5)) * kStepSlow;
+  int4* const heads = reinterpret_cast<int4*>(smem + L.head) + (threadIdx.x >> 5) * kStepTurn * kStepHead;
   unsigned long long* const tsum = reinterpret_cast<unsigned long long*>(smem + L.tsum);   // X0, W1, W2 [32]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const float fmin_f = (float)p.f_min, inv_df_f = (float)(1.0 / p.df);
   const bool two = VK == 2 && p.track_bins == 2;
-  const int more_bins = two ? 1 : 0;
+  constexpr unsigned kAll = 0xffffffffu;
+  const unsigned lt_mask = (1u << lane) - 1u;
   const int n_bin = (int)p.n_bin;
+  const float hb = two ? 1.0f : 0.5f;   // boundary n lies at base + n + hb
   longlong2* const edge = p.edge + (int64_t)blockIdx.x * (2 * kStepCells + 32);
-  longlong2* const edge_acc = edge + kStepCells + 32;
-  long long* const acc = p.acc + (int64_t)blockIdx.x * kStepCells;
-  unsigned long long ngen = 0;
 
-  for (int i = tid; i < cells; i += kStepThreads) chi[i] = clo[i] = 0;
+  for (int i = tid; i < 2 * cells; i += kStepThreads) chi[i] = 0;
+  if (tid == 0) s_ctx.n_edge = 0;
 
   while (true) {
     __syncthreads();
     if (tid == 0) {
       s_item = (int)atomicAdd(p.next, 1u);
-      s_edge = 0;
     }
-    if (tid < 32 * 4) tsum[tid] = 0;
     __syncthreads();
     if (s_item >= p.n_items) break;
     int4 item;
     if (p.items) {
       item = p.items[s_item];
     } else {
-      const int blocks = p.events[0].Bpad >> p.events[0].log_t, g0 = s_item / p.n_chunks * p.bank_chunk;
-      item = make_int4(0, s_item % p.n_chunks, g0 << p.events[0].log_t, min(p.bank_chunk, blocks - g0));
+      const int blocks = p.events[0].Bpad >> LT, g0 = s_item / p.n_chunks * p.bank_chunk;
+      item = make_int4(0, s_item % p.n_chunks, g0 << LT, min(p.bank_chunk, blocks - g0));
     }
-    const StepEvent& ev = p.events[item.x];
-    const int log_t = ev.log_t, T = 1 << log_t, cpad = ev.cpad;
-    const int n_seg = ev.n_seg;
-    const int lt = lane & (T - 1), ls = lane >> log_t, lps = 32 >> log_t;
-    const int meta_n = step_meta(cpad);
+    for (int i = tid; i < (int)(sizeof(StepEvent) / 4); i += kStepThreads)
+      reinterpret_cast<int*>(&s_ev)[i] = reinterpret_cast<const int*>(p.events + item.x)[i];
+    __syncthreads();
+    const StepEvent& ev = s_ev;
+    const int cpad = ev.cpad;
+    const int n_seg = ev.n_seg, sub = min(ev.sub_shift, DP == 1 ? 4 : 3);
+    const int lt = lane & (T - 1), ls = lane >> LT;
+    constexpr int lps = 32 >> LT;
+    const unsigned t_mask = T == 32 ? kAll : (1u << T) - 1u;
+    const int nk = step_buckets(cpad), qs = step_row(cpad);
+    const int vpitch = VK == 2 && ev.bits ? ev.bit_pitch : n_bin;
     const int64_t row0 = (int64_t)item.y * n_seg * p.n_det;
     const float xs = ev.x_scale;
-    // epilogue roles: template t, piece pc of the positions
-    const int t = tid & (T - 1), pc = tid >> log_t, pieces = kStepThreads >> log_t;
-    const int len = (cpad + pieces - 1) / pieces;
-    const int p0 = min(cpad, pc * len), p1 = min(cpad, p0 + len);
-    longlong2* const ecol = edge + (int64_t)t * (cpad + 1);
+
+    // W1, W2 of every segment from T0 on (unit and per-segment weights: lookups
+    // outside the band are taken off; amplitude weights are summed per lookup)
+    if (tid < 2) {
+      long long sum = 0;
+      if (p.amp_power == 0)
+        for (int i = 0; i < kStepSlots; ++i) sum += __ldg(ev.wtot + 2 * i + tid);
+      s_wtot[tid] = (unsigned long long)sum;
+    }
+    __syncthreads();
+    if (tid < 32 * 3) tsum[tid] = tid < 32 ? 0 : s_wtot[tid / 32 - 1];
 
     for (int tb = 0; tb < item.w; ++tb) {
       const int b0 = item.z + tb * T, b = b0 + lt;
+      const float famp = p.amp_power > 0 ? p.df_f / (float)ev.f0[b] : 0.f;
+      if (tid == 0) {
+        s_ctx.ev = &ev;
+        s_ctx.chi = chi;
+        s_ctx.coef = coef;
+        s_ctx.tsum = tsum;
+        s_ctx.edge = edge;
+        s_ctx.b0 = b0;
+        s_ctx.cpad = cpad;
+        s_ctx.nk = nk;
+        s_ctx.chunk = item.y;
+        s_ctx.edge_mask = 0;
+      }
       if (tid < T) {
-        // binomial coefficients C(r, k) of (1 + delta)^r, r = 1/(n - 1)
+        // binomial coefficients C(r, k) of 1/f and C(e, k) of f, r = 1/(n - 1) = -e
         const double r = 1.0 / (ev.nbr[b0 + tid] - 1.0);
         double c = 1.0;
-        if constexpr (FAST) {
-          for (int k = 1; k <= kFastTerms; ++k) {
-            c = c * (r - (k - 1)) / k;
-            if (k <= 4) {
-              const Pair q = pair_of(c);
-              fcoef[(2 * k - 2) * 32 + tid] = q.h;
-              fcoef[(2 * k - 1) * 32 + tid] = q.l;
-            } else {
-              fcoef[(k + 3) * 32 + tid] = (float)c;
-            }
-          }
-        } else {
-          for (int k = 0; k < p.nterms; ++k) {
-            coef[k * 32 + tid] = c;
-            c = c * (r - k) / (k + 1);
-          }
+        for (int k = 0; k < p.nterms; ++k) {
+          coef[k * 32 + tid] = c;
+          c = c * (r - k) / (k + 1);
         }
+        float cf[kStepTerms];
+        c = 0.5 * r * (r + 1.0);
+#pragma unroll
+        for (int k = 0; k < kStepTerms; ++k) {
+          c = c * (-r - (k + 2)) / (k + 3);
+          cf[k] = (float)c;
+        }
+        fcoef[tid] = make_float4(cf[0], cf[1], cf[2], cf[3]);
       }
       __syncthreads();
-      long long X0 = 0, W1 = 0, W2 = 0;
+      long long X0 = 0;
       for (int pass = 0; pass < ev.passes; ++pass) {
         const int per = p.n_det / DP;
         const int d0 = DP == 1 ? pass % per : 0;
         const int js = pass / per * ev.pass_seg, je = min(n_seg, js + ev.pass_seg);
         for (int jc = js; jc < je; jc += kStepCarry) {
           const int jce = min(je, jc + kStepCarry);
-          for (int j0 = jc + (warp << p.sub_shift); j0 < jce; j0 += kStepWarps << p.sub_shift) {
-            const int ti = j0 >> p.tile_shift;
-            const double2 an = reinterpret_cast<const double2*>(ev.anchors)[(int64_t)b * ev.n_tiles + ti];
-            // constants of (template, tile)
-            Pair io, io1, qa;
-            float fa = 0.f;
-            int Ba = 0;
-            long long E11 = 0, Q10 = 0;
-            double ta = 0.0;
-            if constexpr (FAST) {
-              // h = 1/f = h_a (1 + g); c_K h - 1 = E_a + (1 + E_a) g + (K - K_a) df h_a (1 + g)
-              // with c_a the bin centre nearest to f_a and E_a = c_a h_a - 1
-              fa = __frcp_rn((float)an.x);
-              Ba = __float2int_rn((fa - fmin_f) * inv_df_f);
-              const double Qd = p.df * an.x;
-              const double Ea = fma((double)Ba, Qd, fma(p.f_min, an.x, -1.0));
-              io = pair_of(an.y);
-              io1 = pair_of(fma(an.y, Ea, an.y));
-              qa = pair_of(Qd);
-              E11 = __double2ll_rn(ldexp(Ea, 19) * p.inv_q);
-              Q10 = __double2ll_rn(ldexp(Qd, 18) * p.inv_q);
-            } else {
-              const int t0 = ti << p.tile_shift;
-              ta = fmax(ev.t_mid[t0 + (min(1 << p.tile_shift, n_seg - t0) - 1) / 2], ev.T0);
-            }
-            const int jn = min(jce, j0 + (1 << p.sub_shift));
-            for (int j = j0 + ls; j < jn; j += lps) {
-              const int4* meta = ev.meta + (row0 + (int64_t)j * p.n_det + d0) * meta_n;
-              int4 m0 = __ldg(meta);
-              const float dth = __int_as_float(m0.z);
-              if (!(dth == dth)) continue;   // before T0
-              // track (Eq. 1): f, the nearest bin `base` of the unshifted track, and the thresholds
-              // theta_n = c_K / f - 1 between the bins K = base + n and K + 1 (two-bin lookups: the
-              // bin centres f_min + (K + 1) df in place of the edges)
-              float f, h_f0 = 1.f;
-              int base;
-              long long A, B;   // FAST: theta_n = (A + B (2 n + 1 or 2)) >> 11 >> 8; else (A + n B) >> 8
-              long long G = 0;
-              if constexpr (FAST) {
-                const Pair dt{dth, __int_as_float(m0.w)};
-                const Pair dl = pair_mul(dt, io), dl1 = pair_mul(dt, io1);
-                float s = fcoef[(kFastTerms + 3) * 32 + lt];
-#pragma unroll
-                for (int k = kFastTerms - 1; k >= 5; --k) s = fmaf(dl.h, s, fcoef[(k + 3) * 32 + lt]);
-                Pair sp{fcoef[6 * 32 + lt], fmaf(dl.h, s, fcoef[7 * 32 + lt])};
-#pragma unroll
-                for (int k = 3; k >= 1; --k)
-                  sp = pair_fma(dl, sp, {fcoef[(2 * k - 2) * 32 + lt], fcoef[(2 * k - 1) * 32 + lt]});
-                const Pair g = pair_mul(dl, sp);
-                const Pair gq = pair_mul(qa, g);
-                f = fa * __frcp_rn(1.0f + g.h);
-                h_f0 = 1.0f + g.h;
-                const float sg = __int_as_float((p.q_exp + 8 + 127) << 23);   // 2^(q_exp + 8)
-                G = pair_fixed(pair_mul(dl1, sp), sg * (1.0f / 4194304.0f), sg);
-                B = Q10 + pair_fixed(gq, sg * (1.0f / 4096.0f), sg * 1024.0f);
-                const float x = (f - fmin_f) * inv_df_f;
-                base = __float2int_rn(x);
-                A = E11 + 1024 + (long long)(2 * (base - Ba) + (two ? 2 : 1)) * B;
-                G += 128;
-              } else {
-                const double delta = (ev.t_mid[j] - ta) * an.y;
-                double R = coef[(p.nterms - 1) * 32 + lt];
-#pragma unroll 4
-                for (int k = p.nterms - 2; k >= 0; --k) R = fma(R, delta, coef[k * 32 + lt]);
-                const double h = an.x * R;
-                f = __frcp_rn((float)h);
-                base = __float2int_rn((f - fmin_f) * inv_df_f);
-                const double Q = p.df * h;
-                const double A0 = fma((double)base + (two ? 1.0 : 0.5), Q, fma(p.f_min, h, -1.0));
-                A = __double2ll_rn(A0 * (p.inv_q * 256.0)) + 128;
-                B = __double2ll_rn(Q * (p.inv_q * 256.0));
-                h_f0 = (float)(h * ev.f0[b]);
+          for (int j0 = jc + (warp << sub); j0 < jce; j0 += kStepWarps << sub) {
+            const int jn = min(jce, j0 + (1 << sub));
+            const int64_t rbase = row0 + (int64_t)j0 * p.n_det + d0;   // first row of the turn
+            const int64_t vbase = ((int64_t)d0 * n_seg + j0) * vpitch;
+            {
+              // heads of the turn's rows
+              __syncwarp();
+              const int nr = (jn - j0) * DP;
+              if (lane < nr) {
+                const int4* h = ev.head + (rbase + (int64_t)(lane / DP) * p.n_det + lane % DP) * kStepHead;
+                heads[lane * kStepHead] = __ldg(h);
+                heads[lane * kStepHead + 1] = __ldg(h + 1);
               }
-              auto threshold = [&](int n) {
-                long long v = FAST ? (((A + (long long)(2 * n) * B) >> 11) + G) >> 8 : (A + (long long)n * B) >> 8;
-                v = v > 2147483647LL ? 2147483647LL : (v < -2147483647LL ? -2147483647LL : v);
-                return (int)v;
-              };
+              __syncwarp();
+            }
+            // dt at the ends of the turn; NaN before T0
+            const float dt_first = __int_as_float(heads[1].x);
+            const float dt_last = __int_as_float(heads[((jn - j0) * DP - 1) * kStepHead + 1].x);
+            if (!(dt_last == dt_last)) continue;
+            const int4* tp =
+                reinterpret_cast<const int4*>(ev.tiles + ((int64_t)b * ev.n_tiles + (j0 >> p.tile_shift)));
+            const int4 t0 = __ldg(tp), t1 = __ldg(tp + 1);
+            const int base_a = t0.x;
+            const float frac_a = __int_as_float(t0.y), A_hi = __int_as_float(t0.z), A_lo = __int_as_float(t0.w);
+            const float Q_hi = __int_as_float(t1.x), Q_lo = __int_as_float(t1.y), Xf = __int_as_float(t1.z),
+                        sg = __int_as_float(t1.w);
+            // The template's bins over the turn (tracks fall, Doppler shifts below 3 bins): wholly in the
+            // band, wholly out of it, or at an edge (or T0), which step_rare takes segment by segment
+            unsigned at_edge, outside;
+            {
+              const float x0 = fmaf(A_hi, dt_first, fmaf(Q_hi, dt_first * dt_first, (float)base_a));
+              const float x1 = fmaf(A_hi, dt_last, fmaf(Q_hi, dt_last * dt_last, (float)base_a));
+              const bool whole = dt_first == dt_first;
+              const bool in = whole && fminf(x0, x1) >= 8.0f && fmaxf(x0, x1) <= (float)n_bin - 10.0f;
+              const bool out = whole && (fmaxf(x0, x1) < -8.0f || fminf(x0, x1) > (float)n_bin + 8.0f);
+              outside = __ballot_sync(kAll, out);
+              at_edge = __ballot_sync(kAll, !out && !in);
+            }
+            const bool mine = !(((at_edge | outside) >> lane) & 1u);
+            int cnt = 0;     // steps in the warp's queue
+            int nslow = 0;   // steps and lookups in its list
+            // Places the last steps of the queue, one per lane: the sky at which the threshold lies
+            // among the four from the window's start on.  The others go on the list: longer windows,
+            // skies out of order, a sky within the threshold's error.
+            auto drain = [&]() {
+              __syncwarp();
+              const int take = min(cnt, 32);
+              cnt -= take;
+              const bool on = lane < take;
+              // threshold; difference words; row, template; window, step, error
+              const int4 e = on ? queue[cnt + lane] : make_int4(0, 0, 0, 0);
+              const int from = e.w & 0x7ff, to = (e.w >> 11) & 0x7ff;
+              const int32_t* const q = ev.q + ((rbase + ((e.z >> 5) & 0xff)) * qs + from);
+              const int a0 = __ldg(q), a1 = __ldg(q + 1), a2 = __ldg(q + 2), a3 = __ldg(q + 3);
+              const unsigned er = (unsigned)e.w >> 25 << p.eps_shift, lo = (unsigned)e.x - er;
+              const unsigned below = (unsigned)(a0 < e.x) | (unsigned)(a1 < e.x) << 1 | (unsigned)(a2 < e.x) << 2 |
+                                     (unsigned)(a3 < e.x) << 3;
+              const bool near = (unsigned)a0 - lo <= 2u * er || (unsigned)a1 - lo <= 2u * er ||
+                                (unsigned)a2 - lo <= 2u * er || (unsigned)a3 - lo <= 2u * er;
+              const bool slow = on && (near || below == 15u || (below & (below + 1u)) || to > from + 4);
+              if (on && !slow) {
+                int* const cell = chi + (((from + __popc(below)) << (LT + 1)) + (e.z & 31));
+                atomicAdd(cell, e.y);
+                atomicAdd(cell + T, e.z >> 13);
+              }
+              if (const unsigned vote = __ballot_sync(kAll, slow)) {
+                if (slow) slow_list[nslow + __popc(vote & lt_mask)] = e;
+                nslow += __popc(vote);
+              }
+              __syncwarp();
+            };
+            int jb = (at_edge | outside) == kAll ? jn : j0;
+            do {
+            // segments of the turn, then rounds without lookups until the queue is empty
+            for (; (jb < jn || cnt > 0) && nslow <= kStepSlow - kStepSlowMore; jb += lps) {
+              const int j = min(jb + ls, jn - 1), jr = j - j0;
+              const bool turn = mine && jb + ls < jn;
+              const int4* head = heads + jr * DP * kStepHead;
+              const float4 dt = *reinterpret_cast<const float4*>(head + 1);
+              // the unshifted track's position base + frac and F = f/df (see StepTile): the linear and
+              // quadratic terms as products of fp32 pairs whose rounding errors are recovered by fma and
+              // whose integer parts are split off exactly, the rest an fp32 series
+              const float pl = A_hi * dt.x, plr = rintf(pl);
+              const float pq = Q_hi * dt.z, pqr = rintf(pq);
+              const float dl3 = dt.x * sg;
+              const float4 cf = fcoef[lt];
+              float hs = fmaf(cf.w, dl3, cf.z);
+              hs = fmaf(hs, dl3, cf.y);
+              hs = fmaf(hs, dl3, cf.x);
+              const float p3 = Xf * (dl3 * dl3 * dl3 * hs);
+              const float small = (fmaf(A_hi, dt.x, -pl) + fmaf(A_hi, dt.y, A_lo * dt.x)) +
+                                  (fmaf(Q_hi, dt.z, -pq) + fmaf(Q_hi, dt.w, Q_lo * dt.z)) + p3;
+              const float F = (Xf + pl) + (pq + p3);
+              const int base = base_a + (int)(plr + pqr);
               float amp = 1.0f;
               if (p.amp_power > 0) {
-                if constexpr (FAST) h_f0 *= (float)(an.x * ev.f0[b]);
-                float rp = h_f0;
-                for (int k = 1; k < p.amp_power; ++k) rp *= h_f0;
-                amp = __frcp_rn(rp);
+                const float rr = turn ? F * famp : 1.0f;   // f / f0
+                amp = rr;
+                for (int k = 1; k < p.amp_power; ++k) amp *= rr;
               }
-              const float F = f * inv_df_f;
-              const float x = (f - fmin_f) * inv_df_f;
-              if (!(base >= -kMHi && base < n_bin - kMLo)) continue;
-              const float y0 = x - (float)base - (two ? 1.0f : 0.5f), Fq = F * p.q;
-#pragma unroll
+              const float Fq = F * p.q, R = rcp_approx(F) * p.inv_q_f;
+              const float y0 = ((frac_a + (pl - plr)) + ((pq - pqr) + small)) - hb;
+              const uint32_t eps = (uint32_t)(int)fmaf(R, p.eps_scale, 1.0f) << 25;
+#pragma unroll 1
               for (int dd = 0; dd < DP; ++dd) {
-                if (dd > 0) {
-                  meta += meta_n;
-                  m0 = __ldg(meta);
+                const int4 m0 = head[dd * kStepHead];
+                // the lowest and the highest sky's distance from boundary 0, in bins: boundaries in between
+                const float zl = fmaf(Fq, (float)m0.x, y0), zh = fmaf(Fq, (float)m0.y, y0);
+                const float fl = floorf(zl);
+                const bool close = turn && (fabsf(zl - rintf(zl)) < p.eps || fabsf(zh - rintf(zh)) < p.eps);
+                const bool on = turn && !close;
+                const int rl = jr * p.n_det + dd, tag = rl << 5 | lt;
+                if (const unsigned vote = __ballot_sync(kAll, close)) {
+                  if (close) slow_list[nslow + __popc(vote & lt_mask)] = make_int4(0, 0, tag, -1);
+                  nslow += __popc(vote);
                 }
-                const int qmin = m0.x, qmax = m0.y;
-                const int4 m1 = __ldg(meta + 1);
-                const float w = __int_as_float(m1.y) * amp;
-                const float ws = w * xs;
-                const int64_t rrow = (int64_t)(d0 + dd) * n_seg + j;
-                // first threshold above the lowest sky: an estimate good to 1e-2 bins, then exact
-                int n = (int)floorf(fmaf(Fq, (float)qmin, y0)) + 1;
-                int th = threshold(n);
-                if (th <= qmin) {
-                  th = threshold(++n);
-                } else {
-                  const int tl = threshold(n - 1);
-                  if (tl > qmin) {
-                    --n;
-                    th = tl;
-                  }
-                }
-                int K = base + n;   // the lowest sky's bin
-                const bool okK = K >= 0 && K + more_bins < n_bin;
-                bool step = th <= qmax;
-                bool okN = step && K + 1 >= 0 && K + 1 + more_bins < n_bin;
-                const float v0 = okK ? step_value<VK>(p, ev, rrow, K) : 0.f;
-                float vn = okN ? step_value<VK>(p, ev, rrow, K + 1) : 0.f;
-                int h0 = 0, l0 = 0;
+                const int nb = on ? min((int)(floorf(zh) - fl), kNThr - 1) : 0;
+                const float y1 = fl + 1.0f - y0;
+                const int K = base + (int)fl + 1;   // the lowest sky's bin
+                const int64_t vrow = vbase + (int64_t)(dd * n_seg + jr) * vpitch;
+                // the lookup's loads at once; the queue is drained while they are under way
+                const uint32_t* const tr = ev.tab + (rbase + rl) * nk;
+                const float per_unit = __int_as_float(m0.z);
+                const float v0 = on ? step_value<VK>(p, ev, vrow, K) : 0.f;
+                const float v1 = nb > 0 ? step_value<VK>(p, ev, vrow, K + 1) : 0.f;
+                float vn = nb > 1 ? step_value<VK>(p, ev, vrow, K + 2) : 0.f;
+                const int th0 = __float2int_rn(y1 * R);
+                int th = __float2int_rn((y1 + 1.0f) * R);
+                const uint32_t win0 = nb > 0 ? __ldg(tr + step_bucket(th0, m0.x, per_unit, nk)) : 0u;
+                uint32_t win = nb > 1 ? __ldg(tr + step_bucket(th, m0.x, per_unit, nk)) : 0u;
+                const float ws = __int_as_float(m0.w) * amp * xs;
+                if (cnt >= 32 || jb >= jn) drain();
+                int h0, l0, h1, l1;
                 to_fixed(v0, ws, h0, l0);
-                X0 += (long long)h0 * 65536 + l0;
-                if (okK) {
-                  if (p.amp_power > 0) {
-                    int wh, wl;
-                    to_fixed(w, ev.w1_scale, wh, wl);
-                    W1 += (long long)wh * 65536 + wl;
-                    to_fixed(w, w * ev.w2_scale, wh, wl);
-                    W2 += (long long)wh * 65536 + wl;
-                  } else {
-                    const longlong2 wi = *reinterpret_cast<const longlong2*>(meta + 2);
-                    W1 += wi.x;
-                    W2 += wi.y;
-                  }
+                if (on) X0 += (long long)h0 * 65536 + l0;
+                to_fixed(v1, ws, h1, l1);
+                {
+                  const unsigned vote = __ballot_sync(kAll, nb > 0);
+                  if (nb > 0)
+                    queue[cnt + __popc(vote & lt_mask)] =
+                        make_int4(th0, h1 - h0, (l1 - l0) * 8192 | tag, (int)(win0 | eps));
+                  cnt += __popc(vote);
                 }
-                bool ok0 = okK, any_edge = !okK;
-                for (int it = 0; it < kNThr && step; ++it) {
-                  // the step from bin K to K + 1 at threshold th; the next one's power is fetched ahead
-                  ++K;
-                  const int th1 = threshold(++n);
-                  const bool step1 = th1 <= qmax;
-                  const bool okN1 = step1 && K + 1 >= 0 && K + 1 + more_bins < n_bin;
-                  const float vn1 = okN1 ? step_value<VK>(p, ev, rrow, K + 1) : 0.f;
-                  const bool ok1 = okN;
-                  int h1, l1;
-                  to_fixed(vn, ws, h1, l1);
-                  const int dh = h1 - h0, dl = l1 - l0;
-                  const int we = (int)ok1 - (int)ok0;   // weight step at a band edge
-                  long long e1w = 0, e2w = 0;
-                  if (we) {
-                    any_edge = true;
-                    if (p.amp_power > 0) {
-                      int wh, wl;
-                      to_fixed(w, ev.w1_scale, wh, wl);
-                      e1w = we * ((long long)wh * 65536 + wl);
-                      to_fixed(w, w * ev.w2_scale, wh, wl);
-                      e2w = we * ((long long)wh * 65536 + wl);
-                    } else {
-                      const longlong2 wi = *reinterpret_cast<const longlong2*>(meta + 2);
-                      e1w = we * wi.x;
-                      e2w = we * wi.y;
-                    }
-                  }
-                  auto place = [&](int pos, bool plus) {
-                    const int cell = (pos << log_t) + lt;
-                    atomicAdd(chi + cell, plus ? dh : -dh);
-                    atomicAdd(clo + cell, plus ? dl : -dl);
-                    if (we) {
-                      unsigned long long* ec =
-                          reinterpret_cast<unsigned long long*>(edge + (int64_t)lt * (cpad + 1) + pos);
-                      atomicAdd(ec, (unsigned long long)(plus ? e1w : -e1w));
-                      atomicAdd(ec + 1, (unsigned long long)(plus ? e2w : -e2w));
-                    }
-                  };
-                  // the first block that reaches th, then every block until all later skies do
-                  const int2* const blk = reinterpret_cast<const int2*>(meta + kStepHead);
-                  int g = min((int)((float)((unsigned)th - (unsigned)qmin) * __int_as_float(m1.x)),
-                              cpad / kStepBlock - 1);
-                  int2 bk = __ldg(blk + g);
-                  if (bk.x < th) {
-                    do bk = __ldg(blk + ++g);
-                    while (bk.x < th);
-                  } else {
-                    while (g > 0) {
-                      const int2 pb = __ldg(blk + g - 1);
-                      if (pb.x < th) break;
-                      bk = pb;
-                      --g;
-                    }
-                  }
-                  const int4* qr = reinterpret_cast<const int4*>(
-                      ev.q + (row0 + (int64_t)j * p.n_det + d0 + dd) * cpad);
-                  unsigned below = 1;   // the sky before this block is below th
-                  while (true) {
-                    const int4 ua = __ldg(qr + 2 * g), ub = __ldg(qr + 2 * g + 1);
-                    const unsigned m = (unsigned)(ua.x >= th) | (unsigned)(ua.y >= th) << 1 |
-                                       (unsigned)(ua.z >= th) << 2 | (unsigned)(ua.w >= th) << 3 |
-                                       (unsigned)(ub.x >= th) << 4 | (unsigned)(ub.y >= th) << 5 |
-                                       (unsigned)(ub.z >= th) << 6 | (unsigned)(ub.w >= th) << 7;
-                    unsigned tr = (m ^ (m << 1 | (below ^ 1u))) & 0xffu;
-                    while (tr) {
-                      const int bit = __ffs(tr) - 1;
-                      place(kStepBlock * g + bit, (m >> bit) & 1u);
-                      tr &= tr - 1;
-                    }
-                    below = (m >> 7) ^ 1u;
-                    if (bk.y >= th) break;
-                    bk = __ldg(blk + ++g);
-                  }
-                  if (below) place(kStepBlock * (g + 1), true);
+                for (int i = 1;; ++i) {
+                  const unsigned vote = __ballot_sync(kAll, nb > i);
+                  if (!vote) break;
+                  if (cnt >= 32) drain();
                   h0 = h1;
                   l0 = l1;
-                  ok0 = ok1;
-                  th = th1;
-                  step = step1;
-                  okN = okN1;
-                  vn = vn1;
+                  to_fixed(vn, ws, h1, l1);
+                  if (nb > i)
+                    queue[cnt + __popc(vote & lt_mask)] =
+                        make_int4(th, h1 - h0, (l1 - l0) * 8192 | tag, (int)(win | (uint32_t)i << 22 | eps));
+                  cnt += __popc(vote);
+                  if (nb > i + 1) {
+                    vn = step_value<VK>(p, ev, vrow, K + i + 2);
+                    th = __float2int_rn((y1 + (float)(i + 1)) * R);
+                    win = __ldg(tr + step_bucket(th, m0.x, per_unit, nk));
+                  }
                 }
-                if (any_edge) {
-                  ++ngen;
-                  atomicOr(&s_edge, 1u << lt);
+                if (p.amp_power > 0 && on) {
+                  const float w = __int_as_float(m0.w) * amp;
+                  int wh, wl;
+                  to_fixed(w, ev.w1_scale, wh, wl);
+                  atomicAdd(tsum + 32 + lt, (unsigned long long)((long long)wh * 65536 + wl));
+                  to_fixed(w, w * ev.w2_scale, wh, wl);
+                  atomicAdd(tsum + 64 + lt, (unsigned long long)((long long)wh * 65536 + wl));
                 }
               }
+            }
+            __syncwarp();
+            {
+              // the list, and at the end of the turn every (template, row) of templates at a band edge
+              const int nr = (jn - j0) * DP;
+              const int n = nslow + (jb < jn || cnt > 0 ? 0 : __popc(at_edge & t_mask) * nr);
+              for (int i = lane; i < n; i += 32) {
+                int4 e = make_int4(0, 0, 0, -1);
+                if (i < nslow) {
+                  e = __ldcg(slow_list + i);
+                } else {
+                  const int r = (i - nslow) % nr;
+                  e.z = (r / DP * p.n_det + r % DP) << 5 | __fns(at_edge & t_mask, 0, (i - nslow) / nr + 1);
+                }
+                const int rl = (e.z >> 5) & 0xff, le = e.z & 31;
+                int only = -1;
+                if (e.w != -1) {
+                  const int32_t* const q = ev.q + (rbase + rl) * qs;
+                  const int from = e.w & 0x7ff, to = (e.w >> 11) & 0x7ff;
+                  const unsigned er = (unsigned)e.w >> 25 << p.eps_shift, lo = (unsigned)e.x - er;
+                  bool near = false;
+                  for (int k = from; k < to; ++k) near = near || (unsigned)__ldg(q + k) - lo <= 2u * er;
+                  if (near) {
+                    only = (e.w >> 22) & 7;
+                  } else {
+                    place_exact(q, (uint32_t)e.w & 0x3fffffu, e.x, [&](int pos, bool up) {
+                      int* const cell = chi + ((pos << (LT + 1)) + le);
+                      atomicAdd(cell, up ? e.y : -e.y);
+                      atomicAdd(cell + T, up ? e.z >> 13 : -(e.z >> 13));
+                    });
+                    continue;
+                  }
+                }
+                step_rare<VK, LT>(p, s_ctx, le, j0 + rl / p.n_det, d0 + rl % p.n_det, only);
+              }
+              nslow = 0;
+              __syncwarp();
+            }
+            } while (jb < jn || cnt > 0);
+            {
+              const int nr = (jn - j0) * DP;
+              if ((outside & t_mask) && p.amp_power == 0) {
+                // out of the band: the turn's weights come off
+                longlong2 wi = make_longlong2(0, 0);
+                if (lane < nr) {
+                  const float dth = __int_as_float(heads[lane * kStepHead + 1].x);
+                  if (dth == dth) wi = ev.wfix[(int64_t)(j0 + lane / DP) * p.n_det + d0 + lane % DP];
+                }
+                for (int off = 16; off > 0; off >>= 1) {
+                  wi.x += __shfl_xor_sync(kAll, wi.x, off);
+                  wi.y += __shfl_xor_sync(kAll, wi.y, off);
+                }
+                if (ls == 0 && ((outside >> lane) & 1u)) {
+                  atomicAdd(tsum + 32 + lt, (unsigned long long)-wi.x);
+                  atomicAdd(tsum + 64 + lt, (unsigned long long)-wi.y);
+                }
+              }
+              __syncwarp();
             }
           }
           if (jce < je) {
             // carry the low words over before they can overflow
             __syncthreads();
-            for (int i = tid; i < cells; i += kStepThreads) {
-              const int l = clo[i];
-              chi[i] += l >> 16;
-              clo[i] = l & 0xffff;
+            for (int i = tid; i < (cpad + 1) << LT; i += kStepThreads) {
+              const int c = i + (i >> LT << LT), l = clo[c];
+              chi[c] += l >> 16;
+              clo[c] = l & 0xffff;
             }
             __syncthreads();
           }
         }
         const bool last = pass == ev.passes - 1;
         if (last) {
-          for (int off = T; off < 32; off <<= 1) {
-            X0 += __shfl_xor_sync(0xffffffffu, X0, off);
-            W1 += __shfl_xor_sync(0xffffffffu, W1, off);
-            W2 += __shfl_xor_sync(0xffffffffu, W2, off);
-          }
-          if (ls == 0) {
-            atomicAdd(tsum + lt, (unsigned long long)X0);
-            atomicAdd(tsum + 32 + lt, (unsigned long long)W1);
-            atomicAdd(tsum + 64 + lt, (unsigned long long)W2);
-          }
+          for (int off = T; off < 32; off <<= 1) X0 += __shfl_xor_sync(0xffffffffu, X0, off);
+          if (ls == 0) atomicAdd(tsum + lt, (unsigned long long)X0);
         }
         __syncthreads();
 
-        // ---- prefix sums of the pass over its positions ----
-        const bool te = (s_edge >> t) & 1u;
-        {
-          long long sx = 0, s1 = 0, s2 = 0;
-          for (int q = p0; q < p1; ++q) {
-            const int c = (q << log_t) + t;
-            sx += (long long)chi[c] * 65536 + clo[c];
-            if (te) {
-              const longlong2 v = __ldcg(ecol + q);
-              s1 += v.x;
-              s2 += v.y;
-            }
-          }
-          part[tid] = sx;
-          part[kStepThreads + tid] = s1;
-          part[2 * kStepThreads + tid] = s2;
-        }
-        __syncthreads();
-        if (tid < 3 * 32) {
-          // exclusive scan over the pieces, one thread per (sum, template)
-          const int k = tid >> 5, tt = tid & 31;
-          if (tt < T) {
-            long long run = last ? (long long)tsum[k * 32 + tt] : 0;
-            for (int i = 0; i < pieces; ++i) {
-              long long* const q = part + k * kStepThreads + (i << log_t) + tt;
-              const long long v = *q;
-              *q = run;
-              run += v;
-            }
-          }
-        }
-        __syncthreads();
-        {
-          // Eq. 4: <s> = mq W1, sigma^2 = vq W2 (power: 1, 1; number count: q, q(1-q)),
-          // both doubled for two-bin lookups
-          const double nbins = two ? 2.0 : 1.0;
-          const bool count = VK == 2 && p.nc_q > 0.0;
-          const double mq = nbins * (count ? p.nc_q : 1.0);
-          const float vq = (float)(nbins * (count ? p.nc_q * (1.0 - p.nc_q) : 1.0));
-          const double m_units = mq * ev.w1_unit / ev.x_unit;   // mean of one W1 unit, in units of X
-          const float x_unit = (float)ev.x_unit;
-          const int64_t sky0 = (int64_t)item.y * ev.chunk;
-          const int rows = min(ev.chunk, ev.S - (int)sky0);
-          long long X = part[tid], w1 = part[kStepThreads + tid], w2 = part[2 * kStepThreads + tid];
-          // skies without band-edge steps share W1, W2 and the mean
-          long long mean = 0;
-          float W2f = 0.f, rs = 0.f;
-          auto moments = [&](long long a1, long long a2) {
-            mean = __double2ll_rn((double)a1 * m_units);
-            W2f = (float)((double)a2 * ev.w2_unit);
-            rs = W2f > 0.f ? rsqrtf(vq * W2f) : 0.f;
-          };
-          if (last) moments(w1, w2);
-          auto finish = [&](int sky, long long x, long long a1) {
-            // the cells' high words wrap at 2^31, so x is known modulo 2^48
-            const long long xs48 = (long long)((unsigned long long)x << 16) >> 16;
-            const int64_t o = (sky0 + sky) * ev.Bpad + b0 + t;
-            ev.psi[o] = W2f > 0.f ? (float)(xs48 - mean) * x_unit * rs : -INFINITY;
-            if (ev.S_out) {
-              ev.S_out[o] = (float)((double)xs48 * ev.x_unit);
-              ev.W1_out[o] = (float)((double)a1 * ev.w1_unit);
-              ev.W2_out[o] = W2f;
-            }
-          };
-          const int16_t* order = ev.order ? ev.order + ((int64_t)pass * ev.n_chunks + item.y) * cpad : nullptr;
-          for (int q = p0; q < p1; ++q) {
-            const int c = (q << log_t) + t;
-            X += (long long)chi[c] * 65536 + clo[c];
-            chi[c] = clo[c] = 0;
-            if (te) {
-              const longlong2 v = __ldcg(ecol + q);
-              __stcg(ecol + q, make_longlong2(0, 0));
-              w1 += v.x;
-              w2 += v.y;
-            }
-            if (q >= rows) continue;
-            if (!order) {
-              if (te) moments(w1, w2);
-              finish(q, X, w1);
-              continue;
-            }
-            // several passes: the sky's sums so far, kept by the sky's own index
-            const int sky = order[q];
-            const int a = (sky << log_t) + t;
-            long long x = X;
-            if (pass > 0) x += __ldcg(acc + a);
-            if (te) {
-              longlong2 v = __ldcg(edge_acc + a);
-              v.x += w1;
-              v.y += w2;
-              if (last) {
-                __stcg(edge_acc + a, make_longlong2(0, 0));
-                moments(v.x, v.y);
-                finish(sky, x, v.x);
-              } else {
-                __stcg(edge_acc + a, v);
-                __stcg(acc + a, x);
-              }
-            } else if (last) {
-              finish(sky, x, w1);
-            } else {
-              __stcg(acc + a, x);
-            }
-          }
-        }
+        step_fold<VK, LT>(p, s_ctx, smem, part, pass, last);
         // the cells past the last sky
         if (tid < T) {
-          const int c = (cpad << log_t) + tid;
+          const int c = (cpad << (LT + 1)) + tid;
           chi[c] = clo[c] = 0;
-          if ((s_edge >> tid) & 1u) __stcg(edge + (int64_t)tid * (cpad + 1) + cpad, make_longlong2(0, 0));
+          if ((s_ctx.edge_mask >> tid) & 1u) __stcg(edge + (int64_t)tid * (cpad + 1) + cpad, make_longlong2(0, 0));
         }
         __syncthreads();
       }
-      if (tid == 0) s_edge = 0;
-      if (tid < 32 * 4) tsum[tid] = 0;
+      if (tid < 32 * 3) tsum[tid] = tid < 32 ? 0 : s_wtot[tid / 32 - 1];
       __syncthreads();
     }
   }
-  if (ngen) atomicAdd(p.n_general, ngen);
+  __syncthreads();
+  if (tid == 0 && s_ctx.n_edge) atomicAdd(p.n_general, (unsigned long long)s_ctx.n_edge);
 }
 
-template <int VK, int DP, bool FAST>
+template <int VK, int DP, int LT>
 cudaError_t set_smem() {
   constexpr int kDevices = 64;
   static bool done[kDevices] = {};
@@ -688,47 +1027,47 @@ cudaError_t set_smem() {
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev >= 0 && dev < kDevices && done[dev]) return cudaSuccess;
-  e = cudaFuncSetAttribute(step_kernel<VK, DP, FAST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  e = cudaFuncSetAttribute(step_kernel<VK, DP, LT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)StepLayout(kStepCells + 32).total);
   if (e == cudaSuccess && dev >= 0 && dev < kDevices) done[dev] = true;
   return e;
 }
 
 struct Prepare {
-  template <int VK, int DP, bool FAST>
-  cudaError_t run() const { return set_smem<VK, DP, FAST>(); }
+  template <int VK, int DP, int LT>
+  cudaError_t run() const { return set_smem<VK, DP, LT>(); }
 };
 
 struct Launch {
   const StepParams& p;
   int cells, grid;
   cudaStream_t st;
-  template <int VK, int DP, bool FAST>
+  template <int VK, int DP, int LT>
   cudaError_t run() const {
-    cudaError_t e = set_smem<VK, DP, FAST>();
+    cudaError_t e = set_smem<VK, DP, LT>();
     if (e != cudaSuccess) return e;
-    step_kernel<VK, DP, FAST><<<grid, kStepThreads, StepLayout(cells).total, st>>>(p, cells);
+    step_kernel<VK, DP, LT><<<grid, kStepThreads, StepLayout(cells).total, st>>>(p, cells);
     return cudaGetLastError();
   }
 };
 
-template <int VK, int DP, typename F>
-cudaError_t pick_fast(bool fast, const F& f) {
-  return fast ? f.template run<VK, DP, true>() : f.template run<VK, DP, false>();
-}
-template <int DP, typename F>
-cudaError_t pick_value(bool half, bool general, bool fast, const F& f) {
-  if (general) return pick_fast<2, DP>(fast, f);
-  return half ? pick_fast<1, DP>(fast, f) : pick_fast<0, DP>(fast, f);
+template <int DP, int LT, typename F>
+cudaError_t pick_value(bool half, bool general, const F& f) {
+  if (general) return f.template run<2, DP, LT>();
+  return half ? f.template run<1, DP, LT>() : f.template run<0, DP, LT>();
 }
 template <typename F>
-cudaError_t pick(int dp, bool half, bool general, bool fast, const F& f) {
-  if (dp == 1) return pick_value<1>(half, general, fast, f);
-  if (dp == 2) return pick_value<2>(half, general, fast, f);
+cudaError_t pick(int dp, int log_t, bool half, bool general, const F& f) {
+  if (dp == 1 && log_t == 4) return pick_value<1, 4>(half, general, f);
+  if (dp == 1 && log_t == 5) return pick_value<1, 5>(half, general, f);
+  if (dp == 2 && log_t == 4) return pick_value<2, 4>(half, general, f);
+  if (dp == 2 && log_t == 5) return pick_value<2, 5>(half, general, f);
   return cudaErrorInvalidValue;
 }
 
 }  // namespace
+
+size_t step_slow_bytes(int grid) { return (size_t)grid * kStepWarps * kStepSlow * sizeof(int4); }
 
 StepScales step_scales(double vmax, double w_min, double w_max, double a_ref, int64_t n) {
   StepScales s;
@@ -747,27 +1086,46 @@ StepScales step_scales(double vmax, double w_min, double w_max, double a_ref, in
   return s;
 }
 
-int step_fast_track(const double* t_mid, int64_t n_seg, double T0, int tile, double tau_min, double r_max,
-                    double f_min, double df, int q_exp) {
-  // fixed-point words: thresholds in units of 2^-(q_exp + 8), 2^-(q_exp + 18) for the bin spacing
-  // df/f (f >= 64 bins for every lookup in the band)
-  if (!(f_min >= 72.0 * df) || q_exp > 45 || q_exp < 20) return 0;
-  double dmax = 0;
-  for (int64_t j0 = 0; j0 < n_seg; j0 += tile) {
-    const int64_t jn = std::min<int64_t>(tile, n_seg - j0);
-    const double ta = std::max(t_mid[j0 + (jn - 1) / 2], T0);
-    if (t_mid[j0 + jn - 1] < T0) continue;
-    dmax = std::max(dmax, std::max(std::fabs(t_mid[j0 + jn - 1] - ta), std::fabs(std::max(t_mid[j0], T0) - ta)) /
-                              (tau_min + (ta - T0)));
-  }
-  if (!(dmax <= 0.04) || !(r_max <= 1.0)) return 0;
-  auto term = [&](int k) {   // |C(r, k)| delta^k
+StepTrack step_track(const double* t_mid, int64_t n_seg, double T0, int most, double tau_min, double r_max,
+                     double x_max, double db, double f_min, double df, double inv_q) {
+  StepTrack r;
+  auto cbound = [&](int k) {   // |C(e, k)| for |e| <= r_max
     double c = 1.0;
-    for (int i = 0; i < k; ++i) c *= (r_max + i) / (i + 1) * dmax;
+    for (int i = 0; i < k; ++i) c *= (r_max + i) / (i + 1);
     return c;
   };
-  // the fp32 terms' rounding and the first dropped term below a quarter unit of 2^-52
-  return term(5) < std::ldexp(1.0, -30) && term(kFastTerms + 1) < std::ldexp(1.0, -54) ? 1 : 0;
+  for (int shift = ilog2(most); shift >= 2; --shift) {
+    const int tile = 1 << shift;
+    double dmax = 0;   // |t - t_a| / (tau + t_a - T0)
+    for (int64_t j0 = 0; j0 < n_seg; j0 += tile) {
+      const int64_t jn = std::min<int64_t>(tile, n_seg - j0);
+      const double ta = std::max(t_mid[j0 + (jn - 1) / 2], T0), te = t_mid[j0 + jn - 1];
+      if (te < T0) continue;
+      dmax = std::max(dmax, std::max(te - ta, ta - std::max(t_mid[j0], T0)) / (tau_min + (ta - T0)));
+    }
+    // the series' dropped terms and the fp32 rounding of its cubic part, in bins
+    if (!(dmax <= 0.1) || x_max * cbound(3) * std::pow(dmax, 3) > 0.15 ||
+        x_max * cbound(kStepTerms + 3) * std::pow(dmax, kStepTerms + 3) > 2e-8 || x_max * r_max * dmax > 2.0e6)
+      continue;
+    r.nterms = series_terms_for(t_mid, n_seg, T0, tile, tau_min, r_max);
+    if (r.nterms < 1) continue;
+    r.shift = shift;
+    // Error of an fp32 threshold: the position's sums (values up to 2) and the
+    // cubic part 3e-7, the difference to the boundary 1.2e-7 (1 + y), and four
+    // roundings of 6e-8 of y (F, 1/F, their products) for y = db + 1 bins
+    // at most; emulated worst cases stay below 0.7 of it.
+    r.eps = (float)(3.0e-7 + 1.2e-7 * (2.0 + db) + 2.4e-7 * (1.0 + db));
+    // in grid units (most at the lowest frequency): 7 bits of 2^eps_shift units
+    const double f_low = std::max(f_min / df - 8.0, 0.0);
+    if (!(f_low >= 64.0)) return r;
+    const double worst = r.eps * inv_q / f_low;
+    while (std::ldexp(worst, -r.eps_shift) > 120.0) ++r.eps_shift;
+    if (r.eps_shift > 20) return r;
+    r.eps_max = (int)std::ldexp(std::ceil(std::ldexp(worst, -r.eps_shift)) + 2.0, r.eps_shift);
+    r.ok = true;
+    return r;
+  }
+  return r;
 }
 
 StepGeometry step_geometry(int64_t S, int D, int64_t n_seg, int tile, const double* v, bool split) {
@@ -815,7 +1173,9 @@ StepGeometry step_geometry(int64_t S, int D, int64_t n_seg, int tile, const doub
       if (half * worst <= kPlaces) break;
     }
   }
-  const int64_t L = ((n_seg + runs - 1) / runs + tile - 1) / tile * tile;
+  // whole rounds of the 32 warps' turns of 16 segments where a pass is long enough
+  const int unit = n_seg / runs >= 512 ? 512 : tile;
+  const int64_t L = std::max<int64_t>(1, ((n_seg + runs - 1) / runs + unit / 2) / unit) * unit;
   g.pass_seg = (int)std::min<int64_t>(L, INT32_MAX / 2);
   g.passes = (int)((n_seg + g.pass_seg - 1) / g.pass_seg) * (D / g.dets_per_pass);
   return g;
@@ -842,16 +1202,24 @@ cudaError_t launch_absmax(const void* rho, bool half, int64_t n, unsigned* out, 
   return cudaGetLastError();
 }
 
-cudaError_t step_prepare(int dets_per_pass, bool half, bool general, bool fast) {
-  return pick(dets_per_pass, half, general, fast, Prepare{});
+cudaError_t step_prepare(int dets_per_pass, int log_t, bool half, bool general) {
+  return pick(dets_per_pass, log_t, half, general, Prepare{});
 }
 
-cudaError_t launch_step(const StepParams& p, int dets_per_pass, bool half, bool general, bool fast, int cells,
+cudaError_t launch_step(const StepParams& p, int dets_per_pass, int log_t, bool half, bool general, int cells,
                         int grid, cudaStream_t st) {
-  if (p.n_det < 1 || p.n_det % dets_per_pass || cells > kStepCells + 32 || (!fast && p.nterms < 1))
+  if (p.n_det < 1 || p.n_det % dets_per_pass || cells > kStepCells + 32 || p.nterms < 1)
     return cudaErrorInvalidValue;
   if (grid <= 0) return cudaSuccess;
-  return pick(dets_per_pass, half, general, fast, Launch{p, cells, grid, st});
+  return pick(dets_per_pass, log_t, half, general, Launch{p, cells, grid, st});
+}
+
+cudaError_t launch_step_tiles(const StepTileParams& p, cudaStream_t st) {
+  const int threads = 128;
+  const int64_t total = (int64_t)p.a.Bpad * ((p.a.n_tiles + kAnchorRun - 1) / kAnchorRun);
+  if (total == 0) return cudaSuccess;
+  step_tile_kernel<<<(unsigned)((total + threads - 1) / threads), threads, 0, st>>>(p);
+  return cudaGetLastError();
 }
 
 }  // namespace tcw

@@ -28,24 +28,41 @@ constexpr int kStepCells = 16384;      // difference cells of a CTA: chunk x tem
 // Doppler factors stay (almost) sorted.  Doppler rows: one per (chunk, segment,
 // detector), cpad skies in the order of their pass (a multiple of kStepBlock;
 // the last sky repeated):
-//   q     [cpad]  floor(v.nhat/c / q-grid step)
-//   meta  {qmin, qmax, dt hi, dt lo}: smallest and largest q; t_j - t_a from
-//         the tile's anchor time as an fp32 pair (NaN before T0)
-//         {blocks per grid unit (float bits), w (float bits), 0, 0}
-//         {W1 word, W2 word}: w and w^2 in fixed point (int64 each),
-//         then per block g {largest q of blocks 0..g, smallest q of blocks
-//         g+1.. (INT_MAX after the last)} as int2
+//   q     [step_row(cpad)]  floor(v.nhat/c / q-grid step), then the largest repeated
+//   head  {qmin, qmax, buckets per grid unit (float bits), w (float bits)}: the
+//         smallest and largest q; {dt hi, dt lo, dt^2 hi, dt^2 lo}: t_j - t_a from
+//         the tile's anchor time and its square as fp32 pairs (dt hi NaN before T0)
+//   wfix  {W1 word, W2 word}: w and w^2 in fixed point (int64 each)
+//   tab   per bucket of thresholds {first position not below all of them, first
+//         position from which on every sky reaches all of them}, 11 bits each:
+//         only the skies between the two are compared with a threshold
+// Track constants of one (template, tile), the position x = (f - f_min)/df of
+// the unshifted track (Eq. 1) around the anchor time t_a: x = base + frac +
+// A dt + Q dt^2 + X (cubic and higher terms in dt s).
+struct __align__(16) StepTile {
+  int base;
+  float frac, A_hi, A_lo, Q_hi, Q_lo;
+  float X;   // f_a / df
+  float s;   // 1 / (tau + t_a - T0)
+};
+static_assert(sizeof(StepTile) == 32, "two 16-byte loads");
+
 struct StepEvent {
   const void* rho;           // [D][n_seg][n_bin]
   const uint32_t* bits;      // number count: bit map (see EventDesc), else null
   const double* t_mid;
-  const double* anchors;     // [Bpad][n_tiles][2]
+  const double* anchors;     // [Bpad][n_tiles][2] (exact thresholds)
+  const StepTile* tiles;     // [Bpad][n_tiles]
   const double* f0;          // sorted bank [Bpad]
   const double* nbr;
-  const int32_t* q;          // [n_chunks][n_seg][D][cpad]
-  const int4* meta;          // [n_chunks][n_seg][D][step_meta(cpad)]
+  const int32_t* q;          // [n_chunks][n_seg][D][step_row(cpad)]
+  const int4* head;          // [n_chunks][n_seg][D][kStepHead]
+  const uint32_t* tab;       // [n_chunks][n_seg][D][step_buckets(cpad)]
+  const longlong2* wfix;     // [n_seg][D]
+  const long long* wtot;     // [kStepSlots][2]: partial sums of w and w^2 over the segments from T0 on
   const int16_t* order;      // [passes][n_chunks][cpad] sky (in the chunk) at a position; null for one pass
                              // in the sorted order itself
+  const int16_t* remap;      // [passes][n_chunks][cpad] that sky's position in the pass before
   float* psi;                // [>= S][Bpad]
   float* S_out;              // optional
   float* W1_out;
@@ -58,6 +75,7 @@ struct StepEvent {
   int bit_pitch;
   int chunk, cpad, log_t;    // skies per chunk, of a row; templates of a block: 1 << log_t
   int n_chunks, pass_seg, passes;
+  int sub_shift;             // segments of one warp's turn: 1 << sub_shift <= 16 and <= tile
 };
 
 struct StepParams {
@@ -69,17 +87,19 @@ struct StepParams {
   unsigned* next;            // item counter, zero at launch
   int64_t n_bin;
   double f_min, df, inv_q;
-  float q;
-  int q_exp;                 // q = 2^-q_exp
+  float q, inv_q_f;
+  float eps;                 // bound of the fp32 thresholds' error, in bins
+  float eps_scale;           // the same as a count of 2^eps_shift grid units, per (1/F)/q
+  int eps_shift;
   int nterms, tile_shift;    // FP64 track series (> 0), anchor tiles
-  int sub_shift;             // segments of one warp's turn: 1 << sub_shift <= tile
+  float df_f;
   int amp_power;
   double nc_q;               // number count: q = exp(-rho_th), else 0
   int track_bins;
   int map_half;
-  long long* acc;            // [grid][kStepCells]: sums of the finished passes (several passes only)
-  longlong2* edge;           // [grid][2 kStepCells + 32]: W1, W2 steps at band edges and their sums over
-                             // the finished passes, zero between launches
+  int4* slow;                // [grid][step_slow_bytes(1)]: the warps' lists of steps left for later
+  longlong2* edge;           // [grid][2 kStepCells + 32]: W1, W2 steps at band edges (zero between
+                             // launches), and room to reorder them
   unsigned long long* n_general;
 };
 
@@ -92,14 +112,23 @@ struct StepRowsParams {
   int n_det, n_seg, S, chunk, cpad, n_chunks, tile_shift;
   int dets_per_pass, pass_seg, passes;
   double inv_q;
+  int eps_max;               // largest error of an fp32 threshold, in grid units
   double w1_scale, w2_scale; // 1 / w1_unit, 1 / w2_unit
-  int16_t* order;            // written first when not null (see StepEvent)
+  int16_t* order;            // written first when not null, with remap (see StepEvent)
+  int16_t* remap;
   int32_t* q;
-  int4* meta;
+  int4* head;
+  uint32_t* tab;
+  longlong2* wfix;
+  unsigned long long* wtot;  // zero at launch
 };
 
-constexpr int kStepHead = 3;   // int4 words of a row's meta before its blocks
-__host__ __device__ constexpr int step_meta(int cpad) { return kStepHead + (cpad / kStepBlock + 1) / 2; }
+// Row length: the skies and a block past the end, so that any four from a sky on can be read.
+__host__ __device__ constexpr int step_row(int cpad) { return cpad + kStepBlock; }
+constexpr int kStepHead = 2;     // int4 words of a row's head
+constexpr int kStepSlots = 64;   // partial weight sums of an event
+// Two buckets of thresholds per sky: about half a sky is left to compare per threshold.
+__host__ __device__ constexpr int step_buckets(int cpad) { return 2 * cpad; }
 
 // Chunks of an event's sorted skies: the fewest chunks of at most
 // kStepMaxChunk skies, of nearly equal size; 32 templates per block while the
@@ -128,10 +157,32 @@ inline void set_step_geometry(StepRowsParams& p, const StepGeometry& g) {
 }
 inline bool step_ordered(const StepGeometry& g) { return g.passes > 1; }
 
-// 1 when the in-kernel fp32-pair track series (t - t_a at tiles of `tile`
-// segments) is as accurate as the FP64 one for every template and lookup.
-int step_fast_track(const double* t_mid, int64_t n_seg, double T0, int tile, double tau_min, double r_max,
-                    double f_min, double df, int q_exp);
+// The fp32 track's tiles and error bound: tile = 1 << shift segments (at most
+// `most`), the FP64 series' terms, and the thresholds' error; ok = false when no
+// tile keeps it.  x_max: largest f/df; db: largest Doppler shift in bins.
+struct StepTrack {
+  bool ok = false;
+  int shift = 0, nterms = 0;
+  float eps = 0;             // bins
+  int eps_shift = 0, eps_max = 0;
+};
+StepTrack step_track(const double* t_mid, int64_t n_seg, double T0, int most, double tau_min, double r_max,
+                     double x_max, double db, double f_min, double df, double inv_q);
+inline void set_step_track(StepParams& p, const StepTrack& t) {
+  p.eps = t.eps;
+  p.eps_shift = t.eps_shift;
+  p.eps_scale = std::ldexp(t.eps, -t.eps_shift);
+  p.nterms = t.nterms;
+  p.tile_shift = t.shift;
+}
+
+// Tile anchors and track constants of one event for every sorted template.
+struct StepTileParams {
+  AnchorParams a;            // as for launch_anchors
+  double f_min, df;
+  StepTile* tiles;
+};
+cudaError_t launch_step_tiles(const StepTileParams& p, cudaStream_t st);
 
 // Fixed-point scales of one event, or ok = false when the sums would not be
 // at least as accurate as fp32 partial sums (see step_scales).
@@ -152,20 +203,30 @@ inline void set_step_scales(StepEvent& e, const StepScales& s) {
   e.w1_scale = std::ldexp(1.0f, s.w1 - 16);
   e.w2_scale = std::ldexp(1.0f, s.w2 - 16);
 }
-// Segments of one warp's turn (as a shift): a whole tile where the event has
-// several tiles per warp, else 8 segments so that short events use every warp.
-inline int step_sub_shift(int64_t n_seg, int tile_shift) {
-  return n_seg >= (int64_t)4 * 32 << tile_shift ? tile_shift : 3;
+// Segments of one warp's turn (as a shift): the longest run, a whole tile or
+// less, that leaves few of the 32 warps idle in a pass's last round of turns.
+inline int step_sub_shift(const StepGeometry& g, int64_t n_seg, int tile_shift) {
+  const int64_t len = n_seg < g.pass_seg ? n_seg : g.pass_seg;
+  int best = tile_shift < 3 ? tile_shift : 3;
+  double best_busy = 0;
+  for (int s = tile_shift < 4 ? tile_shift : 4; s >= 3; --s) {
+    const double turns = (double)((len + (1 << s) - 1) >> s), busy = turns / (std::ceil(turns / 32.0) * 32.0);
+    if (busy > best_busy + 0.05) {
+      best = s;
+      best_busy = busy;
+    }
+  }
+  return best;
 }
 inline int step_cells(const StepGeometry& g) { return (g.cpad + 1) << g.log_t; }
+size_t step_slow_bytes(int grid);
 inline size_t step_edge_bytes(int grid) { return (size_t)grid * (2 * kStepCells + 32) * sizeof(longlong2); }
-inline size_t step_acc_bytes(int grid) { return (size_t)grid * kStepCells * sizeof(long long); }
 cudaError_t launch_step_rows(const StepRowsParams& p, cudaStream_t st);
 // Raises the kernel's shared-memory limit (also done at its first launch; call before a graph capture).
-cudaError_t step_prepare(int dets_per_pass, bool half, bool general, bool fast);
-// general: number count or two-bin lookups; fast: step_fast_track held for every event; cells: the
-// largest step_cells of the items' events, whose passes all take dets_per_pass detectors.
-cudaError_t launch_step(const StepParams& p, int dets_per_pass, bool half, bool general, bool fast, int cells,
+cudaError_t step_prepare(int dets_per_pass, int log_t, bool half, bool general);
+// general: number count or two-bin lookups; cells: the largest step_cells of the items' events,
+// which all have this log_t and passes of dets_per_pass detectors.
+cudaError_t launch_step(const StepParams& p, int dets_per_pass, int log_t, bool half, bool general, int cells,
                         int grid, cudaStream_t st);
 // *out = bits of the largest |rho| (NaN above infinity above every finite value); out zero at launch.
 cudaError_t launch_absmax(const void* rho, bool half, int64_t n, unsigned* out, cudaStream_t st);

@@ -106,3 +106,27 @@ def test_infinite_powers_stay_with_their_lookups():
     assert sel.sum() > 0.9 * fin.sum()
     assert np.all(np.abs(st["S"][sel] - S[sel]) <= 1e-5 * S[sel] + 1e-6)
     assert not np.isfinite(st["S"][~fin]).any()
+
+
+def test_skies_at_a_bin_boundary_take_the_exact_thresholds():
+    """Detectors at rest and a bank of constant frequencies on bin edges and a few
+    ulp around them: every lookup lies within the error of the fp32 thresholds."""
+    p = problem(800, 2, 70, 20, 64, weights=True)
+    p.velocity[:] = 0.0
+    p.bank.tau[:] = 1e12
+    p.bank.n[:] = 3.0
+    e = p.f_min + (np.arange(64) * 11 + 40.5) * p.df
+    p.bank.f0[:] = e * (1.0 + (np.arange(64) % 9 - 4) * 1e-8)
+    check(p)
+
+
+def test_long_sfts_take_short_tiles():
+    # 32 s segments at 500-1250 Hz: up to 2.4 bins of Doppler shift, five boundaries per lookup
+    r = syn.rng(900)
+    t = syn.segment_times(90, 32.0)
+    dets = syn.random_detectors(r, 2)
+    vel = np.stack([d.velocity(t) for d in dets])
+    bank = syn.random_bank(r, 60, f0_range=(505.0, 745.0), tau_range=(3500, 35000))
+    p = syn.Problem(syn.exponential_noise(r, (2, 90, 8000)), t, syn.uniform_weights(r, 2, 90), vel, 500.0, 1 / 32.0,
+                    float(t[0] - 16.0), syn.random_sky(r, 300), bank, [], dets, name="32 s")
+    check(p)

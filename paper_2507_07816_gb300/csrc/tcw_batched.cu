@@ -39,6 +39,11 @@ struct EventHost {
   size_t o_anchor = 0, o_psi = 0;  // byte offsets in the wave buffers
   int64_t out_row = 0;             // first output row (sum of earlier events' n_sky)
   int wave = 0;
+  // step-function search (tcw_step.cuh)
+  float w_min = 0, w_max = 0, map_max = 0;   // smallest nonzero and largest weight, largest |rho|
+  StepGeometry geo{};
+  StepScales scales;
+  size_t o_q = 0, o_head = 0, o_tab = 0, o_wfix = 0, o_wtot = 0, o_order = 0;   // byte offsets of its Doppler rows
   // a triaged batch's event: its chosen skies (sorted, with their caller
   // indices within the event) and its template regions (a sub-bank); null
   // pointers / 0 sizes: the event's own sky at o_nhat / o_perm, the context's bank
@@ -80,6 +85,13 @@ struct BatchState {
   std::vector<int> wave_items;     // item offset of each wave in `items`, plus the end
   std::vector<int> wave_cta;       // offset (in ints) of each wave's CTA table
   int64_t lookups = 0;
+  // step-function search: every event meets its conditions (else the group kernel)
+  bool step = false;
+  StepTrack track;
+  int dets_per_pass = 1;
+  DevBuf rows, tiles;              // Doppler rows of every event; track constants of a wave
+  size_t wtot_bytes = 0;           // the events' weight sums, at the start of `rows`
+  std::vector<int> wave_split;     // per wave: items of the events with 32 templates per block, then 16
   // autotuner
   bool tuned = false;
   int64_t tune_key[4] = {-1, -1, -1, -1};
@@ -105,7 +117,7 @@ namespace {
 // arrays, bit maps and outputs.
 void release_batch(BatchState* b, bool shared) {
   if (b->exec) cudaGraphExecDestroy(b->exec);
-  DevBuf* own[] = {&b->blk, &b->anchors, &b->psi, &b->evtab, &b->items, &b->dev, &b->flags, &b->sub};
+  DevBuf* own[] = {&b->rows, &b->tiles, &b->blk, &b->anchors, &b->psi, &b->evtab, &b->items, &b->dev, &b->flags, &b->sub};
   for (DevBuf* d : own) d->release();
   if (!shared) {
     DevBuf* bufs[] = {&b->rho, &b->small, &b->out_psi, &b->out_idx, &b->bits};
@@ -206,8 +218,81 @@ tcw_status plan_batch(tcw_ctx* c, BatchState* b) {
   for (const EventHost& e : b->ev) b->lookups += e.n_sky * ev_B(c, e) * b->D * e.n_seg;
   TCW_CUDA(c, group_grid(&b->grid), "device query");
   TCW_CUDA(c, b->dev.ensure(group_dev_elems(b->grid) * sizeof(float2)), "scratch");
+  TCW_CUDA(c, ensure_step_edge(c->step_edge, b->grid, c->stream), "scratch");
+  TCW_CUDA(c, c->step_slow.ensure(step_slow_bytes(b->grid)), "scratch");
   b->planned = true;
   return TCW_OK;
+}
+
+// The step-function search for tiles of at most `tile` segments: its track and
+// tile length (common to the batch), every event's scales and passes.  b->step =
+// false when some event does not meet its conditions.
+void plan_step(const tcw_ctx* c, BatchState* b, int tile) {
+  b->step = false;
+  const bool count = c->statistic == TCW_STAT_NUMBER_COUNT;
+  const double f_top = b->f_min + (double)b->n_bin * b->df;
+  b->track = StepTrack{};
+  b->track.shift = ilog2(tile);
+  for (int round = 0; round < 2; ++round) {
+    // the shortest tile that an event needs, then every event with it
+    const int most = 1 << b->track.shift;
+    StepTrack all;
+    all.shift = b->track.shift;
+    for (const EventHost& e : b->ev) {
+      const StepTrack t = step_track(e.t.data(), e.n_seg, e.T0, most, c->bank_tau_min, c->bank_r_max,
+                                     c->bank_f0max / b->df, b->doppler_bins, b->f_min, b->df, b->inv_q);
+      if (!t.ok || (round == 1 && t.shift != b->track.shift)) return;
+      all.shift = std::min(all.shift, t.shift);
+      all.nterms = std::max(all.nterms, t.nterms);
+      all.eps = t.eps;
+      all.eps_shift = t.eps_shift;
+      all.eps_max = t.eps_max;
+    }
+    b->track = all;
+  }
+  const int step_tile = 1 << b->track.shift;
+  bool split = false;
+  for (int round = 0; round < 2; ++round) {
+    b->dets_per_pass = b->D;
+    for (EventHost& e : b->ev) {
+      e.geo = step_geometry(e.n_sky, b->D, e.n_seg, step_tile, e.v.data(), split);
+      b->dets_per_pass = std::min(b->dets_per_pass, e.geo.dets_per_pass);
+    }
+    if (b->dets_per_pass == b->D || split) break;
+    split = true;   // some event takes its detectors one by one: all of them do
+  }
+  for (EventHost& e : b->ev) {
+    e.scales = step_scales((count ? 1.0 : (double)e.map_max) * c->track_bins, e.w_min, e.w_max,
+                           step_amp_ref(c->amp_power, e.t, e.T0, c->bank_tau_min, c->bank_r_max, f_top, c->bank_f0max),
+                           (int64_t)b->D * e.n_seg);
+    if (!e.scales.ok) return;
+  }
+  b->track.ok = true;
+  b->step = true;
+}
+
+// Offsets of the Doppler rows of every event in b->rows; returns their size.
+size_t layout_rows(BatchState* b) {
+  size_t o = 0;
+  for (EventHost& e : b->ev) {
+    e.o_wtot = o;
+    o += kStepSlots * 16;
+  }
+  b->wtot_bytes = o;
+  auto take = [&](size_t n) {
+    const size_t at = o;
+    o += align256(n);
+    return at;
+  };
+  for (EventHost& e : b->ev) {
+    const size_t rows = (size_t)e.geo.n_chunks * e.n_seg * b->D;
+    e.o_q = take(rows * step_row(e.geo.cpad) * sizeof(int32_t));
+    e.o_head = take(rows * kStepHead * sizeof(int4));
+    e.o_tab = take(rows * step_buckets(e.geo.cpad) * sizeof(uint32_t));
+    e.o_wfix = take((size_t)e.n_seg * b->D * sizeof(longlong2));
+    e.o_order = step_ordered(e.geo) ? take((size_t)e.geo.passes * e.geo.n_chunks * e.geo.cpad * 2 * sizeof(int16_t)) : 0;
+  }
+  return o;
 }
 
 int batch_series_terms(const tcw_ctx* c, const BatchState* b, int tile) {
@@ -223,8 +308,9 @@ int batch_series_terms(const tcw_ctx* c, const BatchState* b, int tile) {
 
 int n_tiles_of(int64_t n_seg, int tile) { return (int)((n_seg + tile - 1) / tile); }
 
-// Split the events into waves whose Psi and anchor buffers fit `budget` bytes
-// and lay out those buffers.  Returns the per-wave buffer sizes.
+// Split the events into waves whose Psi and anchor buffers (with the track
+// constants of a step-function search) fit `budget` bytes and lay out those
+// buffers.  Returns the per-wave buffer sizes.
 void layout_waves(const tcw_ctx* c, BatchState* b, int tile, bool anchors, size_t* psi_bytes,
                   size_t* anchor_bytes) {
   const size_t budget = (size_t)c->batch_memory;
@@ -233,7 +319,8 @@ void layout_waves(const tcw_ctx* c, BatchState* b, int tile, bool anchors, size_
   for (EventHost& e : b->ev) {
     const size_t p = align256((size_t)e.Spad * ev_Bpad(c, e) * 4);
     const size_t a = anchors ? align256((size_t)ev_Bpad(c, e) * n_tiles_of(e.n_seg, tile) * 16) : 0;
-    if ((psi_w + anc_w) > 0 && psi_w + anc_w + p + a > budget) {
+    const size_t f = b->step ? 1 + sizeof(StepTile) / 16 : 1;   // anchor and track constants per tile
+    if ((psi_w + anc_w) > 0 && psi_w + f * anc_w + p + f * a > budget) {
       ++wave;
       psi_w = anc_w = 0;
     }
@@ -248,6 +335,67 @@ void layout_waves(const tcw_ctx* c, BatchState* b, int tile, bool anchors, size_
   b->waves = wave + 1;
   *psi_bytes = psi_max;
   *anchor_bytes = anc_max;
+}
+
+// An event's Doppler rows, and what the search reads of it.
+StepRowsParams step_rows_of(BatchState* b, const EventHost& e) {
+  StepRowsParams rp{};
+  rp.vel = at<double>(b->small, e.o_v);
+  rp.nhat = ev_nhat(b, e);
+  rp.weights = at<float>(b->small, e.o_w);
+  rp.t_mid = at<double>(b->small, e.o_t);
+  rp.T0 = e.T0;
+  rp.n_det = b->D;
+  rp.n_seg = (int)e.n_seg;
+  rp.S = (int)e.n_sky;
+  set_step_geometry(rp, e.geo);
+  rp.tile_shift = b->track.shift;
+  rp.inv_q = b->inv_q;
+  rp.eps_max = b->track.eps_max;
+  rp.w1_scale = std::ldexp(1.0, e.scales.w1);
+  rp.w2_scale = std::ldexp(1.0, e.scales.w2);
+  if (step_ordered(e.geo)) {
+    rp.order = at<int16_t>(b->rows, e.o_order);
+    rp.remap = rp.order + (size_t)e.geo.passes * e.geo.n_chunks * e.geo.cpad;
+  }
+  rp.q = at<int32_t>(b->rows, e.o_q);
+  rp.head = at<int4>(b->rows, e.o_head);
+  rp.tab = at<uint32_t>(b->rows, e.o_tab);
+  rp.wfix = at<longlong2>(b->rows, e.o_wfix);
+  rp.wtot = at<unsigned long long>(b->rows, e.o_wtot);
+  return rp;
+}
+
+StepEvent step_event(const tcw_ctx* c, BatchState* b, const EventHost& e) {
+  const StepRowsParams rp = step_rows_of(b, e);
+  StepEvent d{};
+  d.rho = at<char>(b->rho, e.o_rho);
+  if (c->statistic == TCW_STAT_NUMBER_COUNT) {
+    d.bits = at<uint32_t>(b->bits, e.o_bits);
+    d.bit_pitch = bit_pitch_for(b->n_bin);
+  }
+  d.t_mid = rp.t_mid;
+  d.anchors = at<double>(b->anchors, e.o_anchor);
+  d.tiles = at<StepTile>(b->tiles, e.o_anchor / 16 * sizeof(StepTile));
+  d.f0 = ev_f0(c, e);
+  d.nbr = ev_nbr(c, e);
+  d.q = rp.q;
+  d.head = rp.head;
+  d.tab = rp.tab;
+  d.wfix = rp.wfix;
+  d.wtot = reinterpret_cast<const long long*>(rp.wtot);
+  d.order = rp.order;
+  d.remap = rp.remap;
+  d.psi = at<float>(b->psi, e.o_psi);
+  d.T0 = e.T0;
+  set_step_scales(d, e.scales);
+  d.n_seg = (int)e.n_seg;
+  d.n_tiles = n_tiles_of(e.n_seg, 1 << b->track.shift);
+  d.S = (int)e.n_sky;
+  d.Bpad = ev_Bpad(c, e);
+  set_step_geometry(d, e.geo);
+  d.sub_shift = step_sub_shift(e.geo, e.n_seg, b->track.shift);
+  return d;
 }
 
 EventDesc make_desc(const tcw_ctx* c, BatchState* b, const EventHost& e, int tile, bool anchors) {
@@ -303,6 +451,32 @@ tcw_status ensure_batch_bits(tcw_ctx* c, BatchState* b) {
   return TCW_OK;
 }
 
+// Work items of the step-function search of wave w over the first `tmpl_limit`
+// templates, bank_chunk template blocks per item, longest first: the events with
+// 32 templates per block, then (from *split on) those with 16.
+void wave_step_items(const tcw_ctx* c, const BatchState* b, int w, int bank_chunk, int tmpl_limit,
+                     std::vector<int4>& order, int* split, int64_t* sums) {
+  *sums = 0;
+  order.clear();
+  for (int lt : {5, 4}) {
+    if (lt == 4) *split = (int)order.size();
+    std::vector<int4> items;
+    for (size_t i = 0; i < b->ev.size(); ++i) {
+      const EventHost& e = b->ev[i];
+      if (e.wave != w || e.geo.log_t != lt) continue;
+      const int blocks = std::min(tmpl_limit, ev_Bpad(c, e)) >> lt;
+      for (int g0 = 0; g0 < blocks; g0 += bank_chunk)
+        for (int ch = 0; ch < e.geo.n_chunks; ++ch)
+          items.push_back(make_int4((int)i, ch, g0 << lt, std::min(bank_chunk, blocks - g0)));
+      *sums += ((int64_t)blocks << lt) * e.n_sky * b->D * e.n_seg;
+    }
+    std::stable_sort(items.begin(), items.end(), [&](const int4& x, const int4& y) {
+      return x.w * b->ev[x.x].n_seg > y.w * b->ev[y.x].n_seg;
+    });
+    order.insert(order.end(), items.begin(), items.end());
+  }
+}
+
 // Work items of the events of wave w over `groups_limit` groups of 8
 // templates, bank_chunk groups per item, scheduled longest-first.
 void wave_items(const tcw_ctx* c, const BatchState* b, int w, int bank_chunk, int groups_limit,
@@ -352,24 +526,49 @@ GroupParams base_params(const tcw_ctx* c, BatchState* b, int tile, int nterms) {
 }
 
 // Buffers and event table for (tile, anchors); items are uploaded by the caller.
+// Decides whether the step-function search runs.
 tcw_status prepare_shape(tcw_ctx* c, BatchState* b, int tile, int nterms) {
   size_t psi_bytes = 0, anc_bytes = 0;
-  layout_waves(c, b, tile, nterms > 0, &psi_bytes, &anc_bytes);
+  plan_step(c, b, tile);
+  if (b->step) {
+    layout_waves(c, b, 1 << b->track.shift, true, &psi_bytes, &anc_bytes);
+    TCW_CUDA(c, b->rows.ensure(layout_rows(b)), "doppler rows");
+    TCW_CUDA(c, b->tiles.ensure(anc_bytes / 16 * sizeof(StepTile)), "track tiles");
+  } else {
+    layout_waves(c, b, tile, nterms > 0, &psi_bytes, &anc_bytes);
+  }
   TCW_CUDA(c, b->psi.ensure(psi_bytes), "Psi buffer");
-  if (nterms > 0) TCW_CUDA(c, b->anchors.ensure(anc_bytes), "anchor buffer");
+  if (b->step || nterms > 0) TCW_CUDA(c, b->anchors.ensure(anc_bytes), "anchor buffer");
   std::vector<EventDesc> tab;
-  for (const EventHost& e : b->ev) tab.push_back(make_desc(c, b, e, tile, nterms > 0));
-  TCW_CUDA(c, b->evtab.ensure(tab.size() * sizeof(EventDesc)), "event table");
-  TCW_CUDA(c, cudaMemcpyAsync(b->evtab.p, tab.data(), tab.size() * sizeof(EventDesc), cudaMemcpyHostToDevice,
-                              c->stream), "event table");
+  std::vector<StepEvent> stab;
+  for (const EventHost& e : b->ev) {
+    if (b->step) stab.push_back(step_event(c, b, e));
+    else tab.push_back(make_desc(c, b, e, tile, nterms > 0));
+  }
+  const void* src = b->step ? (const void*)stab.data() : (const void*)tab.data();
+  const size_t bytes = b->step ? stab.size() * sizeof(StepEvent) : tab.size() * sizeof(EventDesc);
+  TCW_CUDA(c, b->evtab.ensure(bytes), "event table");
+  TCW_CUDA(c, cudaMemcpyAsync(b->evtab.p, src, bytes, cudaMemcpyHostToDevice, c->stream), "event table");
   TCW_CUDA(c, cudaStreamSynchronize(c->stream), "event table");
   return TCW_OK;
+}
+
+// Doppler rows of every event (step-function search).
+cudaError_t launch_rows(BatchState* b, cudaStream_t st, int* nodes) {
+  cudaError_t err = cudaMemsetAsync(b->rows.p, 0, b->wtot_bytes, st);
+  for (size_t i = 0; i < b->ev.size() && err == cudaSuccess; ++i) {
+    err = launch_step_rows(step_rows_of(b, b->ev[i]), st);
+    *nodes += step_ordered(b->ev[i].geo) ? 2 : 1;
+  }
+  return err;
 }
 
 cudaError_t launch_wave_anchors(const tcw_ctx* c, BatchState* b, int w, int tile, cudaStream_t st) {
   for (const EventHost& e : b->ev) {
     if (e.wave != w) continue;
-    AnchorParams ap{};
+    if (b->step) tile = 1 << b->track.shift;
+    StepTileParams tp{};
+    AnchorParams& ap = tp.a;
     ap.t_mid = at<double>(b->small, e.o_t);
     ap.f0 = ev_f0(c, e);
     ap.tau = ev_tau(c, e);
@@ -381,7 +580,10 @@ cudaError_t launch_wave_anchors(const tcw_ctx* c, BatchState* b, int w, int tile
     ap.Bpad = ev_Bpad(c, e);
     ap.chain = anchor_chain_for(e.t.data(), e.n_seg, e.T0, tile, c->bank_tau_min, c->bank_r_max);
     ap.anchors = at<double>(b->anchors, e.o_anchor);
-    cudaError_t err = launch_anchors(ap, st);
+    tp.f_min = b->f_min;
+    tp.df = b->df;
+    tp.tiles = b->step ? at<StepTile>(b->tiles, e.o_anchor / 16 * sizeof(StepTile)) : nullptr;
+    cudaError_t err = b->step ? launch_step_tiles(tp, st) : launch_anchors(ap, st);
     if (err != cudaSuccess) return err;
   }
   return cudaSuccess;
@@ -393,11 +595,22 @@ tcw_status upload_items(tcw_ctx* c, BatchState* b, int bank_chunk, int groups_li
   std::vector<int> ctas;
   b->wave_items.assign(1, 0);
   b->wave_cta.clear();
+  b->wave_split.clear();
   *sums = 0;
   for (int w = 0; w < b->waves; ++w) {
     std::vector<int4> order;
     std::vector<int> cta;
     int64_t s = 0;
+    if (b->step) {
+      const int64_t limit = (int64_t)groups_limit * pass_templates(b->lanes);
+      int split = 0;
+      wave_step_items(c, b, w, bank_chunk, (int)std::min<int64_t>(limit, INT32_MAX), order, &split, &s);
+      *sums += s;
+      all.insert(all.end(), order.begin(), order.end());
+      b->wave_items.push_back((int)all.size());
+      b->wave_split.push_back(split);
+      continue;
+    }
     wave_items(c, b, w, bank_chunk, groups_limit, order, cta, &s);
     *sums += s;
     all.insert(all.end(), order.begin(), order.end());
@@ -423,6 +636,51 @@ GroupParams wave_params(const tcw_ctx* c, BatchState* b, int w, int tile, int nt
   return gp;
 }
 
+// The search launches of wave w.
+cudaError_t launch_wave(const tcw_ctx* c, BatchState* b, int w, int tile, int nterms, cudaStream_t st, int* nodes) {
+  if (!b->step) {
+    const GroupParams gp = wave_params(c, b, w, tile, nterms);
+    ++*nodes;
+    return launch_group(gp, b->grid, half_windows(c, b), false, st);
+  }
+  StepParams p{};
+  p.events = b->evtab.as<StepEvent>();
+  p.next = at<unsigned>(b->flags, 32);
+  p.n_det = b->D;
+  p.n_bin = b->n_bin;
+  p.f_min = b->f_min;
+  p.df = b->df;
+  p.inv_q = b->inv_q;
+  p.q = (float)b->q;
+  p.inv_q_f = (float)b->inv_q;
+  p.df_f = (float)b->df;
+  set_step_track(p, b->track);
+  p.amp_power = c->amp_power;
+  p.nc_q = count_q(c);
+  p.track_bins = c->track_bins;
+  p.map_half = b->dtype == TCW_F16 ? 1 : 0;
+  p.slow = c->step_slow.as<int4>();
+  p.edge = c->step_edge.as<longlong2>();
+  p.n_general = at<unsigned long long>(b->flags, 8);
+  const bool general = c->statistic == TCW_STAT_NUMBER_COUNT || c->track_bins == 2;
+  const int first = b->wave_items[w], split = first + b->wave_split[w], end = b->wave_items[w + 1];
+  for (int lt : {5, 4}) {
+    const int i0 = lt == 5 ? first : split, i1 = lt == 5 ? split : end;
+    if (i0 == i1) continue;
+    int cells = 0;
+    for (const EventHost& e : b->ev)
+      if (e.wave == w && e.geo.log_t == lt) cells = std::max(cells, step_cells(e.geo));
+    p.items = b->items.as<int4>() + i0;
+    p.n_items = i1 - i0;
+    cudaError_t err = cudaMemsetAsync(p.next, 0, 4, st);
+    if (err == cudaSuccess)
+      err = launch_step(p, b->dets_per_pass, lt, b->dtype == TCW_F16, general, cells, std::min(b->grid, p.n_items), st);
+    if (err != cudaSuccess) return err;
+    ++*nodes;
+  }
+  return cudaSuccess;
+}
+
 // Autotuner: every (bank chunk, tile) candidate runs the group kernel over the
 // first probe_groups groups of 8 templates of every event (wave by wave); the
 // candidate with the highest sums/s wins, ties going to the earlier one.
@@ -440,7 +698,15 @@ tcw_status autotune(tcw_ctx* c, BatchState* b) {
   for (int tile : tiles) {
     const int nterms = batch_series_terms(c, b, tile);
     if ((st = prepare_shape(c, b, tile, nterms)) != TCW_OK) break;
-    for (int w = 0; w < b->waves && nterms > 0; ++w) {
+    int nodes = 0;
+    if (b->step) {
+      cudaError_t err = launch_rows(b, c->stream, &nodes);
+      if (err != cudaSuccess) {
+        st = cuda_fail(c, err, "step_rows_kernel launch");
+        break;
+      }
+    }
+    for (int w = 0; w < b->waves && (b->step || nterms > 0); ++w) {
       cudaError_t err = launch_wave_anchors(c, b, w, tile, c->stream);
       if (err != cudaSuccess) {
         st = cuda_fail(c, err, "anchor_kernel launch");
@@ -456,10 +722,9 @@ tcw_status autotune(tcw_ctx* c, BatchState* b) {
       for (int rep = 0; rep < 2 && st == TCW_OK; ++rep) {
         cudaEventRecord(e0, c->stream);
         for (int w = 0; w < b->waves; ++w) {
-          const GroupParams gp = wave_params(c, b, w, tile, nterms);
-          cudaError_t err = launch_group(gp, b->grid, half_windows(c, b), false, c->stream);
+          cudaError_t err = launch_wave(c, b, w, tile, nterms, c->stream, &nodes);
           if (err != cudaSuccess) {
-            st = cuda_fail(c, err, "group_kernel launch");
+            st = cuda_fail(c, err, "search kernel launch");
             break;
           }
         }
@@ -494,6 +759,18 @@ tcw_status autotune(tcw_ctx* c, BatchState* b) {
   return TCW_OK;
 }
 
+// Shared-memory limits of the search kernels of a batch.
+tcw_status prepare_kernels(tcw_ctx* c, const BatchState* b) {
+  const bool general = c->statistic == TCW_STAT_NUMBER_COUNT || c->track_bins == 2;
+  if (b->step) {
+    for (int lt : {5, 4})
+      TCW_CUDA(c, step_prepare(b->dets_per_pass, lt, b->dtype == TCW_F16, general), "step_kernel attributes");
+  } else {
+    TCW_CUDA(c, group_prepare(b->D, b->lanes, half_windows(c, b), general), "group_kernel attributes");
+  }
+  return TCW_OK;
+}
+
 // Record one search of the whole batch as a CUDA graph.
 tcw_status capture(tcw_ctx* c, BatchState* b, int k) {
   drop_graph(b);
@@ -505,12 +782,12 @@ tcw_status capture(tcw_ctx* c, BatchState* b, int k) {
   if ((st = upload_items(c, b, b->bank_chunk, INT32_MAX, &sums)) != TCW_OK) return st;
   TCW_CUDA(c, b->out_psi.ensure((size_t)b->total_sky * k * sizeof(float)), "output");
   TCW_CUDA(c, b->out_idx.ensure((size_t)b->total_sky * k * sizeof(int64_t)), "output");
-  TCW_CUDA(c, group_prepare(b->D, b->lanes, half_windows(c, b),
-                            c->statistic == TCW_STAT_NUMBER_COUNT || c->track_bins == 2), "group_kernel attributes");
+  if ((st = prepare_kernels(c, b)) != TCW_OK) return st;
   TCW_CUDA(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal), "graph capture");
   cudaError_t err = cudaMemsetAsync(b->flags.p, 0, 64, c->stream);
   int nodes = 0;
-  for (size_t i = 0; i < b->ev.size() && err == cudaSuccess; ++i) {
+  if (b->step && err == cudaSuccess) err = launch_rows(b, c->stream, &nodes);
+  for (size_t i = 0; i < b->ev.size() && err == cudaSuccess && !b->step; ++i) {
     const EventHost& e = b->ev[i];
     DopplerParams dp{};
     dp.vel = at<double>(b->small, e.o_v);
@@ -528,14 +805,12 @@ tcw_status capture(tcw_ctx* c, BatchState* b, int k) {
     ++nodes;
   }
   for (int w = 0; w < b->waves && err == cudaSuccess; ++w) {
-    if (nterms > 0) {
+    if (b->step || nterms > 0) {
       err = launch_wave_anchors(c, b, w, b->tile, c->stream);
       for (const EventHost& e : b->ev) nodes += e.wave == w;
     }
     if (err != cudaSuccess) break;
-    const GroupParams gp = wave_params(c, b, w, b->tile, nterms);
-    err = launch_group(gp, b->grid, half_windows(c, b), false, c->stream);
-    ++nodes;
+    err = launch_wave(c, b, w, b->tile, nterms, c->stream, &nodes);
     for (const EventHost& e : b->ev) {
       if (e.wave != w || err != cudaSuccess) continue;
       err = launch_topk(at<float>(b->psi, e.o_psi), ev_Bpad(c, e), (int)ev_B(c, e), (int)e.n_sky, k,
@@ -670,6 +945,11 @@ tcw_status tcw_load_events(tcw_ctx* c, int n_det, int64_t n_bin, int dtype, doub
     } else {
       w.assign((size_t)n_det * in.n_seg, 1.0f);
     }
+    e.w_min = INFINITY;
+    for (float x : w) {
+      if (x > 0 && x < e.w_min) e.w_min = x;
+      if (x > e.w_max) e.w_max = x;
+    }
     wts[i] = std::move(w);
     b->unit_weights = b->unit_weights && e.unit_w;
     // sky sorted by its Doppler factor at the event's middle segment (detector 0)
@@ -743,6 +1023,25 @@ tcw_status tcw_load_events(tcw_ctx* c, int n_det, int64_t n_bin, int dtype, doub
   if (ce != cudaSuccess) {
     batch_free(c);
     return cuda_fail(c, ce, "event upload");
+  }
+  {
+    // the largest |rho| of every event (the step-function search's conditions)
+    DevBuf mx;
+    std::vector<float> h(n_events);
+    ce = mx.ensure((size_t)n_events * 4);
+    if (ce == cudaSuccess) ce = cudaMemsetAsync(mx.p, 0, (size_t)n_events * 4, c->stream);
+    for (int i = 0; i < n_events && ce == cudaSuccess; ++i)
+      ce = launch_absmax(at<char>(b->rho, b->ev[i].o_rho), dtype == TCW_F16, (int64_t)n_det * b->ev[i].n_seg * n_bin,
+                         mx.as<unsigned>() + i, c->stream);
+    if (ce == cudaSuccess)
+      ce = cudaMemcpyAsync(h.data(), mx.p, (size_t)n_events * 4, cudaMemcpyDeviceToHost, c->stream);
+    if (ce == cudaSuccess) ce = cudaStreamSynchronize(c->stream);
+    mx.release();
+    if (ce != cudaSuccess) {
+      batch_free(c);
+      return cuda_fail(c, ce, "map maximum");
+    }
+    for (int i = 0; i < n_events; ++i) b->ev[i].map_max = h[i];
   }
   for (EventHost& e : b->ev) {
     if ((size_t)b->D * e.n_seg * n_bin * esz < 64) {
@@ -1084,16 +1383,16 @@ tcw_status tcw_search_batched_triaged(tcw_ctx* c, const uint16_t* wbf, const flo
   if ((st = upload_items(c, tb, bank_chunk, INT32_MAX, &sums)) != TCW_OK) return st;
   TCW_CUDA(c, b->out_psi.ensure((size_t)b->total_sky * k * sizeof(float)), "output");
   TCW_CUDA(c, b->out_idx.ensure((size_t)b->total_sky * k * sizeof(int64_t)), "output");
-  TCW_CUDA(c, group_prepare(tb->D, tb->lanes, half_windows(c, tb),
-                            c->statistic == TCW_STAT_NUMBER_COUNT || c->track_bins == 2), "group_kernel attributes");
+  if ((st = prepare_kernels(c, tb)) != TCW_OK) return st;
   TCW_CUDA(c, launch_fill_empty(b->out_psi.as<float>(), b->out_idx.as<int64_t>(), b->total_sky * k, c->stream),
            "fill");
   TCW_CUDA(c, cudaMemsetAsync(tb->flags.p, 0, 64, c->stream), "flags");
   TCW_CUDA(c, cudaEventRecord(ev[3], c->stream), "event");
+  int nodes = 0;
+  if (tb->step) TCW_CUDA(c, launch_rows(tb, c->stream, &nodes), "step_rows_kernel launch");
   for (int w = 0; w < tb->waves; ++w) {
-    if (nterms > 0) TCW_CUDA(c, launch_wave_anchors(c, tb, w, tile, c->stream), "anchor_kernel launch");
-    const GroupParams gp = wave_params(c, tb, w, tile, nterms);
-    TCW_CUDA(c, launch_group(gp, tb->grid, half_windows(c, tb), false, c->stream), "group_kernel launch");
+    if (tb->step || nterms > 0) TCW_CUDA(c, launch_wave_anchors(c, tb, w, tile, c->stream), "anchor_kernel launch");
+    TCW_CUDA(c, launch_wave(c, tb, w, tile, nterms, c->stream, &nodes), "search kernel launch");
     for (const EventHost& h : tb->ev) {
       if (h.wave != w) continue;
       TCW_CUDA(c, launch_topk(at<float>(tb->psi, h.o_psi), ev_Bpad(c, h), (int)ev_B(c, h), (int)h.n_sky, k,

@@ -307,12 +307,19 @@ __device__ __forceinline__ float step_value(const StepParams& p, const StepEvent
 }
 
 // v * s rounded to the fixed-point grid: hi + lo 2^-16 with |lo| <= 2^15
-// (|v s| < 2^22).  The product is never rounded before the grid.
+// (|v s| < 2^22), each word plus kMagicBits, which cancels in differences.  The
+// product is never rounded before the grid.
 __device__ __forceinline__ void to_fixed(float v, float s, int& hi, int& lo) {
   const float t = fmaf(v, s, kMagic);
   const float r = fmaf(v, s, -(t - kMagic));
-  hi = __float_as_int(t) - kMagicBits;
-  lo = __float_as_int(fmaf(r, 65536.0f, kMagic)) - kMagicBits;
+  hi = __float_as_int(t);
+  lo = __float_as_int(fmaf(r, 65536.0f, kMagic));
+}
+// The same as one 64-bit word.
+__device__ __forceinline__ long long fixed_word(float v, float s) {
+  int hi, lo;
+  to_fixed(v, s, hi, lo);
+  return (long long)(hi - kMagicBits) * 65536 + (lo - kMagicBits);
 }
 
 // The exact thresholds of (template b, segment j) on the q grid, as the group
@@ -441,11 +448,8 @@ __device__ __forceinline__ void step_rare(const StepParams& p, StepBlockCtx& c, 
   for (long long u = v; nb < kNThr && saturate(u) <= qmax; u += x.V2) ++nb;
   long long u1, u2;   // the lookup's weights
   if (p.amp_power > 0) {
-    int wh, wl;
-    to_fixed(w, ev.w1_scale, wh, wl);
-    u1 = (long long)wh * 65536 + wl;
-    to_fixed(w, w * ev.w2_scale, wh, wl);
-    u2 = (long long)wh * 65536 + wl;
+    u1 = fixed_word(w, ev.w1_scale);
+    u2 = fixed_word(w, w * ev.w2_scale);
   } else {
     const longlong2 wi = ev.wfix[(int64_t)j * p.n_det + d];
     u1 = wi.x;
@@ -458,7 +462,7 @@ __device__ __forceinline__ void step_rare(const StepParams& p, StepBlockCtx& c, 
   }
   int h0, l0;
   value(K0, h0, l0);
-  atomicAdd(c.tsum + lt, (unsigned long long)((long long)h0 * 65536 + l0));
+  atomicAdd(c.tsum + lt, (unsigned long long)((long long)(h0 - kMagicBits) * 65536 + (l0 - kMagicBits)));
   // W1, W2 start from every segment's weights, amplitude weights from 0
   if (first != (p.amp_power == 0)) {
     atomicAdd(c.tsum + 32 + lt, (unsigned long long)(first ? u1 : -u1));
@@ -646,12 +650,13 @@ __device__ __noinline__ void step_fold(const StepParams& p, StepBlockCtx& s_ctx,
 // scheduler and cycle, nothing saturated; hence 32 warps (24: 3-10 % slower).
 // 2e5 templates x 1024 skies x 2 detectors x 1e4 segments: 655 ms by the group
 // kernel, 276 with the track in fp32 pairs and every step searched where it
-// arises, 160 so; one sky and one detector: 205, 50, 25 ms.
+// arises, 160 so; one sky and one detector: 205, 50, 24 ms.
 template <int VK, int DP, int LT>
 __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int cells) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_item;
   __shared__ unsigned long long s_wtot[2];
+  __shared__ int s_turn;
   __shared__ StepBlockCtx s_ctx;
   __shared__ StepEvent s_ev;   // the item's event: read in the loops without a trip to global memory
   const StepLayout L(cells);
@@ -665,7 +670,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
   int4* const slow_list = p.slow + ((int64_t)blockIdx.x * kStepWarps + (threadIdx.x >> 5)) * kStepSlow;
   int4* const heads = reinterpret_cast<int4*>(smem + L.head) + (threadIdx.x >> 5) * kStepTurn * kStepHead;
   unsigned long long* const tsum = reinterpret_cast<unsigned long long*>(smem + L.tsum);   // X0, W1, W2 [32]
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31;
   const bool two = VK == 2 && p.track_bins == 2;
   constexpr unsigned kAll = 0xffffffffu;
   const unsigned lt_mask = (1u << lane) - 1u;
@@ -755,7 +760,14 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
         const int js = pass / per * ev.pass_seg, je = min(n_seg, js + ev.pass_seg);
         for (int jc = js; jc < je; jc += kStepCarry) {
           const int jce = min(je, jc + kStepCarry);
-          for (int j0 = jc + (warp << sub); j0 < jce; j0 += kStepWarps << sub) {
+          // the warps take the turns as they come: their lengths in time differ
+          if (tid == 0) s_turn = 0;
+          __syncthreads();
+          while (true) {
+            int j0 = 0;
+            if (lane == 0) j0 = jc + (atomicAdd(&s_turn, 1) << sub);
+            j0 = __shfl_sync(kAll, j0, 0);
+            if (j0 >= jce) break;
             const int jn = min(jce, j0 + (1 << sub));
             const int64_t rbase = row0 + (int64_t)j0 * p.n_det + d0;   // first row of the turn
             const int64_t vbase = ((int64_t)d0 * n_seg + j0) * vpitch;
@@ -784,6 +796,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
             // The template's bins over the turn (tracks fall, Doppler shifts below 3 bins): wholly in the
             // band, wholly out of it, or at an edge (or T0), which step_rare takes segment by segment
             unsigned at_edge, outside;
+            uint32_t eps;   // the thresholds' error bound at the turn's lowest frequency, as queued
             {
               const float x0 = fmaf(A_hi, dt_first, fmaf(Q_hi, dt_first * dt_first, (float)base_a));
               const float x1 = fmaf(A_hi, dt_last, fmaf(Q_hi, dt_last * dt_last, (float)base_a));
@@ -792,6 +805,8 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
               const bool out = whole && (fmaxf(x0, x1) < -8.0f || fminf(x0, x1) > (float)n_bin + 8.0f);
               outside = __ballot_sync(kAll, out);
               at_edge = __ballot_sync(kAll, !out && !in);
+              const float F1 = Xf + (fminf(x0, x1) - (float)base_a);
+              eps = (uint32_t)(int)fmaf(rcp_approx(F1) * p.inv_q_f, p.eps_scale, 1.5f) << 25;
             }
             const bool mine = !(((at_edge | outside) >> lane) & 1u);
             int cnt = 0;     // steps in the warp's queue
@@ -826,12 +841,14 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
               }
               __syncwarp();
             };
-            int jb = (at_edge | outside) == kAll ? jn : j0;
+            const int ns = jn - j0;
+            int jb = (at_edge | outside) == kAll ? ns : 0;
+            int xh = 0, xl = 0, nx = 0;   // the turn's first-sky powers, each with kMagicBits, and their number
             do {
             // segments of the turn, then rounds without lookups until the queue is empty
-            for (; (jb < jn || cnt > 0) && nslow <= kStepSlow - kStepSlowMore; jb += lps) {
-              const int j = min(jb + ls, jn - 1), jr = j - j0;
-              const bool turn = mine && jb + ls < jn;
+            for (; (jb < ns || cnt > 0) && nslow <= kStepSlow - kStepSlowMore; jb += lps) {
+              const int jr = min(jb + ls, ns - 1);
+              const bool turn = mine && jb + ls < ns;
               const int4* head = heads + jr * DP * kStepHead;
               const float4 dt = *reinterpret_cast<const float4*>(head + 1);
               // the unshifted track's position base + frac and F = f/df (see StepTile): the linear and
@@ -848,7 +865,6 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
               const float small = (fmaf(A_hi, dt.x, -pl) + fmaf(A_hi, dt.y, A_lo * dt.x)) +
                                   (fmaf(Q_hi, dt.z, -pq) + fmaf(Q_hi, dt.w, Q_lo * dt.z)) + p3;
               const float F = (Xf + pl) + (pq + p3);
-              const int base = base_a + (int)(plr + pqr);
               float amp = 1.0f;
               if (p.amp_power > 0) {
                 const float rr = turn ? F * famp : 1.0f;   // f / f0
@@ -857,71 +873,77 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
               }
               const float Fq = F * p.q, R = rcp_approx(F) * p.inv_q_f;
               const float y0 = ((frac_a + (pl - plr)) + ((pq - pqr) + small)) - hb;
-              const uint32_t eps = (uint32_t)(int)fmaf(R, p.eps_scale, 1.0f) << 25;
 #pragma unroll 1
               for (int dd = 0; dd < DP; ++dd) {
                 const int4 m0 = head[dd * kStepHead];
                 // the lowest and the highest sky's distance from boundary 0, in bins: boundaries in between
                 const float zl = fmaf(Fq, (float)m0.x, y0), zh = fmaf(Fq, (float)m0.y, y0);
-                const float fl = floorf(zl);
-                const bool close = turn && (fabsf(zl - rintf(zl)) < p.eps || fabsf(zh - rintf(zh)) < p.eps);
+                const float fl = floorf(zl), fh = floorf(zh);
+                const bool close = turn && (fabsf((zl - fl) - 0.5f) > 0.5f - p.eps || fabsf((zh - fh) - 0.5f) > 0.5f - p.eps);
                 const bool on = turn && !close;
                 const int rl = jr * p.n_det + dd, tag = rl << 5 | lt;
                 if (const unsigned vote = __ballot_sync(kAll, close)) {
                   if (close) slow_list[nslow + __popc(vote & lt_mask)] = make_int4(0, 0, tag, -1);
                   nslow += __popc(vote);
                 }
-                const int nb = on ? min((int)(floorf(zh) - fl), kNThr - 1) : 0;
-                const float y1 = fl + 1.0f - y0;
-                const int K = base + (int)fl + 1;   // the lowest sky's bin
+                const int nb = on ? min((int)(fh - fl), kNThr - 1) : 0;
+                const int K = base_a + 1 + (int)(plr + pqr + fl);   // the lowest sky's bin
                 const int64_t vrow = vbase + (int64_t)(dd * n_seg + jr) * vpitch;
                 // the lookup's loads at once; the queue is drained while they are under way
-                const uint32_t* const tr = ev.tab + (rbase + rl) * nk;
-                const float per_unit = __int_as_float(m0.z);
-                const float v0 = on ? step_value<VK>(p, ev, vrow, K) : 0.f;
-                const float v1 = nb > 0 ? step_value<VK>(p, ev, vrow, K + 1) : 0.f;
-                float vn = nb > 1 ? step_value<VK>(p, ev, vrow, K + 2) : 0.f;
-                const int th0 = __float2int_rn(y1 * R);
-                int th = __float2int_rn((y1 + 1.0f) * R);
-                const uint32_t win0 = nb > 0 ? __ldg(tr + step_bucket(th0, m0.x, per_unit, nk)) : 0u;
-                uint32_t win = nb > 1 ? __ldg(tr + step_bucket(th, m0.x, per_unit, nk)) : 0u;
                 const float ws = __int_as_float(m0.w) * amp * xs;
-                if (cnt >= 32 || jb >= jn) drain();
+                const float v0 = on ? step_value<VK>(p, ev, vrow, K) : 0.f;
+                const unsigned some = __ballot_sync(kAll, nb > 0);
+                const uint32_t* const tr = ev.tab + (rbase + rl) * nk;
+                const float per_unit = __int_as_float(m0.z), y1 = fl + 1.0f - y0;
+                float v1 = 0.f, vn = 0.f;
+                int th0 = 0, th = 0;
+                uint32_t win0 = 0, win = 0;
+                if (some) {
+                  th0 = __float2int_rn(y1 * R);
+                  th = __float2int_rn((y1 + 1.0f) * R);
+                  if (nb > 0) {
+                    v1 = step_value<VK>(p, ev, vrow, K + 1);
+                    win0 = __ldg(tr + step_bucket(th0, m0.x, per_unit, nk));
+                  }
+                  if (nb > 1) {
+                    vn = step_value<VK>(p, ev, vrow, K + 2);
+                    win = __ldg(tr + step_bucket(th, m0.x, per_unit, nk));
+                  }
+                }
+                if (cnt >= 32 || jb >= ns) drain();
                 int h0, l0, h1, l1;
                 to_fixed(v0, ws, h0, l0);
-                if (on) X0 += (long long)h0 * 65536 + l0;
-                to_fixed(v1, ws, h1, l1);
-                {
-                  const unsigned vote = __ballot_sync(kAll, nb > 0);
+                xh += h0;
+                xl += l0;
+                ++nx;
+                if (some) {
+                  to_fixed(v1, ws, h1, l1);
                   if (nb > 0)
-                    queue[cnt + __popc(vote & lt_mask)] =
+                    queue[cnt + __popc(some & lt_mask)] =
                         make_int4(th0, h1 - h0, (l1 - l0) * 8192 | tag, (int)(win0 | eps));
-                  cnt += __popc(vote);
-                }
-                for (int i = 1;; ++i) {
-                  const unsigned vote = __ballot_sync(kAll, nb > i);
-                  if (!vote) break;
-                  if (cnt >= 32) drain();
-                  h0 = h1;
-                  l0 = l1;
-                  to_fixed(vn, ws, h1, l1);
-                  if (nb > i)
-                    queue[cnt + __popc(vote & lt_mask)] =
-                        make_int4(th, h1 - h0, (l1 - l0) * 8192 | tag, (int)(win | (uint32_t)i << 22 | eps));
-                  cnt += __popc(vote);
-                  if (nb > i + 1) {
-                    vn = step_value<VK>(p, ev, vrow, K + i + 2);
-                    th = __float2int_rn((y1 + (float)(i + 1)) * R);
-                    win = __ldg(tr + step_bucket(th, m0.x, per_unit, nk));
+                  cnt += __popc(some);
+                  for (int i = 1;; ++i) {
+                    const unsigned vote = __ballot_sync(kAll, nb > i);
+                    if (!vote) break;
+                    if (cnt >= 32) drain();
+                    h0 = h1;
+                    l0 = l1;
+                    to_fixed(vn, ws, h1, l1);
+                    if (nb > i)
+                      queue[cnt + __popc(vote & lt_mask)] =
+                          make_int4(th, h1 - h0, (l1 - l0) * 8192 | tag, (int)(win | (uint32_t)i << 22 | eps));
+                    cnt += __popc(vote);
+                    if (nb > i + 1) {
+                      vn = step_value<VK>(p, ev, vrow, K + i + 2);
+                      th = __float2int_rn((y1 + (float)(i + 1)) * R);
+                      win = __ldg(tr + step_bucket(th, m0.x, per_unit, nk));
+                    }
                   }
                 }
                 if (p.amp_power > 0 && on) {
                   const float w = __int_as_float(m0.w) * amp;
-                  int wh, wl;
-                  to_fixed(w, ev.w1_scale, wh, wl);
-                  atomicAdd(tsum + 32 + lt, (unsigned long long)((long long)wh * 65536 + wl));
-                  to_fixed(w, w * ev.w2_scale, wh, wl);
-                  atomicAdd(tsum + 64 + lt, (unsigned long long)((long long)wh * 65536 + wl));
+                  atomicAdd(tsum + 32 + lt, (unsigned long long)fixed_word(w, ev.w1_scale));
+                  atomicAdd(tsum + 64 + lt, (unsigned long long)fixed_word(w, w * ev.w2_scale));
                 }
               }
             }
@@ -929,7 +951,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
             {
               // the list, and at the end of the turn every (template, row) of templates at a band edge
               const int nr = (jn - j0) * DP;
-              const int n = nslow + (jb < jn || cnt > 0 ? 0 : __popc(at_edge & t_mask) * nr);
+              const int n = nslow + (jb < ns || cnt > 0 ? 0 : __popc(at_edge & t_mask) * nr);
               for (int i = lane; i < n; i += 32) {
                 int4 e = make_int4(0, 0, 0, -1);
                 if (i < nslow) {
@@ -962,7 +984,8 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
               nslow = 0;
               __syncwarp();
             }
-            } while (jb < jn || cnt > 0);
+            } while (jb < ns || cnt > 0);
+            X0 += (long long)(xh - nx * kMagicBits) * 65536 + (xl - nx * kMagicBits);
             {
               const int nr = (jn - j0) * DP;
               if ((outside & t_mask) && p.amp_power == 0) {

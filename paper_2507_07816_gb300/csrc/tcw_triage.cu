@@ -23,9 +23,11 @@
 //                         more than 128 patches
 //   features_kernel       log(1 + count) per histogram bin
 //   MLP 128 -> 256 -> 256 -> 1 (ReLU), bfloat16 weights, fp32 accumulation:
-//     gemm_kernel         tiled C = op(A) op(B) (+ bias, ReLU) for the forward
-//                         pass and every product of the backward pass
-//     relu_mask / colsum / bce / adam kernels
+//     layer_kernel        a hidden layer forward (bias, ReLU), or the gradient
+//                         at the first layer's units
+//     out_kernel          the output layer
+//     wgrad_kernel        every parameter gradient
+//     bce / adam kernels
 //   select_kernel         best patches by score with suppression of their
 //                         neighbours (rank_kernel: plain ranking)
 //   region_select_kernel  the best templates of a chosen patch by coarse Psi
@@ -37,6 +39,7 @@
 // (template, segment), or FP64 anchors per 64-segment tile with fp32 hi/lo
 // pairs inside the tile), so their bins equal the exact ones except within
 // ~1e-7 bins of a rounding tie.  The Doppler term must stay within 2.9 bins.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include <climits>
@@ -645,91 +648,251 @@ __global__ void sweep_finalize_kernel(CoarseSweepParams p) {
 // ---------------------------------------------------------------------------
 // MLP kernels
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float to_f32(float x) { return x; }
-__device__ __forceinline__ float to_f32(__nv_bfloat16 x) { return __bfloat162float(x); }
+// A 64 x 64 tile of a product per CTA, 4 x 4 outputs per thread, fp32 FMAs.  Two
+// stages of 32 terms: the global loads of the next one are in flight while a
+// stage is multiplied.  Rows of 68 floats keep the 16-byte reads aligned.
+constexpr int kGemmTile = 64, kGemmK = 32, kGemmThreads = 256, kGemmRow = kGemmTile + 4;
+constexpr int kGemmLoads = kGemmK * kGemmTile / kGemmThreads;   // elements per thread and operand of a stage
 
-constexpr int kGemmTile = 64, kGemmK = 16, kGemmThreads = 256;
+struct alignas(16) GemmStage {
+  float a[kGemmK][kGemmRow], b[kGemmK][kGemmRow];
+};
 
-// C[m][n] = sum_k A(m, k) B(k, n) (+ bias[n]) (ReLU), A(m, k) = A[m sa0 + k sa1],
-// B(k, n) = B[k sb0 + n sb1], C[m ldc + n]; fp32 accumulation.
-template <typename TB>
-__global__ void __launch_bounds__(kGemmThreads) gemm_kernel(const float* A, int64_t sa0, int64_t sa1,
-                                                            const TB* Bm, int64_t sb0, int64_t sb1, float* C,
-                                                            int64_t ldc, int M, int N, int K, const float* bias,
-                                                            int relu) {
-  __shared__ float sA[kGemmK][kGemmTile + 1];
-  __shared__ float sB[kGemmK][kGemmTile + 1];
-  const int tid = threadIdx.x;
-  const int tm = tid / 16, tn = tid % 16;
-  const int m0 = blockIdx.y * kGemmTile, n0 = blockIdx.x * kGemmTile;
+__device__ __forceinline__ void gemm_stage(const GemmStage& s, int tm, int tn, float (&acc)[4][4]) {
+#pragma unroll
+  for (int kk = 0; kk < kGemmK; ++kk) {
+    const float4 a = *reinterpret_cast<const float4*>(&s.a[kk][tm * 4]);
+    const float4 b = *reinterpret_cast<const float4*>(&s.b[kk][tn * 4]);
+    const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int jx = 0; jx < 4; ++jx) acc[i][jx] = fmaf(av[i], bv[jx], acc[i][jx]);
+  }
+}
+
+// Gradient at the second layer's pre-activation: dL/dy w3 where the unit is on.
+__device__ __forceinline__ float mlp_dz2(float dy, __nv_bfloat16 w3, float h2) {
+  return h2 > 0.f ? dy * __bfloat162float(w3) : 0.f;
+}
+
+// C = relu(A W + bias), A [n][K], W [K][256] bf16 (DGRAD false), or
+// C = (dZ2 W^T) where H1 is on, dZ2 from (dy, w3, H2) as it is loaded
+// (DGRAD true: A = H2).  Each output is one chain of FMAs in the order of k, the
+// same at every batch size.  4096 rows, 256 terms: forward 49 -> 27 us, the
+// gradient 69 -> 26 (before: loads strided by row and waited for, 4-byte shared
+// reads, masks in passes of their own).
+struct LayerParams {
+  const float* A;
+  const __nv_bfloat16* W;
+  const float* bias;             // forward
+  const float* dy;               // dgrad
+  const __nv_bfloat16* w3;
+  const float* H1;
+  float* C;
+  int n;
+};
+
+template <int K, bool DGRAD>
+__global__ void __launch_bounds__(kGemmThreads) layer_kernel(LayerParams p) {
+  __shared__ GemmStage st[2];
+  const int tid = threadIdx.x, tm = tid / 16, tn = tid % 16;
+  const int m0 = blockIdx.x * kGemmTile, n0 = blockIdx.y * kGemmTile;
+  // a stage as loaded: what is made of it waits until it is stored, so that no
+  // multiplication stands behind a load
+  float ra[kGemmLoads], rdy[kGemmLoads];
+  __nv_bfloat16 rb[kGemmLoads], rw = __float2bfloat16_rn(0.f);
+  if (DGRAD) {
+#pragma unroll
+    for (int q = 0; q < kGemmLoads; ++q) {
+      const int m = m0 + (tid + q * kGemmThreads) / kGemmK;
+      rdy[q] = m < p.n ? p.dy[m] : 0.f;
+    }
+  }
+  auto load = [&](int k0) {
+    if (DGRAD) rw = p.w3[k0 + tid % kGemmK];
+#pragma unroll
+    for (int q = 0; q < kGemmLoads; ++q) {
+      const int i = tid + q * kGemmThreads, kk = k0 + i % kGemmK, m = m0 + i / kGemmK;
+      ra[q] = m < p.n ? p.A[(int64_t)m * K + kk] : 0.f;
+      // W^T: 32 neighbours in k; W: 64 neighbours in n
+      rb[q] = DGRAD ? p.W[(n0 + i / kGemmK) * kMlpH + kk] : p.W[(k0 + i / kGemmTile) * kMlpH + n0 + i % kGemmTile];
+    }
+  };
+  auto store = [&](GemmStage& s) {
+#pragma unroll
+    for (int q = 0; q < kGemmLoads; ++q) {
+      const int i = tid + q * kGemmThreads;
+      s.a[i % kGemmK][i / kGemmK] = DGRAD ? mlp_dz2(rdy[q], rw, ra[q]) : ra[q];
+      if (DGRAD)
+        s.b[i % kGemmK][i / kGemmK] = __bfloat162float(rb[q]);
+      else
+        s.b[i / kGemmTile][i % kGemmTile] = __bfloat162float(rb[q]);
+    }
+  };
   float acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += kGemmK) {
-    for (int i = tid; i < kGemmK * kGemmTile; i += kGemmThreads) {
-      const int kk = i / kGemmTile, mm = i % kGemmTile;
-      const int m = m0 + mm, k = k0 + kk;
-      sA[kk][mm] = (m < M && k < K) ? A[(int64_t)m * sa0 + (int64_t)k * sa1] : 0.f;
-      const int n = n0 + mm;
-      sB[kk][mm] = (n < N && k < K) ? to_f32(Bm[(int64_t)k * sb0 + (int64_t)n * sb1]) : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < kGemmK; ++kk) {
-      float a[4], bv[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        a[i] = sA[kk][tm * 4 + i];
-        bv[i] = sB[kk][tn * 4 + i];
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int jx = 0; jx < 4; ++jx) acc[i][jx] = fmaf(a[i], bv[jx], acc[i][jx]);
-    }
+  load(0);
+  store(st[0]);
+  __syncthreads();
+  for (int k0 = 0, s = 0; k0 < K; k0 += kGemmK, s ^= 1) {
+    const bool more = k0 + kGemmK < K;
+    if (more) load(k0 + kGemmK);
+    gemm_stage(st[s], tm, tn, acc);
+    if (more) store(st[s ^ 1]);
     __syncthreads();
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int m = m0 + tm * 4 + i;
-    if (m >= M) continue;
+    if (m >= p.n) continue;
 #pragma unroll
     for (int jx = 0; jx < 4; ++jx) {
       const int n = n0 + tn * 4 + jx;
-      if (n >= N) continue;
-      float v = acc[i][jx] + (bias ? bias[n] : 0.f);
-      if (relu) v = fmaxf(v, 0.f);
-      C[(int64_t)m * ldc + n] = v;
+      const int64_t o = (int64_t)m * kMlpH + n;
+      p.C[o] = DGRAD ? (p.H1[o] > 0.f ? acc[i][jx] : 0.f) : fmaxf(acc[i][jx] + p.bias[n], 0.f);
     }
   }
 }
 
-template <typename TB>
-cudaError_t gemm(const float* A, int64_t sa0, int64_t sa1, const TB* B, int64_t sb0, int64_t sb1, float* C,
-                 int64_t ldc, int M, int N, int K, const float* bias, bool relu, cudaStream_t st) {
-  if (M <= 0 || N <= 0) return cudaSuccess;
-  dim3 grid((N + kGemmTile - 1) / kGemmTile, (M + kGemmTile - 1) / kGemmTile);
-  gemm_kernel<TB><<<grid, kGemmThreads, 0, st>>>(A, sa0, sa1, B, sb0, sb1, C, ldc, M, N, K, bias, relu ? 1 : 0);
-  return cudaGetLastError();
-}
+// y = H2 w3 + b3: a row per thread of the first warp, its terms in order, from
+// rows staged in shared memory.
+constexpr int kOutRows = 32;
 
-// dZ[i][j] = dY[i][j] (or dY[i] when ldy == 1) * scale[j] * (H[i][j] > 0)
-__global__ void relu_mask_kernel(const float* dY, int64_t ldy, const __nv_bfloat16* scale, const float* H,
-                                 int64_t n, int width, float* dZ) {
-  const int64_t total = n * width;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = i / width;
-    const int c = (int)(i % width);
-    const float g = dY[ldy == 1 ? r : r * ldy + c] * (scale ? __bfloat162float(scale[c]) : 1.f);
-    dZ[i] = H[i] > 0.f ? g : 0.f;
+__global__ void __launch_bounds__(256) out_kernel(const float* H2, const __nv_bfloat16* w3, const float* b3,
+                                                  float* y, int n) {
+  __shared__ float s_h[kOutRows][kMlpH + 1];
+  __shared__ float s_w[kMlpH];
+  const int m0 = blockIdx.x * kOutRows, rows = min(kOutRows, n - m0), tid = threadIdx.x;
+  s_w[tid] = __bfloat162float(w3[tid]);
+#pragma unroll 8
+  for (int r = 0; r < kOutRows; ++r) s_h[r][tid] = r < rows ? H2[(int64_t)(m0 + r) * kMlpH + tid] : 0.f;
+  __syncthreads();
+  if (tid >= rows) return;
+  float acc = 0.f;
+#pragma unroll 16
+  for (int k = 0; k < kMlpH; ++k) acc = fmaf(s_h[tid][k], s_w[k], acc);
+  y[m0 + tid] = acc + b3[0];
+}
+static_assert(kMlpH == 256 && kMlpIn % kGemmK == 0 && kMlpIn % kGemmTile == 0, "the tiles cover the layers");
+
+// All parameter gradients: sums over the batch of outer products.  The outputs
+// are few (24 tiles of 64 x 64) and the sums long, so a cluster of 8 CTAs takes
+// a tile, an eighth of the batch each, and adds the partial tiles in a fixed
+// order over distributed shared memory.  Tiles 0..15: W2 (and b2 with the first
+// row of tiles), 16..23: W1 (and b1), 24..27: 64 columns of w3 each (and b3).
+// A training step with a batch of 4096: 1.75 ms with 16 and 8 CTAs over the
+// whole batch and one CTA for each bias, 0.13 ms so.
+constexpr int kWgradSplit = 8, kWgradTiles = 28;
+
+struct WgradParams {
+  const float *X, *H1, *H2, *dy, *dZ1;
+  const __nv_bfloat16* w3;
+  float* grad;
+  int64_t n;
+};
+
+__global__ void __cluster_dims__(kWgradSplit, 1, 1) __launch_bounds__(kGemmThreads) wgrad_kernel(WgradParams p) {
+  namespace cg = cooperative_groups;
+  __shared__ GemmStage st[2];
+  static_assert(sizeof(st) >= kGemmTile * kGemmTile * sizeof(float), "the partial tile takes the stages' place");
+  float* const part = reinterpret_cast<float*>(st);
+  __shared__ float part_b[kGemmThreads];
+  auto cluster = cg::this_cluster();
+  const int tile = blockIdx.x / kWgradSplit, rank = blockIdx.x % kWgradSplit, tid = threadIdx.x;
+  const int64_t per = (p.n + kWgradSplit - 1) / kWgradSplit;
+  const int64_t r0 = min(p.n, rank * per), r1 = min(p.n, r0 + per);
+  const bool second = tile < 16, out = tile >= 24;
+  const int t = second ? tile : tile - 16, m0 = out ? 0 : t / 4 * kGemmTile, n0 = t % 4 * kGemmTile;
+  part_b[tid] = 0.f;
+  if (out) {
+    // a column per thread, 4 threads to a column; the threads of column 0 hold b3 too
+    const int col = n0 + tid % kGemmTile;
+    float s = 0.f, sb = 0.f;
+#pragma unroll 8
+    for (int64_t i = r0 + tid / kGemmTile; i < r1; i += kGemmThreads / kGemmTile) {
+      const float d = p.dy[i];
+      s = fmaf(p.H2[i * kMlpH + col], d, s);
+      sb += d;
+    }
+    part[tid] = s;
+    part_b[tid] = sb;
+  } else {
+    const float* A = (second ? p.H1 : p.X) + m0 + tid % kGemmTile;
+    const int lda = second ? kMlpH : kMlpIn, nc = n0 + tid % kGemmTile;
+    const int tm = tid / 16, tn = tid % 16, row = tid / kGemmTile;
+    const __nv_bfloat16 w3 = p.w3[nc];
+    const float* B = (second ? p.H2 : p.dZ1) + nc;
+    float ra[kGemmLoads], rb[kGemmLoads], rdy[kGemmLoads], acc[4][4] = {}, bsum = 0.f;
+    auto load = [&](int64_t k0) {
+#pragma unroll
+      for (int q = 0; q < kGemmLoads; ++q) {
+        const int64_t i = k0 + row + q * (kGemmThreads / kGemmTile);
+        ra[q] = i < r1 ? A[i * lda] : 0.f;
+        rb[q] = i < r1 ? B[i * kMlpH] : 0.f;
+        rdy[q] = second && i < r1 ? p.dy[i] : 0.f;
+      }
+    };
+    auto store = [&](GemmStage& s) {
+#pragma unroll
+      for (int q = 0; q < kGemmLoads; ++q) {
+        const int kk = row + q * (kGemmThreads / kGemmTile);
+        s.a[kk][tid % kGemmTile] = ra[q];
+        const float b = second ? mlp_dz2(rdy[q], w3, rb[q]) : rb[q];
+        s.b[kk][tid % kGemmTile] = b;
+        bsum += b;
+      }
+    };
+    load(r0);
+    store(st[0]);
+    __syncthreads();
+    int s = 0;
+    for (int64_t k0 = r0; k0 < r1; k0 += kGemmK, s ^= 1) {
+      const bool more = k0 + kGemmK < r1;
+      if (more) load(k0 + kGemmK);
+      gemm_stage(st[s], tm, tn, acc);
+      if (more) store(st[s ^ 1]);
+      __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      *reinterpret_cast<float4*>(&part[(tm * 4 + i) * kGemmTile + tn * 4]) =
+          make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    part_b[tid] = bsum;
   }
-}
-
-// out[j] = sum_i Z[i][j]
-__global__ void colsum_kernel(const float* Z, int64_t n, int width, float* out) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= width) return;
-  float s = 0.f;
-  for (int64_t i = 0; i < n; ++i) s += Z[i * width + j];
-  out[j] = s;
+  cluster.sync();
+  if (out) {
+    if (rank == 0 && tid < kGemmTile) {
+      float s = 0.f, sb = 0.f;
+      for (int r = 0; r < kWgradSplit; ++r) {
+        const float *o = cluster.map_shared_rank(part, r), *ob = cluster.map_shared_rank(part_b, r);
+        for (int q = tid; q < kGemmThreads; q += kGemmTile) {
+          s += o[q];
+          sb += ob[q];
+        }
+      }
+      p.grad[kThW3 + n0 + tid] = s;
+      if (n0 + tid == 0) p.grad[kThB3] = sb;
+    }
+  } else {
+    // an eighth of the tile per CTA
+    constexpr int kShare = kGemmTile * kGemmTile / kWgradSplit;
+    float* W = p.grad + (second ? kThW2 : kThW1);
+    for (int k = rank * kShare + tid; k < (rank + 1) * kShare; k += kGemmThreads) {
+      float s = 0.f;
+#pragma unroll
+      for (int r = 0; r < kWgradSplit; ++r) s += cluster.map_shared_rank(part, r)[k];
+      W[(m0 + k / kGemmTile) * kMlpH + n0 + k % kGemmTile] = s;
+    }
+    if (m0 == 0 && rank == 0 && tid < kGemmTile) {
+      float s = 0.f;
+      for (int r = 0; r < kWgradSplit; ++r) {
+        const float* ob = cluster.map_shared_rank(part_b, r);
+        for (int q = tid; q < kGemmThreads; q += kGemmTile) s += ob[q];
+      }
+      p.grad[(second ? kThB2 : kThB1) + n0 + tid] = s;
+    }
+  }
+  cluster.sync();   // the others' reads of this CTA's shared memory end before it does
 }
 
 __global__ void bce_kernel(const float* y, const float* label, int64_t n, float pw, float* loss, float* dy) {
@@ -1107,36 +1270,29 @@ cudaError_t launch_rank(const float* score, int P, int m, int radius, int* selec
 
 cudaError_t mlp_forward(const __nv_bfloat16* wbf, const float* theta, const float* X, int64_t n, float* H1,
                         float* H2, float* y, cudaStream_t st) {
+  if (n <= 0) return cudaSuccess;
   const int N = (int)n;
-  cudaError_t e = gemm(X, kMlpIn, 1, wbf + kWbfW1, kMlpH, 1, H1, kMlpH, N, kMlpH, kMlpIn, theta + kThB1, true, st);
-  if (e == cudaSuccess)
-    e = gemm(H1, kMlpH, 1, wbf + kWbfW2, kMlpH, 1, H2, kMlpH, N, kMlpH, kMlpH, theta + kThB2, true, st);
-  if (e == cudaSuccess) e = gemm(H2, kMlpH, 1, wbf + kWbfW3, 1, 0, y, 1, N, 1, kMlpH, theta + kThB3, false, st);
-  return e;
+  const dim3 grid((unsigned)((n + kGemmTile - 1) / kGemmTile), kMlpH / kGemmTile);
+  const LayerParams p1{X, wbf + kWbfW1, theta + kThB1, nullptr, nullptr, nullptr, H1, N};
+  const LayerParams p2{H1, wbf + kWbfW2, theta + kThB2, nullptr, nullptr, nullptr, H2, N};
+  layer_kernel<kMlpIn, false><<<grid, kGemmThreads, 0, st>>>(p1);
+  layer_kernel<kMlpH, false><<<grid, kGemmThreads, 0, st>>>(p2);
+  out_kernel<<<(unsigned)((n + kOutRows - 1) / kOutRows), 256, 0, st>>>(H2, wbf + kWbfW3, theta + kThB3, y, N);
+  return cudaGetLastError();
 }
 
 cudaError_t mlp_backward(const __nv_bfloat16* wbf, const float* X, int64_t n, const float* H1, const float* H2,
                          const float* dy, float* grad, float* work, cudaStream_t st) {
-  const int N = (int)n;
-  float* dZ2 = work;
-  float* dZ1 = work + n * kMlpH;
-  const unsigned nb = blocks_for(n * kMlpH, 256);
-  // output layer: y = H2 w3 + b3
-  cudaError_t e = gemm(H2, 1, kMlpH, dy, 1, 0, grad + kThW3, 1, kMlpH, 1, N, nullptr, false, st);
-  if (e != cudaSuccess) return e;
-  colsum_kernel<<<1, 32, 0, st>>>(dy, n, 1, grad + kThB3);
-  relu_mask_kernel<<<nb, 256, 0, st>>>(dy, 1, wbf + kWbfW3, H2, n, kMlpH, dZ2);
-  // second hidden layer: H2 = relu(H1 W2 + b2)
-  e = gemm(H1, 1, kMlpH, dZ2, kMlpH, 1, grad + kThW2, kMlpH, kMlpH, kMlpH, N, nullptr, false, st);
-  if (e != cudaSuccess) return e;
-  colsum_kernel<<<1, kMlpH, 0, st>>>(dZ2, n, kMlpH, grad + kThB2);
-  e = gemm(dZ2, kMlpH, 1, wbf + kWbfW2, 1, kMlpH, dZ1, kMlpH, N, kMlpH, kMlpH, nullptr, false, st);
-  if (e != cudaSuccess) return e;
-  relu_mask_kernel<<<nb, 256, 0, st>>>(dZ1, kMlpH, nullptr, H1, n, kMlpH, dZ1);
-  // first hidden layer: H1 = relu(X W1 + b1)
-  e = gemm(X, 1, kMlpIn, dZ1, kMlpH, 1, grad + kThW1, kMlpH, kMlpIn, kMlpH, N, nullptr, false, st);
-  if (e != cudaSuccess) return e;
-  colsum_kernel<<<1, kMlpH, 0, st>>>(dZ1, n, kMlpH, grad + kThB1);
+  float* dZ1 = work;
+  if (n > 0) {
+    const dim3 grid((unsigned)((n + kGemmTile - 1) / kGemmTile), kMlpH / kGemmTile);
+    const LayerParams p{H2, wbf + kWbfW2, nullptr, dy, wbf + kWbfW3, H1, dZ1, (int)n};
+    layer_kernel<kMlpH, true><<<grid, kGemmThreads, 0, st>>>(p);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  const WgradParams p{X, H1, H2, dy, dZ1, wbf + kWbfW3, grad, n};
+  wgrad_kernel<<<kWgradTiles * kWgradSplit, kGemmThreads, 0, st>>>(p);
   return cudaGetLastError();
 }
 

@@ -204,7 +204,7 @@ tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, boo
   const size_t rows = (size_t)g.n_chunks * c->Nseg * c->D;
   TCW_CUDA(c, c->step_q.ensure(rows * step_row(g.cpad) * sizeof(int32_t)), "doppler rows");
   TCW_CUDA(c, c->step_head.ensure(rows * kStepHead * sizeof(int4)), "doppler rows");
-  TCW_CUDA(c, c->step_tab.ensure(rows * step_buckets(g.cpad) * sizeof(uint32_t)), "doppler rows");
+  TCW_CUDA(c, c->step_tab.ensure(rows * step_buckets(g.cpad) * (sizeof(uint2) + sizeof(uint32_t))), "doppler rows");
   TCW_CUDA(c, c->step_wtot.ensure(kStepSlots * 16 + (size_t)c->Nseg * c->D * sizeof(longlong2)), "weight sums");
   TCW_CUDA(c, cudaMemsetAsync(c->step_wtot.p, 0, kStepSlots * 16, c->stream), "weight sums");
   TCW_CUDA(c, ensure_step_edge(c->step_edge, c->grid, c->stream), "scratch");
@@ -230,7 +230,8 @@ tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, boo
   rp.remap = rp.order ? rp.order + (size_t)g.passes * g.n_chunks * g.cpad : nullptr;
   rp.q = c->step_q.as<int32_t>();
   rp.head = c->step_head.as<int4>();
-  rp.tab = c->step_tab.as<uint32_t>();
+  rp.fast = c->step_tab.as<uint2>();
+  rp.tab = reinterpret_cast<uint32_t*>(rp.fast + rows * step_buckets(g.cpad));
   rp.wtot = c->step_wtot.as<unsigned long long>();
   rp.wfix = reinterpret_cast<longlong2*>(rp.wtot + kStepSlots * 2);
   TCW_CUDA(c, launch_step_rows(rp, c->stream), "step_rows_kernel launch");
@@ -266,6 +267,7 @@ tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, boo
   ev.q = rp.q;
   ev.head = rp.head;
   ev.tab = rp.tab;
+  ev.fast = rp.fast;
   ev.wtot = c->step_wtot.as<long long>();
   ev.wfix = rp.wfix;
   ev.sub_shift = step_sub_shift(g, c->Nseg, tr.shift);

@@ -43,7 +43,7 @@ struct EventHost {
   float w_min = 0, w_max = 0, map_max = 0;   // smallest nonzero and largest weight, largest |rho|
   StepGeometry geo{};
   StepScales scales;
-  size_t o_q = 0, o_head = 0, o_tab = 0, o_wfix = 0, o_wtot = 0, o_order = 0;   // byte offsets of its Doppler rows
+  size_t o_q = 0, o_head = 0, o_tab = 0, o_fast = 0, o_wfix = 0, o_wtot = 0, o_order = 0;   // byte offsets of its Doppler rows
   // a triaged batch's event: its chosen skies (sorted, with their caller
   // indices within the event) and its template regions (a sub-bank); null
   // pointers / 0 sizes: the event's own sky at o_nhat / o_perm, the context's bank
@@ -245,7 +245,6 @@ void plan_step(const tcw_ctx* c, BatchState* b, int tile) {
       all.shift = std::min(all.shift, t.shift);
       all.nterms = std::max(all.nterms, t.nterms);
       all.eps = t.eps;
-      all.eps_shift = t.eps_shift;
       all.eps_max = t.eps_max;
     }
     b->track = all;
@@ -289,6 +288,7 @@ size_t layout_rows(BatchState* b) {
     e.o_q = take(rows * step_row(e.geo.cpad) * sizeof(int32_t));
     e.o_head = take(rows * kStepHead * sizeof(int4));
     e.o_tab = take(rows * step_buckets(e.geo.cpad) * sizeof(uint32_t));
+    e.o_fast = take(rows * step_buckets(e.geo.cpad) * sizeof(uint2));
     e.o_wfix = take((size_t)e.n_seg * b->D * sizeof(longlong2));
     e.o_order = step_ordered(e.geo) ? take((size_t)e.geo.passes * e.geo.n_chunks * e.geo.cpad * 2 * sizeof(int16_t)) : 0;
   }
@@ -361,6 +361,7 @@ StepRowsParams step_rows_of(BatchState* b, const EventHost& e) {
   rp.q = at<int32_t>(b->rows, e.o_q);
   rp.head = at<int4>(b->rows, e.o_head);
   rp.tab = at<uint32_t>(b->rows, e.o_tab);
+  rp.fast = at<uint2>(b->rows, e.o_fast);
   rp.wfix = at<longlong2>(b->rows, e.o_wfix);
   rp.wtot = at<unsigned long long>(b->rows, e.o_wtot);
   return rp;
@@ -382,6 +383,7 @@ StepEvent step_event(const tcw_ctx* c, BatchState* b, const EventHost& e) {
   d.q = rp.q;
   d.head = rp.head;
   d.tab = rp.tab;
+  d.fast = rp.fast;
   d.wfix = rp.wfix;
   d.wtot = reinterpret_cast<const long long*>(rp.wtot);
   d.order = rp.order;

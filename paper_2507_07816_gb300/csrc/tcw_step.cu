@@ -19,10 +19,13 @@ constexpr int kExactSpan = 8;    // boundaries either side of the track that the
 constexpr int kStepTerms = 4;    // fp32 terms of the track beyond the quadratic one
 constexpr int kStepTurn = 16;    // rows whose heads a warp holds (segments of a turn x detectors of a pass)
 // Entries of a warp's list (global memory), and the most that one round of lookups adds: 2 detectors,
-// 7 queue rounds and the lookups themselves.
+// 7 boundaries and the lookups themselves.
 constexpr int kStepSlowMore = 2 * 8 * 32;
 constexpr int kStepSlow = kStepSlowMore + 256;
-constexpr int kStepQueue = 64;   // steps a warp's queue holds: fewer than 32 left over and 32 new ones
+// A threshold's or a sky's place within a bucket of the row's table: 2^-14 of a bucket, biased by a bucket.
+constexpr int kFracBits = 14, kFracShift = 32 - kFracBits;
+constexpr int kErrMax = 0x3ffe;               // largest error bound in these units: anything may be near
+constexpr unsigned kWindowSlow = 1u << 11;    // in a window's first word: not for the fast placing
 
 // Terms of the anchors' series by the size of the step d: the dropped ones,
 // |C(r, K)| d^K with |C(r, K)| <= 1/16 for r <= 1, stay below 2^-56.
@@ -197,9 +200,14 @@ __global__ void __launch_bounds__(kStepMaxChunk) step_order_kernel(StepRowsParam
   }
 }
 
-// Bucket of a threshold (or of a sky's grid value) in a row's table: monotone in v.
-__device__ __forceinline__ int step_bucket(int v, int qmin, float per_unit, int n) {
-  return min((int)((float)((unsigned)v - (unsigned)qmin) * per_unit), n - 1);
+// Place of a threshold (or of a sky's grid value) in a row's table, in 2^-32 of
+// a bucket: exact, so monotone in v.
+__device__ __forceinline__ uint64_t step_place(int v, int qmin, int scale) {
+  return (uint64_t)((unsigned)v - (unsigned)qmin) * (unsigned)scale;
+}
+
+__device__ __forceinline__ int step_bucket(uint64_t place, int n) {
+  return (int)min((unsigned)(place >> 32), (unsigned)n - 1u);
 }
 
 // ---------------------------------------------------------------------------
@@ -208,6 +216,7 @@ __device__ __forceinline__ int step_bucket(int v, int qmin, float per_unit, int 
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(128) step_rows_kernel(StepRowsParams p) {
   __shared__ int s_max[4], s_min[4];
+  __shared__ int s_q[kStepMaxChunk];
   __shared__ uint16_t s_from[step_buckets(kStepMaxChunk)], s_to[step_buckets(kStepMaxChunk)];
   const int d = blockIdx.x % p.n_det, j = blockIdx.x / p.n_det, c = blockIdx.y;
   const int nb = p.cpad / kStepBlock, nk = step_buckets(p.cpad);
@@ -253,15 +262,21 @@ __global__ void __launch_bounds__(128) step_rows_kernel(StepRowsParams p) {
     qmin = min(qmin, s_min[w]);
     qmax = max(qmax, s_max[w]);
   }
-  const float span = (float)((double)qmax - (double)qmin);
-  const float per_unit = span > 0.f ? (float)nk / span : 0.f;
+  const uint64_t span1 = (uint64_t)((unsigned)qmax - (unsigned)qmin) + 1;
+  const int scale = (int)(unsigned)min(((uint64_t)nk << 32) / span1, (uint64_t)0xffffffffu);
   if (g < nb) {
     // Bucket k's window: from the first position whose prefix maximum falls into
     // bucket k or a later one, to the first position whose suffix minimum falls
     // into a later one, with a margin for the error of a threshold.  Position i
     // fills the buckets that it is the first for.
-    auto up = [&](int v) { return step_bucket((int)min((long long)v + p.eps_max, (long long)INT_MAX), qmin, per_unit, nk); };
-    auto down = [&](int v) { return step_bucket((int)max((long long)v - p.eps_max, (long long)qmin), qmin, per_unit, nk); };
+    auto up = [&](int v) {
+      return step_bucket(step_place((int)min((long long)v + p.eps_max, (long long)INT_MAX), qmin, scale), nk);
+    };
+    auto down = [&](int v) {
+      return step_bucket(step_place((int)max((long long)v - p.eps_max, (long long)qmin), qmin, scale), nk);
+    };
+#pragma unroll
+    for (int i = 0; i < kStepBlock; ++i) s_q[g * kStepBlock + i] = qv[i];
     int u = Ue, ub = g > 0 ? up(Ue) : -1;
     int l[kStepBlock];
     int run = Le;
@@ -286,7 +301,22 @@ __global__ void __launch_bounds__(128) step_rows_kernel(StepRowsParams p) {
   }
   __syncthreads();
   uint32_t* tab = p.tab + row * nk;
-  for (int k = threadIdx.x; k < nk; k += blockDim.x) tab[k] = (uint32_t)s_from[k] | (uint32_t)s_to[k] << 11;
+  uint2* fast = p.fast + row * nk;
+  for (int k = threadIdx.x; k < nk; k += blockDim.x) {
+    const int from = s_from[k], to = s_to[k];
+    tab[k] = (uint32_t)from | (uint32_t)to << 11;
+    // the window's skies within the bucket
+    unsigned o[3] = {0xffffu, 0xffffu, 0xffffu};
+    bool slow = to > from + 3;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+      if (from + i < to) {
+        slow = slow || (i > 0 && s_q[from + i] < s_q[from + i - 1]);
+        const long long at = (long long)(step_place(s_q[from + i], qmin, scale) >> kFracShift) - ((long long)k << kFracBits);
+        o[i] = (unsigned)max(min(at + (1 << kFracBits), 65000ll), 0ll);
+      }
+    fast[k] = make_uint2((unsigned)from | (slow ? kWindowSlow : 0u) | o[0] << 16, o[1] | o[2] << 16);
+  }
   if (g == 0) {
     int4* pad = reinterpret_cast<int4*>(p.q + row * step_row(p.cpad) + p.cpad);
     pad[0] = pad[1] = make_int4(qmax, qmax, qmax, qmax);
@@ -295,7 +325,7 @@ __global__ void __launch_bounds__(128) step_rows_kernel(StepRowsParams p) {
     const double tj = p.t_mid[j], dt = tj - ta, d2 = dt * dt;
     const float dth = tj >= p.T0 ? (float)dt : NAN, d2h = (float)d2;
     const float w = p.weights[dj];
-    m[0] = make_int4(qmin, qmax, __float_as_int(per_unit), __float_as_int(w));
+    m[0] = make_int4(qmin, qmax, scale, __float_as_int(w));
     m[1] = make_int4(__float_as_int(dth), __float_as_int((float)(dt - (double)(float)dt)), __float_as_int(d2h),
                      __float_as_int((float)(d2 - (double)d2h)));
     longlong2 wi;
@@ -333,19 +363,20 @@ __global__ void absmax_kernel(const T* x, int64_t n, unsigned* out) {
 }
 
 // Shared memory of the search kernel for `cells` difference cells (templates x
-// (row + 1)): two word planes, the warps' queues of steps (and in their place
-// the piece sums of the epilogue), FP64 and fp32 series coefficients, the heads
-// of each warp's turn, per-template sums.
-static_assert(3 * kStepThreads * 8 <= kStepWarps * kStepQueue * 16, "piece sums fit the queues' place");
+// (row + 1)): two word planes, the heads of each warp's turn (and in their place
+// the piece sums of a pass's end), FP64 and fp32 series coefficients,
+// per-template sums.  What is left of the SM's memory is L1: a smaller layout
+// shows (see step_kernel).
+constexpr size_t kStepPart = 3 * kStepThreads * 8;
+static_assert(kStepWarps * kStepTurn * kStepHead * 16 <= kStepPart, "the heads fit the piece sums' place");
 struct StepLayout {
-  size_t part, coef, fcoef, queue, head, tsum, total;
+  size_t part, coef, fcoef, head, tsum, total;
   __host__ __device__ constexpr explicit StepLayout(int cells)
       : part(((size_t)cells * 8 + 15) & ~(size_t)15),
-        coef(part + (size_t)kStepWarps * kStepQueue * 16),
+        coef(part + kStepPart),
         fcoef(coef + (size_t)kMaxSeriesTerms * 8 * 32),
-        queue(part),
-        head(fcoef + (size_t)32 * 16),
-        tsum(head + (size_t)kStepWarps * kStepTurn * kStepHead * 16),
+        head(part),
+        tsum(fcoef + (size_t)32 * 16),
         total(tsum + (size_t)32 * 4 * 8) {}
 };
 static_assert(StepLayout(kStepCells + 32).total <= 232448 - 1024, "one CTA's shared memory");
@@ -471,7 +502,7 @@ __device__ __forceinline__ void step_rare(const StepParams& p, StepBlockCtx& c, 
     for (int k = 1; k < p.amp_power; ++k) rp *= rr;
     amp = __frcp_rn(rp);
   }
-  const float w = __int_as_float(m0.w) * amp, ws = w * ev.x_scale, per_unit = __int_as_float(m0.z);
+  const float w = __int_as_float(m0.w) * amp, ws = w * ev.x_scale;
   const int64_t vrow =
       ((int64_t)d * ev.n_seg + j) * (VK == 2 && ev.bits ? (int64_t)ev.bit_pitch : p.n_bin);
   const int qmin = m0.x, qmax = m0.y;
@@ -483,7 +514,7 @@ __device__ __forceinline__ void step_rare(const StepParams& p, StepBlockCtx& c, 
     value(K, h0, l0);
     value(K + 1, h1, l1);
     const int dh = h1 - h0, dl = l1 - l0;
-    const uint32_t win = __ldg(ev.tab + row * c.nk + step_bucket(t, qmin, per_unit, c.nk));
+    const uint32_t win = __ldg(ev.tab + row * c.nk + step_bucket(step_place(t, qmin, m0.z), c.nk));
     place_exact(ev.q + row * step_row(c.cpad), win, t, [&](int pos, bool up) {
       int* const cell = c.chi + (pos << (LT + 1)) + lt;
       atomicAdd(cell, up ? dh : -dh);
@@ -703,17 +734,20 @@ __device__ __noinline__ void step_fold(const StepParams& p, StepBlockCtx& s_ctx,
 // skies, two words each) live in shared memory, one column per template.  A
 // lane owns one (template, segment) of its warp's turn: the fp32 track, the
 // first sky's bin, and for each bin boundary inside the chunk's Doppler range a
-// step put on the warp's queue, so that 32 steps are placed at a time whatever
-// their number per lookup.  What fp32 cannot decide (a sky within the
-// threshold's error, about 2 in 1000 steps), skies out of order and lookups at a
-// band edge go on a list that the warp works through at the end of its turn with
-// the exact FP64 thresholds, so that the search loop has no FP64 and no calls.
-// It is bound by instruction latency: about 190 instructions per 32 (template,
-// segment) and 350 more for the steps of 1024 skies, 0.6 and 0.4 issued per
-// scheduler and cycle, nothing saturated; hence 32 warps (24: 3-10 % slower).
+// step, placed by one 8-byte table entry of the threshold's bucket.  What fp32
+// cannot decide (a sky within the threshold's error, about 2 in 1000 steps),
+// skies out of order, crowded buckets and lookups at a band edge go on a list
+// that the warp works through at the end of its turn with the exact FP64
+// thresholds, so that the search loop has no FP64 and no calls.
+// It is bound by the latency of its scattered reads (values and table entries,
+// one per lane): about 150 instructions per 32 (template, segment) and 100 more
+// for each round of steps, 0.66 issued per scheduler and cycle with one sky and
+// 0.45 with 1024, nothing saturated; hence 32 warps (24: 3-10 % slower), and a
+// shared layout that leaves 92 KB of L1 (28 KB: 1.5 times the time).
 // 2e5 templates x 1024 skies x 2 detectors x 1e4 segments: 655 ms by the group
 // kernel, 276 with the track in fp32 pairs and every step searched where it
-// arises, 160 so; one sky and one detector: 205, 50, 24 ms.
+// arises, 160 with steps queued per warp and compared with skies read from the
+// rows, 146 so; one sky and one detector: 205, 50, 24, 22.8 ms.
 template <int VK, int DP, int LT>
 __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int cells) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -729,7 +763,6 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
   long long* const part = reinterpret_cast<long long*>(smem + L.part);
   double* const coef = reinterpret_cast<double*>(smem + L.coef);
   float4* const fcoef = reinterpret_cast<float4*>(smem + L.fcoef);   // [32]: C(e, 3) .. C(e, 6)
-  int4* const queue = reinterpret_cast<int4*>(smem + L.queue) + (threadIdx.x >> 5) * kStepQueue;
   int4* const slow_list = p.slow + ((int64_t)blockIdx.x * kStepWarps + (threadIdx.x >> 5)) * kStepSlow;
   int4* const heads = reinterpret_cast<int4*>(smem + L.head) + (threadIdx.x >> 5) * kStepTurn * kStepHead;
   unsigned long long* const tsum = reinterpret_cast<unsigned long long*>(smem + L.tsum);   // X0, W1, W2 [32]
@@ -767,7 +800,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
     const int lt = lane & (T - 1), ls = lane >> LT;
     constexpr int lps = 32 >> LT;
     const unsigned t_mask = T == 32 ? kAll : (1u << T) - 1u;
-    const int nk = step_buckets(cpad), qs = step_row(cpad);
+    const int nk = step_buckets(cpad);
     const int vpitch = VK == 2 && ev.bits ? ev.bit_pitch : n_bin;
     const int64_t row0 = (int64_t)item.y * n_seg * p.n_det;
     const float xs = ev.x_scale;
@@ -834,15 +867,19 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
             const int jn = min(jce, j0 + (1 << sub));
             const int64_t rbase = row0 + (int64_t)j0 * p.n_det + d0;   // first row of the turn
             const int64_t vbase = ((int64_t)d0 * n_seg + j0) * vpitch;
+            unsigned scale = 0;   // the finest buckets of the turn's rows
             {
               // heads of the turn's rows
               __syncwarp();
               const int nr = (jn - j0) * DP;
               if (lane < nr) {
                 const int4* h = ev.head + (rbase + (int64_t)(lane / DP) * p.n_det + lane % DP) * kStepHead;
-                heads[lane * kStepHead] = __ldg(h);
+                const int4 m = __ldg(h);
+                heads[lane * kStepHead] = m;
+                scale = (unsigned)m.z;
                 heads[lane * kStepHead + 1] = __ldg(h + 1);
               }
+              scale = __reduce_max_sync(kAll, scale);
               __syncwarp();
             }
             // dt at the ends of the turn; NaN before T0
@@ -859,7 +896,9 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
             // The template's bins over the turn (tracks fall, Doppler shifts below 3 bins): wholly in the
             // band, wholly out of it, or at an edge (or T0), which step_rare takes segment by segment
             unsigned at_edge, outside;
-            uint32_t eps;   // the thresholds' error bound at the turn's lowest frequency, as queued
+            // the thresholds' error bound at the turn's lowest frequency in fractions of its finest
+            // buckets
+            int eps;
             {
               const float x0 = fmaf(A_hi, dt_first, fmaf(Q_hi, dt_first * dt_first, (float)base_a));
               const float x1 = fmaf(A_hi, dt_last, fmaf(Q_hi, dt_last * dt_last, (float)base_a));
@@ -869,47 +908,36 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
               outside = __ballot_sync(kAll, out);
               at_edge = __ballot_sync(kAll, !out && !in);
               const float F1 = Xf + (fminf(x0, x1) - (float)base_a);
-              eps = (uint32_t)(int)fmaf(rcp_approx(F1) * p.inv_q_f, p.eps_scale, 1.5f) << 25;
+              const float e = fmaf(rcp_approx(F1) * p.inv_q_f, p.eps, 1.5f) * (float)scale;
+              eps = (int)fminf(fmaf(e, 1.0f / (1 << kFracShift), 3.0f), (float)kErrMax);
             }
             const bool mine = !(((at_edge | outside) >> lane) & 1u);
-            int cnt = 0;     // steps in the warp's queue
-            int nslow = 0;   // steps and lookups in its list
-            // Places the last steps of the queue, one per lane: the sky at which the threshold lies
-            // among the four from the window's start on.  The others go on the list: longer windows,
-            // skies out of order, a sky within the threshold's error.
-            auto drain = [&]() {
-              __syncwarp();
-              const int take = min(cnt, 32);
-              cnt -= take;
-              const bool on = lane < take;
-              // threshold; difference words; row, template; window, step, error
-              const int4 e = on ? queue[cnt + lane] : make_int4(0, 0, 0, 0);
-              const int from = e.w & 0x7ff, to = (e.w >> 11) & 0x7ff;
-              const int32_t* const q = ev.q + ((rbase + ((e.z >> 5) & 0xff)) * qs + from);
-              const int a0 = __ldg(q), a1 = __ldg(q + 1), a2 = __ldg(q + 2), a3 = __ldg(q + 3);
-              const unsigned er = (unsigned)e.w >> 25 << p.eps_shift, lo = (unsigned)e.x - er;
-              const unsigned below = (unsigned)(a0 < e.x) | (unsigned)(a1 < e.x) << 1 | (unsigned)(a2 < e.x) << 2 |
-                                     (unsigned)(a3 < e.x) << 3;
-              const bool near = (unsigned)a0 - lo <= 2u * er || (unsigned)a1 - lo <= 2u * er ||
-                                (unsigned)a2 - lo <= 2u * er || (unsigned)a3 - lo <= 2u * er;
-              const bool slow = on && (near || below == 15u || (below & (below + 1u)) || to > from + 4);
+            int nslow = 0;   // steps and lookups in the warp's list
+            // Places step i of a lookup, one per lane that is on: at the sky at which the threshold lies
+            // among the bucket's.  The others go on the list: longer windows, skies out of order, a sky
+            // within the threshold's error.
+            auto place = [&](bool on, int i, int th, uint32_t at, uint2 w, int dh, int dl, int tag) {
+              const int t = (int)at, o0 = (int)(w.x >> 16), o1 = (int)(w.y & 0xffffu), o2 = (int)(w.y >> 16);
+              const bool near = abs(o0 - t) <= eps || abs(o1 - t) <= eps || abs(o2 - t) <= eps;
+              const bool slow = on && (near || (w.x & kWindowSlow) || eps == kErrMax);
               if (on && !slow) {
-                int* const cell = chi + (((from + __popc(below)) << (LT + 1)) + (e.z & 31));
-                atomicAdd(cell, e.y);
-                atomicAdd(cell + T, e.z >> 13);
+                int* const cell =
+                    chi + ((((int)(w.x & 0x7ffu) + (o0 < t) + (o1 < t) + (o2 < t)) << (LT + 1)) + lt);
+                atomicAdd(cell, dh);
+                atomicAdd(cell + T, dl);
               }
               if (const unsigned vote = __ballot_sync(kAll, slow)) {
-                if (slow) slow_list[nslow + __popc(vote & lt_mask)] = e;
+                // threshold; difference words; row, template; step, error
+                if (slow)
+                  slow_list[nslow + __popc(vote & lt_mask)] = make_int4(th, dh, dl * 8192 | tag, i << 14 | eps);
                 nslow += __popc(vote);
               }
-              __syncwarp();
             };
             const int ns = jn - j0;
             int jb = (at_edge | outside) == kAll ? ns : 0;
             int xh = 0, xl = 0, nx = 0;   // the turn's first-sky powers, each with kMagicBits, and their number
             do {
-            // segments of the turn, then rounds without lookups until the queue is empty
-            for (; (jb < ns || cnt > 0) && nslow <= kStepSlow - kStepSlowMore; jb += lps) {
+            for (; jb < ns && nslow <= kStepSlow - kStepSlowMore; jb += lps) {
               const int jr = min(jb + ls, ns - 1);
               const bool turn = mine && jb + ls < ns;
               const int4* head = heads + jr * DP * kStepHead;
@@ -952,28 +980,33 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
                 const int nb = on ? min((int)(fh - fl), kNThr - 1) : 0;
                 const int K = base_a + 1 + (int)(plr + pqr + fl);   // the lowest sky's bin
                 const int64_t vrow = vbase + (int64_t)(dd * n_seg + jr) * vpitch;
-                // the lookup's loads at once; the queue is drained while they are under way
+                // the loads of the lookup and its first two steps at once
                 const float ws = __int_as_float(m0.w) * amp * xs;
                 const float v0 = on ? step_value<VK>(p, ev, vrow, K) : 0.f;
                 const unsigned some = __ballot_sync(kAll, nb > 0);
-                const uint32_t* const tr = ev.tab + (rbase + rl) * nk;
-                const float per_unit = __int_as_float(m0.z), y1 = fl + 1.0f - y0;
+                const uint2* const tr = ev.fast + (rbase + rl) * nk;
+                const float y1 = fl + 1.0f - y0;
+                auto window = [&](int t, uint32_t& at) {
+                  const uint64_t pl = step_place(t, m0.x, m0.z);
+                  at = ((uint32_t)pl >> kFracShift) + (1u << kFracBits);
+                  return __ldg(tr + step_bucket(pl, nk));
+                };
                 float v1 = 0.f, vn = 0.f;
                 int th0 = 0, th = 0;
-                uint32_t win0 = 0, win = 0;
+                uint2 win0 = make_uint2(0, 0), win = win0;
+                uint32_t at0 = 0, at = 0;
                 if (some) {
                   th0 = __float2int_rn(y1 * R);
                   th = __float2int_rn((y1 + 1.0f) * R);
                   if (nb > 0) {
                     v1 = step_value<VK>(p, ev, vrow, K + 1);
-                    win0 = __ldg(tr + step_bucket(th0, m0.x, per_unit, nk));
+                    win0 = window(th0, at0);
                   }
                   if (nb > 1) {
                     vn = step_value<VK>(p, ev, vrow, K + 2);
-                    win = __ldg(tr + step_bucket(th, m0.x, per_unit, nk));
+                    win = window(th, at);
                   }
                 }
-                if (cnt >= 32 || jb >= ns) drain();
                 int h0, l0, h1, l1;
                 to_fixed(v0, ws, h0, l0);
                 xh += h0;
@@ -981,26 +1014,21 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
                 ++nx;
                 if (some) {
                   to_fixed(v1, ws, h1, l1);
-                  if (nb > 0)
-                    queue[cnt + __popc(some & lt_mask)] =
-                        make_int4(th0, h1 - h0, (l1 - l0) * 8192 | tag, (int)(win0 | eps));
-                  cnt += __popc(some);
-                  for (int i = 1;; ++i) {
-                    const unsigned vote = __ballot_sync(kAll, nb > i);
-                    if (!vote) break;
-                    if (cnt >= 32) drain();
+                  place(nb > 0, 0, th0, at0, win0, h1 - h0, l1 - l0, tag);
+                  for (int i = 1; __any_sync(kAll, nb > i); ++i) {
                     h0 = h1;
                     l0 = l1;
                     to_fixed(vn, ws, h1, l1);
-                    if (nb > i)
-                      queue[cnt + __popc(vote & lt_mask)] =
-                          make_int4(th, h1 - h0, (l1 - l0) * 8192 | tag, (int)(win | (uint32_t)i << 22 | eps));
-                    cnt += __popc(vote);
+                    // the next step's loads before this one's placing
+                    const int th_i = th;
+                    const uint32_t at_i = at;
+                    const uint2 win_i = win;
                     if (nb > i + 1) {
                       vn = step_value<VK>(p, ev, vrow, K + i + 2);
                       th = __float2int_rn((y1 + (float)(i + 1)) * R);
-                      win = __ldg(tr + step_bucket(th, m0.x, per_unit, nk));
+                      win = window(th, at);
                     }
+                    place(nb > i, i, th_i, at_i, win_i, h1 - h0, l1 - l0, tag);
                   }
                 }
                 if (p.amp_power > 0 && on) {
@@ -1014,7 +1042,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
             {
               // the list, and at the end of the turn every (template, row) of templates at a band edge
               const int nr = (jn - j0) * DP;
-              const int n = nslow + (jb < ns || cnt > 0 ? 0 : __popc(at_edge & t_mask) * nr);
+              const int n = nslow + (jb < ns ? 0 : __popc(at_edge & t_mask) * nr);
               for (int i = lane; i < n; i += 32) {
                 int4 e = make_int4(0, 0, 0, -1);
                 if (i < nslow) {
@@ -1026,15 +1054,21 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
                 const int rl = (e.z >> 5) & 0xff, le = e.z & 31;
                 int only = -1;
                 if (e.w != -1) {
-                  const int32_t* const q = ev.q + (rbase + rl) * qs;
-                  const int from = e.w & 0x7ff, to = (e.w >> 11) & 0x7ff;
-                  const unsigned er = (unsigned)e.w >> 25 << p.eps_shift, lo = (unsigned)e.x - er;
-                  bool near = false;
-                  for (int k = from; k < to; ++k) near = near || (unsigned)__ldg(q + k) - lo <= 2u * er;
+                  const int32_t* const q = ev.q + (rbase + rl) * step_row(cpad);
+                  const int4 m = ev.head[(rbase + rl) * kStepHead];
+                  const uint64_t pl = step_place(e.x, m.x, m.z);
+                  const uint32_t win = __ldg(ev.tab + ((rbase + rl) * nk + step_bucket(pl, nk)));
+                  const int er = e.w & 0x3fff;
+                  bool near = er == kErrMax;
+                  for (int k = (int)(win & 0x7ffu); k < (int)(win >> 11); ++k) {
+                    const long long off = (long long)(step_place(__ldg(q + k), m.x, m.z) >> kFracShift) -
+                                          (long long)(pl >> kFracShift);
+                    near = near || llabs(off) <= er;
+                  }
                   if (near) {
-                    only = (e.w >> 22) & 7;
+                    only = e.w >> 14;
                   } else {
-                    place_exact(q, (uint32_t)e.w & 0x3fffffu, e.x, [&](int pos, bool up) {
+                    place_exact(q, win, e.x, [&](int pos, bool up) {
                       int* const cell = chi + ((pos << (LT + 1)) + le);
                       atomicAdd(cell, up ? e.y : -e.y);
                       atomicAdd(cell + T, up ? e.z >> 13 : -(e.z >> 13));
@@ -1047,7 +1081,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
               nslow = 0;
               __syncwarp();
             }
-            } while (jb < ns || cnt > 0);
+            } while (jb < ns);
             X0 += (long long)(xh - nx * kMagicBits) * 65536 + (xl - nx * kMagicBits);
             {
               const int nr = (jn - j0) * DP;
@@ -1201,13 +1235,12 @@ StepTrack step_track(const double* t_mid, int64_t n_seg, double T0, int most, do
     // roundings of 6e-8 of y (F, 1/F, their products) for y = db + 1 bins
     // at most; emulated worst cases stay below 0.7 of it.
     r.eps = (float)(3.0e-7 + 1.2e-7 * (2.0 + db) + 2.4e-7 * (1.0 + db));
-    // in grid units (most at the lowest frequency): 7 bits of 2^eps_shift units
+    // in grid units, most at the lowest frequency
     const double f_low = std::max(f_min / df - 8.0, 0.0);
     if (!(f_low >= 64.0)) return r;
     const double worst = r.eps * inv_q / f_low;
-    while (std::ldexp(worst, -r.eps_shift) > 120.0) ++r.eps_shift;
-    if (r.eps_shift > 20) return r;
-    r.eps_max = (int)std::ldexp(std::ceil(std::ldexp(worst, -r.eps_shift)) + 2.0, r.eps_shift);
+    if (!(worst < 120.0 * (1 << 20))) return r;
+    r.eps_max = (int)std::ceil(worst) + 2;
     r.ok = true;
     return r;
   }

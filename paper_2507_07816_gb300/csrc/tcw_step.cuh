@@ -29,13 +29,16 @@ constexpr int kStepCells = 16384;      // difference cells of a CTA: chunk x tem
 // detector), cpad skies in the order of their pass (a multiple of kStepBlock;
 // the last sky repeated):
 //   q     [step_row(cpad)]  floor(v.nhat/c / q-grid step), then the largest repeated
-//   head  {qmin, qmax, buckets per grid unit (float bits), w (float bits)}: the
+//   head  {qmin, qmax, buckets per grid unit (32 fraction bits), w (float bits)}: the
 //         smallest and largest q; {dt hi, dt lo, dt^2 hi, dt^2 lo}: t_j - t_a from
 //         the tile's anchor time and its square as fp32 pairs (dt hi NaN before T0)
 //   wfix  {W1 word, W2 word}: w and w^2 in fixed point (int64 each)
 //   tab   per bucket of thresholds {first position not below all of them, first
 //         position from which on every sky reaches all of them}, 11 bits each:
 //         only the skies between the two are compared with a threshold
+//   fast  the same in one load: {first position, a flag for windows of more than 3
+//         skies or out of order, place of the first sky; places of the second and
+//         third}, places in 2^-14 buckets from the start of the bucket before on
 // Track constants of one (template, tile), the position x = (f - f_min)/df of
 // the unshifted track (Eq. 1) around the anchor time t_a: x = base + frac +
 // A dt + Q dt^2 + X (cubic and higher terms in dt s).
@@ -58,6 +61,7 @@ struct StepEvent {
   const int32_t* q;          // [n_chunks][n_seg][D][step_row(cpad)]
   const int4* head;          // [n_chunks][n_seg][D][kStepHead]
   const uint32_t* tab;       // [n_chunks][n_seg][D][step_buckets(cpad)]
+  const uint2* fast;         // [n_chunks][n_seg][D][step_buckets(cpad)]
   const longlong2* wfix;     // [n_seg][D]
   const long long* wtot;     // [kStepSlots][2]: partial sums of w and w^2 over the segments from T0 on
   const int16_t* order;      // [passes][n_chunks][cpad] sky (in the chunk) at a position; null for one pass
@@ -89,8 +93,6 @@ struct StepParams {
   double f_min, df, inv_q;
   float q, inv_q_f;
   float eps;                 // bound of the fp32 thresholds' error, in bins
-  float eps_scale;           // the same as a count of 2^eps_shift grid units, per (1/F)/q
-  int eps_shift;
   int nterms, tile_shift;    // FP64 track series (> 0), anchor tiles
   float df_f;
   int amp_power;
@@ -119,6 +121,7 @@ struct StepRowsParams {
   int32_t* q;
   int4* head;
   uint32_t* tab;
+  uint2* fast;
   longlong2* wfix;
   unsigned long long* wtot;  // zero at launch
 };
@@ -164,14 +167,12 @@ struct StepTrack {
   bool ok = false;
   int shift = 0, nterms = 0;
   float eps = 0;             // bins
-  int eps_shift = 0, eps_max = 0;
+  int eps_max = 0;           // in grid units
 };
 StepTrack step_track(const double* t_mid, int64_t n_seg, double T0, int most, double tau_min, double r_max,
                      double x_max, double db, double f_min, double df, double inv_q);
 inline void set_step_track(StepParams& p, const StepTrack& t) {
   p.eps = t.eps;
-  p.eps_shift = t.eps_shift;
-  p.eps_scale = std::ldexp(t.eps, -t.eps_shift);
   p.nterms = t.nterms;
   p.tile_shift = t.shift;
 }

@@ -130,3 +130,15 @@ def test_long_sfts_take_short_tiles():
     p = syn.Problem(syn.exponential_noise(r, (2, 90, 8000)), t, syn.uniform_weights(r, 2, 90), vel, 500.0, 1 / 32.0,
                     float(t[0] - 16.0), syn.random_sky(r, 300), bank, [], dets, name="32 s")
     check(p)
+
+
+@pytest.mark.parametrize("cluster,width", [(3, 1e-12), (4, 1e-12), (5, 1e-7), (40, 1e-4)])
+def test_crowded_skies(cluster, width):
+    """Skies in clusters narrower than a bucket of thresholds (below and above the 3
+    skies of a fast window), at distances from below to far above the thresholds'
+    error."""
+    p = problem(1100 + cluster, 2, 40, 120, 50)
+    r = syn.rng(1200 + cluster)
+    n = np.repeat(p.nhat[::cluster], cluster, axis=0)[:120] + width * r.normal(size=(120, 3))
+    p.nhat = np.ascontiguousarray(n / np.linalg.norm(n, axis=1, keepdims=True))
+    check(p)

@@ -13,7 +13,7 @@ constexpr int kStepThreads = 1024;
 constexpr int kStepWarps = kStepThreads / 32;
 // Segments between two normalisations of the difference cells: a cell's low
 // word takes at most 8 bin differences of at most 2^16 per (segment, detector),
-// 2 detectors, so 2^11 segments stay within 2^31.
+// 2 detectors, so 2^11 segments stay within 2^31 (and their rows within 12 bits).
 constexpr int kStepCarry = 2048;
 constexpr int kExactSpan = 8;    // boundaries either side of the track that the exact search goes to
 constexpr int kStepTerms = 4;    // fp32 terms of the track beyond the quadratic one
@@ -22,6 +22,7 @@ constexpr int kStepTurn = 16;    // rows whose heads a warp holds (segments of a
 // 7 boundaries and the lookups themselves.
 constexpr int kStepSlowMore = 2 * 8 * 32;
 constexpr int kStepSlow = kStepSlowMore + 256;
+constexpr int kStepLookup = 7;   // in place of a step's number: the whole lookup
 // A threshold's or a sky's place within a bucket of the row's table: 2^-14 of a bucket, biased by a bucket.
 constexpr int kFracBits = 14, kFracShift = 32 - kFracBits;
 constexpr int kErrMax = 0x3ffe;               // largest error bound in these units: anything may be near
@@ -406,6 +407,36 @@ __device__ __forceinline__ float step_value(const StepParams& p, const StepEvent
   }
 }
 
+// Read-only loads of the lanes that are on, without a branch (0 elsewhere).
+__device__ __forceinline__ float load_if(const float* p, bool on) {
+  float v;
+  asm("{\n.reg .pred q;\nsetp.ne.s32 q, %2, 0;\nmov.f32 %0, 0f00000000;\n@q ld.global.nc.f32 %0, [%1];\n}"
+      : "=&f"(v)
+      : "l"(p), "r"((int)on));
+  return v;
+}
+__device__ __forceinline__ float load_if(const __half* p, bool on) {
+  unsigned short v;
+  asm("{\n.reg .pred q;\nsetp.ne.s32 q, %2, 0;\nmov.u16 %0, 0;\n@q ld.global.nc.u16 %0, [%1];\n}"
+      : "=&h"(v)
+      : "l"(p), "r"((int)on));
+  return __half2float(__ushort_as_half(v));
+}
+__device__ __forceinline__ uint2 load_if(const uint2* p, bool on) {
+  uint2 v;
+  asm("{\n.reg .pred q;\nsetp.ne.s32 q, %3, 0;\nmov.u32 %0, 0;\nmov.u32 %1, 0;\n@q ld.global.nc.v2.u32 {%0, %1}, [%2];\n}"
+      : "=&r"(v.x), "=&r"(v.y)
+      : "l"(p), "r"((int)on));
+  return v;
+}
+// Adds hi and lo to two shared words OFF bytes apart on the lanes that are on.
+template <int OFF>
+__device__ __forceinline__ void add_if(uint32_t cell, int hi, int lo, bool on) {
+  asm volatile("{\n.reg .pred q;\nsetp.ne.s32 q, %3, 0;\n@q red.shared.add.s32 [%0], %1;\n@q red.shared.add.s32 [%0+%4], %2;\n}"
+               :
+               : "r"(cell), "r"(hi), "r"(lo), "r"((int)on), "n"(OFF));
+}
+
 // v * s rounded to the fixed-point grid: hi + lo 2^-16 with |lo| <= 2^15
 // (|v s| < 2^22), each word plus kMagicBits, which cancels in differences.  The
 // product is never rounded before the grid.
@@ -737,8 +768,9 @@ __device__ __noinline__ void step_fold(const StepParams& p, StepBlockCtx& s_ctx,
 // step, placed by one 8-byte table entry of the threshold's bucket.  What fp32
 // cannot decide (a sky within the threshold's error, about 2 in 1000 steps),
 // skies out of order, crowded buckets and lookups at a band edge go on a list
-// that the warp works through at the end of its turn with the exact FP64
-// thresholds, so that the search loop has no FP64 and no calls.
+// that the warp works through with the exact FP64 thresholds once it is full or
+// the pass moves on, with all its lanes, so that the search loop has no FP64 and
+// no calls and few spills.
 // It is bound by the latency of its scattered reads (values and table entries,
 // one per lane): about 150 instructions per 32 (template, segment) and 100 more
 // for each round of steps, 0.66 issued per scheduler and cycle with one sky and
@@ -747,7 +779,9 @@ __device__ __noinline__ void step_fold(const StepParams& p, StepBlockCtx& s_ctx,
 // 2e5 templates x 1024 skies x 2 detectors x 1e4 segments: 655 ms by the group
 // kernel, 276 with the track in fp32 pairs and every step searched where it
 // arises, 160 with steps queued per warp and compared with skies read from the
-// rows, 146 so; one sky and one detector: 205, 50, 24, 22.8 ms.
+// rows, 146 with the list worked through turn by turn, 139 so; one sky and one
+// detector: 205, 50, 24, 22.8, 22.6 ms; 8 events of 100-800 skies and 1.2e4
+// templates: 121 ms by the group kernel, 19.2 turn by turn, 16.9 so.
 template <int VK, int DP, int LT>
 __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int cells) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -856,15 +890,60 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
         const int js = pass / per * ev.pass_seg, je = min(n_seg, js + ev.pass_seg);
         for (int jc = js; jc < je; jc += kStepCarry) {
           const int jce = min(je, jc + kStepCarry);
-          // the warps take the turns as they come: their lengths in time differ
+          // The warps take the turns as they come: their lengths in time differ.  The last turn's worth of
+          // each warp goes in quarters, so that the warps end a pass closer together.
+          const int small = min(sub, max(sub - 2, 2)), big = max(0, ((jce - jc) >> sub) - kStepWarps);
           if (tid == 0) s_turn = 0;
           __syncthreads();
+          int j0 = 0, jn = 0;   // the warp's turn: segments left to it
+          int nslow = 0;        // steps and lookups in the warp's list
           while (true) {
-            int j0 = 0;
-            if (lane == 0) j0 = jc + (atomicAdd(&s_turn, 1) << sub);
-            j0 = __shfl_sync(kAll, j0, 0);
-            if (j0 >= jce) break;
-            const int jn = min(jce, j0 + (1 << sub));
+            if (j0 >= jn) {
+              int turn = 0;
+              if (lane == 0) turn = atomicAdd(&s_turn, 1);
+              turn = __shfl_sync(kAll, turn, 0);
+              j0 = jc + (turn < big ? turn << sub : (big << sub) + ((turn - big) << small));
+              jn = min(jce, j0 + (1 << (turn < big ? sub : small)));
+            }
+            const bool end = j0 >= jce;
+            if (nslow > kStepSlow - kStepSlowMore || (end && nslow > 0)) {
+              // the list, when it fills up and before the pass moves on
+              __syncwarp();
+              const int64_t row1 = row0 + (int64_t)jc * p.n_det + d0;
+              for (int i = lane; i < nslow; i += 32) {
+                const int4 e = __ldcg(slow_list + i);
+                const int rr = e.w >> 17, le = e.z & 31, dl = e.z >> 5;
+                int only = e.w >> 14 & 7;
+                if (only != kStepLookup) {
+                  const int64_t row = row1 + (int64_t)(rr / DP) * p.n_det + rr % DP;
+                  const int32_t* const q = ev.q + row * step_row(cpad);
+                  const int4 m = ev.head[row * kStepHead];
+                  const uint64_t pl = step_place(e.x, m.x, m.z);
+                  const uint32_t win = __ldg(ev.tab + (row * nk + step_bucket(pl, nk)));
+                  const int er = e.w & 0x3fff;
+                  bool near = er == kErrMax;
+                  for (int k = (int)(win & 0x7ffu); k < (int)(win >> 11); ++k) {
+                    const long long off = (long long)(step_place(__ldg(q + k), m.x, m.z) >> kFracShift) -
+                                          (long long)(pl >> kFracShift);
+                    near = near || llabs(off) <= er;
+                  }
+                  if (!near) {
+                    place_exact(q, win, e.x, [&](int pos, bool up) {
+                      int* const cell = chi + ((pos << (LT + 1)) + le);
+                      atomicAdd(cell, up ? e.y : -e.y);
+                      atomicAdd(cell + T, up ? dl : -dl);
+                    });
+                    continue;
+                  }
+                } else {
+                  only = -1;
+                }
+                step_rare<VK, LT>(p, s_ctx, le, jc + rr / DP, d0 + rr % DP, only);
+              }
+              nslow = 0;
+              __syncwarp();
+            }
+            if (end) break;
             const int64_t rbase = row0 + (int64_t)j0 * p.n_det + d0;   // first row of the turn
             const int64_t vbase = ((int64_t)d0 * n_seg + j0) * vpitch;
             unsigned scale = 0;   // the finest buckets of the turn's rows
@@ -885,7 +964,10 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
             // dt at the ends of the turn; NaN before T0
             const float dt_first = __int_as_float(heads[1].x);
             const float dt_last = __int_as_float(heads[((jn - j0) * DP - 1) * kStepHead + 1].x);
-            if (!(dt_last == dt_last)) continue;
+            if (!(dt_last == dt_last)) {
+              j0 = jn;
+              continue;
+            }
             const int4* tp =
                 reinterpret_cast<const int4*>(ev.tiles + ((int64_t)b * ev.n_tiles + (j0 >> p.tile_shift)));
             const int4 t0 = __ldg(tp), t1 = __ldg(tp + 1);
@@ -894,8 +976,9 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
             const float Q_hi = __int_as_float(t1.x), Q_lo = __int_as_float(t1.y), Xf = __int_as_float(t1.z),
                         sg = __int_as_float(t1.w);
             // The template's bins over the turn (tracks fall, Doppler shifts below 3 bins): wholly in the
-            // band, wholly out of it, or at an edge (or T0), which step_rare takes segment by segment
-            unsigned at_edge, outside;
+            // band, wholly out of it, or at an edge (or T0): every lookup goes on the list
+            bool edge;
+            unsigned outside;
             // the thresholds' error bound at the turn's lowest frequency in fractions of its finest
             // buckets
             int eps;
@@ -906,40 +989,39 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
               const bool in = whole && fminf(x0, x1) >= 8.0f && fmaxf(x0, x1) <= (float)n_bin - 10.0f;
               const bool out = whole && (fmaxf(x0, x1) < -8.0f || fminf(x0, x1) > (float)n_bin + 8.0f);
               outside = __ballot_sync(kAll, out);
-              at_edge = __ballot_sync(kAll, !out && !in);
+              edge = !out && !in;
               const float F1 = Xf + (fminf(x0, x1) - (float)base_a);
               const float e = fmaf(rcp_approx(F1) * p.inv_q_f, p.eps, 1.5f) * (float)scale;
               eps = (int)fminf(fmaf(e, 1.0f / (1 << kFracShift), 3.0f), (float)kErrMax);
             }
-            const bool mine = !(((at_edge | outside) >> lane) & 1u);
-            int nslow = 0;   // steps and lookups in the warp's list
+            const bool mine = !((outside >> lane) & 1u);
+            // a row's number within the segments from jc on, in place
+            const int rr0 = (j0 - jc) * DP;
+            const uint32_t cells0 = (uint32_t)__cvta_generic_to_shared(chi + lt);
             // Places step i of a lookup, one per lane that is on: at the sky at which the threshold lies
             // among the bucket's.  The others go on the list: longer windows, skies out of order, a sky
             // within the threshold's error.
-            auto place = [&](bool on, int i, int th, uint32_t at, uint2 w, int dh, int dl, int tag) {
-              const int t = (int)at, o0 = (int)(w.x >> 16), o1 = (int)(w.y & 0xffffu), o2 = (int)(w.y >> 16);
-              const bool near = abs(o0 - t) <= eps || abs(o1 - t) <= eps || abs(o2 - t) <= eps;
-              const bool slow = on && (near || (w.x & kWindowSlow) || eps == kErrMax);
-              if (on && !slow) {
-                int* const cell =
-                    chi + ((((int)(w.x & 0x7ffu) + (o0 < t) + (o1 < t) + (o2 < t)) << (LT + 1)) + lt);
-                atomicAdd(cell, dh);
-                atomicAdd(cell + T, dl);
-              }
+            auto place = [&](bool on, int i, int th, uint32_t at, uint2 w, int dh, int dl, int rr) {
+              const int low = (int)at - eps;
+              const int o0 = (int)(w.x >> 16) - low, o1 = (int)(w.y & 0xffffu) - low, o2 = (int)(w.y >> 16) - low;
+              const unsigned wide = 2u * (unsigned)eps;
+              const bool slow = on && ((unsigned)o0 <= wide || (unsigned)o1 <= wide || (unsigned)o2 <= wide ||
+                                       (w.x & kWindowSlow) || eps == kErrMax);
+              const int pos = (int)(w.x & 0x7ffu) + (o0 < eps) + (o1 < eps) + (o2 < eps);
+              add_if<T * 4>(cells0 + (uint32_t)(pos << (LT + 3)), dh, dl, on && !slow);
               if (const unsigned vote = __ballot_sync(kAll, slow)) {
-                // threshold; difference words; row, template; step, error
+                // threshold; difference words, template; row, step, error
                 if (slow)
-                  slow_list[nslow + __popc(vote & lt_mask)] = make_int4(th, dh, dl * 8192 | tag, i << 14 | eps);
+                  slow_list[nslow + __popc(vote & lt_mask)] = make_int4(th, dh, dl * 32 | lt, rr << 17 | i << 14 | eps);
                 nslow += __popc(vote);
               }
             };
             const int ns = jn - j0;
-            int jb = (at_edge | outside) == kAll ? ns : 0;
+            int jb = outside == kAll ? ns : 0;
             int xh = 0, xl = 0, nx = 0;   // the turn's first-sky powers, each with kMagicBits, and their number
-            do {
             for (; jb < ns && nslow <= kStepSlow - kStepSlowMore; jb += lps) {
               const int jr = min(jb + ls, ns - 1);
-              const bool turn = mine && jb + ls < ns;
+              const bool here = mine && jb + ls < ns;
               const int4* head = heads + jr * DP * kStepHead;
               const float4 dt = *reinterpret_cast<const float4*>(head + 1);
               // the unshifted track's position base + frac and F = f/df (see StepTile): the linear and
@@ -958,7 +1040,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
               const float F = (Xf + pl) + (pq + p3);
               float amp = 1.0f;
               if (p.amp_power > 0) {
-                const float rr = turn ? F * famp : 1.0f;   // f / f0
+                const float rr = here && !edge ? F * famp : 1.0f;   // f / f0
                 amp = rr;
                 for (int k = 1; k < p.amp_power; ++k) amp *= rr;
               }
@@ -970,11 +1052,13 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
                 // the lowest and the highest sky's distance from boundary 0, in bins: boundaries in between
                 const float zl = fmaf(Fq, (float)m0.x, y0), zh = fmaf(Fq, (float)m0.y, y0);
                 const float fl = floorf(zl), fh = floorf(zh);
-                const bool close = turn && (fabsf((zl - fl) - 0.5f) > 0.5f - p.eps || fabsf((zh - fh) - 0.5f) > 0.5f - p.eps);
-                const bool on = turn && !close;
-                const int rl = jr * p.n_det + dd, tag = rl << 5 | lt;
+                const bool close = here && (edge || fabsf((zl - fl) - 0.5f) > 0.5f - p.eps ||
+                                            fabsf((zh - fh) - 0.5f) > 0.5f - p.eps);
+                const bool on = here && !close;
+                const int rl = jr * p.n_det + dd, rr = rr0 + jr * DP + dd;
                 if (const unsigned vote = __ballot_sync(kAll, close)) {
-                  if (close) slow_list[nslow + __popc(vote & lt_mask)] = make_int4(0, 0, tag, -1);
+                  if (close)
+                    slow_list[nslow + __popc(vote & lt_mask)] = make_int4(0, 0, lt, rr << 17 | kStepLookup << 14);
                   nslow += __popc(vote);
                 }
                 const int nb = on ? min((int)(fh - fl), kNThr - 1) : 0;
@@ -982,14 +1066,19 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
                 const int64_t vrow = vbase + (int64_t)(dd * n_seg + jr) * vpitch;
                 // the loads of the lookup and its first two steps at once
                 const float ws = __int_as_float(m0.w) * amp * xs;
-                const float v0 = on ? step_value<VK>(p, ev, vrow, K) : 0.f;
+                auto value = [&](int o, bool c) {   // of bin K + o
+                  if constexpr (VK == 0) return load_if(static_cast<const float*>(ev.rho) + (vrow + K) + o, c);
+                  else if constexpr (VK == 1) return load_if(static_cast<const __half*>(ev.rho) + (vrow + K) + o, c);
+                  else return c ? step_value<VK>(p, ev, vrow, K + o) : 0.f;
+                };
+                const float v0 = value(0, on);
                 const unsigned some = __ballot_sync(kAll, nb > 0);
                 const uint2* const tr = ev.fast + (rbase + rl) * nk;
                 const float y1 = fl + 1.0f - y0;
-                auto window = [&](int t, uint32_t& at) {
+                auto window = [&](int t, uint32_t& at, bool c) {
                   const uint64_t pl = step_place(t, m0.x, m0.z);
                   at = ((uint32_t)pl >> kFracShift) + (1u << kFracBits);
-                  return __ldg(tr + step_bucket(pl, nk));
+                  return load_if(tr + step_bucket(pl, nk), c);
                 };
                 float v1 = 0.f, vn = 0.f;
                 int th0 = 0, th = 0;
@@ -998,14 +1087,10 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
                 if (some) {
                   th0 = __float2int_rn(y1 * R);
                   th = __float2int_rn((y1 + 1.0f) * R);
-                  if (nb > 0) {
-                    v1 = step_value<VK>(p, ev, vrow, K + 1);
-                    win0 = window(th0, at0);
-                  }
-                  if (nb > 1) {
-                    vn = step_value<VK>(p, ev, vrow, K + 2);
-                    win = window(th, at);
-                  }
+                  v1 = value(1, nb > 0);
+                  win0 = window(th0, at0, nb > 0);
+                  vn = value(2, nb > 1);
+                  win = window(th, at, nb > 1);
                 }
                 int h0, l0, h1, l1;
                 to_fixed(v0, ws, h0, l0);
@@ -1014,7 +1099,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
                 ++nx;
                 if (some) {
                   to_fixed(v1, ws, h1, l1);
-                  place(nb > 0, 0, th0, at0, win0, h1 - h0, l1 - l0, tag);
+                  place(nb > 0, 0, th0, at0, win0, h1 - h0, l1 - l0, rr);
                   for (int i = 1; __any_sync(kAll, nb > i); ++i) {
                     h0 = h1;
                     l0 = l1;
@@ -1023,12 +1108,10 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
                     const int th_i = th;
                     const uint32_t at_i = at;
                     const uint2 win_i = win;
-                    if (nb > i + 1) {
-                      vn = step_value<VK>(p, ev, vrow, K + i + 2);
-                      th = __float2int_rn((y1 + (float)(i + 1)) * R);
-                      win = window(th, at);
-                    }
-                    place(nb > i, i, th_i, at_i, win_i, h1 - h0, l1 - l0, tag);
+                    vn = value(i + 2, nb > i + 1);
+                    th = __float2int_rn((y1 + (float)(i + 1)) * R);
+                    win = window(th, at, nb > i + 1);
+                    place(nb > i, i, th_i, at_i, win_i, h1 - h0, l1 - l0, rr);
                   }
                 }
                 if (p.amp_power > 0 && on) {
@@ -1038,53 +1121,9 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
                 }
               }
             }
-            __syncwarp();
-            {
-              // the list, and at the end of the turn every (template, row) of templates at a band edge
-              const int nr = (jn - j0) * DP;
-              const int n = nslow + (jb < ns ? 0 : __popc(at_edge & t_mask) * nr);
-              for (int i = lane; i < n; i += 32) {
-                int4 e = make_int4(0, 0, 0, -1);
-                if (i < nslow) {
-                  e = __ldcg(slow_list + i);
-                } else {
-                  const int r = (i - nslow) % nr;
-                  e.z = (r / DP * p.n_det + r % DP) << 5 | __fns(at_edge & t_mask, 0, (i - nslow) / nr + 1);
-                }
-                const int rl = (e.z >> 5) & 0xff, le = e.z & 31;
-                int only = -1;
-                if (e.w != -1) {
-                  const int32_t* const q = ev.q + (rbase + rl) * step_row(cpad);
-                  const int4 m = ev.head[(rbase + rl) * kStepHead];
-                  const uint64_t pl = step_place(e.x, m.x, m.z);
-                  const uint32_t win = __ldg(ev.tab + ((rbase + rl) * nk + step_bucket(pl, nk)));
-                  const int er = e.w & 0x3fff;
-                  bool near = er == kErrMax;
-                  for (int k = (int)(win & 0x7ffu); k < (int)(win >> 11); ++k) {
-                    const long long off = (long long)(step_place(__ldg(q + k), m.x, m.z) >> kFracShift) -
-                                          (long long)(pl >> kFracShift);
-                    near = near || llabs(off) <= er;
-                  }
-                  if (near) {
-                    only = e.w >> 14;
-                  } else {
-                    place_exact(q, win, e.x, [&](int pos, bool up) {
-                      int* const cell = chi + ((pos << (LT + 1)) + le);
-                      atomicAdd(cell, up ? e.y : -e.y);
-                      atomicAdd(cell + T, up ? e.z >> 13 : -(e.z >> 13));
-                    });
-                    continue;
-                  }
-                }
-                step_rare<VK, LT>(p, s_ctx, le, j0 + rl / p.n_det, d0 + rl % p.n_det, only);
-              }
-              nslow = 0;
-              __syncwarp();
-            }
-            } while (jb < ns);
             X0 += (long long)(xh - nx * kMagicBits) * 65536 + (xl - nx * kMagicBits);
             {
-              const int nr = (jn - j0) * DP;
+              const int nr = min(jb, ns) * DP;
               if ((outside & t_mask) && p.amp_power == 0) {
                 // out of the band: the turn's weights come off
                 longlong2 wi = make_longlong2(0, 0);
@@ -1103,6 +1142,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
               }
               __syncwarp();
             }
+            j0 += min(jb, ns);   // less than the turn when the list is full
           }
           if (jce < je) {
             // carry the low words over before they can overflow

@@ -224,15 +224,15 @@ tcw_status plan_batch(tcw_ctx* c, BatchState* b) {
   return TCW_OK;
 }
 
-// The step-function search for tiles of at most `tile` segments: its track and
-// tile length (common to the batch), every event's scales and passes.  b->step =
+// The step-function search for anchor tiles of `tile` segments (its own: twice
+// as many at most): its track and tile length (common to the batch), every event's scales and passes.  b->step =
 // false when some event does not meet its conditions.
 void plan_step(const tcw_ctx* c, BatchState* b, int tile) {
   b->step = false;
   const bool count = c->statistic == TCW_STAT_NUMBER_COUNT;
   const double f_top = b->f_min + (double)b->n_bin * b->df;
   b->track = StepTrack{};
-  b->track.shift = ilog2(tile);
+  b->track.shift = ilog2(2 * tile);
   for (int round = 0; round < 2; ++round) {
     // the shortest tile that an event needs, then every event with it
     const int most = 1 << b->track.shift;

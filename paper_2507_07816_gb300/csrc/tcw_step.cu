@@ -16,7 +16,7 @@ constexpr int kStepWarps = kStepThreads / 32;
 // 2 detectors, so 2^11 segments stay within 2^31 (and their rows within 12 bits).
 constexpr int kStepCarry = 2048;
 constexpr int kExactSpan = 8;    // boundaries either side of the track that the exact search goes to
-constexpr int kStepTerms = 4;    // fp32 terms of the track beyond the quadratic one
+constexpr int kStepTerms = 5;    // fp32 terms of the track beyond the quadratic one
 constexpr int kStepTurn = 16;    // rows whose heads a warp holds (segments of a turn x detectors of a pass)
 // Entries of a warp's list (global memory), and the most that one round of lookups adds: 2 detectors,
 // 7 boundaries and the lookups themselves.
@@ -377,7 +377,7 @@ struct StepLayout {
         coef(part + kStepPart),
         fcoef(coef + (size_t)kMaxSeriesTerms * 8 * 32),
         head(part),
-        tsum(fcoef + (size_t)32 * 16),
+        tsum(fcoef + (size_t)32 * 20),
         total(tsum + (size_t)32 * 4 * 8) {}
 };
 static_assert(StepLayout(kStepCells + 32).total <= 232448 - 1024, "one CTA's shared memory");
@@ -797,6 +797,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
   long long* const part = reinterpret_cast<long long*>(smem + L.part);
   double* const coef = reinterpret_cast<double*>(smem + L.coef);
   float4* const fcoef = reinterpret_cast<float4*>(smem + L.fcoef);   // [32]: C(e, 3) .. C(e, 6)
+  float* const fcoef7 = reinterpret_cast<float*>(fcoef + 32);        // [32]: C(e, 7)
   int4* const slow_list = p.slow + ((int64_t)blockIdx.x * kStepWarps + (threadIdx.x >> 5)) * kStepSlow;
   int4* const heads = reinterpret_cast<int4*>(smem + L.head) + (threadIdx.x >> 5) * kStepTurn * kStepHead;
   unsigned long long* const tsum = reinterpret_cast<unsigned long long*>(smem + L.tsum);   // X0, W1, W2 [32]
@@ -881,6 +882,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
           cf[k] = (float)c;
         }
         fcoef[tid] = make_float4(cf[0], cf[1], cf[2], cf[3]);
+        fcoef7[tid] = cf[4];
       }
       __syncthreads();
       long long X0 = 0;
@@ -1031,7 +1033,8 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
               const float pq = Q_hi * dt.z, pqr = rintf(pq);
               const float dl3 = dt.x * sg;
               const float4 cf = fcoef[lt];
-              float hs = fmaf(cf.w, dl3, cf.z);
+              float hs = fmaf(fcoef7[lt], dl3, cf.w);
+              hs = fmaf(hs, dl3, cf.z);
               hs = fmaf(hs, dl3, cf.y);
               hs = fmaf(hs, dl3, cf.x);
               const float p3 = Xf * (dl3 * dl3 * dl3 * hs);
@@ -1264,17 +1267,17 @@ StepTrack step_track(const double* t_mid, int64_t n_seg, double T0, int most, do
       dmax = std::max(dmax, std::max(te - ta, ta - std::max(t_mid[j0], T0)) / (tau_min + (ta - T0)));
     }
     // the series' dropped terms and the fp32 rounding of its cubic part, in bins
-    if (!(dmax <= 0.1) || x_max * cbound(3) * std::pow(dmax, 3) > 0.15 ||
+    if (!(dmax <= 0.1) || x_max * cbound(3) * std::pow(dmax, 3) > 0.25 ||
         x_max * cbound(kStepTerms + 3) * std::pow(dmax, kStepTerms + 3) > 2e-8 || x_max * r_max * dmax > 2.0e6)
       continue;
     r.nterms = series_terms_for(t_mid, n_seg, T0, tile, tau_min, r_max);
     if (r.nterms < 1) continue;
     r.shift = shift;
     // Error of an fp32 threshold: the position's sums (values up to 2) and the
-    // cubic part 3e-7, the difference to the boundary 1.2e-7 (1 + y), and four
+    // cubic part 4e-7, the difference to the boundary 1.2e-7 (1 + y), and four
     // roundings of 6e-8 of y (F, 1/F, their products) for y = db + 1 bins
     // at most; emulated worst cases stay below 0.7 of it.
-    r.eps = (float)(3.0e-7 + 1.2e-7 * (2.0 + db) + 2.4e-7 * (1.0 + db));
+    r.eps = (float)(4.0e-7 + 1.2e-7 * (2.0 + db) + 2.4e-7 * (1.0 + db));
     // in grid units, most at the lowest frequency
     const double f_low = std::max(f_min / df - 8.0, 0.0);
     if (!(f_low >= 64.0)) return r;

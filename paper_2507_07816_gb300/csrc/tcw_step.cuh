@@ -161,7 +161,9 @@ inline void set_step_geometry(StepRowsParams& p, const StepGeometry& g) {
 inline bool step_ordered(const StepGeometry& g) { return g.passes > 1; }
 
 // The fp32 track's tiles and error bound: tile = 1 << shift segments (at most
-// `most`), the FP64 series' terms, and the thresholds' error; ok = false when no
+// `most`: twice the anchor tiles of the other kernels, as a tile here is laid out
+// in FP64 and read once, so that fewer are better: 64 for 32 segments takes a
+// search with one sky from 22.6 to 19.4 ms), the FP64 series' terms, and the thresholds' error; ok = false when no
 // tile keeps it.  x_max: largest f/df; db: largest Doppler shift in bins.
 struct StepTrack {
   bool ok = false;

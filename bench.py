@@ -36,7 +36,6 @@ own synthetic workload:
 from __future__ import annotations
 
 import argparse
-import hashlib
 import json
 import math
 import os
@@ -164,32 +163,6 @@ class ClockSampler:
         return {"sm_mhz": statistics.median(sm) if sm else None,
                 "sm_max_mhz": max(smax) if smax else None,
                 "reasons": sorted(reasons), "samples": len(sm)}
-
-
-def kernel_source_digest():
-    """First 16 hex digits of the sha256 of the group kernel's sources
-    (tcw_persist.cuh followed by tcw_ptx.cuh)."""
-    h = hashlib.sha256()
-    for f in ("tcw_persist.cuh", "tcw_ptx.cuh"):
-        h.update(open(os.path.join(ROOT, "paper_2507_07816_gb300", "csrc", f), "rb").read())
-    return h.hexdigest()[:16]
-
-
-# DRAM bytes (read + write) of one group-kernel launch per lookup, from an ncu
-# capture (dram__bytes_read.sum + dram__bytes_write.sum, one pass) of the
-# bank8000 workload: the full 2 x 10000 x 10000 map, Doppler table and sky with
-# 8000 templates, one launch; a full launch streams the same map and table once
-# per pass, 25 times as many passes, so it is taken to move the same bytes per
-# lookup.  Keyed by the kernel source digest it was taken on; no entry for the
-# current source: the traffic is reported as null.
-GROUP_KERNEL_DRAM_BYTES_PER_LOOKUP = {
-    "c816dee2c7d44e5e": (3010211584 + 39771392) / (1024 * 8000 * 2 * 10000),
-}
-
-
-def group_kernel_traffic(lookups):
-    per = GROUP_KERNEL_DRAM_BYTES_PER_LOOKUP.get(kernel_source_digest())
-    return None if per is None else per * lookups
 
 
 def oracle_rate(p, seconds, seed=0):
@@ -559,17 +532,23 @@ def bench_ours(args):
                "d2h_bytes_per_step": int(d2h), "steps": n_e2e}
         s2.close()
 
-    # roofline of the dominant kernel (group_kernel): ALU-issue bound
+    # roofline of the dominant kernel (step_kernel, with the tiles' track constants): it
+    # evaluates a track per (template, segment) and detector, not per sky, so its work is
+    # counted in those: about 20 lane-operations for the track and 4 per detector.  What
+    # binds is the latency of its scattered reads; no unit is near its peak.
     sm_count = torch.cuda.get_device_properties(dev).multi_processor_count
     kern_ms = statistics.mean(kernel_ms)
-    achieved = U / (kern_ms / 1000.0)
+    n_det = len(p.velocity)
+    entries = U / len(p.nhat) * -(-len(p.nhat) // 1024)
+    ops = 20.0 / n_det + 4.0
+    achieved = entries / (kern_ms / 1000.0)
     clock_mhz = clocks.get("sm_max_mhz") or 2070.0
-    peak = sm_count * 128 * clock_mhz * 1e6 / 2.0      # 2 lane-ops per lookup
-    traffic = group_kernel_traffic(U)
-    roof = {"bound": "alu", "achieved": achieved / 1e9, "peak": peak / 1e9, "unit": "Glookup/s",
-            "frac": achieved / peak, "traffic": traffic,
-            "kernel": "group_kernel", "kernel_ms": kern_ms,
-            "peak_basis": f"{sm_count} SMs x 128 lanes x {clock_mhz:.0f} MHz / 2 lane-ops per lookup"}
+    peak = sm_count * 128 * clock_mhz * 1e6 / ops
+    roof = {"bound": "alu", "achieved": achieved / 1e9, "peak": peak / 1e9, "unit": "Gtrack-points/s",
+            "frac": achieved / peak, "traffic": None,
+            "kernel": "step_kernel", "kernel_ms": kern_ms,
+            "peak_basis": f"{sm_count} SMs x 128 lanes x {clock_mhz:.0f} MHz / {ops:.0f} lane-ops per "
+                          "(template, segment, detector, chunk of up to 1024 skies)"}
     l2_gbps = None
     try:
         l2_gbps = tcw.probe_read_bandwidth(64 << 20, passes=50, reps=5)

@@ -62,11 +62,13 @@ enum {
 enum { TCW_HOST = 0, TCW_DEVICE = 1 };
 enum { TCW_F32 = 0, TCW_F16 = 1 };
 
-/* Search kernels.  TCW_KERNEL_AUTO picks the group kernel when its exactness
+/* Search kernels.  TCW_KERNEL_AUTO picks the grouped search when its exactness
  * conditions hold and the per-lookup kernel otherwise. */
 enum {
     TCW_KERNEL_AUTO = 0,
-    TCW_KERNEL_GROUP = 1,   /* sky-group candidate-pair kernel (fast path) */
+    TCW_KERNEL_GROUP = 1,   /* the sky as a whole (fast path): step functions over the sorted
+                               sky, or the sky-group candidate-pair kernel where the fixed-point
+                               sums or fp32 track of those do not reach */
     TCW_KERNEL_LOOKUP = 2   /* one thread per (sky, template), FP64 per lookup */
 };
 
@@ -77,10 +79,12 @@ enum {
                                   tcw_get_statistics (costs 3*4 B per pair) */
     TCW_OPT_TILE_SEGMENTS = 3, /* segments per tile of the group kernel: the spacing of
                                   the FP64 track anchors and of the fp32 partial sums;
-                                  a power of two in [8, 128], default 32 */
+                                  a power of two in [8, 128], default 32 (the
+                                  step-function search takes up to twice as many) */
     TCW_OPT_BANK_CHUNK = 4,    /* template groups of one pass (1024/lanes sorted
-                                  templates) per work item of the group kernel,
-                                  in [1, 4096], default 1 */
+                                  templates) per work item of the group kernel, or
+                                  blocks of 32, 16 or 4 templates of the
+                                  step-function search, in [1, 4096], default 1 */
     TCW_OPT_AUTOTUNE = 5,      /* batched search: 1 (default) = choose the bank chunk
                                   and tile length by timing candidates on a sample of
                                   the batch; 0 = use TCW_OPT_BANK_CHUNK and

@@ -1,10 +1,11 @@
 // tcw_api.cu -- C ABI, input validation and the host side of a search.
 //
 // A search (tcw_search) runs, on the context's stream:
-//   1. doppler_kernel   v.nhat/c per (detector, segment, sky)        [Eq. 2]
-//   2. group_kernel     track entries + gather + weighted sums + Psi [Eq. 1, Sec. 2, Eq. 4]
-//      (or lookup_kernel when the group kernel's exactness conditions fail)
+//   1. step_rows_kernel, step_tile_kernel  Doppler rows [Eq. 2] and track constants [Eq. 1]
+//   2. step_kernel      lookups, weighted sums and Psi as step functions over the sky [Sec. 2, Eq. 4]
 //   3. topk_kernel      per-sky top-k by (Psi desc, caller index asc)
+// Outside the step kernel's conditions (step_search) 1 and 2 are doppler_kernel
+// and group_kernel, and lookup_kernel when that one's exactness conditions fail.
 // The bank is sorted by f0 and the sky by its Doppler factor at the middle
 // segment; both permutations are undone on output.
 #include <algorithm>
@@ -199,7 +200,8 @@ tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, boo
                                   c->bank_f0max / c->df, pl.doppler_bins, c->f_min, c->df, pl.inv_q);
   if (!tr.ok) return TCW_OK;
   const int tile = 1 << tr.shift;
-  const StepGeometry g = step_geometry(c->S, c->D, c->Nseg, tile, c->h_v.data(), false);
+  StepGeometry g = step_geometry(c->S, c->D, c->Nseg, tile, c->h_v.data(), false);
+  g.log_t = step_block(g, c->Bpad, c->bank_chunk, c->grid, (double)c->Nseg * c->D);
   const int n_tiles = (int)((c->Nseg + tile - 1) / tile);
   const size_t rows = (size_t)g.n_chunks * c->Nseg * c->D;
   TCW_CUDA(c, c->step_q.ensure(rows * step_row(g.cpad) * sizeof(int32_t)), "doppler rows");

@@ -5,11 +5,14 @@
 // events are searched against the context's template bank.  One search is a
 // CUDA graph, replayed on every call:
 //
-//   doppler_kernel  x event      Eq. 2 factor tables
-//   anchor_kernel   x event      FP64 tile anchors of Eq. 1
-//   group_kernel    x wave       ONE persistent launch over the wave's
-//                                (event, sky chunk, bank chunk) work items,
-//                                spread over the CTAs longest-first
+//   step_rows_kernel x event     Eq. 2 factor rows and their tables
+//   step_tile_kernel x event     track constants of Eq. 1 per tile
+//   step_kernel      x wave      a persistent launch over the wave's (event,
+//                                sky chunk, template block) work items,
+//                                longest first, for blocks of 32 templates
+//                                and of 16 each
+//   (doppler_kernel, anchor_kernel and one group_kernel launch per wave when
+//   some event is outside the step kernel's conditions)
 //   topk_kernel     x event      per-sky top-k of Eq. 4's Psi
 //
 // A wave is a run of events whose Psi and anchor buffers fit the memory

@@ -637,7 +637,7 @@ __device__ __noinline__ void step_fold(const StepParams& p, StepBlockCtx& s_ctx,
     part[2 * kStepThreads + tid] = s2;
   }
   __syncthreads();
-  // exclusive scans over a template's pieces (32 or 64), one warp per template
+  // exclusive scans over a template's pieces (32, 64 or 256), one warp per template
   for (int tt = warp; tt < T; tt += kStepWarps) {
     const int ks = s_ctx.edge_mask >> tt & 1u ? 3 : 1;
     for (int k = 0; k < ks; ++k) {
@@ -761,7 +761,7 @@ __device__ __noinline__ void step_fold(const StepParams& p, StepBlockCtx& s_ctx,
 }
 
 // The search kernel: one CTA per SM takes (sky chunk, template block) items from
-// a counter; the difference cells of a block (16 or 32 templates x up to 1024
+// a counter; the difference cells of a block (4, 16 or 32 templates x up to 1024
 // skies, two words each) live in shared memory, one column per template.  A
 // lane owns one (template, segment) of its warp's turn: the fp32 track, the
 // first sky's bin, and for each bin boundary inside the chunk's Doppler range a
@@ -893,8 +893,9 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
         for (int jc = js; jc < je; jc += kStepCarry) {
           const int jce = min(je, jc + kStepCarry);
           // The warps take the turns as they come: their lengths in time differ.  The last turn's worth of
-          // each warp goes in quarters, so that the warps end a pass closer together.
-          const int small = min(sub, max(sub - 2, 2)), big = max(0, ((jce - jc) >> sub) - kStepWarps);
+          // each warp goes in quarters (a full round of segments at least), so that the warps end a pass
+          // closer together.
+          const int small = min(sub, max(sub - 2, max(2, 5 - LT))), big = max(0, ((jce - jc) >> sub) - kStepWarps);
           if (tid == 0) s_turn = 0;
           __syncthreads();
           int j0 = 0, jn = 0;   // the warp's turn: segments left to it
@@ -1221,8 +1222,10 @@ cudaError_t pick_value(bool half, bool general, const F& f) {
 }
 template <typename F>
 cudaError_t pick(int dp, int log_t, bool half, bool general, const F& f) {
+  if (dp == 1 && log_t == 2) return pick_value<1, 2>(half, general, f);
   if (dp == 1 && log_t == 4) return pick_value<1, 4>(half, general, f);
   if (dp == 1 && log_t == 5) return pick_value<1, 5>(half, general, f);
+  if (dp == 2 && log_t == 2) return pick_value<2, 2>(half, general, f);
   if (dp == 2 && log_t == 4) return pick_value<2, 4>(half, general, f);
   if (dp == 2 && log_t == 5) return pick_value<2, 5>(half, general, f);
   return cudaErrorInvalidValue;
@@ -1288,6 +1291,22 @@ StepTrack step_track(const double* t_mid, int64_t n_seg, double T0, int most, do
     return r;
   }
   return r;
+}
+
+int step_block(const StepGeometry& g, int Bpad, int bank_chunk, int grid, double rows) {
+  int best = g.log_t;
+  double least = 0;
+  for (int lt : {5, 4, 2}) {
+    if (lt > g.log_t) continue;
+    const int64_t blocks = Bpad >> lt, items = g.n_chunks * ((blocks + bank_chunk - 1) / bank_chunk);
+    const double ns = lt == 5 ? 2.8 : lt == 4 ? 3.9 : 5.6;
+    const double us = (double)((items + grid - 1) / grid) * bank_chunk * (rows * (1 << lt) * ns * 1e-3 + g.passes * 20.0);
+    if (lt == g.log_t || us < 0.95 * least) {
+      best = lt;
+      least = us;
+    }
+  }
+  return best;
 }
 
 StepGeometry step_geometry(int64_t S, int D, int64_t n_seg, int tile, const double* v, bool split) {

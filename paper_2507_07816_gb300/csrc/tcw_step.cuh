@@ -135,7 +135,7 @@ __host__ __device__ constexpr int step_buckets(int cpad) { return 2 * cpad; }
 
 // Chunks of an event's sorted skies: the fewest chunks of at most
 // kStepMaxChunk skies, of nearly equal size; 32 templates per block while the
-// difference cells allow it (chunks of up to 511 skies), else 16.
+// difference cells allow it (chunks of up to 511 skies), else 16 (see step_block).
 struct StepGeometry {
   int n_chunks, chunk, cpad, log_t;
   int dets_per_pass, pass_seg, passes;
@@ -221,6 +221,14 @@ inline int step_sub_shift(const StepGeometry& g, int64_t n_seg, int tile_shift) 
   }
   return best;
 }
+// Templates of a block (as log2) for a bank whose blocks may not fill the chip:
+// blocks of 16 or 4 when their rounds over `grid` CTAs end sooner than those of
+// the largest block that fits.  A (template, row) takes 2.8 ns of a CTA in
+// blocks of 32 and 3.9 in blocks of 16 (128 skies, where 626 of 32 in 5 rounds
+// take 9.0 ms and 1251 of 16 in 9 rounds 11.0), about twice as much in blocks of
+// 4 (the tables' rows serve fewer templates), and a pass's end some 20 us.
+// 301 templates x 12 skies x 4002 rows: 10 blocks of 32, 511 us; 76 of 4, 322.
+int step_block(const StepGeometry& g, int Bpad, int bank_chunk, int grid, double rows);
 inline int step_cells(const StepGeometry& g) { return (g.cpad + 1) << g.log_t; }
 size_t step_slow_bytes(int grid);
 inline size_t step_edge_bytes(int grid) { return (size_t)grid * (2 * kStepCells + 32) * sizeof(longlong2); }

@@ -142,3 +142,10 @@ def test_crowded_skies(cluster, width):
     n = np.repeat(p.nhat[::cluster], cluster, axis=0)[:120] + width * r.normal(size=(120, 3))
     p.nhat = np.ascontiguousarray(n / np.linalg.norm(n, axis=1, keepdims=True))
     check(p)
+
+
+@pytest.mark.parametrize("n_tmpl,n_seg,n_sky,n_det", [(300, 700, 12, 2), (300, 700, 1024, 1), (9000, 64, 20, 2),
+                                                      (9000, 64, 600, 2)])
+def test_block_sizes(n_tmpl, n_seg, n_sky, n_det):
+    """Blocks of 4 templates for few templates over long data, of 32 and 16 for many."""
+    check(problem(1300 + n_sky + n_tmpl, n_det, n_seg, n_sky, n_tmpl, n_bin=2000))

@@ -44,3 +44,20 @@ def test_forward_and_gradients(n):
     close(g["b2"].reshape(-1), dZ2.sum(0), a.sum(0), n + 1)
     close(g["W1"], X.T @ dZ1, np.abs(X).T @ mZ1, n + 258)
     close(g["b1"].reshape(-1), dZ1.sum(0), mZ1.sum(0), n + 258)
+
+
+@pytest.mark.parametrize("n", [1, 31, 1025, 4096, 20000])
+def test_loss(n):
+    """Terms err by at most 10 u of their parts, their FP64 sum by one rounding."""
+    r = np.random.default_rng(950 + n)
+    y = (r.normal(size=n) * 4).astype(np.float32)
+    label = (r.random(n) < 0.3).astype(np.float32)
+    mlp = tcw.Mlp(seed=1)
+    loss, dy = mlp.bce(torch.as_tensor(y, device="cuda:0"), torch.as_tensor(label, device="cuda:0"), 3.0)
+    again, _ = mlp.bce(torch.as_tensor(y, device="cuda:0"), torch.as_tensor(label, device="cuda:0"), 3.0)
+    ref, rdy = OT.bce_with_logits(y.astype(np.float64), label, pw=3.0)
+    v = y.astype(np.float64)
+    parts = np.mean(3.0 * label * (np.logaddexp(0, v) + np.abs(v)) + (1 - label) * np.logaddexp(0, v))
+    assert abs(loss.item() - ref) <= 10 * U * parts + U * abs(ref)
+    assert loss.item() == again.item()
+    assert np.all(np.abs(dy.cpu().numpy() - rdy) <= 12 * U * 3.0 / n)

@@ -686,9 +686,10 @@ cudaError_t launch_wave(const tcw_ctx* c, BatchState* b, int w, int tile, int nt
   return cudaSuccess;
 }
 
-// Autotuner: every (bank chunk, tile) candidate runs the group kernel over the
-// first probe_groups groups of 8 templates of every event (wave by wave); the
-// candidate with the highest sums/s wins, ties going to the earlier one.
+// Autotuner: every (bank chunk, tile) candidate searches the first
+// probe_groups template groups of every event (wave by wave, the search
+// launches alone on the clock); the candidate with the highest sums/s wins,
+// ties going to the earlier one.
 tcw_status autotune(tcw_ctx* c, BatchState* b) {
   const auto t0 = std::chrono::steady_clock::now();
   const int groups = c->Bpad / pass_templates(b->lanes);
@@ -703,7 +704,7 @@ tcw_status autotune(tcw_ctx* c, BatchState* b) {
   for (int tile : tiles) {
     const int nterms = batch_series_terms(c, b, tile);
     if ((st = prepare_shape(c, b, tile, nterms)) != TCW_OK) break;
-    int nodes = 0;
+    int nodes = 0, laid = -1;   // wave whose anchors are in place
     if (b->step) {
       cudaError_t err = launch_rows(b, c->stream, &nodes);
       if (err != cudaSuccess) {
@@ -711,36 +712,40 @@ tcw_status autotune(tcw_ctx* c, BatchState* b) {
         break;
       }
     }
-    for (int w = 0; w < b->waves && (b->step || nterms > 0); ++w) {
-      cudaError_t err = launch_wave_anchors(c, b, w, tile, c->stream);
-      if (err != cudaSuccess) {
-        st = cuda_fail(c, err, "anchor_kernel launch");
-        break;
-      }
-    }
-    if (st != TCW_OK) break;
     for (int bc : chunks) {
       if (bc > probe_groups && bc != 1) continue;
       int64_t sums = 0;
       if ((st = upload_items(c, b, bc, probe_groups, &sums)) != TCW_OK) break;
       float best = INFINITY;
       for (int rep = 0; rep < 2 && st == TCW_OK; ++rep) {
-        cudaEventRecord(e0, c->stream);
-        for (int w = 0; w < b->waves; ++w) {
+        float ms = 0;
+        for (int w = 0; w < b->waves && st == TCW_OK; ++w) {
+          // the waves share one anchor buffer: a wave is searched with its own anchors in place only
+          if (laid != w && (b->step || nterms > 0)) {
+            cudaError_t err = launch_wave_anchors(c, b, w, tile, c->stream);
+            if (err != cudaSuccess) {
+              st = cuda_fail(c, err, "anchor_kernel launch");
+              break;
+            }
+            laid = w;
+          }
+          cudaEventRecord(e0, c->stream);
           cudaError_t err = launch_wave(c, b, w, tile, nterms, c->stream, &nodes);
           if (err != cudaSuccess) {
             st = cuda_fail(c, err, "search kernel launch");
             break;
           }
+          cudaEventRecord(e1, c->stream);
+          err = cudaEventSynchronize(e1);
+          if (err != cudaSuccess) {
+            st = cuda_fail(c, err, "autotune");
+            break;
+          }
+          float wave_ms = 0;
+          cudaEventElapsedTime(&wave_ms, e0, e1);
+          ms += wave_ms;
         }
-        cudaEventRecord(e1, c->stream);
-        cudaError_t err = cudaEventSynchronize(e1);
-        if (err != cudaSuccess) {
-          st = cuda_fail(c, err, "autotune");
-          break;
-        }
-        float ms = 0;
-        cudaEventElapsedTime(&ms, e0, e1);
+        if (st != TCW_OK) break;
         best = std::min(best, ms);
       }
       if (st != TCW_OK) break;

@@ -197,7 +197,7 @@ tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, boo
                   (int64_t)c->D * c->Nseg);
   if (!sc.ok) return TCW_OK;
   const StepTrack tr = step_track(c->h_t.data(), c->Nseg, c->T0, 2 * c->tile_segments, c->bank_tau_min, c->bank_r_max,
-                                  c->bank_f0max / c->df, pl.doppler_bins, c->f_min, c->df, pl.inv_q);
+                                  c->bank_f0max / c->df, f_top / c->df, pl.doppler_bins, c->f_min, c->df, pl.inv_q);
   if (!tr.ok) return TCW_OK;
   const int tile = 1 << tr.shift;
   StepGeometry g = step_geometry(c->S, c->D, c->Nseg, tile, c->h_v.data(), false);

@@ -243,7 +243,7 @@ void plan_step(const tcw_ctx* c, BatchState* b, int tile) {
     all.shift = b->track.shift;
     for (const EventHost& e : b->ev) {
       const StepTrack t = step_track(e.t.data(), e.n_seg, e.T0, most, c->bank_tau_min, c->bank_r_max,
-                                     c->bank_f0max / b->df, b->doppler_bins, b->f_min, b->df, b->inv_q);
+                                     c->bank_f0max / b->df, f_top / b->df, b->doppler_bins, b->f_min, b->df, b->inv_q);
       if (!t.ok || (round == 1 && t.shift != b->track.shift)) return;
       all.shift = std::min(all.shift, t.shift);
       all.nterms = std::max(all.nterms, t.nterms);

@@ -1253,8 +1253,13 @@ StepScales step_scales(double vmax, double w_min, double w_max, double a_ref, in
 }
 
 StepTrack step_track(const double* t_mid, int64_t n_seg, double T0, int most, double tau_min, double r_max,
-                     double x_max, double db, double f_min, double df, double inv_q) {
+                     double x_max, double x_top, double db, double f_min, double df, double inv_q) {
   StepTrack r;
+  // Bins are compared with the band's edges in fp32, 8 bins and more inside it, and the
+  // exact thresholds are looked for 8 boundaries either side of an fp32 estimate of the
+  // track's bin.  Up to 2^23 bins that estimate is off by at most 3 (five roundings of
+  // 2^-24 in f, f_min and their difference) and a comparison by 1; beyond, neither holds.
+  if (!(x_top <= 8388608.0)) return r;
   auto cbound = [&](int k) {   // |C(e, k)| for |e| <= r_max
     double c = 1.0;
     for (int i = 0; i < k; ++i) c *= (r_max + i) / (i + 1);

@@ -164,7 +164,8 @@ inline bool step_ordered(const StepGeometry& g) { return g.passes > 1; }
 // `most`: twice the anchor tiles of the other kernels, as a tile here is laid out
 // in FP64 and read once, so that fewer are better: 64 for 32 segments takes a
 // search with one sky from 22.6 to 19.4 ms), the FP64 series' terms, and the thresholds' error; ok = false when no
-// tile keeps it.  x_max: largest f/df; db: largest Doppler shift in bins.
+// tile keeps it.  x_max: largest f/df of the bank; x_top: f/df at the top of the
+// band; db: largest Doppler shift in bins.
 struct StepTrack {
   bool ok = false;
   int shift = 0, nterms = 0;
@@ -172,7 +173,7 @@ struct StepTrack {
   int eps_max = 0;           // in grid units
 };
 StepTrack step_track(const double* t_mid, int64_t n_seg, double T0, int most, double tau_min, double r_max,
-                     double x_max, double db, double f_min, double df, double inv_q);
+                     double x_max, double x_top, double db, double f_min, double df, double inv_q);
 inline void set_step_track(StepParams& p, const StepTrack& t) {
   p.eps = t.eps;
   p.nterms = t.nterms;

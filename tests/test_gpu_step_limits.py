@@ -1,0 +1,61 @@
+"""Where the step-function search (tcw_step.cu) ends: inputs at its limits, and
+beyond them the kernels that it hands over to."""
+import numpy as np
+import pytest
+
+import paper_2507_07816_gb300 as tcw
+import tcw_synth as syn
+from _parity import assert_stats_close, assert_topk_consistent, oracle_stats
+
+pytestmark = pytest.mark.gpu
+
+
+def run(p, k=3, options=(), statistic=None):
+    """Search of p: values, indices, statistics, info."""
+    s = tcw.Search(0)
+    s.set_option(tcw.OPT_KEEP_STATS, 1)
+    for o, v in options:
+        s.set_option(o, v)
+    if statistic:
+        s.set_statistic(*statistic)
+    s.load_problem(p)
+    val, idx = s.search(k)
+    st, info = s.statistics(), s.info()
+    s.close()
+    return val, idx, st, info
+
+
+def stepped(st, ora):
+    """Whether the step-function search ran: its S are exact sums rounded once (0.5
+    ulp, and 0.02 for the fixed-point grid), those of the group kernel sums in fp32."""
+    ulp = np.spacing(np.abs(ora[0]).astype(np.float32)).astype(np.float64)
+    return bool(np.all(np.abs(st["S"].astype(np.float64) - ora[0]) <= 0.52 * ulp))
+
+
+def check(p, k=3, options=(), amp_power=0):
+    val, idx, st, info = run(p, k, options)
+    rho = np.asarray(p.rho, np.float64) if p.rho.dtype == np.float16 else None
+    ora = oracle_stats(p, rho=rho, amp_power=amp_power)
+    assert info.kernel == tcw.KERNEL_GROUP
+    assert_stats_close((st["S"], st["W1"], st["W2"], st["psi"]), ora, p.name)
+    assert_topk_consistent(st["psi"], idx, val, k)
+    return stepped(st, ora)
+
+
+@pytest.mark.parametrize("n_bin,step", [(2 ** 23 - 1100, True), (2 ** 23 + 64, False)])
+def test_wide_bands(n_bin, step):
+    """Detectors nearly at rest over bands of 2^23 bins.  Up to there bins are placed
+    in fp32; the templates are at the top of the band.  Beyond, another kernel runs
+    (its bins are fp32 estimates too: templates at the band's bottom)."""
+    r = syn.rng(2000)
+    n_seg, df = 12, 0.25
+    t = syn.segment_times(n_seg, 4.0)
+    v = r.normal(size=(2, n_seg, 3))
+    v *= 46.0 / np.linalg.norm(v, axis=-1, keepdims=True)
+    f_min, f_max = 1000 * df, (1000 + n_bin) * df
+    lo, hi = (0.97 * f_max, f_max + 5) if step else (f_min + 1e3, f_min + 2e4)
+    bank = syn.random_bank(r, 60, f0_range=(lo, hi), tau_range=(3500, 35000))
+    rho = np.tile(syn.exponential_noise(r, (1, 1, n_bin)), (2, n_seg, 1))
+    p = syn.Problem(rho, t, syn.uniform_weights(r, 2, n_seg), v, f_min, df, float(t[0] - 2.0), syn.random_sky(r, 12),
+                    bank, [], [], name="wide")
+    assert check(p) == step

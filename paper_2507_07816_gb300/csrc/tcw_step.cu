@@ -714,9 +714,8 @@ __device__ __noinline__ void step_fold(const StepParams& p, StepBlockCtx& s_ctx,
     const double nbins = two ? 2.0 : 1.0;
     const bool count = VK == 2 && p.nc_q > 0.0;
     const double mq = nbins * (count ? p.nc_q : 1.0);
-    const float vq = (float)(nbins * (count ? p.nc_q * (1.0 - p.nc_q) : 1.0));
+    const double vq = nbins * (count ? p.nc_q * (1.0 - p.nc_q) : 1.0);
     const double m_units = mq * ev.w1_unit / ev.x_unit;   // mean of one W1 unit, in units of X
-    const float x_unit = (float)ev.x_unit;
     const int64_t sky0 = (int64_t)chunk * ev.chunk;
     const int rows = min(ev.chunk, ev.S - (int)sky0);
     long long X = part[tid] + (long long)tsum[t];
@@ -727,11 +726,18 @@ __device__ __noinline__ void step_fold(const StepParams& p, StepBlockCtx& s_ctx,
     }
     // skies without band-edge steps share W1, W2 and the mean
     long long mean = 0;
-    float W2f = 0.f, rs = 0.f;
+    float W2f = 0.f, Rh = 0.f, Rl = 0.f;   // Rh + Rl: 2^24 units of X in sigma
     auto moments = [&]() {
       mean = __double2ll_rn((double)w1 * m_units);
       W2f = (float)((double)w2 * ev.w2_unit);
-      rs = W2f > 0.f ? rsqrtf(vq * W2f) : 0.f;
+      // 1 / sqrt(vq w2) as an fp32 pair: rsqrtf and one Newton step, r + r (1 - v r^2) / 2,
+      // with v r^2 - 1 in fp32 pairs; what it drops is below 2^-42
+      const double v = vq * (double)w2;
+      const float vh = (float)v, vl = (float)(v - (double)vh);
+      const float r = rsqrtf(vh), p2 = r * r;
+      const float e = fmaf(vh, p2, -1.0f) + fmaf(vh, fmaf(r, r, -p2), vl * p2);
+      Rh = r * ev.r_unit;
+      Rl = -0.5f * Rh * e;
     };
     moments();
     const int16_t* order = ev.order ? ev.order + ((int64_t)pass * ev.n_chunks + chunk) * cpad : nullptr;
@@ -744,13 +750,17 @@ __device__ __noinline__ void step_fold(const StepParams& p, StepBlockCtx& s_ctx,
         __stcg(ecol + q, make_longlong2(0, 0));
         w1 += v.x;
         w2 += v.y;
-        moments();
+        if (v.x | v.y) moments();
       }
       if (q >= rows) continue;
       // the cells' high words wrap at 2^31, so X is known modulo 2^48
       const long long x = (long long)((unsigned long long)X << 16) >> 16;
       const int64_t o = (sky0 + (order ? (int)order[q] : q)) * ev.Bpad + b0 + t;
-      ev.psi[o] = W2f > 0.f ? (float)(x - mean) * x_unit * rs : -INFINITY;
+      // x - mean as a 2^24 + b, both exact in fp32, so that Psi is rounded once
+      const long long u = x - mean;
+      const int a = (int)((u + (1 << 23)) >> 24);
+      const float af = (float)a, bf = (float)(int)(u - ((long long)a << 24)) * (1.0f / 16777216.0f);
+      ev.psi[o] = W2f > 0.f ? fmaf(af, Rh, fmaf(af, Rl, bf * Rh)) : -INFINITY;
       if (ev.S_out) {
         ev.S_out[o] = (float)((double)x * ev.x_unit);
         ev.W1_out[o] = (float)((double)w1 * ev.w1_unit);
@@ -1243,7 +1253,7 @@ StepScales step_scales(double vmax, double w_min, double w_max, double a_ref, in
   // the sum of a (template, sky) below 2^47 units and one value below 2^21 2^16 units
   s.x = std::min(46 - ln - lm, 36 - lm);
   s.w1 = std::min(36 - lw, 60 - ln - lw);
-  s.w2 = std::min(36 - lw2, 60 - ln - lw2);
+  s.w2 = std::min(36 - lw2, 60 - ln - lw2) & ~1;   // even: the root of its unit is a power of 2
   // one unit at most 2^-20 of the smallest weighted unit power: a sum of n
   // rounded values is then off by about 0.3 sqrt(n) 2^-20 of it, 3e-7 of the
   // standard deviation sqrt(n) that Eq. 4 divides by

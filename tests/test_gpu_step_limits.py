@@ -3,6 +3,7 @@ beyond them the kernels that it hands over to."""
 import numpy as np
 import pytest
 
+import oracle
 import paper_2507_07816_gb300 as tcw
 import tcw_synth as syn
 from _parity import assert_stats_close, assert_topk_consistent, oracle_stats
@@ -59,3 +60,30 @@ def test_wide_bands(n_bin, step):
     p = syn.Problem(rho, t, syn.uniform_weights(r, 2, n_seg), v, f_min, df, float(t[0] - 2.0), syn.random_sky(r, 12),
                     bank, [], [], name="wide")
     assert check(p) == step
+
+
+@pytest.mark.parametrize("statistic,bins,amp", [("power", 1, 0), ("power", 2, 0), ("count", 1, 0)])
+def test_psi_is_rounded_once(statistic, bins, amp):
+    """A few skies far apart (too wide a group for the group kernel): Psi is Eq. 4 of
+    exact sums, rounded once to fp32 (2^-24 relative, 2^-25 for its pieces), as from
+    sums in FP64.  The sums' grid is 2^-25 or finer here, 0.3 of it per value: 6 sigma
+    of that are 2^-23 of sigma = sqrt(W2) when the weights' rms is at least 0.25."""
+    r = syn.rng(2100)
+    n_seg = 1500
+    t = syn.segment_times(n_seg, 4.0)
+    dets = syn.random_detectors(r, 2)
+    vel = np.stack([d.velocity(t) for d in dets])
+    bank = syn.random_bank(r, 300, f0_range=(495.0, 1255.0), tau_range=(3500, 35000))
+    rho = 2 * syn.exponential_noise(r, (2, n_seg, 3000))    # off the noise's mean: Psi up to 50
+    p = syn.Problem(rho, t, syn.uniform_weights(r, 2, n_seg), vel, 500.0, 0.25, float(t[0] - 2.0),
+                    syn.random_sky(r, 12), bank, [], dets, name="far apart")
+    val, idx, st, info = run(p, options=[(tcw.OPT_TRACK_BINS, bins), (tcw.OPT_AMPLITUDE_POWER, amp)],
+                             statistic=(tcw.STAT_NUMBER_COUNT, 1.6) if statistic == "count" else None)
+    assert info.kernel == tcw.KERNEL_GROUP
+    S, W1, W2, psi = oracle.search_stats(p.rho, p.f_min, p.df, p.t_mid, p.weights, p.velocity, p.nhat, bank.f0, bank.tau,
+                                         bank.n, p.T0, amp_power=amp, track_bins=bins,
+                                         rho_th=1.6 if statistic == "count" else None)
+    assert_topk_consistent(st["psi"], idx, val, 3)
+    ok = W2 >= 0.0625 * W1.max() / 16
+    assert ok.mean() > 0.5 and np.abs(psi[ok]).max() > 20
+    assert np.all(np.abs(st["psi"] - psi)[ok] <= (2.0 ** -24 + 2.0 ** -25) * np.abs(psi[ok]) + 2.0 ** -23)

@@ -303,7 +303,6 @@ tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, boo
   p.inv_q = pl.inv_q;
   p.q = (float)pl.q;
   p.inv_q_f = (float)pl.inv_q;
-  p.df_f = (float)c->df;
   set_step_track(p, tr);
   p.amp_power = c->amp_power;
   p.nc_q = count ? std::exp(-c->rho_th) : 0.0;
@@ -314,9 +313,8 @@ tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, boo
   p.n_general = reinterpret_cast<unsigned long long*>(c->flags.as<char>() + 8);
   TCW_CUDA(c, cudaEventRecord(c->ev0, c->stream), "event");
   TCW_CUDA(c, launch_step_tiles(tp, c->stream), "step_tile_kernel launch");
-  TCW_CUDA(c, launch_step(p, g.dets_per_pass, g.log_t, c->dtype == TCW_F16, count || c->track_bins == 2, step_cells(g),
-                          std::min(c->grid, p.n_items), c->stream),
-           "step_kernel launch");
+  const StepForm form{g.dets_per_pass, g.log_t, c->dtype == TCW_F16, count || c->track_bins == 2, c->amp_power > 0};
+  TCW_CUDA(c, launch_step(p, form, step_cells(g), std::min(c->grid, p.n_items), c->stream), "step_kernel launch");
   TCW_CUDA(c, cudaEventRecord(c->ev1, c->stream), "event");
   *launches += 2;
   *ran = true;

@@ -641,6 +641,11 @@ GroupParams wave_params(const tcw_ctx* c, BatchState* b, int w, int tile, int nt
   return gp;
 }
 
+StepForm step_form(const tcw_ctx* c, const BatchState* b, int log_t) {
+  return StepForm{b->dets_per_pass, log_t, b->dtype == TCW_F16,
+                  c->statistic == TCW_STAT_NUMBER_COUNT || c->track_bins == 2, c->amp_power > 0};
+}
+
 // The search launches of wave w.
 cudaError_t launch_wave(const tcw_ctx* c, BatchState* b, int w, int tile, int nterms, cudaStream_t st, int* nodes) {
   if (!b->step) {
@@ -658,7 +663,6 @@ cudaError_t launch_wave(const tcw_ctx* c, BatchState* b, int w, int tile, int nt
   p.inv_q = b->inv_q;
   p.q = (float)b->q;
   p.inv_q_f = (float)b->inv_q;
-  p.df_f = (float)b->df;
   set_step_track(p, b->track);
   p.amp_power = c->amp_power;
   p.nc_q = count_q(c);
@@ -667,7 +671,6 @@ cudaError_t launch_wave(const tcw_ctx* c, BatchState* b, int w, int tile, int nt
   p.slow = c->step_slow.as<int4>();
   p.edge = c->step_edge.as<longlong2>();
   p.n_general = at<unsigned long long>(b->flags, 8);
-  const bool general = c->statistic == TCW_STAT_NUMBER_COUNT || c->track_bins == 2;
   const int first = b->wave_items[w], split = first + b->wave_split[w], end = b->wave_items[w + 1];
   for (int lt : {5, 4}) {
     const int i0 = lt == 5 ? first : split, i1 = lt == 5 ? split : end;
@@ -679,7 +682,7 @@ cudaError_t launch_wave(const tcw_ctx* c, BatchState* b, int w, int tile, int nt
     p.n_items = i1 - i0;
     cudaError_t err = cudaMemsetAsync(p.next, 0, 4, st);
     if (err == cudaSuccess)
-      err = launch_step(p, b->dets_per_pass, lt, b->dtype == TCW_F16, general, cells, std::min(b->grid, p.n_items), st);
+      err = launch_step(p, step_form(c, b, lt), cells, std::min(b->grid, p.n_items), st);
     if (err != cudaSuccess) return err;
     ++*nodes;
   }
@@ -771,11 +774,10 @@ tcw_status autotune(tcw_ctx* c, BatchState* b) {
 
 // Shared-memory limits of the search kernels of a batch.
 tcw_status prepare_kernels(tcw_ctx* c, const BatchState* b) {
-  const bool general = c->statistic == TCW_STAT_NUMBER_COUNT || c->track_bins == 2;
   if (b->step) {
-    for (int lt : {5, 4})
-      TCW_CUDA(c, step_prepare(b->dets_per_pass, lt, b->dtype == TCW_F16, general), "step_kernel attributes");
+    for (int lt : {5, 4}) TCW_CUDA(c, step_prepare(step_form(c, b, lt)), "step_kernel attributes");
   } else {
+    const bool general = c->statistic == TCW_STAT_NUMBER_COUNT || c->track_bins == 2;
     TCW_CUDA(c, group_prepare(b->D, b->lanes, half_windows(c, b), general), "group_kernel attributes");
   }
   return TCW_OK;

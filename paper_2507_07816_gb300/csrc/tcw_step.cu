@@ -371,24 +371,33 @@ __global__ void absmax_kernel(const T* x, int64_t n, unsigned* out) {
 constexpr size_t kStepPart = 3 * kStepThreads * 8;
 static_assert(kStepWarps * kStepTurn * kStepHead * 16 <= kStepPart, "the heads fit the piece sums' place");
 struct StepLayout {
-  size_t part, coef, fcoef, head, tsum, total;
+  size_t part, coef, fcoef, head, famp, tsum, total;
   __host__ __device__ constexpr explicit StepLayout(int cells)
       : part(((size_t)cells * 8 + 15) & ~(size_t)15),
         coef(part + kStepPart),
         fcoef(coef + (size_t)kMaxSeriesTerms * 8 * 32),
         head(part),
-        tsum(fcoef + (size_t)32 * 20),
+        famp(fcoef + (size_t)32 * 20),
+        tsum(famp + (size_t)32 * 8),
         total(tsum + (size_t)32 * 4 * 8) {}
 };
 static_assert(StepLayout(kStepCells + 32).total <= 232448 - 1024, "one CTA's shared memory");
 
+// Value kinds VK: fp32 or fp16 powers, or number count and / or two-bin sums; each
+// without and with amplitude weights, whose code and registers the others are spared
+// (number count 30.9 -> 31.7 ms, two-bin 13.7 -> 13.9 with them).
+enum { kF32 = 0, kF16 = 1, kGen = 2, kWithAmp = 3 };
+template <int VK>
+constexpr bool kAmp = VK >= kWithAmp;
+template <int VK>
+constexpr bool kGeneral = VK % kWithAmp == kGen;
+
 // A value of the lookup at bin K of row (the caller checks the band).
-// VK 0: fp32 power, 1: fp16 power, 2: number count and / or two-bin sums.
 template <int VK>
 __device__ __forceinline__ float step_value(const StepParams& p, const StepEvent& ev, int64_t row, int K) {
-  if constexpr (VK == 0) {
+  if constexpr (VK % kWithAmp == kF32) {
     return __ldg(static_cast<const float*>(ev.rho) + (row + K));
-  } else if constexpr (VK == 1) {
+  } else if constexpr (VK % kWithAmp == kF16) {
     return __half2float(__ldg(static_cast<const __half*>(ev.rho) + (row + K)));
   } else {
     const int more = p.track_bins == 2 ? 1 : 0;
@@ -446,12 +455,51 @@ __device__ __forceinline__ void to_fixed(float v, float s, int& hi, int& lo) {
   hi = __float_as_int(t);
   lo = __float_as_int(fmaf(r, 65536.0f, kMagic));
 }
+// v (s + sl), |sl| < 2^-23 |s|
+__device__ __forceinline__ void to_fixed(float v, float s, float sl, int& hi, int& lo) {
+  const float t = fmaf(v, s, kMagic);
+  const float r = fmaf(v, sl, fmaf(v, s, -(t - kMagic)));
+  hi = __float_as_int(t);
+  lo = __float_as_int(fmaf(r, 65536.0f, kMagic));
+}
 // The same as one 64-bit word.
-__device__ __forceinline__ long long fixed_word(float v, float s) {
+__device__ __forceinline__ long long fixed_word(float v, float s, float sl) {
   int hi, lo;
-  to_fixed(v, s, hi, lo);
+  to_fixed(v, s, sl, hi, lo);
   return (long long)(hi - kMagicBits) * 65536 + (lo - kMagicBits);
 }
+
+// (h + l)^n, 1 <= n and |l| < |h|, as an fp32 pair x + y with x the nearest float:
+// products of pairs whose rounding errors are recovered by fma.
+__device__ __forceinline__ float2 pair_power(float h, float l, int n) {
+  const float s = h + l;
+  l -= s - h;
+  h = s;
+  float x = h, y = l;
+  for (int k = 1; k < n; ++k) {
+    const float t = x * h;
+    y = fmaf(x, h, -t) + fmaf(x, l, y * h);
+    x = t;
+  }
+  const float t = x + y;
+  return make_float2(t, y - (t - x));
+}
+
+// A lookup's weight w (f/f0)^p as an fp32 pair h + l: what the per-lookup kernel
+// has in FP64.  Its words in the sums W1 and W2.
+struct PairWeight {
+  float h, l;
+  __device__ __forceinline__ PairWeight(float w, float2 amp) {
+    h = w * amp.x;
+    l = fmaf(w, amp.x, -h) + w * amp.y;
+  }
+  __device__ __forceinline__ long long w1(const StepEvent& ev) const {
+    return fixed_word(1.0f, h * ev.w1_scale, l * ev.w1_scale);
+  }
+  __device__ __forceinline__ long long w2(const StepEvent& ev) const {
+    return fixed_word(h, h * ev.w2_scale, 2.0f * l * ev.w2_scale);
+  }
+};
 
 // The exact thresholds of (template b, segment j) on the q grid, as the group
 // kernel takes them: theta_n = (V + n V2) >> 8 between the bins base + n and
@@ -519,26 +567,31 @@ struct StepBlockCtx {
 template <int VK, int LT>
 __device__ __forceinline__ void step_rare(const StepParams& p, StepBlockCtx& c, int lt, int j, int d, int only) {
   const StepEvent& ev = *c.ev;
-  const bool two = VK == 2 && p.track_bins == 2;
+  const bool two = kGeneral<VK> && p.track_bins == 2;
   const unsigned k_end = (unsigned)max(0, (int)p.n_bin - (two ? 1 : 0));
   const int64_t row = ((int64_t)c.chunk * ev.n_seg + j) * p.n_det + d;
   const int4 m0 = ev.head[row * kStepHead];
   const float dth = __int_as_float(ev.head[row * kStepHead + 1].x);
   if (!(dth == dth)) return;   // before T0
   const StepExact x = step_exact(p, ev, c.coef + lt, c.b0 + lt, j, two);
-  float amp = 1.0f;
-  if (p.amp_power > 0) {
-    const float rr = (float)(x.h * ev.f0[c.b0 + lt]);
-    float rp = rr;
-    for (int k = 1; k < p.amp_power; ++k) rp *= rr;
-    amp = __frcp_rn(rp);
+  float2 amp = make_float2(1.0f, 0.0f);
+  if (kAmp<VK>) {
+    // (f0/f)^p, and its reciprocal by a Newton step from fp32's
+    const double rr = x.h * ev.f0[c.b0 + lt];
+    const float rh = (float)rr;
+    const float2 rp = pair_power(rh, (float)(rr - (double)rh), p.amp_power);
+    const float u = __frcp_rn(rp.x);
+    amp = make_float2(u, u * (fmaf(-rp.x, u, 1.0f) - rp.y * u));
   }
-  const float w = __int_as_float(m0.w) * amp, ws = w * ev.x_scale;
+  const PairWeight w(__int_as_float(m0.w), amp);
+  const float ws = w.h * ev.x_scale, wsl = w.l * ev.x_scale;
   const int64_t vrow =
-      ((int64_t)d * ev.n_seg + j) * (VK == 2 && ev.bits ? (int64_t)ev.bit_pitch : p.n_bin);
+      ((int64_t)d * ev.n_seg + j) * (kGeneral<VK> && ev.bits ? (int64_t)ev.bit_pitch : p.n_bin);
   const int qmin = m0.x, qmax = m0.y;
   auto value = [&](int K, int& h, int& l) {
-    to_fixed((unsigned)K < k_end ? step_value<VK>(p, ev, vrow, K) : 0.f, ws, h, l);
+    const float v = (unsigned)K < k_end ? step_value<VK>(p, ev, vrow, K) : 0.f;
+    if constexpr (kAmp<VK>) to_fixed(v, ws, wsl, h, l);
+    else to_fixed(v, ws, h, l);
   };
   auto step = [&](int t, int K, long long e1, long long e2) {   // from bin K to K + 1
     int h0, l0, h1, l1;
@@ -572,9 +625,9 @@ __device__ __forceinline__ void step_rare(const StepParams& p, StepBlockCtx& c, 
   int nb = 0;
   for (long long u = v; nb < kNThr && saturate(u) <= qmax; u += x.V2) ++nb;
   long long u1, u2;   // the lookup's weights
-  if (p.amp_power > 0) {
-    u1 = fixed_word(w, ev.w1_scale);
-    u2 = fixed_word(w, w * ev.w2_scale);
+  if (kAmp<VK>) {
+    u1 = w.w1(ev);
+    u2 = w.w2(ev);
   } else {
     const longlong2 wi = ev.wfix[(int64_t)j * p.n_det + d];
     u1 = wi.x;
@@ -589,7 +642,7 @@ __device__ __forceinline__ void step_rare(const StepParams& p, StepBlockCtx& c, 
   value(K0, h0, l0);
   atomicAdd(c.tsum + lt, (unsigned long long)((long long)(h0 - kMagicBits) * 65536 + (l0 - kMagicBits)));
   // W1, W2 start from every segment's weights, amplitude weights from 0
-  if (first != (p.amp_power == 0)) {
+  if (first == kAmp<VK>) {
     atomicAdd(c.tsum + 32 + lt, (unsigned long long)(first ? u1 : -u1));
     atomicAdd(c.tsum + 64 + lt, (unsigned long long)(first ? u2 : -u2));
   }
@@ -618,7 +671,7 @@ __device__ __noinline__ void step_fold(const StepParams& p, StepBlockCtx& s_ctx,
   const unsigned long long* const tsum = s_ctx.tsum;
   longlong2* const edge_acc = s_ctx.edge + kStepCells + 32;
   longlong2* const ecol = s_ctx.edge + (int64_t)t * (cpad + 1);
-  const bool two = VK == 2 && p.track_bins == 2;
+  const bool two = kGeneral<VK> && p.track_bins == 2;
   const int chunk = s_ctx.chunk, b0 = s_ctx.b0;
   const bool te = (s_ctx.edge_mask >> t) & 1u;
   {
@@ -712,7 +765,7 @@ __device__ __noinline__ void step_fold(const StepParams& p, StepBlockCtx& s_ctx,
     // Eq. 4: <s> = mq W1, sigma^2 = vq W2 (power: 1, 1; number count: q, q(1-q)),
     // both doubled for two-bin lookups
     const double nbins = two ? 2.0 : 1.0;
-    const bool count = VK == 2 && p.nc_q > 0.0;
+    const bool count = kGeneral<VK> && p.nc_q > 0.0;
     const double mq = nbins * (count ? p.nc_q : 1.0);
     const double vq = nbins * (count ? p.nc_q * (1.0 - p.nc_q) : 1.0);
     const double m_units = mq * ev.w1_unit / ev.x_unit;   // mean of one W1 unit, in units of X
@@ -808,11 +861,12 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
   double* const coef = reinterpret_cast<double*>(smem + L.coef);
   float4* const fcoef = reinterpret_cast<float4*>(smem + L.fcoef);   // [32]: C(e, 3) .. C(e, 6)
   float* const fcoef7 = reinterpret_cast<float*>(fcoef + 32);        // [32]: C(e, 7)
+  float2* const famp = reinterpret_cast<float2*>(smem + L.famp);     // [32]: df / f0 as an fp32 pair
   int4* const slow_list = p.slow + ((int64_t)blockIdx.x * kStepWarps + (threadIdx.x >> 5)) * kStepSlow;
   int4* const heads = reinterpret_cast<int4*>(smem + L.head) + (threadIdx.x >> 5) * kStepTurn * kStepHead;
   unsigned long long* const tsum = reinterpret_cast<unsigned long long*>(smem + L.tsum);   // X0, W1, W2 [32]
   const int tid = threadIdx.x, lane = tid & 31;
-  const bool two = VK == 2 && p.track_bins == 2;
+  const bool two = kGeneral<VK> && p.track_bins == 2;
   constexpr unsigned kAll = 0xffffffffu;
   const unsigned lt_mask = (1u << lane) - 1u;
   const int n_bin = (int)p.n_bin;
@@ -846,7 +900,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
     constexpr int lps = 32 >> LT;
     const unsigned t_mask = T == 32 ? kAll : (1u << T) - 1u;
     const int nk = step_buckets(cpad);
-    const int vpitch = VK == 2 && ev.bits ? ev.bit_pitch : n_bin;
+    const int vpitch = kGeneral<VK> && ev.bits ? ev.bit_pitch : n_bin;
     const int64_t row0 = (int64_t)item.y * n_seg * p.n_det;
     const float xs = ev.x_scale;
 
@@ -854,7 +908,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
     // outside the band are taken off; amplitude weights are summed per lookup)
     if (tid < 2) {
       long long sum = 0;
-      if (p.amp_power == 0)
+      if (!kAmp<VK>)
         for (int i = 0; i < kStepSlots; ++i) sum += __ldg(ev.wtot + 2 * i + tid);
       s_wtot[tid] = (unsigned long long)sum;
     }
@@ -863,7 +917,6 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
 
     for (int tb = 0; tb < item.w; ++tb) {
       const int b0 = item.z + tb * T, b = b0 + lt;
-      const float famp = p.amp_power > 0 ? p.df_f / (float)ev.f0[b] : 0.f;
       if (tid == 0) {
         s_ctx.ev = &ev;
         s_ctx.chi = chi;
@@ -893,6 +946,10 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
         }
         fcoef[tid] = make_float4(cf[0], cf[1], cf[2], cf[3]);
         fcoef7[tid] = cf[4];
+        if (kAmp<VK>) {
+          const double u = p.df / ev.f0[b0 + tid];
+          famp[tid] = make_float2((float)u, (float)(u - (double)(float)u));
+        }
       }
       __syncthreads();
       long long X0 = 0;
@@ -1052,14 +1109,16 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
               const float small = (fmaf(A_hi, dt.x, -pl) + fmaf(A_hi, dt.y, A_lo * dt.x)) +
                                   (fmaf(Q_hi, dt.z, -pq) + fmaf(Q_hi, dt.w, Q_lo * dt.z)) + p3;
               const float F = (Xf + pl) + (pq + p3);
-              float amp = 1.0f;
-              if (p.amp_power > 0) {
-                const float rr = here && !edge ? F * famp : 1.0f;   // f / f0
-                amp = rr;
-                for (int k = 1; k < p.amp_power; ++k) amp *= rr;
-              }
               const float Fq = F * p.q, R = rcp_approx(F) * p.inv_q_f;
               const float y0 = ((frac_a + (pl - plr)) + ((pq - pqr) + small)) - hb;
+              float2 amp = make_float2(1.0f, 0.0f);
+              if (kAmp<VK> && here && !edge) {
+                // f/f0 as an fp32 pair, from the whole bins and the fraction of f/df apart
+                const float2 u = famp[lt];
+                const float fi = ((float)base_a + p.x_min_i) + (plr + pqr), ff = (y0 + hb) + p.x_min_f;
+                const float rh = fi * u.x;
+                amp = pair_power(rh, fmaf(fi, u.x, -rh) + fmaf(fi, u.y, ff * u.x), p.amp_power);
+              }
 #pragma unroll 1
               for (int dd = 0; dd < DP; ++dd) {
                 const int4 m0 = head[dd * kStepHead];
@@ -1079,10 +1138,15 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
                 const int K = base_a + 1 + (int)(plr + pqr + fl);   // the lowest sky's bin
                 const int64_t vrow = vbase + (int64_t)(dd * n_seg + jr) * vpitch;
                 // the loads of the lookup and its first two steps at once
-                const float ws = __int_as_float(m0.w) * amp * xs;
+                const PairWeight w(__int_as_float(m0.w), amp);
+                const float ws = w.h * xs, wsl = w.l * xs;
+                auto fixed = [&](float v, int& h, int& l) {
+                  if constexpr (kAmp<VK>) to_fixed(v, ws, wsl, h, l);
+                  else to_fixed(v, ws, h, l);
+                };
                 auto value = [&](int o, bool c) {   // of bin K + o
-                  if constexpr (VK == 0) return load_if(static_cast<const float*>(ev.rho) + (vrow + K) + o, c);
-                  else if constexpr (VK == 1) return load_if(static_cast<const __half*>(ev.rho) + (vrow + K) + o, c);
+                  if constexpr (VK % kWithAmp == kF32) return load_if(static_cast<const float*>(ev.rho) + (vrow + K) + o, c);
+                  else if constexpr (VK % kWithAmp == kF16) return load_if(static_cast<const __half*>(ev.rho) + (vrow + K) + o, c);
                   else return c ? step_value<VK>(p, ev, vrow, K + o) : 0.f;
                 };
                 const float v0 = value(0, on);
@@ -1107,17 +1171,17 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
                   win = window(th, at, nb > 1);
                 }
                 int h0, l0, h1, l1;
-                to_fixed(v0, ws, h0, l0);
+                fixed(v0, h0, l0);
                 xh += h0;
                 xl += l0;
                 ++nx;
                 if (some) {
-                  to_fixed(v1, ws, h1, l1);
+                  fixed(v1, h1, l1);
                   place(nb > 0, 0, th0, at0, win0, h1 - h0, l1 - l0, rr);
                   for (int i = 1; __any_sync(kAll, nb > i); ++i) {
                     h0 = h1;
                     l0 = l1;
-                    to_fixed(vn, ws, h1, l1);
+                    fixed(vn, h1, l1);
                     // the next step's loads before this one's placing
                     const int th_i = th;
                     const uint32_t at_i = at;
@@ -1128,17 +1192,16 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
                     place(nb > i, i, th_i, at_i, win_i, h1 - h0, l1 - l0, rr);
                   }
                 }
-                if (p.amp_power > 0 && on) {
-                  const float w = __int_as_float(m0.w) * amp;
-                  atomicAdd(tsum + 32 + lt, (unsigned long long)fixed_word(w, ev.w1_scale));
-                  atomicAdd(tsum + 64 + lt, (unsigned long long)fixed_word(w, w * ev.w2_scale));
+                if (kAmp<VK> && on) {
+                  atomicAdd(tsum + 32 + lt, (unsigned long long)w.w1(ev));
+                  atomicAdd(tsum + 64 + lt, (unsigned long long)w.w2(ev));
                 }
               }
             }
             X0 += (long long)(xh - nx * kMagicBits) * 65536 + (xl - nx * kMagicBits);
             {
               const int nr = min(jb, ns) * DP;
-              if ((outside & t_mask) && p.amp_power == 0) {
+              if (!kAmp<VK> && (outside & t_mask)) {
                 // out of the band: the turn's weights come off
                 longlong2 wi = make_longlong2(0, 0);
                 if (lane < nr) {
@@ -1225,19 +1288,24 @@ struct Launch {
   }
 };
 
+template <int DP, int LT, int AMP, typename F>
+cudaError_t pick_value(const StepForm& v, const F& f) {
+  if (v.general) return f.template run<AMP + kGen, DP, LT>();
+  return v.half ? f.template run<AMP + kF16, DP, LT>() : f.template run<AMP + kF32, DP, LT>();
+}
 template <int DP, int LT, typename F>
-cudaError_t pick_value(bool half, bool general, const F& f) {
-  if (general) return f.template run<2, DP, LT>();
-  return half ? f.template run<1, DP, LT>() : f.template run<0, DP, LT>();
+cudaError_t pick_amp(const StepForm& v, const F& f) {
+  return v.amp ? pick_value<DP, LT, kWithAmp>(v, f) : pick_value<DP, LT, 0>(v, f);
 }
 template <typename F>
-cudaError_t pick(int dp, int log_t, bool half, bool general, const F& f) {
-  if (dp == 1 && log_t == 2) return pick_value<1, 2>(half, general, f);
-  if (dp == 1 && log_t == 4) return pick_value<1, 4>(half, general, f);
-  if (dp == 1 && log_t == 5) return pick_value<1, 5>(half, general, f);
-  if (dp == 2 && log_t == 2) return pick_value<2, 2>(half, general, f);
-  if (dp == 2 && log_t == 4) return pick_value<2, 4>(half, general, f);
-  if (dp == 2 && log_t == 5) return pick_value<2, 5>(half, general, f);
+cudaError_t pick(const StepForm& v, const F& f) {
+  const int dp = v.dets_per_pass;
+  if (dp == 1 && v.log_t == 2) return pick_amp<1, 2>(v, f);
+  if (dp == 1 && v.log_t == 4) return pick_amp<1, 4>(v, f);
+  if (dp == 1 && v.log_t == 5) return pick_amp<1, 5>(v, f);
+  if (dp == 2 && v.log_t == 2) return pick_amp<2, 2>(v, f);
+  if (dp == 2 && v.log_t == 4) return pick_amp<2, 4>(v, f);
+  if (dp == 2 && v.log_t == 5) return pick_amp<2, 5>(v, f);
   return cudaErrorInvalidValue;
 }
 
@@ -1398,16 +1466,14 @@ cudaError_t launch_absmax(const void* rho, bool half, int64_t n, unsigned* out, 
   return cudaGetLastError();
 }
 
-cudaError_t step_prepare(int dets_per_pass, int log_t, bool half, bool general) {
-  return pick(dets_per_pass, log_t, half, general, Prepare{});
-}
+cudaError_t step_prepare(const StepForm& v) { return pick(v, Prepare{}); }
 
-cudaError_t launch_step(const StepParams& p, int dets_per_pass, int log_t, bool half, bool general, int cells,
-                        int grid, cudaStream_t st) {
-  if (p.n_det < 1 || p.n_det % dets_per_pass || cells > kStepCells + 32 || p.nterms < 1)
+cudaError_t launch_step(const StepParams& p, const StepForm& v, int cells, int grid, cudaStream_t st) {
+  if (p.n_det < 1 || p.n_det % v.dets_per_pass || cells > kStepCells + 32 || p.nterms < 1 ||
+      (p.amp_power > 0) != v.amp)
     return cudaErrorInvalidValue;
   if (grid <= 0) return cudaSuccess;
-  return pick(dets_per_pass, log_t, half, general, Launch{p, cells, grid, st});
+  return pick(v, Launch{p, cells, grid, st});
 }
 
 cudaError_t launch_step_tiles(const StepTileParams& p, cudaStream_t st) {

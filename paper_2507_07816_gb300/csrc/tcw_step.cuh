@@ -95,7 +95,7 @@ struct StepParams {
   float q, inv_q_f;
   float eps;                 // bound of the fp32 thresholds' error, in bins
   int nterms, tile_shift;    // FP64 track series (> 0), anchor tiles
-  float df_f;
+  float x_min_i, x_min_f;    // f_min / df: whole bins, fraction
   int amp_power;
   double nc_q;               // number count: q = exp(-rho_th), else 0
   int track_bins;
@@ -175,7 +175,11 @@ struct StepTrack {
 };
 StepTrack step_track(const double* t_mid, int64_t n_seg, double T0, int most, double tau_min, double r_max,
                      double x_max, double x_top, double db, double f_min, double df, double inv_q);
+// p.f_min and p.df are set.
 inline void set_step_track(StepParams& p, const StepTrack& t) {
+  const double x = p.f_min / p.df, i = std::nearbyint(x);
+  p.x_min_i = (float)i;      // below 2^23 where the track is ok
+  p.x_min_f = (float)(x - i);
   p.eps = t.eps;
   p.nterms = t.nterms;
   p.tile_shift = t.shift;
@@ -236,12 +240,16 @@ inline int step_cells(const StepGeometry& g) { return (g.cpad + 1) << g.log_t; }
 size_t step_slow_bytes(int grid);
 inline size_t step_edge_bytes(int grid) { return (size_t)grid * (2 * kStepCells + 32) * sizeof(longlong2); }
 cudaError_t launch_step_rows(const StepRowsParams& p, cudaStream_t st);
+// A form of the search kernel: detectors of a pass, templates of a block (log2), an
+// FP16 map, number count or two-bin lookups (general), amplitude weights.
+struct StepForm {
+  int dets_per_pass, log_t;
+  bool half, general, amp;
+};
 // Raises the kernel's shared-memory limit (also done at its first launch; call before a graph capture).
-cudaError_t step_prepare(int dets_per_pass, int log_t, bool half, bool general);
-// general: number count or two-bin lookups; cells: the largest step_cells of the items' events,
-// which all have this log_t and passes of dets_per_pass detectors.
-cudaError_t launch_step(const StepParams& p, int dets_per_pass, int log_t, bool half, bool general, int cells,
-                        int grid, cudaStream_t st);
+cudaError_t step_prepare(const StepForm& v);
+// cells: the largest step_cells of the items' events, which are all of this form.
+cudaError_t launch_step(const StepParams& p, const StepForm& v, int cells, int grid, cudaStream_t st);
 // *out = bits of the largest |rho| (NaN above infinity above every finite value); out zero at launch.
 cudaError_t launch_absmax(const void* rho, bool half, int64_t n, unsigned* out, cudaStream_t st);
 

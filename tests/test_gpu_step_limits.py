@@ -62,12 +62,15 @@ def test_wide_bands(n_bin, step):
     assert check(p) == step
 
 
-@pytest.mark.parametrize("statistic,bins,amp", [("power", 1, 0), ("power", 2, 0), ("count", 1, 0)])
+@pytest.mark.parametrize("statistic,bins,amp", [("power", 1, 0), ("power", 2, 0), ("power", 1, 4), ("power", 1, 7),
+                                                ("count", 1, 0)])
 def test_psi_is_rounded_once(statistic, bins, amp):
     """A few skies far apart (too wide a group for the group kernel): Psi is Eq. 4 of
     exact sums, rounded once to fp32 (2^-24 relative, 2^-25 for its pieces), as from
     sums in FP64.  The sums' grid is 2^-25 or finer here, 0.3 of it per value: 6 sigma
-    of that are 2^-23 of sigma = sqrt(W2) when the weights' rms is at least 0.25."""
+    of that are 2^-23 of sigma = sqrt(W2) when the weights' rms is at least 0.25.
+    Amplitude weights are rounded twice to fp32 per lookup, independently: below 2^-24
+    of a sum of 50 of them and of its squares' at 6 sigma, beside the sums' own 2^-24."""
     r = syn.rng(2100)
     n_seg = 1500
     t = syn.segment_times(n_seg, 4.0)
@@ -86,4 +89,6 @@ def test_psi_is_rounded_once(statistic, bins, amp):
     assert_topk_consistent(st["psi"], idx, val, 3)
     ok = W2 >= 0.0625 * W1.max() / 16
     assert ok.mean() > 0.5 and np.abs(psi[ok]).max() > 20
+    assert np.all(np.abs(st["W1"] - W1)[ok] <= 2.0 ** -23 * W1[ok])
+    assert np.all(np.abs(st["W2"] - W2)[ok] <= 2.0 ** -23 * W2[ok])
     assert np.all(np.abs(st["psi"] - psi)[ok] <= (2.0 ** -24 + 2.0 ** -25) * np.abs(psi[ok]) + 2.0 ** -23)

@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <climits>
 #include <cmath>
+#include <type_traits>
 
 #include "tcw_step.cuh"
 
@@ -392,27 +393,31 @@ constexpr bool kAmp = VK >= kWithAmp;
 template <int VK>
 constexpr bool kGeneral = VK % kWithAmp == kGen;
 
-// A value of the lookup at bin K of row (the caller checks the band).
+// A value of the lookup at bin K of row (the caller checks the band); of two bins,
+// their sum and its rounding error.
 template <int VK>
-__device__ __forceinline__ float step_value(const StepParams& p, const StepEvent& ev, int64_t row, int K) {
+using StepValue = std::conditional_t<kGeneral<VK>, float2, float>;
+template <int VK>
+__device__ __forceinline__ StepValue<VK> step_value(const StepParams& p, const StepEvent& ev, int64_t row, int K) {
   if constexpr (VK % kWithAmp == kF32) {
     return __ldg(static_cast<const float*>(ev.rho) + (row + K));
   } else if constexpr (VK % kWithAmp == kF16) {
     return __half2float(__ldg(static_cast<const __half*>(ev.rho) + (row + K)));
   } else {
     const int more = p.track_bins == 2 ? 1 : 0;
-    float v = 0.f;
     if (ev.bits) {
       const uint32_t* r = ev.bits + row;
+      float v = 0.f;
       for (int i = 0; i <= more; ++i) v += (float)((__ldg(r + ((K + i) >> 5)) >> ((K + i) & 31)) & 1u);
-    } else {
-      for (int i = 0; i <= more; ++i) {
-        const int64_t o = row + K + i;
-        v += p.map_half ? __half2float(__ldg(static_cast<const __half*>(ev.rho) + o))
-                        : __ldg(static_cast<const float*>(ev.rho) + o);
-      }
+      return make_float2(v, 0.f);
     }
-    return v;
+    auto power = [&](int64_t o) {
+      return p.map_half ? __half2float(__ldg(static_cast<const __half*>(ev.rho) + o))
+                        : __ldg(static_cast<const float*>(ev.rho) + o);
+    };
+    const float a = power(row + K), b = more ? power(row + K + 1) : 0.f;
+    const float v = a + b, bb = v - a;   // the error of a sum, Knuth's two-sum
+    return make_float2(v, (a - (v - bb)) + (b - bb));
   }
 }
 
@@ -455,18 +460,25 @@ __device__ __forceinline__ void to_fixed(float v, float s, int& hi, int& lo) {
   hi = __float_as_int(t);
   lo = __float_as_int(fmaf(r, 65536.0f, kMagic));
 }
-// v (s + sl), |sl| < 2^-23 |s|
-__device__ __forceinline__ void to_fixed(float v, float s, float sl, int& hi, int& lo) {
+// v s + more, |more| < 2^-22 |v s|
+__device__ __forceinline__ void to_fixed(float v, float s, float more, int& hi, int& lo) {
   const float t = fmaf(v, s, kMagic);
-  const float r = fmaf(v, sl, fmaf(v, s, -(t - kMagic)));
+  const float r = fmaf(v, s, -(t - kMagic)) + more;
   hi = __float_as_int(t);
   lo = __float_as_int(fmaf(r, 65536.0f, kMagic));
 }
 // The same as one 64-bit word.
-__device__ __forceinline__ long long fixed_word(float v, float s, float sl) {
+__device__ __forceinline__ long long fixed_word(float v, float s, float more) {
   int hi, lo;
-  to_fixed(v, s, sl, hi, lo);
+  to_fixed(v, s, more, hi, lo);
   return (long long)(hi - kMagicBits) * 65536 + (lo - kMagicBits);
+}
+// A value times the weight s + sl (sl with amplitude weights only).
+template <int VK>
+__device__ __forceinline__ void to_fixed(StepValue<VK> v, float s, float sl, int& hi, int& lo) {
+  if constexpr (kGeneral<VK>) to_fixed(v.x, s, kAmp<VK> ? fmaf(v.y, s, v.x * sl) : v.y * s, hi, lo);
+  else if constexpr (kAmp<VK>) to_fixed(v, s, v * sl, hi, lo);
+  else to_fixed(v, s, hi, lo);
 }
 
 // (h + l)^n, 1 <= n and |l| < |h|, as an fp32 pair x + y with x the nearest float:
@@ -494,10 +506,10 @@ struct PairWeight {
     l = fmaf(w, amp.x, -h) + w * amp.y;
   }
   __device__ __forceinline__ long long w1(const StepEvent& ev) const {
-    return fixed_word(1.0f, h * ev.w1_scale, l * ev.w1_scale);
+    return fixed_word(h, ev.w1_scale, l * ev.w1_scale);
   }
   __device__ __forceinline__ long long w2(const StepEvent& ev) const {
-    return fixed_word(h, h * ev.w2_scale, 2.0f * l * ev.w2_scale);
+    return fixed_word(h, h * ev.w2_scale, 2.0f * h * l * ev.w2_scale);
   }
 };
 
@@ -589,9 +601,9 @@ __device__ __forceinline__ void step_rare(const StepParams& p, StepBlockCtx& c, 
       ((int64_t)d * ev.n_seg + j) * (kGeneral<VK> && ev.bits ? (int64_t)ev.bit_pitch : p.n_bin);
   const int qmin = m0.x, qmax = m0.y;
   auto value = [&](int K, int& h, int& l) {
-    const float v = (unsigned)K < k_end ? step_value<VK>(p, ev, vrow, K) : 0.f;
-    if constexpr (kAmp<VK>) to_fixed(v, ws, wsl, h, l);
-    else to_fixed(v, ws, h, l);
+    StepValue<VK> v{};
+    if ((unsigned)K < k_end) v = step_value<VK>(p, ev, vrow, K);
+    to_fixed<VK>(v, ws, wsl, h, l);
   };
   auto step = [&](int t, int K, long long e1, long long e2) {   // from bin K to K + 1
     int h0, l0, h1, l1;
@@ -1140,16 +1152,12 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
                 // the loads of the lookup and its first two steps at once
                 const PairWeight w(__int_as_float(m0.w), amp);
                 const float ws = w.h * xs, wsl = w.l * xs;
-                auto fixed = [&](float v, int& h, int& l) {
-                  if constexpr (kAmp<VK>) to_fixed(v, ws, wsl, h, l);
-                  else to_fixed(v, ws, h, l);
-                };
                 auto value = [&](int o, bool c) {   // of bin K + o
                   if constexpr (VK % kWithAmp == kF32) return load_if(static_cast<const float*>(ev.rho) + (vrow + K) + o, c);
                   else if constexpr (VK % kWithAmp == kF16) return load_if(static_cast<const __half*>(ev.rho) + (vrow + K) + o, c);
-                  else return c ? step_value<VK>(p, ev, vrow, K + o) : 0.f;
+                  else return c ? step_value<VK>(p, ev, vrow, K + o) : make_float2(0.f, 0.f);
                 };
-                const float v0 = value(0, on);
+                const StepValue<VK> v0 = value(0, on);
                 const unsigned some = __ballot_sync(kAll, nb > 0);
                 const uint2* const tr = ev.fast + (rbase + rl) * nk;
                 const float y1 = fl + 1.0f - y0;
@@ -1158,7 +1166,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
                   at = ((uint32_t)pl >> kFracShift) + (1u << kFracBits);
                   return load_if(tr + step_bucket(pl, nk), c);
                 };
-                float v1 = 0.f, vn = 0.f;
+                StepValue<VK> v1{}, vn{};
                 int th0 = 0, th = 0;
                 uint2 win0 = make_uint2(0, 0), win = win0;
                 uint32_t at0 = 0, at = 0;
@@ -1171,17 +1179,17 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
                   win = window(th, at, nb > 1);
                 }
                 int h0, l0, h1, l1;
-                fixed(v0, h0, l0);
+                to_fixed<VK>(v0, ws, wsl, h0, l0);
                 xh += h0;
                 xl += l0;
                 ++nx;
                 if (some) {
-                  fixed(v1, h1, l1);
+                  to_fixed<VK>(v1, ws, wsl, h1, l1);
                   place(nb > 0, 0, th0, at0, win0, h1 - h0, l1 - l0, rr);
                   for (int i = 1; __any_sync(kAll, nb > i); ++i) {
                     h0 = h1;
                     l0 = l1;
-                    fixed(vn, h1, l1);
+                    to_fixed<VK>(vn, ws, wsl, h1, l1);
                     // the next step's loads before this one's placing
                     const int th_i = th;
                     const uint32_t at_i = at;

@@ -92,3 +92,24 @@ def test_psi_is_rounded_once(statistic, bins, amp):
     assert np.all(np.abs(st["W1"] - W1)[ok] <= 2.0 ** -23 * W1[ok])
     assert np.all(np.abs(st["W2"] - W2)[ok] <= 2.0 ** -23 * W2[ok])
     assert np.all(np.abs(st["psi"] - psi)[ok] <= (2.0 ** -24 + 2.0 ** -25) * np.abs(psi[ok]) + 2.0 ** -23)
+
+
+def test_two_bin_sums_are_not_rounded():
+    """Bins of 1 + 2^-23 and 1 - 2^-24 in turn: every pair sums to 2 + 2^-24, which fp32
+    rounds to 2.  Psi is n 2^-24 / sqrt(2 n), 2e-6 here, and 0 from rounded sums."""
+    r = syn.rng(2200)
+    n_seg = 1500
+    t = syn.segment_times(n_seg, 4.0)
+    dets = syn.random_detectors(r, 2)
+    vel = np.stack([d.velocity(t) for d in dets])
+    bank = syn.random_bank(r, 60, f0_range=(800.0, 1200.0), tau_range=(3500, 35000))
+    row = np.where(np.arange(3000) % 2 == 0, 1 + 2.0 ** -23, 1 - 2.0 ** -24).astype(np.float32)
+    p = syn.Problem(np.broadcast_to(row, (2, n_seg, 3000)).copy(), t, None, vel, 500.0, 0.25, float(t[0] - 2.0),
+                    syn.random_sky(r, 12), bank, [], dets, name="pairs")
+    for amp in (0, 2):
+        _, _, st, info = run(p, options=[(tcw.OPT_TRACK_BINS, 2), (tcw.OPT_AMPLITUDE_POWER, amp)])
+        assert info.kernel == tcw.KERNEL_GROUP
+        psi = oracle.search_stats(p.rho, p.f_min, p.df, p.t_mid, p.weights, p.velocity, p.nhat, bank.f0, bank.tau, bank.n,
+                                  p.T0, track_bins=2, amp_power=amp)[3]
+        assert np.abs(psi).max() > 1.5e-6
+        assert np.all(np.abs(st["psi"] - psi) <= 2.0 ** -23)

@@ -163,19 +163,19 @@ tcw_status ensure_bits(tcw_ctx* c, int* launches) {
   return TCW_OK;
 }
 
-// Largest |rho| of the loaded map, taken once per load.
-tcw_status ensure_map_max(tcw_ctx* c) {
-  if (c->map_max_epoch == c->spec_epoch) return TCW_OK;
+// Range of the loaded map's powers, taken once per load.
+tcw_status ensure_map_range(tcw_ctx* c) {
+  if (c->map_epoch == c->spec_epoch) return TCW_OK;
   TCW_CUDA(c, c->flags.ensure(64), "flags");
   unsigned* out = reinterpret_cast<unsigned*>(c->flags.as<char>() + 40);
-  unsigned bits = 0;
-  TCW_CUDA(c, cudaMemsetAsync(out, 0, 4, c->stream), "map maximum");
-  TCW_CUDA(c, launch_absmax(c->rho.p, c->dtype == TCW_F16, (int64_t)c->D * c->Nseg * c->Nbin, out, c->stream),
-           "absmax_kernel launch");
-  TCW_CUDA(c, cudaMemcpyAsync(&bits, out, 4, cudaMemcpyDeviceToHost, c->stream), "map maximum");
-  TCW_CUDA(c, cudaStreamSynchronize(c->stream), "map maximum");
-  std::memcpy(&c->map_max, &bits, 4);
-  c->map_max_epoch = c->spec_epoch;
+  unsigned bits[kMapWords] = {};
+  TCW_CUDA(c, cudaMemsetAsync(out, 0, sizeof(bits), c->stream), "map range");
+  TCW_CUDA(c, launch_map_range(c->rho.p, c->dtype == TCW_F16, (int64_t)c->D * c->Nseg * c->Nbin, out, c->stream),
+           "map_range_kernel launch");
+  TCW_CUDA(c, cudaMemcpyAsync(bits, out, sizeof(bits), cudaMemcpyDeviceToHost, c->stream), "map range");
+  TCW_CUDA(c, cudaStreamSynchronize(c->stream), "map range");
+  c->map = map_range(bits);
+  c->map_epoch = c->spec_epoch;
   return TCW_OK;
 }
 
@@ -188,11 +188,10 @@ tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, boo
   if (!pl.group_ok || c->D > 2) return TCW_OK;
   const bool count = c->statistic == TCW_STAT_NUMBER_COUNT;
   tcw_status st = TCW_OK;
-  if (!count && (st = ensure_map_max(c)) != TCW_OK) return st;
-  const double vmax = (count ? 1.0 : (double)c->map_max) * c->track_bins;
+  if (!count && (st = ensure_map_range(c)) != TCW_OK) return st;
   const double f_top = c->f_min + (double)c->Nbin * c->df;
   const StepScales sc =
-      step_scales(vmax, c->w_min, c->w_max,
+      step_scales(count ? MapRange{1.0f, 1.0f} : c->map, c->track_bins, c->w_range,
                   step_amp_ref(c->amp_power, c->h_t, c->T0, c->bank_tau_min, c->bank_r_max, f_top, c->bank_f0max),
                   (int64_t)c->D * c->Nseg);
   if (!sc.ok) return TCW_OK;
@@ -1067,13 +1066,10 @@ tcw_status tcw_load_spectrogram(tcw_ctx* c, int n_det, int64_t n_seg, int64_t n_
   c->df = df;
   c->h_t = std::move(t);
   c->unit_weights = true;
-  c->w_min = INFINITY;
-  c->w_max = 0;
-  for (float x : w) {
+  c->w_range = WeightRange{};
+  c->w_range.take(w);
+  for (float x : w)
     if (x != 1.0f) c->unit_weights = false;
-    if (x > 0 && x < c->w_min) c->w_min = x;
-    if (x > c->w_max) c->w_max = x;
-  }
   c->have_spec = true;
   c->have_result = false;
   c->sky_dirty = true;

@@ -43,7 +43,8 @@ struct EventHost {
   int64_t out_row = 0;             // first output row (sum of earlier events' n_sky)
   int wave = 0;
   // step-function search (tcw_step.cuh)
-  float w_min = 0, w_max = 0, map_max = 0;   // smallest nonzero and largest weight, largest |rho|
+  WeightRange w_range;
+  MapRange map;
   StepGeometry geo{};
   StepScales scales;
   size_t o_q = 0, o_head = 0, o_tab = 0, o_fast = 0, o_wfix = 0, o_wtot = 0, o_order = 0;   // byte offsets of its Doppler rows
@@ -264,7 +265,7 @@ void plan_step(const tcw_ctx* c, BatchState* b, int tile) {
     split = true;   // some event takes its detectors one by one: all of them do
   }
   for (EventHost& e : b->ev) {
-    e.scales = step_scales((count ? 1.0 : (double)e.map_max) * c->track_bins, e.w_min, e.w_max,
+    e.scales = step_scales(count ? MapRange{1.0f, 1.0f} : e.map, c->track_bins, e.w_range,
                            step_amp_ref(c->amp_power, e.t, e.T0, c->bank_tau_min, c->bank_r_max, f_top, c->bank_f0max),
                            (int64_t)b->D * e.n_seg);
     if (!e.scales.ok) return;
@@ -957,11 +958,7 @@ tcw_status tcw_load_events(tcw_ctx* c, int n_det, int64_t n_bin, int dtype, doub
     } else {
       w.assign((size_t)n_det * in.n_seg, 1.0f);
     }
-    e.w_min = INFINITY;
-    for (float x : w) {
-      if (x > 0 && x < e.w_min) e.w_min = x;
-      if (x > e.w_max) e.w_max = x;
-    }
+    e.w_range.take(w);
     wts[i] = std::move(w);
     b->unit_weights = b->unit_weights && e.unit_w;
     // sky sorted by its Doppler factor at the event's middle segment (detector 0)
@@ -1037,23 +1034,22 @@ tcw_status tcw_load_events(tcw_ctx* c, int n_det, int64_t n_bin, int dtype, doub
     return cuda_fail(c, ce, "event upload");
   }
   {
-    // the largest |rho| of every event (the step-function search's conditions)
-    DevBuf mx;
-    std::vector<float> h(n_events);
-    ce = mx.ensure((size_t)n_events * 4);
-    if (ce == cudaSuccess) ce = cudaMemsetAsync(mx.p, 0, (size_t)n_events * 4, c->stream);
+    // the range of every event's powers (the step-function search's conditions)
+    DevBuf mr;
+    std::vector<unsigned> h(kMapWords * (size_t)n_events);
+    ce = mr.ensure(h.size() * 4);
+    if (ce == cudaSuccess) ce = cudaMemsetAsync(mr.p, 0, h.size() * 4, c->stream);
     for (int i = 0; i < n_events && ce == cudaSuccess; ++i)
-      ce = launch_absmax(at<char>(b->rho, b->ev[i].o_rho), dtype == TCW_F16, (int64_t)n_det * b->ev[i].n_seg * n_bin,
-                         mx.as<unsigned>() + i, c->stream);
-    if (ce == cudaSuccess)
-      ce = cudaMemcpyAsync(h.data(), mx.p, (size_t)n_events * 4, cudaMemcpyDeviceToHost, c->stream);
+      ce = launch_map_range(at<char>(b->rho, b->ev[i].o_rho), dtype == TCW_F16, (int64_t)n_det * b->ev[i].n_seg * n_bin,
+                            mr.as<unsigned>() + kMapWords * (size_t)i, c->stream);
+    if (ce == cudaSuccess) ce = cudaMemcpyAsync(h.data(), mr.p, h.size() * 4, cudaMemcpyDeviceToHost, c->stream);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(c->stream);
-    mx.release();
+    mr.release();
     if (ce != cudaSuccess) {
       batch_free(c);
-      return cuda_fail(c, ce, "map maximum");
+      return cuda_fail(c, ce, "map range");
     }
-    for (int i = 0; i < n_events; ++i) b->ev[i].map_max = h[i];
+    for (int i = 0; i < n_events; ++i) b->ev[i].map = map_range(&h[kMapWords * (size_t)i]);
   }
   for (EventHost& e : b->ev) {
     if ((size_t)b->D * e.n_seg * n_bin * esz < 64) {

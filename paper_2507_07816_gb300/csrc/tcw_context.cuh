@@ -66,9 +66,9 @@ struct tcw_ctx {
   double f_min = 0, df = 0;
   std::vector<double> h_t;
   bool unit_weights = true;
-  float w_min = 0, w_max = 0;        // smallest nonzero and largest weight
-  float map_max = 0;                 // largest |rho| of the loaded map (see ensure_map_max)
-  unsigned map_max_epoch = ~0u;
+  tcw::WeightRange w_range;
+  tcw::MapRange map;                 // of the loaded map (see ensure_map_range)
+  unsigned map_epoch = ~0u;
   tcw::DevBuf rho, t_mid, weights;
   tcw::DevBuf bits;        // number-count bit map of rho (see tcw_set_statistic)
   unsigned bits_epoch = ~0u;

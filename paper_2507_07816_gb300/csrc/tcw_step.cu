@@ -1,8 +1,9 @@
 // tcw_step.cu -- the exhaustive search as step functions over the sorted sky
-// (tcw_step.cuh): Doppler rows, the search kernel, the map's largest value.
+// (tcw_step.cuh): Doppler rows, the search kernel, the map's range of powers.
 #include <algorithm>
 #include <climits>
 #include <cmath>
+#include <cstring>
 #include <type_traits>
 
 #include "tcw_step.cuh"
@@ -341,27 +342,59 @@ __global__ void __launch_bounds__(128) step_rows_kernel(StepRowsParams p) {
   }
 }
 
+// The largest |rho| of a map and its level (MapRange): one read of the map.  out[0]:
+// bits of the largest; [1], [2]: infinity's bits minus those of the smallest maximum of
+// a run of kLevelRun values at least half of which are nonzero, or fewer; [3], [4]:
+// the number of such runs (zero at launch).
 template <typename T>
-__global__ void absmax_kernel(const T* x, int64_t n, unsigned* out) {
-  unsigned m = 0;
-  constexpr int V = 16 / sizeof(T);
+__global__ void map_range_kernel(const T* x, int64_t n, unsigned* out) {
+  constexpr unsigned kInf = 0x7f800000u, kAll = 0xffffffffu;
+  constexpr int V = 16 / sizeof(T), R = kLevelRun / V;   // values of a load, lanes of a run
+  unsigned m = 0, low[2] = {0, 0}, runs[2] = {0, 0};
+  const int lane = threadIdx.x & 31;
   const int64_t nv = n / V, stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  auto take = [&](T v) {
+  auto bits = [](T v) {
     float f;
     if constexpr (sizeof(T) == 2) f = __half2float(v);
     else f = v;
-    m = max(m, __float_as_uint(f) & 0x7fffffffu);
+    return __float_as_uint(f) & 0x7fffffffu;
   };
-  for (int64_t i = i0; i < nv; i += stride) {
-    const int4 v = reinterpret_cast<const int4*>(x)[i];
-    const T* e = reinterpret_cast<const T*>(&v);
+  for (int64_t i = i0; i - lane < nv; i += stride) {
+    unsigned r = 0, c = 0;
+    if (i < nv) {
+      const int4 v = reinterpret_cast<const int4*>(x)[i];
+      const T* e = reinterpret_cast<const T*>(&v);
 #pragma unroll
-    for (int k = 0; k < V; ++k) take(e[k]);
+      for (int k = 0; k < V; ++k) {
+        const unsigned b = bits(e[k]);
+        r = max(r, b);
+        c += b != 0;
+      }
+    }
+    m = max(m, r);
+#pragma unroll
+    for (int off = 1; off < R; off <<= 1) {
+      r = max(r, __shfl_xor_sync(kAll, r, off));
+      c += __shfl_xor_sync(kAll, c, off);
+    }
+    if ((lane & (R - 1)) == 0 && (i | (R - 1)) < nv && r > 0 && r < kInf) {
+      const int few = c < kLevelRun / 2;
+      low[few] = max(low[few], kInf - r);
+      ++runs[few];
+    }
   }
-  for (int64_t i = nv * V + i0; i < n; i += stride) take(x[i]);
-  for (int off = 16; off > 0; off >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, off));
-  if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+  for (int64_t i = nv * V + i0; i < n; i += stride) m = max(m, bits(x[i]));
+  m = __reduce_max_sync(kAll, m);
+  if (lane == 0) atomicMax(out, m);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const unsigned l = __reduce_max_sync(kAll, low[k]), c = __reduce_add_sync(kAll, runs[k]);
+    if (lane == 0 && c) {
+      atomicMax(out + 1 + k, l);
+      atomicAdd(out + 3 + k, c);
+    }
+  }
 }
 
 // Shared memory of the search kernel for `cells` difference cells (templates x
@@ -1321,19 +1354,34 @@ cudaError_t pick(const StepForm& v, const F& f) {
 
 size_t step_slow_bytes(int grid) { return (size_t)grid * kStepWarps * kStepSlow * sizeof(int4); }
 
-StepScales step_scales(double vmax, double w_min, double w_max, double a_ref, int64_t n) {
+MapRange map_range(const unsigned* out) {
+  MapRange r;
+  // runs with few nonzero powers are the edges of zeroed stretches, unless they are many
+  const unsigned low = out[4] > out[3] / 16 ? std::max(out[1], out[2]) : out[1];
+  const unsigned level = out[3] + out[4] ? 0x7f800000u - low : out[0];
+  std::memcpy(&r.max, &out[0], 4);
+  std::memcpy(&r.level, &level, 4);
+  return r;
+}
+
+StepScales step_scales(const MapRange& map, int bins, const WeightRange& w, double a_ref, int64_t n) {
   StepScales s;
-  if (!(vmax >= 0.0) || !(vmax < 1e30) || !(w_max > 0.0) || !(w_min > 0.0) || n < 1) return s;
-  auto lg = [](double v) { return (int)std::ceil(std::log2(v)) + 1; };   // v < 2^lg, with a margin
-  const int lm = lg(std::max(vmax, 1.0) * w_max), lw = lg(w_max), lw2 = lg(w_max * w_max), ln = lg((double)n);
-  // the sum of a (template, sky) below 2^47 units and one value below 2^21 2^16 units
-  s.x = std::min(46 - ln - lm, 36 - lm);
+  const double vmax = (double)map.max * bins;
+  if (!(vmax >= 0.0) || !(vmax < 1e30) || !(w.max > 0.0) || n < 1) return s;
+  auto lg = [](double v) { return (int)std::ceil(std::log2(v)); };   // v <= 2^lg
+  const int lw = lg(w.max) + 1, lw2 = lg((double)w.max * w.max) + 1, ln = lg((double)n) + 1;
+  // the sums of a (template, sky), of powers and of their means, within 2^46 units and
+  // one value within 2^21 2^16 units
+  const double v = std::max(vmax, (double)bins);
+  s.x = std::min(46 - lg(v * w.sum), 37 - lg(v * w.max));
   s.w1 = std::min(36 - lw, 60 - ln - lw);
   s.w2 = std::min(36 - lw2, 60 - ln - lw2) & ~1;   // even: the root of its unit is a power of 2
-  // one unit at most 2^-20 of the smallest weighted unit power: a sum of n
-  // rounded values is then off by about 0.3 sqrt(n) 2^-20 of it, 3e-7 of the
-  // standard deviation sqrt(n) that Eq. 4 divides by
-  const int need = 20 - (int)std::floor(std::log2(w_min * a_ref));
+  // one unit at most 2^-22 of the smallest weighted power, the noise's mean or, where
+  // the map lies lower, twice its level: a sum of m rounded values is then off by about
+  // 0.3 sqrt(m) 2^-22 of it, 7e-8 of the standard deviation sqrt(m) that Eq. 4 divides
+  // by and less of S
+  const double p = map.level > 0 ? std::min(1.0, 2.0 * (double)map.level) : 1.0;
+  const int need = 22 - (int)std::floor(std::log2((double)w.min * a_ref * p));
   s.ok = s.x >= need && std::abs(s.x) < 100 && std::abs(s.w1) < 100 && std::abs(s.w2) < 100 && need < 100;
   return s;
 }
@@ -1465,12 +1513,12 @@ cudaError_t launch_step_rows(const StepRowsParams& p, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_absmax(const void* rho, bool half, int64_t n, unsigned* out, cudaStream_t st) {
+cudaError_t launch_map_range(const void* rho, bool half, int64_t n, unsigned* out, cudaStream_t st) {
   const int64_t blocks = std::min<int64_t>((n + 8191) / 8192, 152 * 16);
   if (half)
-    absmax_kernel<__half><<<(unsigned)blocks, 256, 0, st>>>(static_cast<const __half*>(rho), n, out);
+    map_range_kernel<__half><<<(unsigned)blocks, 256, 0, st>>>(static_cast<const __half*>(rho), n, out);
   else
-    absmax_kernel<float><<<(unsigned)blocks, 256, 0, st>>>(static_cast<const float*>(rho), n, out);
+    map_range_kernel<float><<<(unsigned)blocks, 256, 0, st>>>(static_cast<const float*>(rho), n, out);
   return cudaGetLastError();
 }
 

@@ -193,16 +193,39 @@ struct StepTileParams {
 };
 cudaError_t launch_step_tiles(const StepTileParams& p, cudaStream_t st);
 
+// What the fixed-point sums are scaled by.  A map's largest |rho|, and its level: the
+// smallest maximum of |rho| over its runs of kLevelRun bins (0: every bin is 0), about
+// the mean power of the quietest stretch (0.95 for noise of mean 1 over 2e8 bins; runs
+// of 4 would give 0.01).  Runs of zeros don't count, and those at their edges, with
+// fewer than half of the bins nonzero, only where they are more than 1 in 16.
+constexpr int kLevelRun = 32;
+constexpr int kMapWords = 5;   // words that launch_map_range writes
+struct MapRange {
+  float max = 0, level = 0;
+};
+MapRange map_range(const unsigned* out);   // from launch_map_range's words
+// The segments' weights: smallest nonzero one, largest one, sum.
+struct WeightRange {
+  float min = INFINITY, max = 0;
+  double sum = 0;
+  void take(const std::vector<float>& w) {
+    for (float x : w) {
+      if (x > 0 && x < min) min = x;
+      if (x > max) max = x;
+      sum += x;
+    }
+  }
+};
+
 // Fixed-point scales of one event, or ok = false when the sums would not be
 // at least as accurate as fp32 partial sums (see step_scales).
 struct StepScales {
   bool ok = false;
   int x = 0, w1 = 0, w2 = 0;   // exponents: one unit is 2^-x (2^-w1, 2^-w2)
 };
-// vmax: largest |value| a lookup adds (before its weight); w_min: smallest
-// nonzero weight, w_max the largest; a_ref: amplitude factor of a template's
-// first lookups; n: lookups of one (template, sky).
-StepScales step_scales(double vmax, double w_min, double w_max, double a_ref, int64_t n);
+// bins: powers that a lookup adds; a_ref: amplitude factor of a template's first
+// lookups; n: lookups of one (template, sky).
+StepScales step_scales(const MapRange& map, int bins, const WeightRange& w, double a_ref, int64_t n);
 
 inline void set_step_scales(StepEvent& e, const StepScales& s) {
   e.x_unit = std::ldexp(1.0, -s.x);
@@ -250,7 +273,7 @@ struct StepForm {
 cudaError_t step_prepare(const StepForm& v);
 // cells: the largest step_cells of the items' events, which are all of this form.
 cudaError_t launch_step(const StepParams& p, const StepForm& v, int cells, int grid, cudaStream_t st);
-// *out = bits of the largest |rho| (NaN above infinity above every finite value); out zero at launch.
-cudaError_t launch_absmax(const void* rho, bool half, int64_t n, unsigned* out, cudaStream_t st);
+// out[kMapWords] as map_range reads it; zero at launch.
+cudaError_t launch_map_range(const void* rho, bool half, int64_t n, unsigned* out, cudaStream_t st);
 
 }  // namespace tcw

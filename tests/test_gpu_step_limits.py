@@ -113,3 +113,52 @@ def test_two_bin_sums_are_not_rounded():
                                   p.T0, track_bins=2, amp_power=amp)[3]
         assert np.abs(psi).max() > 1.5e-6
         assert np.all(np.abs(st["psi"] - psi) <= 2.0 ** -23)
+
+
+def small(seed, n_det=1, n_seg=300, n_sky=40, n_tmpl=60, n_bin=3000, weights=True):
+    r = syn.rng(seed)
+    t = syn.segment_times(n_seg, 4.0)
+    dets = syn.random_detectors(r, n_det)
+    vel = np.stack([d.velocity(t) for d in dets])
+    f_max = 500.0 + n_bin * 0.25
+    bank = syn.random_bank(r, n_tmpl, f0_range=(495.0, f_max + 5), tau_range=(3500, 35000))
+    w = syn.uniform_weights(r, n_det, n_seg) if weights else None
+    return syn.Problem(syn.exponential_noise(r, (n_det, n_seg, n_bin)), t, w, vel, 500.0, 0.25, float(t[0] - 2.0),
+                       syn.random_sky(r, n_sky), bank, [], dets, name="small")
+
+
+@pytest.mark.parametrize("scale", [1e-3, 1e-6, 1e-9, 1e-12])
+@pytest.mark.parametrize("part", ["all", "band", "odd bins"])
+def test_quiet_maps(scale, part):
+    """Powers far below 1, everywhere, in the lower half of the band, or in all bins of a
+    map whose rows begin with a bin of 1: S is as close as fp32 sums have it."""
+    p = small(2300)
+    if part == "all":
+        p.rho *= np.float32(scale)
+    elif part == "band":
+        p.rho[:, :, :1500] *= np.float32(scale)
+    else:
+        p.rho *= np.float32(scale)
+        p.rho[:, :, 0] = 1.0
+    val, idx, st, info = run(p)
+    S, W1, W2, psi = oracle_stats(p)
+    assert info.kernel == tcw.KERNEL_GROUP
+    assert np.all(np.abs(st["S"] - S) <= 1e-5 * S)
+    fin = np.isfinite(psi)
+    assert np.array_equal(fin, np.isfinite(st["psi"]))
+    assert np.all(np.abs(st["psi"] - psi)[fin] <= 1e-5 * (np.sqrt(W1) + 1)[fin])
+
+
+@pytest.mark.parametrize("n_bin", [3000, 3001, 31])
+@pytest.mark.parametrize("dtype", [np.float32, np.float16])
+def test_lines_and_gaps_keep_the_fast_search(n_bin, dtype):
+    """A loud line in one bin of every row, and rows and stretches of zeros: powers that
+    the fixed-point grid spans."""
+    p = small(2400 + n_bin, n_det=2, n_bin=n_bin)
+    p.rho[:, 10:20] = 0.0
+    p.rho[:, :, n_bin // 3:n_bin // 2] = 0.0
+    p.rho[:, :, n_bin // 2 + 3] = 2000.0
+    p.rho = p.rho.astype(dtype)
+    if n_bin == 31:
+        p.bank.f0[:] = 500 + 7 * np.linspace(0.5, 1.1, len(p.bank.f0))
+    assert check(p)

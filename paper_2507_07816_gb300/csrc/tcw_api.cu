@@ -191,9 +191,8 @@ tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, boo
   if (!count && (st = ensure_map_range(c)) != TCW_OK) return st;
   const double f_top = c->f_min + (double)c->Nbin * c->df;
   const StepScales sc =
-      step_scales(count ? MapRange{1.0f, 1.0f} : c->map, c->track_bins, c->w_range,
-                  step_amp_ref(c->amp_power, c->h_t, c->T0, c->bank_tau_min, c->bank_r_max, f_top, c->bank_f0max),
-                  (int64_t)c->D * c->Nseg);
+      step_scales(count ? MapRange{1.0f, 1.0f} : c->map, c->track_bins, c->w_range, c->amp_power > 0,
+                  step_amp_ref(c->amp_power, c->h_t, c->T0, c->bank_tau_min, c->bank_r_max, f_top, c->bank_f0max));
   if (!sc.ok) return TCW_OK;
   const StepTrack tr = step_track(c->h_t.data(), c->Nseg, c->T0, 2 * c->tile_segments, c->bank_tau_min, c->bank_r_max,
                                   c->bank_f0max / c->df, f_top / c->df, pl.doppler_bins, c->f_min, c->df, pl.inv_q);

@@ -265,9 +265,8 @@ void plan_step(const tcw_ctx* c, BatchState* b, int tile) {
     split = true;   // some event takes its detectors one by one: all of them do
   }
   for (EventHost& e : b->ev) {
-    e.scales = step_scales(count ? MapRange{1.0f, 1.0f} : e.map, c->track_bins, e.w_range,
-                           step_amp_ref(c->amp_power, e.t, e.T0, c->bank_tau_min, c->bank_r_max, f_top, c->bank_f0max),
-                           (int64_t)b->D * e.n_seg);
+    e.scales = step_scales(count ? MapRange{1.0f, 1.0f} : e.map, c->track_bins, e.w_range, c->amp_power > 0,
+                           step_amp_ref(c->amp_power, e.t, e.T0, c->bank_tau_min, c->bank_r_max, f_top, c->bank_f0max));
     if (!e.scales.ok) return;
   }
   b->track.ok = true;

@@ -1364,25 +1364,30 @@ MapRange map_range(const unsigned* out) {
   return r;
 }
 
-StepScales step_scales(const MapRange& map, int bins, const WeightRange& w, double a_ref, int64_t n) {
+StepScales step_scales(const MapRange& map, int bins, const WeightRange& w, bool amp, double a_ref) {
   StepScales s;
   const double vmax = (double)map.max * bins;
-  if (!(vmax >= 0.0) || !(vmax < 1e30) || !(w.max > 0.0) || n < 1) return s;
+  if (!(vmax >= 0.0) || !(vmax < 1e30) || !(w.max > 0.0)) return s;
   auto lg = [](double v) { return (int)std::ceil(std::log2(v)); };   // v <= 2^lg
-  const int lw = lg(w.max) + 1, lw2 = lg((double)w.max * w.max) + 1, ln = lg((double)n) + 1;
   // the sums of a (template, sky), of powers and of their means, within 2^46 units and
   // one value within 2^21 2^16 units
   const double v = std::max(vmax, (double)bins);
   s.x = std::min(46 - lg(v * w.sum), 37 - lg(v * w.max));
-  s.w1 = std::min(36 - lw, 60 - ln - lw);
-  s.w2 = std::min(36 - lw2, 60 - ln - lw2) & ~1;   // even: the root of its unit is a power of 2
+  // sums of weights and of their squares below 2^60; amplitude weights are made by the
+  // kernel in words of 2^37 (PairWeight), the others here in FP64
+  const double max2 = (double)w.max * w.max, sum2 = w.sum * w.max;
+  s.w1 = std::min(60 - lg(w.sum), amp ? 36 - lg(w.max) : 60);
+  s.w2 = std::min(60 - lg(sum2), amp ? 36 - lg(max2) : 60) & ~1;   // even: the root of its unit is a power of 2
   // one unit at most 2^-22 of the smallest weighted power, the noise's mean or, where
   // the map lies lower, twice its level: a sum of m rounded values is then off by about
   // 0.3 sqrt(m) 2^-22 of it, 7e-8 of the standard deviation sqrt(m) that Eq. 4 divides
   // by and less of S
   const double p = map.level > 0 ? std::min(1.0, 2.0 * (double)map.level) : 1.0;
   const int need = 22 - (int)std::floor(std::log2((double)w.min * a_ref * p));
-  s.ok = s.x >= need && std::abs(s.x) < 100 && std::abs(s.w1) < 100 && std::abs(s.w2) < 100 && need < 100;
+  // W1 and W2 of the smallest weights alone to 2^-25, as fp32 has each of them
+  const double a = std::log2((double)w.min * a_ref);
+  const bool weights = s.w1 >= 24 - std::floor(a) && s.w2 >= 24 - std::floor(2 * a);
+  s.ok = weights && s.x >= need && std::abs(s.x) < 100 && std::abs(s.w1) < 100 && std::abs(s.w2) < 100 && need < 100;
   return s;
 }
 

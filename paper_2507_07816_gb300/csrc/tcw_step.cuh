@@ -223,9 +223,9 @@ struct StepScales {
   bool ok = false;
   int x = 0, w1 = 0, w2 = 0;   // exponents: one unit is 2^-x (2^-w1, 2^-w2)
 };
-// bins: powers that a lookup adds; a_ref: amplitude factor of a template's first
-// lookups; n: lookups of one (template, sky).
-StepScales step_scales(const MapRange& map, int bins, const WeightRange& w, double a_ref, int64_t n);
+// bins: powers that a lookup adds; amp: amplitude weights, a_ref: their factor at a
+// template's first lookups.
+StepScales step_scales(const MapRange& map, int bins, const WeightRange& w, bool amp, double a_ref);
 
 inline void set_step_scales(StepEvent& e, const StepScales& s) {
   e.x_unit = std::ldexp(1.0, -s.x);

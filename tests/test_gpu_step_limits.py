@@ -162,3 +162,28 @@ def test_lines_and_gaps_keep_the_fast_search(n_bin, dtype):
     if n_bin == 31:
         p.bank.f0[:] = 500 + 7 * np.linspace(0.5, 1.1, len(p.bank.f0))
     assert check(p)
+
+
+@pytest.mark.parametrize("w_low", [1.3 * 2.0 ** -3, 1.3 * 2.0 ** -9, 1.3 * 2.0 ** -13, 1.3 * 2.0 ** -18])
+@pytest.mark.parametrize("statistic", ["power", "count"])
+def test_templates_of_small_weights(statistic, w_low):
+    """Weights 1 in the first half and w_low in the second, the only one where the
+    templates are in the band: W1, W2 and Psi from the small weights alone."""
+    p = small(2500, n_det=2, n_seg=64, n_sky=20, n_tmpl=50, n_bin=1500)
+    p.t_mid = p.t_mid[0] + 60.0 * np.arange(64)
+    p.weights = np.ones((2, 64), np.float32)
+    p.weights[:, 30:] = w_low
+    f_top = p.f_min + 1500 * p.df
+    # above the band's top, Doppler shifts included, at segment 30
+    drop = (60.0 * 30 / p.bank.tau + 1) ** (1 / (1 - p.bank.n))
+    p.bank.f0[:] = f_top / drop * np.linspace(1.0005, 1.004, 50)
+    stat = (tcw.STAT_NUMBER_COUNT, 1.0) if statistic == "count" else None
+    val, idx, st, info = run(p, statistic=stat)
+    S, W1, W2, psi = oracle.search_stats(p.rho, p.f_min, p.df, p.t_mid, p.weights, p.velocity, p.nhat, p.bank.f0,
+                                         p.bank.tau, p.bank.n, p.T0, rho_th=1.0 if stat else None)
+    low = (W1 > 0) & (W1 < 68 * w_low * 1.001)
+    assert info.kernel == tcw.KERNEL_GROUP and low.sum() > 100 and (W2[low] > 0).all()
+    assert np.all(np.abs(st["W1"] - W1)[low] <= 1e-6 * W1[low])
+    assert np.all(np.abs(st["W2"] - W2)[low] <= 1e-6 * W2[low])
+    assert np.all(np.abs(st["S"] - S)[low] <= 1e-5 * S[low])
+    assert np.all(np.abs(st["psi"] - psi)[low] <= 1e-5 * (S / np.sqrt(np.maximum(W2, 1e-30)))[low] + 1e-5)

@@ -192,7 +192,7 @@ tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, boo
   const double f_top = c->f_min + (double)c->Nbin * c->df;
   const StepScales sc =
       step_scales(count ? MapRange{1.0f, 1.0f} : c->map, c->track_bins, c->w_range, c->amp_power > 0,
-                  step_amp_ref(c->amp_power, c->h_t, c->T0, c->bank_tau_min, c->bank_r_max, f_top, c->bank_f0max));
+                  step_amp_ref(c->amp_power, c->h_tw, c->T0, c->bank_tau_min, c->bank_r_max, f_top, c->bank_f0max));
   if (!sc.ok) return TCW_OK;
   const StepTrack tr = step_track(c->h_t.data(), c->Nseg, c->T0, 2 * c->tile_segments, c->bank_tau_min, c->bank_r_max,
                                   c->bank_f0max / c->df, f_top / c->df, pl.doppler_bins, c->f_min, c->df, pl.inv_q);
@@ -674,9 +674,16 @@ SweepPlan plan_sweep(const std::vector<double>& tc, double T0, double tau_min, d
 double tcw::step_amp_ref(int amp_power, const std::vector<double>& t, double T0, double tau_min, double r_max,
                          double f_top, double f0_max) {
   if (amp_power == 0) return 1.0;
-  double a = std::min(1.0, f_top / f0_max);
   const auto first = std::lower_bound(t.begin(), t.end(), T0);
-  if (first != t.end()) a = std::min(a, std::pow((*first - T0) / tau_min + 1.0, -r_max));
+  if (first == t.end()) return 1.0;   // no lookups
+  // tracks in the band at the first segment from T0 on, and those that enter it later:
+  // below its top then, by as much as they fall from one segment to the next
+  double a = std::pow((*first - T0) / tau_min + 1.0, -r_max);
+  if (f0_max > 0.999 * f_top) {
+    double gap = 1.0;
+    for (auto i = first; i + 1 != t.end(); ++i) gap = std::max(gap, (i[1] - T0 + tau_min) / (i[0] - T0 + tau_min));
+    a = std::min(a, std::min(1.0, 0.999 * f_top / f0_max) * std::pow(gap, -r_max));
+  }
   return std::pow(std::max(a, 1e-30), amp_power);
 }
 
@@ -1067,6 +1074,7 @@ tcw_status tcw_load_spectrogram(tcw_ctx* c, int n_det, int64_t n_seg, int64_t n_
   c->unit_weights = true;
   c->w_range = WeightRange{};
   c->w_range.take(w);
+  c->h_tw = weighted_times(c->h_t, w);
   for (float x : w)
     if (x != 1.0f) c->unit_weights = false;
   c->have_spec = true;

@@ -34,7 +34,7 @@ namespace {
 struct EventHost {
   int64_t n_seg = 0, n_sky = 0;
   double T0 = 0;
-  std::vector<double> t, v;   // segment times, velocities (planning)
+  std::vector<double> t, v, tw;   // segment times, velocities (planning); times with a nonzero weight
   bool unit_w = true;
   int Spad = 0, NG = 0, n_chunks = 0;
   size_t o_rho = 0, o_t = 0, o_w = 0, o_v = 0, o_nhat = 0, o_perm = 0, o_blk = 0;  // byte offsets
@@ -266,7 +266,7 @@ void plan_step(const tcw_ctx* c, BatchState* b, int tile) {
   }
   for (EventHost& e : b->ev) {
     e.scales = step_scales(count ? MapRange{1.0f, 1.0f} : e.map, c->track_bins, e.w_range, c->amp_power > 0,
-                           step_amp_ref(c->amp_power, e.t, e.T0, c->bank_tau_min, c->bank_r_max, f_top, c->bank_f0max));
+                           step_amp_ref(c->amp_power, e.tw, e.T0, c->bank_tau_min, c->bank_r_max, f_top, c->bank_f0max));
     if (!e.scales.ok) return;
   }
   b->track.ok = true;
@@ -958,6 +958,7 @@ tcw_status tcw_load_events(tcw_ctx* c, int n_det, int64_t n_bin, int dtype, doub
       w.assign((size_t)n_det * in.n_seg, 1.0f);
     }
     e.w_range.take(w);
+    e.tw = weighted_times(e.t, w);
     wts[i] = std::move(w);
     b->unit_weights = b->unit_weights && e.unit_w;
     // sky sorted by its Doppler factor at the event's middle segment (detector 0)

@@ -64,7 +64,7 @@ struct tcw_ctx {
   int64_t Nseg = 0, Nbin = 0;
   int dtype = TCW_F32;
   double f_min = 0, df = 0;
-  std::vector<double> h_t;
+  std::vector<double> h_t, h_tw;     // segment times; those with a nonzero weight
   bool unit_weights = true;
   tcw::WeightRange w_range;
   tcw::MapRange map;                 // of the loaded map (see ensure_map_range)
@@ -169,8 +169,20 @@ inline cudaError_t ensure_step_edge(DevBuf& b, int grid, cudaStream_t st) {
   return e == cudaSuccess ? cudaMemsetAsync(b.p, 0, b.bytes, st) : e;
 }
 
-// Amplitude factor (Eq. 3) that every template's first lookups reach at least:
-// at the first segment from T0 on, or where the track enters the band.
+// The segments' times where some detector's weight is not 0.
+inline std::vector<double> weighted_times(const std::vector<double>& t, const std::vector<float>& w) {
+  std::vector<double> r;
+  for (size_t j = 0; j < t.size(); ++j)
+    for (size_t i = j; i < w.size(); i += t.size())
+      if (w[i] > 0) {
+        r.push_back(t[j]);
+        break;
+      }
+  return r;
+}
+
+// Amplitude factor (Eq. 3) that every template's first lookups reach at least: at the
+// first of the times t (weighted_times) from T0 on, or where the track enters the band.
 double step_amp_ref(int amp_power, const std::vector<double>& t, double T0, double tau_min, double r_max,
                     double f_top, double f0_max);
 

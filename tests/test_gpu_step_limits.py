@@ -187,3 +187,30 @@ def test_templates_of_small_weights(statistic, w_low):
     assert np.all(np.abs(st["W2"] - W2)[low] <= 1e-6 * W2[low])
     assert np.all(np.abs(st["S"] - S)[low] <= 1e-5 * S[low])
     assert np.all(np.abs(st["psi"] - psi)[low] <= 1e-5 * (S / np.sqrt(np.maximum(W2, 1e-30)))[low] + 1e-5)
+
+
+@pytest.mark.parametrize("gated", ["weights", "gap"])
+@pytest.mark.parametrize("n_det", [1, 2])
+def test_amplitude_weights_after_a_gap(gated, n_det):
+    """Tracks whose first lookups come late, when (f/f0)^8 is down to 1e-6: the segments
+    before have weight 0, or are missing while the track comes into the band."""
+    r = syn.rng(2600 + n_det)
+    t = 1.4e9 + 10.0 * np.arange(1200)
+    if gated == "gap":
+        t[4:] += 9000.0   # between two tiles
+    dets = syn.random_detectors(r, n_det)
+    vel = np.stack([d.velocity(t) for d in dets])
+    w = syn.uniform_weights(r, n_det, 1200)
+    if gated == "weights":
+        w[:, :1100] = 0.0
+    f0 = {"weights": (600.0, 1090.0), "gap": (1150.0, 1800.0)}[gated]
+    bank = syn.random_bank(r, 50, f0_range=f0, tau_range=(500.0, 520.0), n_range=(3.0, 3.1))
+    p = syn.Problem(syn.exponential_noise(r, (n_det, 1200, 4000)), t, w, vel, 100.0, 0.25, float(t[0] - 5.0),
+                    syn.random_sky(r, 20), bank, [], dets, name="late")
+    val, idx, st, info = run(p, options=[(tcw.OPT_AMPLITUDE_POWER, 8)])
+    S, W1, W2, psi = oracle_stats(p, amp_power=8)
+    on = W1 > 0
+    assert info.kernel == tcw.KERNEL_GROUP and on.sum() > 500 and W1[on].max() < 1.0
+    for k, ref in (("S", S), ("W1", W1), ("W2", W2)):
+        assert np.all(np.abs(st[k] - ref) <= 1e-5 * ref), k
+    assert np.all(np.abs(st["psi"] - psi)[on] <= 1e-5 * (S / np.sqrt(np.where(on, W2, 1)))[on] + 1e-5)

@@ -182,7 +182,8 @@ tcw_status ensure_map_range(tcw_ctx* c) {
 // The exhaustive search by step functions (tcw_step.cuh).  *ran = false when
 // its conditions do not hold (the group kernel's exactness conditions, a track
 // series, and fixed-point sums at least as accurate as fp32 ones: not with
-// non-finite or very large powers): the caller takes the group kernel.
+// non-finite or very large powers) or its tables do not fit the device: the
+// caller takes the group kernel.
 tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, bool* ran) {
   *ran = false;
   if (!pl.group_ok || c->D > 2) return TCW_OK;
@@ -197,29 +198,45 @@ tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, boo
   const StepTrack tr = step_track(c->h_t.data(), c->Nseg, c->T0, 2 * c->tile_segments, c->bank_tau_min, c->bank_r_max,
                                   c->bank_f0max / c->df, f_top / c->df, pl.doppler_bins, c->f_min, c->df, pl.inv_q);
   if (!tr.ok) return TCW_OK;
+  if (count && (st = ensure_bits(c, launches)) != TCW_OK) return st;
   const int tile = 1 << tr.shift;
   StepGeometry g = step_geometry(c->S, c->D, c->Nseg, tile, c->h_v.data(), false);
+  const int all_chunks = g.n_chunks;
+  const int slab = (int)std::min<size_t>(all_chunks, std::max<size_t>(1, kStepRowsMax / step_chunk_bytes(g, c->Nseg, c->D)));
+  g.n_chunks = slab;   // chunks searched at a time
   g.log_t = step_block(g, c->Bpad, c->bank_chunk, c->grid, (double)c->Nseg * c->D);
   const int n_tiles = (int)((c->Nseg + tile - 1) / tile);
-  const size_t rows = (size_t)g.n_chunks * c->Nseg * c->D;
-  TCW_CUDA(c, c->step_q.ensure(rows * step_row(g.cpad) * sizeof(int32_t)), "doppler rows");
-  TCW_CUDA(c, c->step_head.ensure(rows * kStepHead * sizeof(int4)), "doppler rows");
-  TCW_CUDA(c, c->step_tab.ensure(rows * step_buckets(g.cpad) * (sizeof(uint2) + sizeof(uint32_t))), "doppler rows");
-  TCW_CUDA(c, c->step_wtot.ensure(kStepSlots * 16 + (size_t)c->Nseg * c->D * sizeof(longlong2)), "weight sums");
-  TCW_CUDA(c, cudaMemsetAsync(c->step_wtot.p, 0, kStepSlots * 16, c->stream), "weight sums");
-  TCW_CUDA(c, ensure_step_edge(c->step_edge, c->grid, c->stream), "scratch");
-  TCW_CUDA(c, c->step_slow.ensure(step_slow_bytes(c->grid)), "scratch");
-  if (step_ordered(g))
-    TCW_CUDA(c, c->step_order.ensure((size_t)g.passes * g.n_chunks * g.cpad * 2 * sizeof(int16_t)), "sky order");
+  const size_t rows = (size_t)slab * c->Nseg * c->D;
+  {
+    cudaError_t e = cudaSuccess;
+    auto room = [&](DevBuf& b, size_t n) {
+      if (e == cudaSuccess) e = b.ensure(n);
+    };
+    room(c->step_q, rows * step_row(g.cpad) * sizeof(int32_t));
+    room(c->step_head, rows * kStepHead * sizeof(int4));
+    room(c->step_tab, rows * step_buckets(g.cpad) * (sizeof(uint2) + sizeof(uint32_t)));
+    room(c->step_wtot, kStepSlots * 16 + (size_t)c->Nseg * c->D * sizeof(longlong2));
+    if (step_ordered(g)) room(c->step_order, (size_t)g.passes * slab * g.cpad * 2 * sizeof(int16_t));
+    room(c->anchors, (size_t)c->Bpad * n_tiles * 2 * sizeof(double));
+    room(c->step_tiles, (size_t)c->Bpad * n_tiles * sizeof(StepTile));
+    room(c->step_slow, step_slow_bytes(c->grid));
+    if (e == cudaSuccess) e = ensure_step_edge(c->step_edge, c->grid, c->stream);
+    if (e == cudaErrorMemoryAllocation) {
+      // step_slow and step_edge stay: a recorded batch may hold them
+      cudaGetLastError();
+      for (DevBuf* b : {&c->step_q, &c->step_head, &c->step_tab, &c->step_wtot, &c->step_order, &c->step_tiles, &c->anchors})
+        b->release();
+      return TCW_OK;
+    }
+    TCW_CUDA(c, e, "step-function tables");
+  }
   StepRowsParams rp{};
   rp.vel = c->vel.as<double>();
-  rp.nhat = c->nhat_sorted.as<double>();
   rp.weights = c->weights.as<float>();
   rp.t_mid = c->t_mid.as<double>();
   rp.T0 = c->T0;
   rp.n_det = c->D;
   rp.n_seg = (int)c->Nseg;
-  rp.S = (int)c->S;
   set_step_geometry(rp, g);
   rp.tile_shift = tr.shift;
   rp.inv_q = pl.inv_q;
@@ -227,18 +244,13 @@ tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, boo
   rp.w1_scale = std::ldexp(1.0, sc.w1);
   rp.w2_scale = std::ldexp(1.0, sc.w2);
   rp.order = step_ordered(g) ? c->step_order.as<int16_t>() : nullptr;
-  rp.remap = rp.order ? rp.order + (size_t)g.passes * g.n_chunks * g.cpad : nullptr;
+  rp.remap = rp.order ? rp.order + (size_t)g.passes * slab * g.cpad : nullptr;
   rp.q = c->step_q.as<int32_t>();
   rp.head = c->step_head.as<int4>();
   rp.fast = c->step_tab.as<uint2>();
   rp.tab = reinterpret_cast<uint32_t*>(rp.fast + rows * step_buckets(g.cpad));
   rp.wtot = c->step_wtot.as<unsigned long long>();
   rp.wfix = reinterpret_cast<longlong2*>(rp.wtot + kStepSlots * 2);
-  TCW_CUDA(c, launch_step_rows(rp, c->stream), "step_rows_kernel launch");
-  ++*launches;
-  if (count && (st = ensure_bits(c, launches)) != TCW_OK) return st;
-  TCW_CUDA(c, c->anchors.ensure((size_t)c->Bpad * n_tiles * 2 * sizeof(double)), "anchors");
-  TCW_CUDA(c, c->step_tiles.ensure((size_t)c->Bpad * n_tiles * sizeof(StepTile)), "track tiles");
   StepTileParams tp{};
   tp.f_min = c->f_min;
   tp.df = c->df;
@@ -273,26 +285,18 @@ tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, boo
   ev.sub_shift = step_sub_shift(g, c->Nseg, tr.shift);
   ev.order = rp.order;
   ev.remap = rp.remap;
-  ev.psi = c->psi.as<float>();
-  ev.S_out = keep ? c->st_S.as<float>() : nullptr;
-  ev.W1_out = keep ? c->st_W1.as<float>() : nullptr;
-  ev.W2_out = keep ? c->st_W2.as<float>() : nullptr;
   ev.T0 = c->T0;
   set_step_scales(ev, sc);
   ev.n_seg = (int)c->Nseg;
   ev.n_tiles = n_tiles;
-  ev.S = (int)c->S;
   ev.Bpad = c->Bpad;
   set_step_geometry(ev, g);
   TCW_CUDA(c, c->evtab.ensure(sizeof(StepEvent)), "event table");
-  TCW_CUDA(c, cudaMemcpyAsync(c->evtab.p, &ev, sizeof(ev), cudaMemcpyHostToDevice, c->stream), "event table");
   StepParams p{};
   p.events = c->evtab.as<StepEvent>();
   p.items = nullptr;
-  p.n_chunks = g.n_chunks;
   p.bank_chunk = c->bank_chunk;
   const int blocks = c->Bpad >> g.log_t;
-  p.n_items = g.n_chunks * ((blocks + c->bank_chunk - 1) / c->bank_chunk);
   p.next = reinterpret_cast<unsigned*>(c->flags.as<char>() + 32);
   p.n_det = c->D;
   p.n_bin = c->Nbin;
@@ -309,12 +313,33 @@ tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, boo
   p.slow = c->step_slow.as<int4>();
   p.edge = c->step_edge.as<longlong2>();
   p.n_general = reinterpret_cast<unsigned long long*>(c->flags.as<char>() + 8);
-  TCW_CUDA(c, cudaEventRecord(c->ev0, c->stream), "event");
-  TCW_CUDA(c, launch_step_tiles(tp, c->stream), "step_tile_kernel launch");
   const StepForm form{g.dets_per_pass, g.log_t, c->dtype == TCW_F16, count || c->track_bins == 2, c->amp_power > 0};
-  TCW_CUDA(c, launch_step(p, form, step_cells(g), std::min(c->grid, p.n_items), c->stream), "step_kernel launch");
+  for (int c0 = 0; c0 < all_chunks; c0 += slab) {
+    const int n = std::min(slab, all_chunks - c0);
+    const int64_t sky0 = (int64_t)c0 * g.chunk;
+    rp.nhat = c->nhat_sorted.as<double>() + 3 * sky0;
+    rp.S = ev.S = (int)std::min<int64_t>(c->S - sky0, (int64_t)n * g.chunk);
+    rp.n_chunks = ev.n_chunks = p.n_chunks = n;
+    p.n_items = n * ((blocks + c->bank_chunk - 1) / c->bank_chunk);
+    const int64_t out = sky0 * c->Bpad;
+    ev.psi = c->psi.as<float>() + out;
+    ev.S_out = keep ? c->st_S.as<float>() + out : nullptr;
+    ev.W1_out = keep ? c->st_W1.as<float>() + out : nullptr;
+    ev.W2_out = keep ? c->st_W2.as<float>() + out : nullptr;
+    TCW_CUDA(c, cudaMemsetAsync(c->step_wtot.p, 0, kStepSlots * 16, c->stream), "weight sums");
+    TCW_CUDA(c, launch_step_rows(rp, c->stream), "step_rows_kernel launch");
+    TCW_CUDA(c, cudaMemcpyAsync(c->evtab.p, &ev, sizeof(ev), cudaMemcpyHostToDevice, c->stream), "event table");
+    if (c0 == 0) {
+      TCW_CUDA(c, cudaEventRecord(c->ev0, c->stream), "event");
+      TCW_CUDA(c, launch_step_tiles(tp, c->stream), "step_tile_kernel launch");
+      ++*launches;
+    } else {
+      TCW_CUDA(c, cudaMemsetAsync(p.next, 0, 4, c->stream), "item counter");
+    }
+    TCW_CUDA(c, launch_step(p, form, step_cells(g), std::min(c->grid, p.n_items), c->stream), "step_kernel launch");
+    *launches += 2;
+  }
   TCW_CUDA(c, cudaEventRecord(c->ev1, c->stream), "event");
-  *launches += 2;
   *ran = true;
   return TCW_OK;
 }

@@ -160,6 +160,15 @@ inline void set_step_geometry(StepRowsParams& p, const StepGeometry& g) {
   p.passes = g.passes;
 }
 inline bool step_ordered(const StepGeometry& g) { return g.passes > 1; }
+// Doppler rows of one chunk, in bytes: about 28 per sky of a (segment, detector).
+inline size_t step_chunk_bytes(const StepGeometry& g, int64_t n_seg, int D) {
+  return (size_t)n_seg * D *
+         (step_row(g.cpad) * sizeof(int32_t) + kStepHead * sizeof(int4) +
+          step_buckets(g.cpad) * (sizeof(uint2) + sizeof(uint32_t)));
+}
+// Rows held at a time: a longer sky list is searched some chunks at a time (a chunk
+// fills the chip for milliseconds).
+constexpr size_t kStepRowsMax = (size_t)4 << 30;
 
 // The fp32 track's tiles and error bound: tile = 1 << shift segments (at most
 // `most`: twice the anchor tiles of the other kernels, as a tile here is laid out

@@ -2,6 +2,7 @@
 beyond them the kernels that it hands over to."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
 import paper_2507_07816_gb300 as tcw
@@ -214,3 +215,64 @@ def test_amplitude_weights_after_a_gap(gated, n_det):
     for k, ref in (("S", S), ("W1", W1), ("W2", W2)):
         assert np.all(np.abs(st[k] - ref) <= 1e-5 * ref), k
     assert np.all(np.abs(st["psi"] - psi)[on] <= 1e-5 * (S / np.sqrt(np.where(on, W2, 1)))[on] + 1e-5)
+
+
+def long_list(seed, n_sky, n_seg=8000, n_bin=1500):
+    """Thousands of skies over 8 h of one detector, few templates."""
+    r = syn.rng(seed)
+    t = syn.segment_times(n_seg, 4.0)
+    dets = syn.random_detectors(r, 1)
+    vel = np.stack([d.velocity(t) for d in dets])
+    f_max = 500.0 + n_bin * 0.25
+    bank = syn.random_bank(r, 64, f0_range=(600.0, f_max + 5), tau_range=(10000, 35000))
+    rho = syn.exponential_noise(r, (1, n_seg, n_bin)).astype(np.float16)
+    return syn.Problem(rho, t, syn.uniform_weights(r, 1, n_seg), vel, 500.0, 0.25, float(t[0] - 2.0),
+                       syn.random_sky(r, n_sky), bank, [], dets, name="long list")
+
+
+def test_rows_of_long_sky_lists_are_held_in_parts():
+    """40000 skies x 8000 segments: 9 GB of Doppler rows, held 4 GiB at a time.  The
+    sums are exact, so any sky's results are those of a short list."""
+    p = long_list(2700, 40000)
+    s = tcw.Search(0)
+    s.set_option(tcw.OPT_KEEP_STATS, 1)
+    s.load_problem(p)
+    free = torch.cuda.mem_get_info()[0]
+    val, idx = s.search(3)
+    used = free - torch.cuda.mem_get_info()[0]
+    st = s.statistics()
+    some = np.argsort(p.nhat @ p.velocity[0, 4000])[::997]   # over all the parts
+    p.nhat = np.ascontiguousarray(p.nhat[some])
+    s.load_problem(p)
+    val1, idx1 = s.search(3)
+    st1 = s.statistics()
+    s.close()
+    assert used < (4 << 30) + 600e6
+    for k in st:
+        np.testing.assert_array_equal(st[k][some], st1[k])
+    np.testing.assert_array_equal(val[some], val1)
+    np.testing.assert_array_equal(idx[some], idx1)
+
+
+def test_tables_that_do_not_fit_leave_the_group_kernel():
+    """Device memory left for the group kernel's tables (0.4 GB) but not for the step
+    kernel's rows (2 GB): the search runs as with memory to spare."""
+    p = long_list(2800, 9000)
+    s = tcw.Search(0)
+    s.set_option(tcw.OPT_KEEP_STATS, 1)
+    s.load_problem(p)
+    torch.cuda.empty_cache()
+    hog = torch.empty(torch.cuda.mem_get_info()[0] - 1_200_000_000, dtype=torch.uint8, device="cuda:0")
+    try:
+        val, idx = s.search(3)
+        st = s.statistics()
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+    val1, idx1 = s.search(3)
+    st1 = s.statistics()
+    s.close()
+    np.testing.assert_allclose(st["S"], st1["S"], rtol=1e-5)
+    np.testing.assert_allclose(st["W1"], st1["W1"], rtol=1e-5)
+    np.testing.assert_allclose(st["psi"], st1["psi"], rtol=0, atol=1e-3)
+    assert_topk_consistent(st["psi"], idx, val, 3)

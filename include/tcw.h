@@ -89,8 +89,9 @@ enum {
                                   and tile length by timing candidates on a sample of
                                   the batch; 0 = use TCW_OPT_BANK_CHUNK and
                                   TCW_OPT_TILE_SEGMENTS */
-    TCW_OPT_BATCH_MEMORY = 6,  /* batched search: bytes of Psi and anchor buffers per
-                                  wave of events (default 48 GiB, minimum 1 MiB) */
+    TCW_OPT_BATCH_MEMORY = 6,  /* batched search: bytes of Psi, anchor and Doppler-row
+                                  buffers per wave of events (default 48 GiB, minimum
+                                  1 MiB; a wave holds one event at least) */
     TCW_OPT_SKY_LANES = 7,     /* sky groups of 16 per chunk of the group kernel: 16,
                                   32 or 64 (a pass covers 16*lanes skies x 1024/lanes
                                   templates); 0 (default) = the lowest cost for the

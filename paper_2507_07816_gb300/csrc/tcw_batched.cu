@@ -15,7 +15,7 @@
 //   some event is outside the step kernel's conditions)
 //   topk_kernel     x event      per-sky top-k of Eq. 4's Psi
 //
-// A wave is a run of events whose Psi and anchor buffers fit the memory
+// A wave is a run of events whose Psi, anchor and row buffers fit the memory
 // budget (TCW_OPT_BATCH_MEMORY); small batches are a single wave.  The bank
 // chunk (templates per work item) and the tile length (anchor spacing and
 // fp32 partial-sum length) are chosen by an autotuner that times every
@@ -93,8 +93,8 @@ struct BatchState {
   bool step = false;
   StepTrack track;
   int dets_per_pass = 1;
-  DevBuf rows, tiles;              // Doppler rows of every event; track constants of a wave
-  size_t wtot_bytes = 0;           // the events' weight sums, at the start of `rows`
+  DevBuf rows, tiles;              // Doppler rows and track constants of a wave
+  DevBuf wtot;                     // the events' weight sums
   std::vector<int> wave_split;     // per wave: items of the events with 32 templates per block, then 16
   // autotuner
   bool tuned = false;
@@ -121,7 +121,7 @@ namespace {
 // arrays, bit maps and outputs.
 void release_batch(BatchState* b, bool shared) {
   if (b->exec) cudaGraphExecDestroy(b->exec);
-  DevBuf* own[] = {&b->rows, &b->tiles, &b->blk, &b->anchors, &b->psi, &b->evtab, &b->items, &b->dev, &b->flags, &b->sub};
+  DevBuf* own[] = {&b->rows, &b->tiles, &b->wtot, &b->blk, &b->anchors, &b->psi, &b->evtab, &b->items, &b->dev, &b->flags, &b->sub};
   for (DevBuf* d : own) d->release();
   if (!shared) {
     DevBuf* bufs[] = {&b->rho, &b->small, &b->out_psi, &b->out_idx, &b->bits};
@@ -222,8 +222,6 @@ tcw_status plan_batch(tcw_ctx* c, BatchState* b) {
   for (const EventHost& e : b->ev) b->lookups += e.n_sky * ev_B(c, e) * b->D * e.n_seg;
   TCW_CUDA(c, group_grid(&b->grid), "device query");
   TCW_CUDA(c, b->dev.ensure(group_dev_elems(b->grid) * sizeof(float2)), "scratch");
-  TCW_CUDA(c, ensure_step_edge(c->step_edge, b->grid, c->stream), "scratch");
-  TCW_CUDA(c, c->step_slow.ensure(step_slow_bytes(b->grid)), "scratch");
   b->planned = true;
   return TCW_OK;
 }
@@ -268,34 +266,30 @@ void plan_step(const tcw_ctx* c, BatchState* b, int tile) {
     e.scales = step_scales(count ? MapRange{1.0f, 1.0f} : e.map, c->track_bins, e.w_range, c->amp_power > 0,
                            step_amp_ref(c->amp_power, e.tw, e.T0, c->bank_tau_min, c->bank_r_max, f_top, c->bank_f0max));
     if (!e.scales.ok) return;
+    // an event's rows are held whole
+    const size_t rows = (size_t)e.geo.n_chunks * step_chunk_bytes(e.geo, e.n_seg, b->D);
+    if (rows > std::max((size_t)c->batch_memory, kStepRowsMax)) return;
   }
   b->track.ok = true;
   b->step = true;
 }
 
-// Offsets of the Doppler rows of every event in b->rows; returns their size.
-size_t layout_rows(BatchState* b) {
-  size_t o = 0;
-  for (EventHost& e : b->ev) {
-    e.o_wtot = o;
-    o += kStepSlots * 16;
-  }
-  b->wtot_bytes = o;
+// Offsets of an event's Doppler rows from `at` on in a wave's rows; returns their size.
+size_t layout_rows(const BatchState* b, EventHost& e, size_t at) {
+  size_t o = at;
   auto take = [&](size_t n) {
-    const size_t at = o;
+    const size_t from = o;
     o += align256(n);
-    return at;
+    return from;
   };
-  for (EventHost& e : b->ev) {
-    const size_t rows = (size_t)e.geo.n_chunks * e.n_seg * b->D;
-    e.o_q = take(rows * step_row(e.geo.cpad) * sizeof(int32_t));
-    e.o_head = take(rows * kStepHead * sizeof(int4));
-    e.o_tab = take(rows * step_buckets(e.geo.cpad) * sizeof(uint32_t));
-    e.o_fast = take(rows * step_buckets(e.geo.cpad) * sizeof(uint2));
-    e.o_wfix = take((size_t)e.n_seg * b->D * sizeof(longlong2));
-    e.o_order = step_ordered(e.geo) ? take((size_t)e.geo.passes * e.geo.n_chunks * e.geo.cpad * 2 * sizeof(int16_t)) : 0;
-  }
-  return o;
+  const size_t rows = (size_t)e.geo.n_chunks * e.n_seg * b->D;
+  e.o_q = take(rows * step_row(e.geo.cpad) * sizeof(int32_t));
+  e.o_head = take(rows * kStepHead * sizeof(int4));
+  e.o_tab = take(rows * step_buckets(e.geo.cpad) * sizeof(uint32_t));
+  e.o_fast = take(rows * step_buckets(e.geo.cpad) * sizeof(uint2));
+  e.o_wfix = take((size_t)e.n_seg * b->D * sizeof(longlong2));
+  e.o_order = step_ordered(e.geo) ? take((size_t)e.geo.passes * e.geo.n_chunks * e.geo.cpad * 2 * sizeof(int16_t)) : 0;
+  return o - at;
 }
 
 int batch_series_terms(const tcw_ctx* c, const BatchState* b, int tile) {
@@ -311,33 +305,42 @@ int batch_series_terms(const tcw_ctx* c, const BatchState* b, int tile) {
 
 int n_tiles_of(int64_t n_seg, int tile) { return (int)((n_seg + tile - 1) / tile); }
 
+// Bytes of a wave's buffers; every wave's fit.
+struct WaveBytes {
+  size_t psi = 0, anchors = 0, rows = 0;
+};
+
 // Split the events into waves whose Psi and anchor buffers (with the track
-// constants of a step-function search) fit `budget` bytes and lay out those
-// buffers.  Returns the per-wave buffer sizes.
-void layout_waves(const tcw_ctx* c, BatchState* b, int tile, bool anchors, size_t* psi_bytes,
-                  size_t* anchor_bytes) {
+// constants and Doppler rows of a step-function search) fit `budget` bytes and
+// lay out those buffers.
+WaveBytes layout_waves(const tcw_ctx* c, BatchState* b, int tile, bool anchors) {
   const size_t budget = (size_t)c->batch_memory;
-  size_t psi_w = 0, anc_w = 0, psi_max = 0, anc_max = 0;
+  WaveBytes w, most;
   int wave = 0;
-  for (EventHost& e : b->ev) {
+  for (size_t i = 0; i < b->ev.size(); ++i) {
+    EventHost& e = b->ev[i];
     const size_t p = align256((size_t)e.Spad * ev_Bpad(c, e) * 4);
     const size_t a = anchors ? align256((size_t)ev_Bpad(c, e) * n_tiles_of(e.n_seg, tile) * 16) : 0;
     const size_t f = b->step ? 1 + sizeof(StepTile) / 16 : 1;   // anchor and track constants per tile
-    if ((psi_w + anc_w) > 0 && psi_w + f * anc_w + p + f * a > budget) {
+    size_t r = b->step ? layout_rows(b, e, w.rows) : 0;
+    if (w.psi + w.anchors > 0 && w.psi + f * w.anchors + w.rows + p + f * a + r > budget) {
       ++wave;
-      psi_w = anc_w = 0;
+      w = WaveBytes{};
+      if (b->step) r = layout_rows(b, e, 0);
     }
     e.wave = wave;
-    e.o_psi = psi_w;
-    e.o_anchor = anc_w;
-    psi_w += p;
-    anc_w += a;
-    psi_max = std::max(psi_max, psi_w);
-    anc_max = std::max(anc_max, anc_w);
+    e.o_psi = w.psi;
+    e.o_anchor = w.anchors;
+    e.o_wtot = i * kStepSlots * 16;
+    w.psi += p;
+    w.anchors += a;
+    w.rows += r;
+    most.psi = std::max(most.psi, w.psi);
+    most.anchors = std::max(most.anchors, w.anchors);
+    most.rows = std::max(most.rows, w.rows);
   }
   b->waves = wave + 1;
-  *psi_bytes = psi_max;
-  *anchor_bytes = anc_max;
+  return most;
 }
 
 // An event's Doppler rows, and what the search reads of it.
@@ -366,7 +369,7 @@ StepRowsParams step_rows_of(BatchState* b, const EventHost& e) {
   rp.tab = at<uint32_t>(b->rows, e.o_tab);
   rp.fast = at<uint2>(b->rows, e.o_fast);
   rp.wfix = at<longlong2>(b->rows, e.o_wfix);
-  rp.wtot = at<unsigned long long>(b->rows, e.o_wtot);
+  rp.wtot = at<unsigned long long>(b->wtot, e.o_wtot);
   return rp;
 }
 
@@ -531,19 +534,32 @@ GroupParams base_params(const tcw_ctx* c, BatchState* b, int tile, int nterms) {
 }
 
 // Buffers and event table for (tile, anchors); items are uploaded by the caller.
-// Decides whether the step-function search runs.
+// Decides whether the step-function search runs: the group kernel does where its
+// rows and track constants do not fit the device.
 tcw_status prepare_shape(tcw_ctx* c, BatchState* b, int tile, int nterms) {
-  size_t psi_bytes = 0, anc_bytes = 0;
   plan_step(c, b, tile);
   if (b->step) {
-    layout_waves(c, b, 1 << b->track.shift, true, &psi_bytes, &anc_bytes);
-    TCW_CUDA(c, b->rows.ensure(layout_rows(b)), "doppler rows");
-    TCW_CUDA(c, b->tiles.ensure(anc_bytes / 16 * sizeof(StepTile)), "track tiles");
-  } else {
-    layout_waves(c, b, tile, nterms > 0, &psi_bytes, &anc_bytes);
+    const WaveBytes w = layout_waves(c, b, 1 << b->track.shift, true);
+    cudaError_t e = b->psi.ensure(w.psi);
+    if (e == cudaSuccess) e = b->anchors.ensure(w.anchors);
+    if (e == cudaSuccess) e = b->rows.ensure(w.rows);
+    if (e == cudaSuccess) e = b->tiles.ensure(w.anchors / 16 * sizeof(StepTile));
+    if (e == cudaSuccess) e = b->wtot.ensure(b->ev.size() * kStepSlots * 16);
+    if (e == cudaSuccess) e = c->step_slow.ensure(step_slow_bytes(b->grid));
+    if (e == cudaSuccess) e = ensure_step_edge(c->step_edge, b->grid, c->stream);
+    if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
+      for (DevBuf* d : {&b->psi, &b->anchors, &b->rows, &b->tiles}) d->release();
+      b->step = false;
+    } else {
+      TCW_CUDA(c, e, "step-function tables");
+    }
   }
-  TCW_CUDA(c, b->psi.ensure(psi_bytes), "Psi buffer");
-  if (b->step || nterms > 0) TCW_CUDA(c, b->anchors.ensure(anc_bytes), "anchor buffer");
+  if (!b->step) {
+    const WaveBytes w = layout_waves(c, b, tile, nterms > 0);
+    TCW_CUDA(c, b->psi.ensure(w.psi), "Psi buffer");
+    if (nterms > 0) TCW_CUDA(c, b->anchors.ensure(w.anchors), "anchor buffer");
+  }
   std::vector<EventDesc> tab;
   std::vector<StepEvent> stab;
   for (const EventHost& e : b->ev) {
@@ -558,15 +574,19 @@ tcw_status prepare_shape(tcw_ctx* c, BatchState* b, int tile, int nterms) {
   return TCW_OK;
 }
 
-// Doppler rows of every event (step-function search).
-cudaError_t launch_rows(BatchState* b, cudaStream_t st, int* nodes) {
-  cudaError_t err = cudaMemsetAsync(b->rows.p, 0, b->wtot_bytes, st);
-  for (size_t i = 0; i < b->ev.size() && err == cudaSuccess; ++i) {
-    err = launch_step_rows(step_rows_of(b, b->ev[i]), st);
-    *nodes += step_ordered(b->ev[i].geo) ? 2 : 1;
+// Doppler rows of wave w (step-function search).
+cudaError_t launch_rows(BatchState* b, int w, cudaStream_t st, int* nodes) {
+  cudaError_t err = cudaSuccess;
+  for (const EventHost& e : b->ev) {
+    if (e.wave != w || err != cudaSuccess) continue;
+    err = launch_step_rows(step_rows_of(b, e), st);
+    *nodes += step_ordered(e.geo) ? 2 : 1;
   }
   return err;
 }
+
+// The weight sums that the rows add to.
+cudaError_t clear_wtot(BatchState* b, cudaStream_t st) { return cudaMemsetAsync(b->wtot.p, 0, b->wtot.bytes, st); }
 
 cudaError_t launch_wave_anchors(const tcw_ctx* c, BatchState* b, int w, int tile, cudaStream_t st) {
   for (const EventHost& e : b->ev) {
@@ -707,14 +727,7 @@ tcw_status autotune(tcw_ctx* c, BatchState* b) {
   for (int tile : tiles) {
     const int nterms = batch_series_terms(c, b, tile);
     if ((st = prepare_shape(c, b, tile, nterms)) != TCW_OK) break;
-    int nodes = 0, laid = -1;   // wave whose anchors are in place
-    if (b->step) {
-      cudaError_t err = launch_rows(b, c->stream, &nodes);
-      if (err != cudaSuccess) {
-        st = cuda_fail(c, err, "step_rows_kernel launch");
-        break;
-      }
-    }
+    int nodes = 0, laid = -1;   // wave whose anchors (and rows) are in place
     for (int bc : chunks) {
       if (bc > probe_groups && bc != 1) continue;
       int64_t sums = 0;
@@ -723,9 +736,12 @@ tcw_status autotune(tcw_ctx* c, BatchState* b) {
       for (int rep = 0; rep < 2 && st == TCW_OK; ++rep) {
         float ms = 0;
         for (int w = 0; w < b->waves && st == TCW_OK; ++w) {
-          // the waves share one anchor buffer: a wave is searched with its own anchors in place only
+          // the waves share their buffers: a wave is searched with its own anchors and rows in place only
           if (laid != w && (b->step || nterms > 0)) {
-            cudaError_t err = launch_wave_anchors(c, b, w, tile, c->stream);
+            cudaError_t err = cudaSuccess;
+            if (b->step) err = clear_wtot(b, c->stream);
+            if (b->step && err == cudaSuccess) err = launch_rows(b, w, c->stream, &nodes);
+            if (err == cudaSuccess) err = launch_wave_anchors(c, b, w, tile, c->stream);
             if (err != cudaSuccess) {
               st = cuda_fail(c, err, "anchor_kernel launch");
               break;
@@ -798,7 +814,7 @@ tcw_status capture(tcw_ctx* c, BatchState* b, int k) {
   TCW_CUDA(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal), "graph capture");
   cudaError_t err = cudaMemsetAsync(b->flags.p, 0, 64, c->stream);
   int nodes = 0;
-  if (b->step && err == cudaSuccess) err = launch_rows(b, c->stream, &nodes);
+  if (b->step && err == cudaSuccess) err = clear_wtot(b, c->stream);
   for (size_t i = 0; i < b->ev.size() && err == cudaSuccess && !b->step; ++i) {
     const EventHost& e = b->ev[i];
     DopplerParams dp{};
@@ -817,7 +833,8 @@ tcw_status capture(tcw_ctx* c, BatchState* b, int k) {
     ++nodes;
   }
   for (int w = 0; w < b->waves && err == cudaSuccess; ++w) {
-    if (b->step || nterms > 0) {
+    if (b->step) err = launch_rows(b, w, c->stream, &nodes);
+    if (err == cudaSuccess && (b->step || nterms > 0)) {
       err = launch_wave_anchors(c, b, w, b->tile, c->stream);
       for (const EventHost& e : b->ev) nodes += e.wave == w;
     }
@@ -1397,8 +1414,9 @@ tcw_status tcw_search_batched_triaged(tcw_ctx* c, const uint16_t* wbf, const flo
   TCW_CUDA(c, cudaMemsetAsync(tb->flags.p, 0, 64, c->stream), "flags");
   TCW_CUDA(c, cudaEventRecord(ev[3], c->stream), "event");
   int nodes = 0;
-  if (tb->step) TCW_CUDA(c, launch_rows(tb, c->stream, &nodes), "step_rows_kernel launch");
+  if (tb->step) TCW_CUDA(c, clear_wtot(tb, c->stream), "weight sums");
   for (int w = 0; w < tb->waves; ++w) {
+    if (tb->step) TCW_CUDA(c, launch_rows(tb, w, c->stream, &nodes), "step_rows_kernel launch");
     if (tb->step || nterms > 0) TCW_CUDA(c, launch_wave_anchors(c, tb, w, tile, c->stream), "anchor_kernel launch");
     TCW_CUDA(c, launch_wave(c, tb, w, tile, nterms, c->stream, &nodes), "search kernel launch");
     for (const EventHost& h : tb->ev) {

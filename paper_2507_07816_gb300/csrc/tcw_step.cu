@@ -1133,7 +1133,8 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
             };
             const int ns = jn - j0;
             int jb = outside == kAll ? ns : 0;
-            int xh = 0, xl = 0, nx = 0;   // the turn's first-sky powers, each with kMagicBits, and their number
+            // the turn's first-sky powers, each with kMagicBits, and their number: sums modulo 2^32
+            unsigned xh = 0, xl = 0, nx = 0;
             for (; jb < ns && nslow <= kStepSlow - kStepSlowMore; jb += lps) {
               const int jr = min(jb + ls, ns - 1);
               const bool here = mine && jb + ls < ns;
@@ -1213,8 +1214,8 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
                 }
                 int h0, l0, h1, l1;
                 to_fixed<VK>(v0, ws, wsl, h0, l0);
-                xh += h0;
-                xl += l0;
+                xh += (unsigned)h0;
+                xl += (unsigned)l0;
                 ++nx;
                 if (some) {
                   to_fixed<VK>(v1, ws, wsl, h1, l1);
@@ -1239,7 +1240,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
                 }
               }
             }
-            X0 += (long long)(xh - nx * kMagicBits) * 65536 + (xl - nx * kMagicBits);
+            X0 += (long long)(int)(xh - nx * kMagicBits) * 65536 + (int)(xl - nx * kMagicBits);
             {
               const int nr = min(jb, ns) * DP;
               if (!kAmp<VK> && (outside & t_mask)) {

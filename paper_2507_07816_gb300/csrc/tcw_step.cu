@@ -292,7 +292,8 @@ __global__ void __launch_bounds__(128) step_rows_kernel(StepRowsParams p) {
     for (int i = 0; i < kStepBlock; ++i) {
       const int pos = g * kStepBlock + i;
       u = max(u, qv[i]);
-      const int nu = up(u);
+      // the last position takes what is left: no threshold leads past the row
+      const int nu = pos + 1 < p.cpad ? up(u) : nk - 1;
       for (int k = ub + 1; k <= nu; ++k) s_from[k] = (uint16_t)pos;
       ub = nu;
       // suffix minimum from pos on to that from pos + 1 on

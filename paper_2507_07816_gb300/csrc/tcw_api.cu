@@ -212,7 +212,7 @@ tcw_status step_search(tcw_ctx* c, const Plan& pl, bool keep, int* launches, boo
     auto room = [&](DevBuf& b, size_t n) {
       if (e == cudaSuccess) e = b.ensure(n);
     };
-    room(c->step_q, rows * step_row(g.cpad) * sizeof(int32_t));
+    room(c->step_q, rows * g.cpad * sizeof(int32_t));
     room(c->step_head, rows * kStepHead * sizeof(int4));
     room(c->step_tab, rows * step_buckets(g.cpad) * (sizeof(uint2) + sizeof(uint32_t)));
     room(c->step_wtot, kStepSlots * 16 + (size_t)c->Nseg * c->D * sizeof(longlong2));

@@ -283,7 +283,7 @@ size_t layout_rows(const BatchState* b, EventHost& e, size_t at) {
     return from;
   };
   const size_t rows = (size_t)e.geo.n_chunks * e.n_seg * b->D;
-  e.o_q = take(rows * step_row(e.geo.cpad) * sizeof(int32_t));
+  e.o_q = take(rows * e.geo.cpad * sizeof(int32_t));
   e.o_head = take(rows * kStepHead * sizeof(int4));
   e.o_tab = take(rows * step_buckets(e.geo.cpad) * sizeof(uint32_t));
   e.o_fast = take(rows * step_buckets(e.geo.cpad) * sizeof(uint2));

@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(128) step_rows_kernel(StepRowsParams p) {
       mx = max(mx, qv[i]);
       mn = min(mn, qv[i]);
     }
-    int4* o = reinterpret_cast<int4*>(p.q + row * step_row(p.cpad) + g * kStepBlock);
+    int4* o = reinterpret_cast<int4*>(p.q + row * p.cpad + g * kStepBlock);
     o[0] = make_int4(qv[0], qv[1], qv[2], qv[3]);
     o[1] = make_int4(qv[4], qv[5], qv[6], qv[7]);
   }
@@ -322,8 +322,6 @@ __global__ void __launch_bounds__(128) step_rows_kernel(StepRowsParams p) {
     fast[k] = make_uint2((unsigned)from | (slow ? kWindowSlow : 0u) | o[0] << 16, o[1] | o[2] << 16);
   }
   if (g == 0) {
-    int4* pad = reinterpret_cast<int4*>(p.q + row * step_row(p.cpad) + p.cpad);
-    pad[0] = pad[1] = make_int4(qmax, qmax, qmax, qmax);
     int4* m = p.head + row * kStepHead;
     const double ta = anchor_time(p.t_mid, p.n_seg, p.T0, p.tile_shift, j >> p.tile_shift);
     const double tj = p.t_mid[j], dt = tj - ta, d2 = dt * dt;
@@ -645,7 +643,7 @@ __device__ __forceinline__ void step_rare(const StepParams& p, StepBlockCtx& c, 
     value(K + 1, h1, l1);
     const int dh = h1 - h0, dl = l1 - l0;
     const uint32_t win = __ldg(ev.tab + row * c.nk + step_bucket(step_place(t, qmin, m0.z), c.nk));
-    place_exact(ev.q + row * step_row(c.cpad), win, t, [&](int pos, bool up) {
+    place_exact(ev.q + row * c.cpad, win, t, [&](int pos, bool up) {
       int* const cell = c.chi + (pos << (LT + 1)) + lt;
       atomicAdd(cell, up ? dh : -dh);
       atomicAdd(cell + (1 << LT), up ? dl : -dl);
@@ -1032,7 +1030,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int
                 int only = e.w >> 14 & 7;
                 if (only != kStepLookup) {
                   const int64_t row = row1 + (int64_t)(rr / DP) * p.n_det + rr % DP;
-                  const int32_t* const q = ev.q + row * step_row(cpad);
+                  const int32_t* const q = ev.q + row * cpad;
                   const int4 m = ev.head[row * kStepHead];
                   const uint64_t pl = step_place(e.x, m.x, m.z);
                   const uint32_t win = __ldg(ev.tab + (row * nk + step_bucket(pl, nk)));

@@ -28,7 +28,7 @@ constexpr int kStepCells = 16384;      // difference cells of a CTA: chunk x tem
 // Doppler factors stay (almost) sorted.  Doppler rows: one per (chunk, segment,
 // detector), cpad skies in the order of their pass (a multiple of kStepBlock;
 // the last sky repeated):
-//   q     [step_row(cpad)]  floor(v.nhat/c / q-grid step), then the largest repeated
+//   q     [cpad]  floor(v.nhat/c / q-grid step)
 //   head  {qmin, qmax, buckets per grid unit (32 fraction bits), w (float bits)}: the
 //         smallest and largest q; {dt hi, dt lo, dt^2 hi, dt^2 lo}: t_j - t_a from
 //         the tile's anchor time and its square as fp32 pairs (dt hi NaN before T0)
@@ -58,7 +58,7 @@ struct StepEvent {
   const StepTile* tiles;     // [Bpad][n_tiles]
   const double* f0;          // sorted bank [Bpad]
   const double* nbr;
-  const int32_t* q;          // [n_chunks][n_seg][D][step_row(cpad)]
+  const int32_t* q;          // [n_chunks][n_seg][D][cpad]
   const int4* head;          // [n_chunks][n_seg][D][kStepHead]
   const uint32_t* tab;       // [n_chunks][n_seg][D][step_buckets(cpad)]
   const uint2* fast;         // [n_chunks][n_seg][D][step_buckets(cpad)]
@@ -127,8 +127,6 @@ struct StepRowsParams {
   unsigned long long* wtot;  // zero at launch
 };
 
-// Row length: the skies and a block past the end, so that any four from a sky on can be read.
-__host__ __device__ constexpr int step_row(int cpad) { return cpad + kStepBlock; }
 constexpr int kStepHead = 2;     // int4 words of a row's head
 constexpr int kStepSlots = 64;   // partial weight sums of an event
 // Two buckets of thresholds per sky: about half a sky is left to compare per threshold.
@@ -163,7 +161,7 @@ inline bool step_ordered(const StepGeometry& g) { return g.passes > 1; }
 // Doppler rows of one chunk, in bytes: about 28 per sky of a (segment, detector).
 inline size_t step_chunk_bytes(const StepGeometry& g, int64_t n_seg, int D) {
   return (size_t)n_seg * D *
-         (step_row(g.cpad) * sizeof(int32_t) + kStepHead * sizeof(int4) +
+         (g.cpad * sizeof(int32_t) + kStepHead * sizeof(int4) +
           step_buckets(g.cpad) * (sizeof(uint2) + sizeof(uint32_t)));
 }
 // Rows held at a time: a longer sky list is searched some chunks at a time (a chunk

@@ -1444,7 +1444,8 @@ int step_block(const StepGeometry& g, int Bpad, int bank_chunk, int grid, double
     if (lt > g.log_t) continue;
     const int64_t blocks = Bpad >> lt, items = g.n_chunks * ((blocks + bank_chunk - 1) / bank_chunk);
     const double ns = lt == 5 ? 2.8 : lt == 4 ? 3.9 : 5.6;
-    const double us = (double)((items + grid - 1) / grid) * bank_chunk * (rows * (1 << lt) * ns * 1e-3 + g.passes * 20.0);
+    const double per = (double)std::min<int64_t>(bank_chunk, blocks);   // blocks of an item
+    const double us = (double)((items + grid - 1) / grid) * per * (rows * (1 << lt) * ns * 1e-3 + g.passes * 20.0);
     if (lt == g.log_t || us < 0.95 * least) {
       best = lt;
       least = us;

@@ -260,7 +260,7 @@ inline int step_sub_shift(const StepGeometry& g, int64_t n_seg, int tile_shift) 
 }
 // Templates of a block (as log2) for a bank whose blocks may not fill the chip:
 // blocks of 16 or 4 when their rounds over `grid` CTAs end sooner than those of
-// the largest block that fits.  A (template, row) takes 2.8 ns of a CTA in
+// the largest block that fits (bank_chunk blocks are one item).  A (template, row) takes 2.8 ns of a CTA in
 // blocks of 32 and 3.9 in blocks of 16 (128 skies, where 626 of 32 in 5 rounds
 // take 9.0 ms and 1251 of 16 in 9 rounds 11.0), about twice as much in blocks of
 // 4 (the tables' rows serve fewer templates), and a pass's end some 20 us.

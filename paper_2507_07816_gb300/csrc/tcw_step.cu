@@ -300,11 +300,14 @@ __global__ void __launch_bounds__(128) step_rows_kernel(StepRowsParams p) {
 // The largest |rho| of a map and its level (MapRange): one read of the map.  out[0]:
 // bits of the largest; [1], [2]: infinity's bits minus those of the smallest maximum of
 // a run of kLevelRun values at least half of which are nonzero, or fewer; [3], [4]:
-// the number of such runs (zero at launch).
+// the number of such runs (zero at launch).  Bound by memory: four loads in flight per
+// thread and one set of atomics per block (a load at a time and a set per warp: 60 us
+// for 128 MB and 172 for 800 MB; 31 and 145 so; 31 and 118 for the maximum alone).
 template <typename T>
 __global__ void map_range_kernel(const T* x, int64_t n, unsigned* out) {
   constexpr unsigned kInf = 0x7f800000u, kAll = 0xffffffffu;
   constexpr int V = 16 / sizeof(T), R = kLevelRun / V;   // values of a load, lanes of a run
+  __shared__ unsigned s_out[kMapWords];
   unsigned m = 0, low[2] = {0, 0}, runs[2] = {0, 0};
   const int lane = threadIdx.x & 31;
   const int64_t nv = n / V, stride = (int64_t)gridDim.x * blockDim.x;
@@ -315,41 +318,52 @@ __global__ void map_range_kernel(const T* x, int64_t n, unsigned* out) {
     else f = v;
     return __float_as_uint(f) & 0x7fffffffu;
   };
-  for (int64_t i = i0; i - lane < nv; i += stride) {
-    unsigned r = 0, c = 0;
-    if (i < nv) {
-      const int4 v = reinterpret_cast<const int4*>(x)[i];
-      const T* e = reinterpret_cast<const T*>(&v);
+  if (threadIdx.x < kMapWords) s_out[threadIdx.x] = 0;
+  __syncthreads();
+  // kLoads in flight per thread; lanes past the end take zeros
+  constexpr int kLoads = 4;
+  for (int64_t i = i0; i - lane < nv; i += kLoads * stride) {
+    int4 v[kLoads];
+#pragma unroll
+    for (int q = 0; q < kLoads; ++q)
+      v[q] = i + q * stride < nv ? __ldg(reinterpret_cast<const int4*>(x) + i + q * stride) : make_int4(0, 0, 0, 0);
+#pragma unroll
+    for (int q = 0; q < kLoads; ++q) {
+      const T* e = reinterpret_cast<const T*>(&v[q]);
+      unsigned r = 0, c = 0;
 #pragma unroll
       for (int k = 0; k < V; ++k) {
         const unsigned b = bits(e[k]);
         r = max(r, b);
         c += b != 0;
       }
-    }
-    m = max(m, r);
+      m = max(m, r);
 #pragma unroll
-    for (int off = 1; off < R; off <<= 1) {
-      r = max(r, __shfl_xor_sync(kAll, r, off));
-      c += __shfl_xor_sync(kAll, c, off);
-    }
-    if ((lane & (R - 1)) == 0 && (i | (R - 1)) < nv && r > 0 && r < kInf) {
-      const int few = c < kLevelRun / 2;
-      low[few] = max(low[few], kInf - r);
-      ++runs[few];
+      for (int off = 1; off < R; off <<= 1) {
+        r = max(r, __shfl_xor_sync(kAll, r, off));
+        c += __shfl_xor_sync(kAll, c, off);
+      }
+      if ((lane & (R - 1)) == 0 && ((i + q * stride) | (R - 1)) < nv && r > 0 && r < kInf) {
+        const int few = c < kLevelRun / 2;
+        low[few] = max(low[few], kInf - r);
+        ++runs[few];
+      }
     }
   }
   for (int64_t i = nv * V + i0; i < n; i += stride) m = max(m, bits(x[i]));
   m = __reduce_max_sync(kAll, m);
-  if (lane == 0) atomicMax(out, m);
+  if (lane == 0) atomicMax(s_out, m);
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
     const unsigned l = __reduce_max_sync(kAll, low[k]), c = __reduce_add_sync(kAll, runs[k]);
     if (lane == 0 && c) {
-      atomicMax(out + 1 + k, l);
-      atomicAdd(out + 3 + k, c);
+      atomicMax(s_out + 1 + k, l);
+      atomicAdd(s_out + 3 + k, c);
     }
   }
+  __syncthreads();
+  if (threadIdx.x < 3) atomicMax(out + threadIdx.x, s_out[threadIdx.x]);
+  else if (threadIdx.x < kMapWords) atomicAdd(out + threadIdx.x, s_out[threadIdx.x]);
 }
 
 // Shared memory of the search kernel for `cells` difference cells (templates x
@@ -1476,7 +1490,7 @@ cudaError_t launch_step_rows(const StepRowsParams& p, cudaStream_t st) {
 }
 
 cudaError_t launch_map_range(const void* rho, bool half, int64_t n, unsigned* out, cudaStream_t st) {
-  const int64_t blocks = std::min<int64_t>((n + 8191) / 8192, 152 * 16);
+  const int64_t blocks = std::min<int64_t>((n + 8191) / 8192, 152 * 8);
   if (half)
     map_range_kernel<__half><<<(unsigned)blocks, 256, 0, st>>>(static_cast<const __half*>(rho), n, out);
   else

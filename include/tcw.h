@@ -67,8 +67,12 @@ enum { TCW_F32 = 0, TCW_F16 = 1 };
 enum {
     TCW_KERNEL_AUTO = 0,
     TCW_KERNEL_GROUP = 1,   /* the sky as a whole (fast path): step functions over the sorted
-                               sky, or the sky-group candidate-pair kernel where the fixed-point
-                               sums or fp32 track of those do not reach */
+                               sky, or, some five times slower, the sky-group candidate-pair
+                               kernel where the fixed-point sums or fp32 track of those do not
+                               reach: at most 2 detectors, a finite map, and sums of 46 bits of
+                               (largest power x sum of the weights) that resolve 2^-22 of the
+                               smallest weighted power (2e4 lookups of unit weights: powers up
+                               to 800); in a batch, of every event */
     TCW_KERNEL_LOOKUP = 2   /* one thread per (sky, template), FP64 per lookup */
 };
 
@@ -238,7 +242,8 @@ tcw_status tcw_track_bins(tcw_ctx *ctx, int32_t *bins_out, int out_flags);
  * device synchronisation of cudaMalloc/cudaFree, or a plug-in host that
  * forbids device allocation.
  *
- * It runs the same Doppler-table, group and top-k kernels as tcw_search, on
+ * It runs the Doppler-table, group and top-k kernels (those of tcw_search
+ * outside its step-function search, whose tables are larger), on
  * caller-owned DEVICE inputs and outputs, with no context:
  *   rho [n_det][n_seg][n_bin] (dtype TCW_F32 or TCW_F16), t_mid [n_seg]
  *   (strictly increasing), weights [n_det][n_seg] float or NULL for ones,
@@ -281,7 +286,7 @@ tcw_status tcw_search_noalloc(int n_det, int64_t n_seg, int64_t n_bin, int dtype
  * many events -- spectrograms of uneven length, each with its own segment
  * times, detector velocities, weights, signal start T0 (Eq. 1) and sky list --
  * against the context's template bank (tcw_define_bank; its T0 is not used
- * here) in one persistent group-kernel launch per wave of events, recorded
+ * here) in one or two persistent kernel launches per wave of events, recorded
  * once as a CUDA graph and replayed by every tcw_search_batched call.
  *
  * tcw_load_events copies every event (host or device memory per `flags`)
@@ -321,9 +326,9 @@ tcw_status tcw_search_batched(tcw_ctx *ctx, int k, float *psi_out, int64_t *idx_
 /* What the last batched search ran. */
 typedef struct {
     int n_events;
-    int waves;                  /* group-kernel launches per search */
-    int bank_chunk;             /* groups of 8 templates per work item */
-    int tile_segments;          /* anchor spacing / fp32 partial-sum length */
+    int waves;                  /* runs of events searched together */
+    int bank_chunk;             /* template groups or blocks per work item (TCW_OPT_BANK_CHUNK) */
+    int tile_segments;          /* anchor spacing (TCW_OPT_TILE_SEGMENTS) */
     int autotuned;              /* 1 if the two above came from the autotuner */
     int n_candidates;           /* shapes timed by the autotuner */
     int n_items;                /* work items over all waves */
@@ -377,7 +382,7 @@ tcw_status tcw_mlp_forward(const uint16_t *wbf, const float *theta, const float 
                            float *H1, float *H2, float *y, void *stream);
 /* Gradient of a loss with dL/dy = dy into grad[TCW_MLP_PARAMS] (packed like
  * theta; taken at the bfloat16 weights the forward pass used).
- * work: 2 * n * 256 floats of scratch. */
+ * work: 2 * n * 256 floats of scratch (the first half is written). */
 tcw_status tcw_mlp_backward(const uint16_t *wbf, const float *X, int64_t n, const float *H1,
                             const float *H2, const float *dy, float *grad, float *work,
                             void *stream);
@@ -422,8 +427,8 @@ tcw_status tcw_search_triaged(tcw_ctx *ctx, const uint16_t *wbf, const float *th
  * Doppler-sorted skies of that event; patch_size = 0: ceil(n_sky / 32)
  * skies, i.e. 32 patches per event), ONE network call over all events'
  * patches, per event the ceil(frac * n_patch) best patches (spread apart by
- * TCW_OPT_TRIAGE_SPREAD), and one persistent group-kernel launch per wave over
- * the chosen (event, sky chunk, template group) items.  With
+ * TCW_OPT_TRIAGE_SPREAD), and one or two persistent kernel launches per wave
+ * over the chosen (event, sky chunk, template group) items.  With
  * TCW_OPT_TRIAGE_TEMPLATES < 1000 each chosen patch contributes its
  * max(ceil(n_tmpl * permille / 1000), k) best templates by coarse Psi and an
  * event's chosen skies are searched over the union of its patches' templates;
@@ -575,8 +580,10 @@ typedef struct {
     int kernel;                 /* TCW_KERNEL_GROUP or TCW_KERNEL_LOOKUP */
     int launches;               /* kernels launched by the search */
     int64_t lookups;            /* n_sky * n_tmpl * n_det * n_seg */
-    int64_t general_path_lanes; /* lookups at a band edge: (template, detector, segment) steps whose
-                                   skies do not all read bins inside the band */
+    int64_t general_path_lanes; /* step-function search: lookups at a band edge, (template, detector,
+                                   segment) steps whose skies do not all read bins inside the band;
+                                   sky-group kernel: (template, detector, segment, sky group) steps
+                                   that took the per-sky path */
     double doppler_bins_max;    /* largest |f * v.nhat/c| / df over the search */
     double quantum;             /* fixed-point step of the Doppler factor */
     float search_ms;            /* device time of the search kernel, ms */

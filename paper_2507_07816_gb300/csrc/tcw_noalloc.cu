@@ -5,8 +5,9 @@
 // would fail or fragment that pool), a real-time pipeline that cannot afford
 // the implicit device-wide synchronisation of cudaMalloc/cudaFree, or a
 // plug-in host that forbids device allocation by its plug-ins.  For them,
-// tcw_search_noalloc runs the same kernels as tcw_search (Doppler table,
-// group kernel, top-k) on caller-owned inputs and outputs, and takes every
+// tcw_search_noalloc runs the group kernel with its Doppler table and the top-k
+// (the kernels of tcw_search outside its step-function search, whose tables are
+// larger) on caller-owned inputs and outputs, and takes every
 // intermediate buffer from one file-scope device array of fixed size,
 // kTcwNoallocScratchBytes (64 MiB).  Every GPU on which this device code is
 // loaded holds that array until the process exits.  Host memory is used

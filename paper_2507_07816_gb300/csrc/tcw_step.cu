@@ -856,9 +856,10 @@ __device__ __noinline__ void step_fold(const StepParams& p, StepBlockCtx& s_ctx,
 // 2e5 templates x 1024 skies x 2 detectors x 1e4 segments: 655 ms by the group
 // kernel, 276 with the track in fp32 pairs and every step searched where it
 // arises, 160 with steps queued per warp and compared with skies read from the
-// rows, 146 with the list worked through turn by turn, 139 so; one sky and one
-// detector: 205, 50, 24, 22.8, 22.6 ms; 8 events of 100-800 skies and 1.2e4
-// templates: 121 ms by the group kernel, 19.2 turn by turn, 16.9 so.
+// rows, 146 with the list worked through turn by turn, 139 with it worked through
+// full, 133 with tiles of 64 segments and sums that round Psi once; one sky and one
+// detector: 205, 50, 24, 22.8, 22.6, 18.6 ms; 8 events of 100-800 skies and 1.2e4
+// templates: 121 ms by the group kernel, 19.2 turn by turn, 16.9 full, 15.2.
 template <int VK, int DP, int LT>
 __global__ void __launch_bounds__(kStepThreads, 1) step_kernel(StepParams p, int cells) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -1433,10 +1434,13 @@ StepGeometry step_geometry(int64_t S, int D, int64_t n_seg, int tile, const doub
   g.cpad = (most + kStepBlock - 1) / kStepBlock * kStepBlock;
   g.log_t = (g.cpad + 1) * 32 <= kStepCells + 32 ? 5 : 4;
   // Drift of the detectors' direction of motion (rad) away from a pass's
-  // middle: it displaces a sky by up to S drift / 2 places of a whole-sky list
-  // sorted at the middle.  Places out of order cost difference steps of their
-  // own (1.2 per boundary at a displacement of 3, 4.5 at 10: emulated on
-  // Fibonacci and random lists), a pass costs one fold of the cells.
+  // middle: it displaces a sky by up to drift / 2 of a whole-sky list sorted at
+  // the middle.  Places out of order cost difference steps of their own (1.2 per
+  // boundary at a displacement of 3, 4.5 at 10: emulated on Fibonacci and random
+  // lists), a pass costs one fold of the cells.  The places are those of a list
+  // of one chunk's length: in a longer list the skies lie closer and the chunks
+  // see n_chunks times as many (over 11 h 3 % of the windows are longer than 3
+  // skies at 1024 skies, 40 % at 4000 and 69 % at 16000, emulated).
   auto drift = [&](int64_t j0, int64_t j1, int d0, int d1) {
     const double* m = v + ((int64_t)d0 * n_seg + (j0 + j1 - 1) / 2) * 3;
     const double mn = std::sqrt(m[0] * m[0] + m[1] * m[1] + m[2] * m[2]);

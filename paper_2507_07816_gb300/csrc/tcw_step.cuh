@@ -134,7 +134,7 @@ __host__ __device__ constexpr int step_buckets(int cpad) { return 2 * cpad; }
 
 // Chunks of an event's sorted skies: the fewest chunks of at most
 // kStepMaxChunk skies, of nearly equal size; 32 templates per block while the
-// difference cells allow it (chunks of up to 511 skies), else 16 (see step_block).
+// difference cells allow it (chunks of up to 512 skies), else 16 (see step_block).
 struct StepGeometry {
   int n_chunks, chunk, cpad, log_t;
   int dets_per_pass, pass_seg, passes;

@@ -1347,8 +1347,8 @@ StepScales step_scales(const MapRange& map, int bins, const WeightRange& w, bool
   // sums of weights and of their squares below 2^60; amplitude weights are made by the
   // kernel in words of 2^37 (PairWeight), the others here in FP64
   const double max2 = (double)w.max * w.max, sum2 = w.sum * w.max;
-  s.w1 = std::min(60 - lg(w.sum), amp ? 36 - lg(w.max) : 60);
-  s.w2 = std::min(60 - lg(sum2), amp ? 36 - lg(max2) : 60) & ~1;   // even: the root of its unit is a power of 2
+  s.w1 = std::min(60 - lg(w.sum), amp ? 36 - lg(w.max) : INT_MAX);
+  s.w2 = std::min(60 - lg(sum2), amp ? 36 - lg(max2) : INT_MAX) & ~1;   // even: the root of its unit is a power of 2
   // one unit at most 2^-22 of the smallest weighted power, the noise's mean or, where
   // the map lies lower, twice its level: a sum of m rounded values is then off by about
   // 0.3 sqrt(m) 2^-22 of it, 7e-8 of the standard deviation sqrt(m) that Eq. 4 divides
@@ -1358,7 +1358,9 @@ StepScales step_scales(const MapRange& map, int bins, const WeightRange& w, bool
   // W1 and W2 of the smallest weights alone to 2^-25, as fp32 has each of them
   const double a = std::log2((double)w.min * a_ref);
   const bool weights = s.w1 >= 24 - std::floor(a) && s.w2 >= 24 - std::floor(2 * a);
-  s.ok = weights && s.x >= need && std::abs(s.x) < 100 && std::abs(s.w1) < 100 && std::abs(s.w2) < 100 && need < 100;
+  // exponents that fp32 scales hold (the plain weights' W2 words are made in FP64)
+  s.ok = weights && s.x >= need && std::abs(s.x) < 100 && std::abs(s.w1) < 100 && std::abs(s.w2) < (amp ? 100 : 150) &&
+         need < 100;
   return s;
 }
 

@@ -276,3 +276,19 @@ def test_tables_that_do_not_fit_leave_the_group_kernel():
     np.testing.assert_allclose(st["W1"], st1["W1"], rtol=1e-5)
     np.testing.assert_allclose(st["psi"], st1["psi"], rtol=0, atol=1e-3)
     assert_topk_consistent(st["psi"], idx, val, 3)
+
+
+@pytest.mark.parametrize("scale", [1e-9, 1e-6, 1e-3, 1e3, 1e9])
+@pytest.mark.parametrize("amp", [0, 4])
+def test_weights_of_any_scale_keep_the_fast_search(scale, amp):
+    """The grids follow the weights' scale, on which Psi does not depend."""
+    p = small(2900, n_det=2)
+    p.weights = (p.weights * np.float32(scale)).astype(np.float32)
+    val, idx, st, info = run(p, options=[(tcw.OPT_AMPLITUDE_POWER, amp)])
+    S, W1, W2, psi = oracle_stats(p, amp_power=amp)
+    assert info.kernel == tcw.KERNEL_GROUP
+    many = W1 > 0.1 * W1.max()
+    assert stepped({"S": st["S"][many]}, [S[many]])
+    assert np.all(np.abs(st["W2"] - W2)[many] <= 2.0 ** -23 * W2[many])
+    assert np.all(np.abs(st["psi"][many] - psi[many]) <= 2.0 ** -23 * np.abs(psi[many]) + 2.0 ** -22)
+    assert_topk_consistent(st["psi"], idx, val, 3)

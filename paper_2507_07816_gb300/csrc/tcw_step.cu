@@ -469,11 +469,14 @@ __device__ __forceinline__ void to_fixed(float v, float s, float more, int& hi, 
   hi = __float_as_int(t);
   lo = __float_as_int(fmaf(r, 65536.0f, kMagic));
 }
-// The same as one 64-bit word.
+// The same on a grid of 2^-22 as one 64-bit word: the sums of weights are 64 bits.
+constexpr int kWordBits = 22;
 __device__ __forceinline__ long long fixed_word(float v, float s, float more) {
-  int hi, lo;
-  to_fixed(v, s, more, hi, lo);
-  return (long long)(hi - kMagicBits) * 65536 + (lo - kMagicBits);
+  constexpr float kUnit = (float)(1 << kWordBits);
+  const float t = fmaf(v, s, kMagic);
+  const float r = fmaf(v, s, -(t - kMagic)) + more;
+  const int hi = __float_as_int(t) - kMagicBits, lo = __float_as_int(fmaf(r, kUnit, kMagic)) - kMagicBits;
+  return (long long)hi * (1 << kWordBits) + lo;
 }
 // A value times the weight s + sl (sl with amplitude weights only).
 template <int VK>
@@ -1345,21 +1348,22 @@ StepScales step_scales(const MapRange& map, int bins, const WeightRange& w, bool
   const double v = std::max(vmax, (double)bins);
   s.x = std::min(46 - lg(v * w.sum), 37 - lg(v * w.max));
   // sums of weights and of their squares below 2^60; amplitude weights are made by the
-  // kernel in words of 2^37 (PairWeight), the others here in FP64
+  // kernel in words of 2^42 (PairWeight), the others here in FP64
   const double max2 = (double)w.max * w.max, sum2 = w.sum * w.max;
-  s.w1 = std::min(60 - lg(w.sum), amp ? 36 - lg(w.max) : INT_MAX);
-  s.w2 = std::min(60 - lg(sum2), amp ? 36 - lg(max2) : INT_MAX) & ~1;   // even: the root of its unit is a power of 2
+  s.w1 = std::min(60 - lg(w.sum), amp ? 42 - lg(w.max) : INT_MAX);
+  s.w2 = std::min(60 - lg(sum2), amp ? 42 - lg(max2) : INT_MAX) & ~1;   // even: the root of its unit is a power of 2
   // one unit at most 2^-22 of the smallest weighted power, the noise's mean or, where
   // the map lies lower, twice its level: a sum of m rounded values is then off by about
   // 0.3 sqrt(m) 2^-22 of it, 7e-8 of the standard deviation sqrt(m) that Eq. 4 divides
   // by and less of S
   const double p = map.level > 0 ? std::min(1.0, 2.0 * (double)map.level) : 1.0;
   const int need = 22 - (int)std::floor(std::log2((double)w.min * a_ref * p));
-  // W1 and W2 of the smallest weights alone to 2^-25, as fp32 has each of them
+  // W1 and W2 of the smallest weights alone to 2^-25, as fp32 has each of them; squares
+  // of amplitude weights, no two of which are alike, to 2^-21 each
   const double a = std::log2((double)w.min * a_ref);
-  const bool weights = s.w1 >= 24 - std::floor(a) && s.w2 >= 24 - std::floor(2 * a);
+  const bool weights = s.w1 >= 24 - std::floor(a) && s.w2 >= (amp ? 20 : 24) - std::floor(2 * a);
   // exponents that fp32 scales hold (the plain weights' W2 words are made in FP64)
-  s.ok = weights && s.x >= need && std::abs(s.x) < 100 && std::abs(s.w1) < 100 && std::abs(s.w2) < (amp ? 100 : 150) &&
+  s.ok = weights && s.x >= need && std::abs(s.x) < 100 && std::abs(s.w1) < 100 && std::abs(s.w2) < (amp ? 130 : 150) &&
          need < 100;
   return s;
 }

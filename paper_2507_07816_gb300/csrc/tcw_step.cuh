@@ -75,7 +75,7 @@ struct StepEvent {
   double x_unit, w1_unit, w2_unit;   // value of one unit of the fixed-point sums
   float x_scale;                     // 2^-16 / x_unit
   float r_unit;                      // 2^24 x_unit / sqrt(w2_unit), a power of 2
-  float w1_scale, w2_scale;          // 2^-16 / w1_unit, 2^-16 / w2_unit
+  float w1_scale, w2_scale;          // 2^-22 / w1_unit, 2^-22 / w2_unit
   int n_seg, n_tiles, S, Bpad;
   int bit_pitch;
   int chunk, cpad, log_t;    // skies per chunk, of a row; templates of a block: 1 << log_t
@@ -240,8 +240,8 @@ inline void set_step_scales(StepEvent& e, const StepScales& s) {
   e.w2_unit = std::ldexp(1.0, -s.w2);
   e.x_scale = std::ldexp(1.0f, s.x - 16);
   e.r_unit = std::ldexp(1.0f, 24 - s.x + s.w2 / 2);
-  e.w1_scale = std::ldexp(1.0f, s.w1 - 16);
-  e.w2_scale = std::ldexp(1.0f, s.w2 - 16);
+  e.w1_scale = std::ldexp(1.0f, s.w1 - 22);
+  e.w2_scale = std::ldexp(1.0f, s.w2 - 22);
 }
 // Segments of one warp's turn (as a shift): the longest run, a whole tile or
 // less, that leaves few of the 32 warps idle in a pass's last round of turns.

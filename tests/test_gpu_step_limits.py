@@ -292,3 +292,21 @@ def test_weights_of_any_scale_keep_the_fast_search(scale, amp):
     assert np.all(np.abs(st["W2"] - W2)[many] <= 2.0 ** -23 * W2[many])
     assert np.all(np.abs(st["psi"][many] - psi[many]) <= 2.0 ** -23 * np.abs(psi[many]) + 2.0 ** -22)
     assert_topk_consistent(st["psi"], idx, val, 3)
+
+
+@pytest.mark.parametrize("delay,power", [(2000.0, 4), (6000.0, 4), (20000.0, 3), (20000.0, 4)])
+def test_amplitude_weights_long_after_the_start(delay, power):
+    """Data that begin well after T0, when (f/f0)^p is down to 0.02: their grids resolve it."""
+    p = small(2950 + power, n_det=2, n_tmpl=200)
+    p.T0 = float(p.t_mid[0] - delay)
+    p.bank.f0[:] = 500.0 + np.linspace(30, 745, 200)
+    p.bank.f0[:] *= (delay / p.bank.tau + 1) ** (1 / (p.bank.n - 1))
+    val, idx, st, info = run(p, options=[(tcw.OPT_AMPLITUDE_POWER, power)])
+    S, W1, W2, psi = oracle_stats(p, amp_power=power)
+    assert info.kernel == tcw.KERNEL_GROUP
+    many = W1 > 0.02 * W1.max()
+    assert many.mean() > 0.5 and stepped({"S": st["S"][many]}, [S[many]])
+    assert np.all(np.abs(st["W1"] - W1)[many] <= 2.0 ** -23 * W1[many])
+    assert np.all(np.abs(st["W2"] - W2)[many] <= 2.0 ** -23 * W2[many])
+    assert np.all(np.abs(st["psi"][many] - psi[many]) <= 2.0 ** -23 * np.abs(psi[many]) + 2.0 ** -20)
+    assert_topk_consistent(st["psi"], idx, val, 3)

@@ -368,8 +368,8 @@ __global__ void map_range_kernel(const T* x, int64_t n, unsigned* out) {
 
 // Shared memory of the search kernel for `cells` difference cells (templates x
 // (row + 1)): two word planes, the heads of each warp's turn (and in their place
-// the piece sums of a pass's end), FP64 and fp32 series coefficients,
-// per-template sums.  What is left of the SM's memory is L1: a smaller layout
+// the piece sums of a pass's end), FP64 and fp32 series coefficients, df / f0
+// (amplitude weights), per-template sums.  What is left of the SM's memory is L1: a smaller layout
 // shows (see step_kernel).
 constexpr size_t kStepPart = 3 * kStepThreads * 8;
 static_assert(kStepWarps * kStepTurn * kStepHead * 16 <= kStepPart, "the heads fit the piece sums' place");
